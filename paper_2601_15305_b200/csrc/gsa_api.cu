@@ -420,14 +420,14 @@ static int attn_fwd_impl(const gsa_params_t* p, const void* Q, const void* K, co
         if (wp.prepass && ws_bytes >= attn_ws_bytes(*p, true)) {
             bf16* Vg = (bf16*)(wsb + attn_ws_bytes(*p, false));
             cudaError_t e = launch_value_gate((const bf16*)V, (const bf16*)g2_logits, Vg,
-                                              (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st);
+                                              (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st, t_dev_status + kStatusGeneralWord);
             if (e != cudaSuccess) return cuda_rc(e);
             Vuse = Vg;
             g2use = nullptr;
         }
     }
     return cuda_rc(launch_sparse_attn(*p, rr, (const bf16*)Q, (const bf16*)K, Vuse, (const bf16*)g1_logits,
-                                      g2use, idx, kt, il, (bf16*)out, scratch, st, nullptr, lse));
+                                      g2use, idx, kt, il, (bf16*)out, scratch, st, nullptr, lse, g2_logits != nullptr));
 }
 
 int gsa_sparse_gated_attn_fwd(const gsa_params_t* p, const void* Q, const void* K, const void* V,
@@ -512,7 +512,7 @@ static int forward_impl(const gsa_params_t* p, const void* Q, const void* K, con
     if (g2_logits && wp.prepass) {
         bf16* Vg = (bf16*)(wsb + wp.vg_off);
         e = launch_value_gate((const bf16*)V, (const bf16*)g2_logits, Vg,
-                              (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st);
+                              (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st, t_dev_status + kStatusGeneralWord);
         if (e != cudaSuccess) return cuda_rc(e);
         timeline_mark(kStageValueGate, st);
         Vuse = Vg;
@@ -521,7 +521,7 @@ static int forward_impl(const gsa_params_t* p, const void* Q, const void* K, con
     // Eq. 11, 12, 10 over all rows
     RowRange all{0, p->B, 0, p->Lq};
     e = launch_sparse_attn(*p, all, (const bf16*)Q, (const bf16*)K, Vuse, (const bf16*)g1_logits, g2use, idx,
-                           kt, il, (bf16*)out, wsb + wp.attn_off, st, progress);
+                           kt, il, (bf16*)out, wsb + wp.attn_off, st, progress, nullptr, g2_logits != nullptr);
     if (g_prof_ev[2]) cudaEventRecord(g_prof_ev[2], st);
     return cuda_rc(e);
 }

@@ -1,4 +1,5 @@
-// Sparse gated attention (Eq. 9, 11, 12, 10).
+// Sparse gated attention (Eq. 9, 11, 12, 10): the gather kernels, for sets that hold a small share of the visible keys
+// (larger shares: masked tiles, gsa_masked_attn.cu; masked_rows_end below draws the line) and for decode.
 //
 // Work item = (query token, KV head, segment of the token's index set S_t); one warp per item,
 // 16 warps per CTA, items dealt to warps round-robin so that the warps of a CTA work on the same
@@ -34,6 +35,7 @@
 // of a tile then arrive in two shared-memory tiles, both are read transposed into the same A-fragment
 // layout, and the gate is applied to the fragments in registers right before the MMA.
 #include "gsa_common.cuh"
+#include "gsa_masked.cuh"
 
 namespace gsa {
 
@@ -522,7 +524,9 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
 // Eq. 9 as a streaming pre-pass: Vg = bf16(V * sigmoid(g2)), 8 elements per thread.
 __global__ void __launch_bounds__(256) gsa_value_gate_kernel(const uint4* __restrict__ V,
                                                              const uint4* __restrict__ g2,
-                                                             uint4* __restrict__ Vg, int64_t n_vec) {
+                                                             uint4* __restrict__ Vg, int64_t n_vec,
+                                                             int32_t* nonfinite) {
+    uint32_t bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec;
          i += (int64_t)gridDim.x * blockDim.x) {
         uint4 vv = __ldg(V + i);
@@ -535,7 +539,9 @@ __global__ void __launch_bounds__(256) gsa_value_gate_kernel(const uint4* __rest
             v2[e] = __floats2bfloat162_rn(vf.x * gate_sigmoid(gf.x), vf.y * gate_sigmoid(gf.y));
         }
         Vg[i] = vv;
+        bad |= nonfinite_bf16x8(vv);
     }
+    if (bad && nonfinite) *nonfinite = 1;
 }
 
 int g_range_keys = kRangeKeysDefault;
@@ -645,6 +651,51 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
     return finalize(finalized_to, q_end);
 }
 
+// First row from which the gather is the cheaper path (rr.q_begin: all of them; its end: none).
+// A gathered pair costs 36 ps per KV head at d_h = 128 and 24 ps at 64 (L2 rate, measured at L = 16K for 1, 2, 4 and 8
+// query heads per KV head), a visible pair of a masked tile 0.53 / 0.43 ps per query head: the tiles win while a row sees
+// fewer than 68 / G (56 / G) times the keys it selects.  The sets' sizes are on the device; the budget they centre on
+// stands for them.  Fewer CTAs than two thirds of the SMs leave too much of the GPU idle.
+int masked_rows_end(const gsa_params_t& p, const RowRange& rr) {
+    const int G = p.n_h / p.n_kv, q_end = rr.q_begin + rr.R;
+    int64_t t_end = q_end;
+    if (p.k_mode != 3) {
+        const int64_t k = p.k_base < p.k_min ? p.k_min : (p.k_base > p.k_max ? p.k_max : p.k_base);
+        t_end = k * (p.d_h == 128 ? 68 : 56) / G - (p.Lk - p.Lq);
+    }
+    const int block = masked_block_rows(p);
+    if (t_end <= rr.q_begin) return rr.q_begin;
+    if (t_end + 4 * block >= q_end) t_end = q_end;                 // (a short rest is not worth the gather's launches)
+    else t_end = rr.q_begin + (t_end - rr.q_begin) / block * block;
+    const int64_t ctas = (t_end - rr.q_begin + block - 1) / block * p.n_kv * rr.nb;
+    return ctas * 3 >= 2 * sm_count() ? (int)t_end : rr.q_begin;
+}
+
+cudaError_t launch_masked_rows(const gsa_params_t& p, const RowRange& rr, int t_end, const __nv_bfloat16* Q,
+                               const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const int32_t* idx,
+                               const int32_t* kt, IdxLayout il, __nv_bfloat16* out, void* scratch, size_t scratch_bytes,
+                               cudaStream_t st, AttnProgress* prog, float* lse) {
+    const int block = masked_block_rows(p);
+    const size_t row_bytes = mask_plan(p, 0, kMaskRowAlign).bytes(p.B) / kMaskRowAlign;
+    int64_t per = (int64_t)(scratch_bytes / row_bytes) / block * block;
+    if (per < block) return cudaErrorInvalidValue;
+    for (int q = rr.q_begin; q < t_end; q += (int)per) {
+        const MaskPlan mp = mask_plan(p, q, (int)(t_end - q < per ? t_end - q : per));
+        cudaError_t e = launch_build_masks(p, mp, block, idx, kt, il, (uint4*)scratch, t_dev_status + kStatusGeneralWord, st);
+        if (e != cudaSuccess) return e;
+        timeline_mark(kStageRangeCuts, st);
+        e = launch_masked_attn_fwd(p, mp, (const uint4*)scratch, Q, K, Vg, g1, out, lse, idx, kt, il, t_dev_status, st);
+        if (e != cudaSuccess) return e;
+        timeline_mark(kStageAttn, st);
+        if (prog && prog->n < prog->cap && prog->n < 64) {
+            if ((e = cudaEventRecord(prog->events[prog->n], st)) != cudaSuccess) return e;
+            prog->t_lo[prog->n] = q; prog->t_hi[prog->n] = q + mp.rows;
+            ++prog->n;
+        }
+    }
+    return cudaSuccess;
+}
+
 template <int DH, bool FUSE_G2>
 cudaError_t launch_attn_g(const AttnArgs& a, const gsa_params_t& p, const AttnPlan& pl, const __nv_bfloat16* g1,
                           __nv_bfloat16* out, int32_t* cuts, int G, cudaStream_t st, AttnProgress* prog) {
@@ -668,13 +719,13 @@ void set_attn_range_keys(int keys) { g_range_keys = keys >= 1024 ? keys : kRange
 int attn_range_keys() { return g_range_keys; }
 
 cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, __nv_bfloat16* Vg,
-                              int64_t n_elems, cudaStream_t st) {
+                              int64_t n_elems, cudaStream_t st, int32_t* nonfinite) {
     const int64_t n_vec = n_elems / 8;
     if (n_vec <= 0) return cudaSuccess;
     const int blocks = (int)((n_vec + 255) / 256 < sm_count() * 16 ? (n_vec + 255) / 256 : sm_count() * 16);
     gsa_value_gate_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const uint4*>(V),
                                                   reinterpret_cast<const uint4*>(g2),
-                                                  reinterpret_cast<uint4*>(Vg), n_vec);
+                                                  reinterpret_cast<uint4*>(Vg), n_vec, nonfinite);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -683,9 +734,24 @@ cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bf
                                const __nv_bfloat16* K, const __nv_bfloat16* V,
                                const __nv_bfloat16* g1, const __nv_bfloat16* g2, const int32_t* idx,
                                const int32_t* kt, IdxLayout il, __nv_bfloat16* out, void* scratch,
-                               cudaStream_t st, AttnProgress* progress, float* lse) {
+                               cudaStream_t st, AttnProgress* progress, float* lse, bool values_scanned) {
     if (rr.rows() <= 0) return cudaSuccess;
     const AttnPlan pl = plan_attn(p);
+    if (!g2 && pl.mode == 0 && t_dev_status) {
+        // rows whose sets hold a large enough share of what they see: masked tiles, in chunks whose masks fit the scratch
+        const int t_end = masked_rows_end(p, rr);
+        if (t_end > rr.q_begin) {
+            cudaError_t e = cudaSuccess;
+            if (!values_scanned)
+                e = launch_check_finite(V, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, t_dev_status + kStatusGeneralWord, st);
+            if (e != cudaSuccess) return e;
+            e = launch_masked_rows(p, rr, t_end, Q, K, V, g1, idx, kt, il, out, scratch,
+                                               (pl.state_bytes + 255) / 256 * 256 + pl.cuts_bytes, st, progress, lse);
+            if (e != cudaSuccess || t_end >= rr.q_begin + rr.R) return e;
+            rr.R = rr.q_begin + rr.R - t_end;
+            rr.q_begin = t_end;
+        }
+    }
     AttnArgs a;
     a.lse = lse;
     a.dev_status = t_dev_status;

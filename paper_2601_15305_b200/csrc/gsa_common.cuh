@@ -29,6 +29,7 @@ struct IdxLayout {
 
 constexpr int kStatusBytes = 256;   // head of every workspace: device status word, counters, padding
 constexpr int kStatusFallbackWord = 1;   // int32 word: rows on which top-k selection took its whole-row fallback
+constexpr int kStatusGeneralWord = 2;    // int32 word: nonzero if the call's inputs rule the masked tiles out (gsa_masked.cuh)
 
 // device status word values: which bounded wait of a tensor-core pipeline ran out (copy producer, MMA
 // issuer, epilogue), or that a kernel met an index set entry / budget outside its range
@@ -66,7 +67,7 @@ cudaError_t launch_select(const gsa_params_t& p, RowRange rr, const float* score
                           IdxLayout il, int32_t* fallback_rows /*nullable counter*/, cudaStream_t st);
 
 cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, __nv_bfloat16* Vg,
-                              int64_t n_elems, cudaStream_t st);
+                              int64_t n_elems, cudaStream_t st, int32_t* nonfinite = nullptr /*raised if a gated value is*/);
 
 // Backward of sparse gated attention.  Query-major half (gsa_attn_bwd.cu): dQ, dg1 for the rows of rr, and
 // per (row, head) do = dout * sigmoid(g1), the softmax statistics lse2 and delta for the key-major half
@@ -122,7 +123,8 @@ cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bf
                                const __nv_bfloat16* g1, const __nv_bfloat16* g2 /*nullable*/,
                                const int32_t* idx, const int32_t* kt, IdxLayout il,
                                __nv_bfloat16* out, void* scratch, cudaStream_t st,
-                               AttnProgress* progress = nullptr, float* lse = nullptr);
+                               AttnProgress* progress = nullptr, float* lse = nullptr,
+                               bool values_scanned = false /*launch_value_gate wrote V and watched the status head*/);
 
 // bytes of device scratch launch_sparse_attn needs for `p` (softmax state slots, range cuts)
 size_t attn_scratch_bytes(const gsa_params_t& p);
@@ -263,6 +265,14 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
     for (uint32_t p = 0; p < kDrainPolls; ++p)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
+}
+
+// nonzero if one of eight bf16 values is infinite or NaN
+__device__ __forceinline__ uint32_t nonfinite_bf16x8(uint4 v) {
+    auto f = [](uint32_t x) -> uint32_t {       // an exponent of all ones carries into the bit above it
+        return (((x & 0x7F807F80u) + 0x00800080u) & 0x80008000u);
+    };
+    return f(v.x) | f(v.y) | f(v.z) | f(v.w);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {

@@ -1,0 +1,181 @@
+// Masked tiles: the attention stage as dense 128-row x 128-key tiles on the 5th-generation tensor cores, with the
+// index sets S_t as bit masks.  Shared by the forward (gsa_masked_attn.cu) and backward kernels.
+//
+// Why: the gather kernels move n_kv * d_h * 4 bytes per selected (query, key) pair through the L2 (0.30 ns per pair
+// and forward at 16 heads of 128), a tile costs 4 * d_h flops per (query, key, head) whether selected or not.  Once
+// more than a few per cent of the visible keys are selected the tensor cores win.
+//
+// Mask layout: one uint4 (128 bits, bit k of word w = key 32 w + k of the tile) per (batch element, key tile, query
+// row): mask[(b * n_key_tiles + tile) * row_pitch + row], so that the threads of a tile (consecutive rows) read
+// consecutive 16-byte pieces.
+#pragma once
+
+#include "gsa_common.cuh"
+#include "gsa_tc.cuh"
+
+namespace gsa {
+
+constexpr int kMaskTileKeys = 128;
+constexpr int kMaskRowAlign = 8;           // row_pitch is a multiple of this (rows a mask-building CTA handles)
+
+struct MaskPlan {
+    int32_t q0, rows;          // query rows q0 .. q0 + rows - 1 of every batch element
+    int32_t row_pitch;         // rows rounded up to kMaskRowAlign
+    int32_t key_tiles;         // ceil(Lk / 128)
+    size_t bytes(int B) const { return (size_t)B * key_tiles * row_pitch * 16; }
+};
+
+inline MaskPlan mask_plan(const gsa_params_t& p, int q0, int rows) {
+    MaskPlan m;
+    m.q0 = q0; m.rows = rows;
+    m.row_pitch = (rows + kMaskRowAlign - 1) / kMaskRowAlign * kMaskRowAlign;
+    m.key_tiles = (p.Lk + kMaskTileKeys - 1) / kMaskTileKeys;
+    return m;
+}
+
+// Builds the masks of rows mp.q0 .. of every batch element.  Row r gets the key tiles that the last row of its block
+// of `block_rows` rows (counted from mp.q0) can see.  A set that a mask cannot stand for (not strictly ascending, an
+// entry that the row cannot see, a budget out of range) raises *general.
+cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int block_rows, const int32_t* idx,
+                               const int32_t* kt, IdxLayout il, uint4* mask, int32_t* general, cudaStream_t st);
+
+// Raises *general if one of n_elems (a multiple of 8) values is infinite or NaN.
+cudaError_t launch_check_finite(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st);
+
+// query rows of a forward CTA (two M = 128 tiles of (query, head of the group) rows)
+inline int masked_block_rows(const gsa_params_t& p) { return 256 / (p.n_h / p.n_kv); }
+
+// Attention of the rows of mp.  dev_status: the call's status head, whose `general` word says whether the tiles may be
+// used (the masks and the scan of the values come first on the stream); if not, the same launch pair does the rows one
+// set entry at a time.
+cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, const uint4* mask, const __nv_bfloat16* Q,
+                                   const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1,
+                                   __nv_bfloat16* out, float* lse, const int32_t* idx, const int32_t* kt, IdxLayout il,
+                                   int32_t* dev_status, cudaStream_t st);
+
+// ---- device helpers --------------------------------------------------------------------------------------
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+
+// A operand in TMEM (bf16 pairs, one 32-bit column per two contraction elements), B in shared memory
+__device__ __forceinline__ void tc_mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+#define GSA_R32_OUT(r)                                                                                              \
+    "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),    \
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),     \
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),    \
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+#define GSA_R32_TIE(r)                                                                                              \
+    "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),    \
+        "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),     \
+        "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),    \
+        "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+#define GSA_R32_IN(r)                                                                                               \
+    "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),  \
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),            \
+        "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]),            \
+        "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+
+// 32 columns of this thread's TMEM lane
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,"
+        "%29,%30,%31}, [%32];"
+        : GSA_R32_OUT(r)
+        : "r"(taddr)
+        : "memory");
+}
+// waits for every tcgen05.ld of this thread; the registers of r may be used from here on (tc_tie32 for others)
+__device__ __forceinline__ void tc_wait_ld32(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : GSA_R32_TIE(r) : : "memory");
+}
+__device__ __forceinline__ void tc_tie32(uint32_t (&r)[32]) { asm volatile("" : GSA_R32_TIE(r) : : "memory"); }
+__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,"
+        "%29,%30,%31};" ::GSA_R32_IN(r), "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};"
+        ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// shared-memory descriptor of a [contraction rows][64-column chunks] operand tile whose 128-byte rows run along the
+// M / N dimension ("MN-major", 128-byte swizzle): 8-row groups 1024 bytes apart, 64-column chunks chunk_bytes apart
+__device__ __forceinline__ uint64_t make_mnmajor_desc(uint32_t smem_addr, uint32_t chunk_bytes) {
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(chunk_bytes >> 4) << 16;                           // leading byte offset: next 64 of M / N
+    d |= (uint64_t)(1024u >> 4) << 32;                                 // stride byte offset: next 8 contraction rows
+    d |= 1ull << 46;
+    d |= 2ull << 61;                                                   // SWIZZLE_128B
+    return d;
+}
+constexpr uint32_t kIdescTransA = 1u << 15, kIdescTransB = 1u << 16;   // operand is MN-major
+
+__device__ __forceinline__ uint64_t pack_f32x2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(__float_as_uint(a)), "r"(__float_as_uint(b)));
+    return r;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& a, float& b) {
+    uint32_t x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(x), "=r"(y) : "l"(v));
+    a = __uint_as_float(x); b = __uint_as_float(y);
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// tokens x heads x d_h bf16 (row-major); box = tokens_box x heads_box x 64 values (one 128-byte swizzle span).  Tokens
+// past the end read as zero.
+inline bool make_heads_tmap(CUtensorMap* tm, const void* base, uint64_t tokens, uint64_t heads, uint64_t d_h,
+                            uint32_t tokens_box, uint32_t heads_box) {
+    auto fn = get_encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)d_h, (cuuint64_t)heads, (cuuint64_t)tokens};
+    cuuint64_t strides[2] = {(cuuint64_t)d_h * 2, (cuuint64_t)(heads * d_h) * 2};
+    cuuint32_t box[3] = {64u, heads_box, tokens_box};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace gsa

@@ -1,0 +1,555 @@
+// Sparse gated attention forward (Eq. 9, 11, 12, 10) on masked dense tiles (see gsa_masked.cuh): for index sets that
+// hold more than a few per cent of the visible keys.
+//
+// One CTA = one KV head and 256 rows, a row being a (query, head of the group) pair: two M = 128 tiles whose chains
+//     S = Q K^T (tcgen05, fp32 in TMEM) -> mask, softmax numerators P (registers) -> P as bf16 into the columns of S
+//     -> O += P V' (tcgen05, A operand in TMEM, V' tile read as it lies: keys are the contraction, d runs along N)
+// run against each other: while four warps work on one tile's scores, the tensor cores run the other's products.  A
+// K and a V' tile are fetched once for both.  Thread = row: no shuffles anywhere.
+//
+// Softmax reference: as in the gather kernel, it moves only when a selected score exceeds it by more than 2^8, so the
+// accumulator in TMEM is touched by the softmax warps on a row's first tiles only.  Masked scores are replaced by
+// -inf before the maximum and the exponentials; fp32 everywhere except P (bf16, as in the gather kernel).
+//
+// Bound: the two tiles' softmax chains against their products; 16 exponentials and 4 * 128 * d_h flops per (row, key) column
+// make special-function unit and tensor cores about equally long (1024 cycles per tile at d_h = 128).  Measured at 16 heads
+// of 128 on 8 KV heads: L = 32K 3.92 ms = 1.12 PFLOP/s over the visible pairs (the gather kernel: 19.6 ms), 8K 0.35 ms
+// (4.6 ms), dense 2 x 3072 0.14 ms (2.7 ms).
+//
+// Warps 0-3 / 4-7: softmax and epilogue of tile 0 / 1; warp 8: TMA; warp 9: MMA issue and TMEM allocation; 10, 11
+// only complete their warpgroup.
+// TMEM: S0 | S1 (128 columns each, P overlays the first 64) | O0 | O1.
+#include "gsa_masked.cuh"
+
+namespace gsa {
+
+namespace {
+
+// ---- masks -----------------------------------------------------------------------------------------------
+constexpr int kMaskWindowWords = 1024;                 // 32768 keys of every row at a time
+constexpr int kMaskRowWords = kMaskWindowWords + 4;    // (padded: the rows' pieces of a key tile fall into different banks)
+
+__global__ void __launch_bounds__(kMaskRowAlign * 32)
+gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ kt, uint4* __restrict__ mask,
+                       IdxLayout il, int q0, int rows, int row_pitch, int key_tiles, int block_rows, int k_max, int off,
+                       int32_t* __restrict__ general) {
+    __shared__ __align__(16) uint32_t s_bits[kMaskRowAlign * kMaskRowWords];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = blockIdx.y, r0 = blockIdx.x * kMaskRowAlign, r = r0 + warp;
+    const int blk_end = min((r0 / block_rows + 1) * block_rows, rows);
+    const int tiles = min((off + q0 + blk_end + kMaskTileKeys - 1) / kMaskTileKeys, key_tiles);
+    const int n_vis = off + q0 + r + 1;
+    const int64_t irow = r < rows ? il.row(b, q0 + r) : 0;
+    const int k = r < rows ? clamp_budget(kt[irow], k_max) : 0;
+    const int32_t* __restrict__ row = idx + irow * k_max;
+    const bool vec = (k_max & 3) == 0;                 // rows start on 16-byte boundaries
+    uint32_t* const bits = s_bits + warp * kMaskRowWords;
+    int at = 0;                                        // entries below `at` have been placed
+    bool regular = r >= rows || k == kt[irow];
+    for (int w0 = 0; w0 < tiles * 4; w0 += kMaskWindowWords) {
+        const int words = min(kMaskWindowWords, tiles * 4 - w0);
+        for (int i = lane; i < words / 4; i += 32) reinterpret_cast<uint4*>(bits)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+        const int lo = w0 * 32, hi = min((w0 + words) * 32, n_vis);
+        int last = -1;                                 // entry in front of the batch (-1: compared already)
+        while (at < k) {
+            // 256 entries a time, eight consecutive ones per lane: neighbours mostly share a word, which then takes
+            // one shared-memory atomic
+            const int j0 = at + lane * 8;
+            int32_t e[8];
+            if (vec && (at & 3) == 0 && j0 + 8 <= k) {
+                const int4 a = *reinterpret_cast<const int4*>(row + j0), c = *reinterpret_cast<const int4*>(row + j0 + 4);
+                e[0] = a.x; e[1] = a.y; e[2] = a.z; e[3] = a.w; e[4] = c.x; e[5] = c.y; e[6] = c.z; e[7] = c.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) e[j] = j0 + j < k ? row[j0 + j] : 0x7FFFFFFF;
+            }
+            int before = __shfl_up_sync(0xFFFFFFFFu, e[7], 1);
+            if (lane == 0) before = last;
+            int taken = 0, word = -1;
+            uint32_t acc = 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (j0 + j < k && e[j] <= before) regular = false;       // not strictly ascending from 0 on
+                before = e[j];
+                if (e[j] < hi) {
+                    ++taken;
+                    if (e[j] >= lo) {
+                        const int w = (e[j] - lo) >> 5;
+                        if (w != word) {
+                            if (acc) atomicOr(bits + word, acc);
+                            word = w; acc = 0;
+                        }
+                        acc |= 1u << (e[j] & 31);
+                    }
+                }
+            }
+            if (acc) atomicOr(bits + word, acc);
+            taken = __reduce_add_sync(0xFFFFFFFFu, taken);
+            at += taken;
+            if (taken < 256) break;
+            last = __shfl_sync(0xFFFFFFFFu, e[7], 31);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < words / 4 * kMaskRowAlign; i += kMaskRowAlign * 32) {
+            const int tile = i / kMaskRowAlign, rr = i % kMaskRowAlign;
+            mask[((int64_t)b * key_tiles + w0 / 4 + tile) * row_pitch + r0 + rr] =
+                *reinterpret_cast<const uint4*>(&s_bits[rr * kMaskRowWords + tile * 4]);
+        }
+        __syncthreads();
+    }
+    if (at < k || !regular) *general = 1;              // (at < k: an entry past what the row can see, or out of order)
+}
+
+// ---- what the tiles cannot take -----------------------------------------------------------------------------
+// A tile multiplies every value row of its 128 keys, by zero where the key is not in the set, and a bit mask holds a
+// key once.  So a call whose gated values are not all finite (0 * inf), or whose sets are not strictly ascending
+// positions that the row can see, raises the `general` word; the tile kernels then leave at once and this plain
+// kernel (one warp per row and KV head, the set walked entry by entry) does the work.  Otherwise it costs a launch.
+template <int DH, int G>
+__global__ void __launch_bounds__(256)
+gsa_general_attn_kernel(const int32_t* __restrict__ general, const __nv_bfloat16* __restrict__ Q,
+                        const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
+                        const __nv_bfloat16* __restrict__ g1, const int32_t* __restrict__ idx,
+                        const int32_t* __restrict__ kt, IdxLayout il, __nv_bfloat16* __restrict__ out,
+                        float* __restrict__ lse, int32_t* dev_status, int q0, int rows, int B, int Lq, int Lk, int n_kv,
+                        int k_max, float scale_log2) {
+    if (*general == 0) return;
+    constexpr int NV = DH / 32;
+    const int lane = threadIdx.x & 31, n_h = n_kv * G;
+    auto load = [&](const __nv_bfloat16* p, float (&f)[NV]) {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) f[c] = __bfloat162float(p[lane * NV + c]);
+    };
+    const int64_t items = (int64_t)B * rows * n_kv;
+    for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < items; item += (int64_t)gridDim.x * 8) {
+        const int g = (int)(item % n_kv), b = (int)(item / n_kv / rows), t = q0 + (int)(item / n_kv % rows);
+        const int64_t irow = il.row(b, t);
+        const int k = checked_budget(kt[irow], k_max, dev_status);
+        float q[G][NV], o[G][NV], m[G], l[G];
+#pragma unroll
+        for (int e = 0; e < G; ++e) {
+            load(Q + (((size_t)b * Lq + t) * n_h + g * G + e) * DH, q[e]);
+            m[e] = -INFINITY; l[e] = 0.f;
+#pragma unroll
+            for (int c = 0; c < NV; ++c) o[e][c] = 0.f;
+        }
+        for (int j = 0; j < k; ++j) {
+            const int s = checked_pos(idx[irow * k_max + j], Lk, dev_status);
+            const size_t at = (((size_t)b * Lk + s) * n_kv + g) * DH;
+            float kr[NV], vr[NV];
+            load(K + at, kr);
+            load(V + at, vr);
+#pragma unroll
+            for (int e = 0; e < G; ++e) {
+                float z = 0.f;
+#pragma unroll
+                for (int c = 0; c < NV; ++c) z = fmaf(q[e][c], kr[c], z);
+#pragma unroll
+                for (int d = 16; d > 0; d >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, d);
+                z *= scale_log2;
+                if (z > m[e]) {
+                    const float alpha = exp2f(m[e] - z);
+                    m[e] = z; l[e] *= alpha;
+#pragma unroll
+                    for (int c = 0; c < NV; ++c) o[e][c] *= alpha;
+                }
+                const float pz = exp2f(z - m[e]);
+                l[e] += pz;
+#pragma unroll
+                for (int c = 0; c < NV; ++c) o[e][c] = fmaf(pz, vr[c], o[e][c]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < G; ++e) {
+            const size_t at = (((size_t)b * Lq + t) * n_h + g * G + e) * DH;
+            float gl[NV];
+            load(g1 + at, gl);
+#pragma unroll
+            for (int c = 0; c < NV; ++c)
+                out[at + lane * NV + c] = __float2bfloat16_rn(k > 0 ? o[e][c] / l[e] * fast_sigmoid(gl[c]) : 0.f);
+            if (lse && lane == 0) lse[((size_t)b * Lq + t) * n_h + g * G + e] = (m[e] + log2f(l[e])) * 0.6931471805599453f;
+        }
+    }
+}
+
+// raises `general` if a bf16 value is infinite or NaN
+__global__ void __launch_bounds__(256) gsa_check_finite_kernel(const uint4* __restrict__ x, int64_t n_vec, int32_t* general) {
+    uint32_t bad = 0;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * blockDim.x)
+        bad |= nonfinite_bf16x8(__ldg(x + i));
+    if (bad) *general = 1;
+}
+
+// ---- forward ---------------------------------------------------------------------------------------------
+// Three warpgroups launched at 168 registers a thread; the two softmax groups take 216 (a row's 128 scores live in
+// registers), the copy / MMA group keeps 72: 2 * 216 + 72 = 504 of the 504 the block was launched with.
+constexpr int kFwdThreads = 384;
+
+template <int DH>
+struct FwdSmem {
+    static constexpr int CHUNKS = DH / 64;
+    static constexpr int CHUNK_BYTES = 128 * 128;                  // 128 rows of 64 bf16
+    static constexpr int TILE_BYTES = CHUNKS * CHUNK_BYTES;
+    static constexpr int SLOTS = DH == 128 ? 5 : 8;                // K / V' tiles in flight
+    static constexpr int OFF_RING = 2 * TILE_BYTES;
+    static constexpr int OFF_BAR = OFF_RING + SLOTS * TILE_BYTES;
+    static constexpr int N_BARS = 2 * SLOTS + 2 + 2 + 2 + 2 + 1;   // ring full / empty, Q, S, P, O, drain
+    static constexpr int OFF_TMEM = OFF_BAR + N_BARS * 8;
+    static constexpr int OFF_ABORT = OFF_TMEM + 8;
+    static constexpr int ALLOC = OFF_ABORT + 8 + 1024;
+};
+
+struct MaskedFwdArgs {
+    const uint4* mask;
+    const __nv_bfloat16* g1;
+    __nv_bfloat16* out;
+    float* lse;                    // nullable
+    int32_t* dev_status;
+    const int32_t* general;
+    int32_t q0, rows, row_pitch, key_tiles;      // MaskPlan
+    int32_t Lq, Lk, n_h, n_kv, row_blocks;
+    float scale_log2;
+    long long wait_cycles;
+};
+
+template <int DH, int G>
+__global__ void __launch_bounds__(kFwdThreads, 1)
+gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                           const __grid_constant__ CUtensorMap tm_v, const MaskedFwdArgs a) {
+    using P = FwdSmem<DH>;
+    constexpr int QT = 128 / G;                                    // queries per M tile
+    constexpr int CH = P::CHUNKS;
+    constexpr uint32_t kTmS = 0, kTmO = 256;                       // TMEM columns: S / P at kTmS + 128 s, O at kTmO + 128 s
+    constexpr uint32_t kIdescS = make_idesc_bf16(128, kMaskTileKeys);
+    constexpr uint32_t kIdescO = make_idesc_bf16(128, DH) | kIdescTransB;
+
+    extern __shared__ unsigned char dyn_smem_raw[];
+    const uint32_t raw_u32 = smem_u32(dyn_smem_raw);
+    const uint32_t pad = (1024u - (raw_u32 & 1023u)) & 1023u;
+    unsigned char* smem = dyn_smem_raw + pad;
+    const uint32_t sbase = raw_u32 + pad;
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + P::OFF_TMEM);
+    volatile int* s_abort = reinterpret_cast<volatile int*>(smem + P::OFF_ABORT);
+    const uint32_t bar0 = sbase + P::OFF_BAR;
+    auto bar_full = [&](int s) { return bar0 + 8u * s; };
+    auto bar_empty = [&](int s) { return bar0 + 8u * (P::SLOTS + s); };
+    auto bar_q = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + s); };
+    auto bar_s = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 2 + s); };
+    auto bar_p = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 4 + s); };
+    auto bar_o = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 6 + s); };
+    const uint32_t bar_drain = bar0 + 8u * (2 * P::SLOTS + 8);
+
+    if (*a.general) return;                                        // (uniform: written by earlier launches only)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (batch element, KV head) outermost, so that the CTAs of a wave share K and V' in the L2; late (long) rows first
+    const int blk = a.row_blocks - 1 - (int)(blockIdx.x % a.row_blocks);
+    const int bh = blockIdx.x / a.row_blocks;
+    const int g = bh % a.n_kv, b = bh / a.n_kv;
+    const int r0 = blk * 2 * QT;                                   // first query row of the CTA (from q0)
+    const int off = a.Lk - a.Lq;
+    const int r_end = min(r0 + 2 * QT, a.rows);
+    const int ntiles = min((off + a.q0 + r_end + kMaskTileKeys - 1) / kMaskTileKeys, a.key_tiles);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < P::SLOTS; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_q(s), 1); mbar_init(bar_s(s), 1); mbar_init(bar_p(s), 4); mbar_init(bar_o(s), 1); }
+        mbar_init(bar_drain, 1);
+        *s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 9) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(sbase + P::OFF_TMEM) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *s_tmem;
+    int copies_issued = 0, q_issued = 0;                           // by the copy producer
+    int slots_released = 0;                                        // by the MMA issuer
+
+    if (warp < 8) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        // ================= softmax, then the epilogue: thread = row ==================================
+        const int s = warp >> 2, quad = warp & 3;
+        const int m = quad * 32 + lane;                            // row of the tile = TMEM lane
+        const int r = r0 + s * QT + m / G;                         // query row from q0
+        const bool live = r < a.rows;
+        const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
+        const uint32_t ts = lane_base + kTmS + 128 * s, to = lane_base + kTmO + 128 * s;
+        const uint4* __restrict__ mrow = a.mask + (int64_t)b * a.key_tiles * a.row_pitch + r;
+        float m_ref = -INFINITY;
+        uint64_t l2[2] = {0ull, 0ull};                             // (pairs of fp32 partial sums)
+        uint4 mk_next = live ? __ldg(mrow) : make_uint4(0u, 0u, 0u, 0u);
+        const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
+        bool ok = true;
+        for (int i = 0; i < ntiles; ++i) {
+            const uint4 mk = mk_next;
+            if (live && i + 1 < ntiles) mk_next = __ldg(mrow + (int64_t)(i + 1) * a.row_pitch);
+            if (!mbar_wait(bar_s(s), i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
+            tc_fence_after();
+            uint32_t v[4][32];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) tc_ld32(ts + 32 * c, v[c]);
+            tc_wait_ld32(v[0]);
+            tc_tie32(v[1]); tc_tie32(v[2]); tc_tie32(v[3]);
+            const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
+            float mx[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                mx[c] = -INFINITY;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float x = (mw[c] >> j) & 1u ? __uint_as_float(v[c][j]) : -INFINITY;
+                    v[c][j] = __float_as_uint(x);
+                    mx[c] = fmaxf(mx[c], x);
+                }
+            }
+            const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * a.scale_log2;
+            if (__any_sync(0xFFFFFFFFu, top > m_ref + 8.0f)) {
+                const float m_new = fmaxf(m_ref, top);
+                const float alpha = m_ref == -INFINITY ? 0.f : ex2_approx(m_ref - m_new);
+                m_ref = m_new;
+                const uint64_t al2 = pack_f32x2(alpha, alpha);
+                l2[0] = mul_f32x2(l2[0], al2); l2[1] = mul_f32x2(l2[1], al2);
+                if (i > 0) {                                       // every product into O so far has completed (bar_s)
+                    uint32_t o[32];
+#pragma unroll
+                    for (int c = 0; c < DH / 32; ++c) {
+                        tc_ld32(to + 32 * c, o);
+                        tc_wait_ld32(o);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
+                        tc_st32(to + 32 * c, o);
+                    }
+                }
+            }
+            const float neg = m_ref == -INFINITY ? 0.f : -m_ref;
+            const uint64_t neg2 = pack_f32x2(neg, neg);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                uint32_t pk[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const uint64_t x = fma_f32x2(pack_f32x2(__uint_as_float(v[c][2 * j]), __uint_as_float(v[c][2 * j + 1])), scale2, neg2);
+                    float x0, x1;
+                    unpack_f32x2(x, x0, x1);
+                    x0 = ex2_approx(x0); x1 = ex2_approx(x1);
+                    l2[j & 1] = add_f32x2(l2[j & 1], pack_f32x2(x0, x1));
+                    pk[j] = pack_bf16(x0, x1);
+                }
+                tc_st16(ts + 16 * c, pk);
+            }
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_p(s));
+        }
+        if (ok && !mbar_wait(bar_o(s), 0, s_abort, a.wait_cycles)) ok = false;
+        if (!ok) {
+            if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
+        } else {
+            tc_fence_after();
+            float la, lb, lc, ld;
+            unpack_f32x2(l2[0], la, lb); unpack_f32x2(l2[1], lc, ld);
+            const float l = (la + lb) + (lc + ld);
+            const int h = g * G + m % G, t = a.q0 + r;
+            const size_t at = (((size_t)b * a.Lq + (live ? t : 0)) * a.n_h + h) * DH;
+            const float inv = l > 0.f ? 1.0f / l : 0.f;            // (an empty set: a zero row)
+            if (a.lse && live) a.lse[((size_t)b * a.Lq + t) * a.n_h + h] = (m_ref + log2f(l)) * 0.6931471805599453f;
+#pragma unroll
+            for (int c = 0; c < DH / 32; ++c) {
+                uint32_t o[32];
+                tc_ld32(to + 32 * c, o);
+                tc_wait_ld32(o);
+                if (!live) continue;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint4 gv = *reinterpret_cast<const uint4*>(a.g1 + at + c * 32 + q * 8);
+                    const __nv_bfloat162* gp = reinterpret_cast<const __nv_bfloat162*>(&gv);
+                    uint32_t w[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 gf = __bfloat1622float2(gp[e]);
+                        const float o0 = l > 0.f ? __uint_as_float(o[q * 8 + 2 * e]) * inv : 0.f;
+                        const float o1 = l > 0.f ? __uint_as_float(o[q * 8 + 2 * e + 1]) * inv : 0.f;
+                        w[e] = pack_bf16(o0 * fast_sigmoid(gf.x), o1 * fast_sigmoid(gf.y));
+                    }
+                    *reinterpret_cast<uint4*>(a.out + at + c * 32 + q * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        if (warp == 8) {
+            // ================= copies: Q tiles, then K_0 V_0 K_1 V_1 ... ================================
+            if (lane == 0) {
+                for (int s = 0; s < 2; ++s) {
+                    mbar_expect_tx(bar_q(s), P::TILE_BYTES);
+                    for (int c = 0; c < CH; ++c)
+                        tma_load_3d(sbase + s * P::TILE_BYTES + c * P::CHUNK_BYTES, &tm_q, c * 64, g * G,
+                                    b * a.Lq + a.q0 + r0 + s * QT, bar_q(s));
+                    q_issued = s + 1;
+                }
+                bool ok = true;
+                for (int n = 0; ok && n < 2 * ntiles; ++n) {
+                    const int s = n % P::SLOTS;
+                    if (!mbar_wait(bar_empty(s), ((n / P::SLOTS) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                    mbar_expect_tx(bar_full(s), P::TILE_BYTES);
+                    for (int c = 0; c < CH; ++c)
+                        tma_load_3d(sbase + P::OFF_RING + s * P::TILE_BYTES + c * P::CHUNK_BYTES, (n & 1) ? &tm_v : &tm_k,
+                                    c * 64, g, b * a.Lk + (n >> 1) * kMaskTileKeys, bar_full(s));
+                    copies_issued = n + 1;
+                }
+                if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
+            }
+        } else if (warp == 9) {
+            // ================= MMA issuer ===============================================================
+            if (lane == 0) {
+                bool ok = true;
+                auto wait_slot = [&](int n) {                          // ring entry n has landed
+                    ok = ok && mbar_wait(bar_full(n % P::SLOTS), (n / P::SLOTS) & 1, s_abort, a.wait_cycles);
+                    tc_fence_after();
+                };
+                auto slot_addr = [&](int n) { return sbase + P::OFF_RING + (n % P::SLOTS) * P::TILE_BYTES; };
+                auto issue_s = [&](int s, int i) {                     // S_s = Q_s K_i^T
+                    const uint64_t qd = make_kmajor_desc<128>(sbase + s * P::TILE_BYTES);
+                    const uint64_t kd = make_kmajor_desc<128>(slot_addr(2 * i));
+    #pragma unroll
+                    for (int k = 0; k < DH / 16; ++k) {
+                        const uint64_t step = (uint64_t)((k >> 2) * (P::CHUNK_BYTES >> 4) + 2 * (k & 3));
+                        tc_mma_bf16(tmem + kTmS + 128 * s, qd + step, kd + step, kIdescS, k > 0);
+                    }
+                };
+                auto issue_o = [&](int s, int i) {                     // O_s += P_s V'_i
+                    const uint64_t vd = make_mnmajor_desc(slot_addr(2 * i + 1), P::CHUNK_BYTES);
+    #pragma unroll
+                    for (int k = 0; k < kMaskTileKeys / 16; ++k)       // 16 keys = 2048 bytes of the V' tile, 8 columns of P
+                        tc_mma_bf16_ts(tmem + kTmO + 128 * s, tmem + kTmS + 128 * s + 8 * k, vd + 128 * k, kIdescO, (i | k) != 0);
+                };
+                auto release = [&](int n) { tc_commit(bar_empty(n % P::SLOTS)); slots_released = n + 1; };
+                wait_slot(0);
+                for (int s = 0; ok && s < 2; ++s) {
+                    ok = mbar_wait(bar_q(s), 0, s_abort, a.wait_cycles);
+                    tc_fence_after();
+                    if (ok) { issue_s(s, 0); tc_commit(bar_s(s)); }
+                }
+                if (ok) release(0);
+                for (int i = 0; ok && i < ntiles; ++i) {
+                    wait_slot(2 * i + 1);
+                    for (int s = 0; ok && s < 2; ++s) {
+                        ok = mbar_wait(bar_p(s), i & 1, s_abort, a.wait_cycles);
+                        tc_fence_after();
+                        if (!ok) break;
+                        issue_o(s, i);
+                        if (i + 1 < ntiles) {
+                            if (s == 0) wait_slot(2 * i + 2);
+                            if (!ok) break;
+                            // (in order behind the product that reads P from these columns)
+                            issue_s(s, i + 1);
+                            tc_commit(bar_s(s));
+                        } else {
+                            tc_commit(bar_o(s));
+                        }
+                    }
+                    if (!ok) break;
+                    release(2 * i + 1);
+                    if (i + 1 < ntiles) release(2 * i + 2);
+                }
+                if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (*s_abort) {
+        // give-up path: let what was issued complete (each poll is bounded) before shared memory and TMEM are released
+        if (warp == 8 && lane == 0) {
+            for (int s = 0; s < q_issued; ++s) mbar_drain(bar_q(s), 0);
+            for (int n = max(0, copies_issued - P::SLOTS); n < copies_issued; ++n)
+                mbar_drain(bar_full(n % P::SLOTS), (n / P::SLOTS) & 1);
+        }
+        if (warp == 9 && lane == 0) {
+            tc_commit(bar_drain);
+            mbar_drain(bar_drain, 0);
+            for (int n = max(0, slots_released - P::SLOTS); n < slots_released; ++n)
+                mbar_drain(bar_empty(n % P::SLOTS), (n / P::SLOTS) & 1);
+        }
+        tc_fence_before();
+        __syncthreads();
+    }
+    if (warp == 9) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+    }
+}
+
+template <int DH, int G>
+cudaError_t launch_fwd_t(const MaskedFwdArgs& a, const gsa_params_t& p, const CUtensorMap& tq, const CUtensorMap& tk,
+                         const CUtensorMap& tv, cudaStream_t st) {
+    constexpr int kSmem = FwdSmem<DH>::ALLOC;
+    auto kern = gsa_masked_attn_fwd_kernel<DH, G>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)(a.row_blocks * p.n_kv * p.B), kFwdThreads, kSmem, st>>>(tq, tk, tv, a);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int block_rows, const int32_t* idx,
+                               const int32_t* kt, IdxLayout il, uint4* mask, int32_t* general, cudaStream_t st) {
+    const dim3 grid((unsigned)(mp.row_pitch / kMaskRowAlign), (unsigned)p.B);
+    gsa_build_masks_kernel<<<grid, kMaskRowAlign * 32, 0, st>>>(idx, kt, mask, il, mp.q0, mp.rows, mp.row_pitch, mp.key_tiles,
+                                                               block_rows, p.k_max, p.Lk - p.Lq, general);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_check_finite(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st) {
+    const int64_t n_vec = n_elems / 8;
+    const int64_t want = (n_vec + 255) / 256, cap = (int64_t)sm_count() * 8;
+    gsa_check_finite_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(reinterpret_cast<const uint4*>(x), n_vec, general);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, const uint4* mask, const __nv_bfloat16* Q,
+                                   const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1,
+                                   __nv_bfloat16* out, float* lse, const int32_t* idx, const int32_t* kt, IdxLayout il,
+                                   int32_t* dev_status, cudaStream_t st) {
+    const int G = p.n_h / p.n_kv;
+    CUtensorMap tq, tk, tv;
+    if (!make_heads_tmap(&tq, Q, (uint64_t)p.B * p.Lq, p.n_h, p.d_h, 128 / G, G)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&tk, K, (uint64_t)p.B * p.Lk, p.n_kv, p.d_h, kMaskTileKeys, 1)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&tv, Vg, (uint64_t)p.B * p.Lk, p.n_kv, p.d_h, kMaskTileKeys, 1)) return cudaErrorUnknown;
+    MaskedFwdArgs a;
+    a.mask = mask; a.g1 = g1; a.out = out; a.lse = lse; a.dev_status = dev_status; a.general = dev_status + kStatusGeneralWord;
+    a.q0 = mp.q0; a.rows = mp.rows; a.row_pitch = mp.row_pitch; a.key_tiles = mp.key_tiles;
+    a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv;
+    a.row_blocks = (mp.rows + masked_block_rows(p) - 1) / masked_block_rows(p);
+    const float sc = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
+    a.scale_log2 = sc * 1.4426950408889634f;
+    a.wait_cycles = wait_limit_cycles();
+    const int ctas = sm_count() * 4;
+#define GSA_CASE(DH_, G_)                                                                                              \
+    if (p.d_h == DH_ && G == G_) {                                                                                     \
+        cudaError_t e = launch_fwd_t<DH_, G_>(a, p, tq, tk, tv, st);                                                   \
+        if (e != cudaSuccess) return e;                                                                                \
+        gsa_general_attn_kernel<DH_, G_><<<ctas, 256, 0, st>>>(a.general, Q, K, Vg, g1, idx, kt, il, out, lse,         \
+                                                               dev_status, mp.q0, mp.rows, p.B, p.Lq, p.Lk, p.n_kv,   \
+                                                               p.k_max, a.scale_log2);                                \
+        ++g_launches;                                                                                                  \
+        return cudaGetLastError();                                                                                     \
+    }
+    GSA_CASE(128, 1); GSA_CASE(128, 2); GSA_CASE(128, 4); GSA_CASE(128, 8);
+    GSA_CASE(64, 1); GSA_CASE(64, 2); GSA_CASE(64, 4); GSA_CASE(64, 8);
+#undef GSA_CASE
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace gsa

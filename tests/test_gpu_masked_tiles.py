@@ -1,0 +1,113 @@
+"""Masked dense tiles of the attention stage against the oracle: sizes at the edges of the 128-key tiles and of the
+128-row tiles, every grouping of query heads, rows without keys, and inputs that the tiles must leave to the plain path."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2601_15305_b200 import binding as gsa
+from paper_2601_15305_b200.inputs import CONFIGS, make_inputs
+
+import gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+def _sets(cfg, seed, empty=()):
+    """Random ascending index sets of 1 .. k_max keys."""
+    g = torch.Generator().manual_seed(seed)
+    vis = cfg.Lk - cfg.Lq + 1 + torch.arange(cfg.Lq)
+    kt = torch.minimum(torch.randint(1, cfg.k_max + 1, (cfg.B, cfg.Lq), generator=g), vis)
+    for b, t in empty:
+        kt[b, t] = 0
+    r = torch.rand(cfg.B, cfg.Lq, cfg.Lk, generator=g).masked_fill(torch.arange(cfg.Lk) >= vis[:, None], 2.0)
+    order = r.argsort(-1)[..., :cfg.k_max]
+    order = order.masked_fill(torch.arange(order.shape[-1]) >= kt[..., None], 1 << 30).sort(-1).values
+    idx = torch.full((cfg.B, cfg.Lq, cfg.k_max), -1, dtype=torch.int32)
+    idx[..., :order.shape[-1]] = order.masked_fill(order >= 1 << 30, -1).to(torch.int32)
+    return idx, kt.to(torch.int32)
+
+
+def _run(cfg, d, idx, kt):
+    p = gsa.make_params(cfg)
+    out = torch.full_like(d["Q"], float("nan"))
+    lse = torch.full((cfg.B, cfg.Lq, cfg.n_h), float("nan"), dtype=torch.float32, device="cuda")
+    ws = torch.empty(gsa.gsa_attn_workspace_bytes(p, True), dtype=torch.uint8, device="cuda").fill_(0xFF)
+    n0 = gsa.gsa_launch_count()
+    gsa.gsa_sparse_gated_attn_fwd_lse(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx.cuda(), kt.cuda(), out, lse, ws)
+    assert gsa.gsa_launch_count() - n0 == 4          # value gate, masks, tiles, plain path (the gather takes 3 here)
+    return out, lse, gsa.gsa_device_status(ws)
+
+
+def _rows(cfg):
+    return np.unique(np.concatenate([np.arange(0, cfg.Lq, 29), np.arange(min(4, cfg.Lq)), [cfg.Lq - 2, cfg.Lq - 1]]))
+
+
+def _check(cfg, x, out, lse, idx, kt, rows):
+    for b in range(cfg.B):
+        want = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx[b][rows].numpy(),
+                           kt[b][rows].numpy(), rows, np.full_like(rows, b))
+        U.check_out(out[b][torch.from_numpy(rows).cuda()].float().cpu().numpy(), want)
+        for t in rows[::7]:
+            S = idx[b, t, :int(kt[b, t])].long()
+            if len(S):
+                z = (x["K"][b, S].double().repeat_interleave(cfg.n_h // cfg.n_kv, 1) * x["Q"][b, t].double()).sum(-1) / cfg.d_h ** 0.5
+                # bf16 inputs, fp32 sums of d_h products of order 1: 1e-5 absolute
+                assert (lse[b, t].cpu().double() - torch.logsumexp(z, 0)).abs().max() < 1e-5
+
+
+@pytest.mark.parametrize("B,Lq,Lk,n_h,n_kv,d_h", [
+    (1, 1664, 1664, 16, 8, 128),      # whole tiles
+    (2, 1025, 1793, 16, 8, 128),      # one row and one key past a tile
+    (1, 3327, 3327, 8, 8, 128),       # one row and one key short of a tile, no head sharing
+    (1, 1665, 1801, 16, 2, 128),      # eight heads per KV head
+    (2, 865, 1153, 32, 8, 64),        # d_h = 64, four heads
+    (1, 707, 900, 64, 8, 64),
+    (5, 2561, 2561, 2, 2, 64),
+])
+def test_masked_tiles_match_the_oracle(B, Lq, Lk, n_h, n_kv, d_h):
+    cfg = CONFIGS["tiny"].with_(name="masked", B=B, Lq=Lq, Lk=Lk, n_h=n_h, n_kv=n_kv, d_h=d_h, k_base=300, k_min=1, k_max=419,
+                                seed=200 + Lq)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 201, empty=[(0, 0), (B - 1, Lq - 1)])
+    out, lse, status = _run(cfg, U.to_dev(x), idx, kt)
+    assert status == 0 and (out[0, 0] == 0).all() and (out[B - 1, Lq - 1] == 0).all()
+    _check(cfg, x, out, lse, idx, kt, _rows(cfg))
+
+
+@pytest.mark.parametrize("what", ["unsorted", "duplicate", "inf_value", "nan_key", "large_scores", "position_too_large", "budget_too_large"])
+def test_inputs_that_a_mask_cannot_stand_for(what):
+    """Sets out of order or with an entry twice, and values that are not finite, give what walking the sets gives: a
+    value that is not finite reaches exactly the rows that select it.  Corrupt sets are reported, not followed."""
+    cfg = CONFIGS["tiny"].with_(name="general", B=2, Lq=900, Lk=1300, n_h=16, n_kv=8, d_h=128, k_base=300, k_min=1, k_max=419, seed=210)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 211)
+    kt[1, 500] = 7
+    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, 900, 1000], dtype=torch.int32)
+    idx[1, 500, 7:] = -1
+    hit = torch.zeros(cfg.B, cfg.Lq, dtype=torch.bool)
+    status_want = 0
+    if what == "unsorted":
+        idx[1, 500, :7] = idx[1, 500, :7].flip(0)
+    elif what == "duplicate":
+        idx[1, 500, 4] = 400
+    elif what in ("inf_value", "nan_key"):
+        x["V" if what == "inf_value" else "K"][0, 700, 3, 5] = float("inf" if what == "inf_value" else "nan")
+        hit[0] = ((idx[0] == 700) & (torch.arange(cfg.k_max) < kt[0, :, None])).any(-1)
+    elif what == "large_scores":
+        x["Q"] = x["Q"] * 300.0                      # softmax over scores that span hundreds
+    elif what == "position_too_large":
+        idx[1, 500, 6], status_want = cfg.Lk + 5, 6
+    else:
+        kt[1, 500], status_want = cfg.k_max + 1, 6
+    if status_want:
+        hit[1, 500] = True
+    out, lse, status = _run(cfg, U.to_dev(x), idx, kt)
+    assert status == status_want
+    bad = ~torch.isfinite(out.float().cpu()).all(-1).all(-1)
+    assert not (bad & ~hit).any()
+    if what in ("inf_value", "nan_key"):
+        assert hit.any() and (bad == hit).all()
+    rows = _rows(cfg)
+    keep = rows[~hit[:, rows].any(0).numpy()]
+    _check(cfg, x, out, lse, idx, kt, np.unique(np.concatenate([keep, [500]])) if not hit[:, 500].any() else keep)
