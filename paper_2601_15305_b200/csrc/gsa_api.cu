@@ -3,7 +3,7 @@
 #include <math.h>
 #include <stdio.h>
 
-#include "gsa_common.cuh"
+#include "gsa_masked.cuh"
 
 namespace gsa {
 
@@ -261,6 +261,7 @@ static size_t attn_ws_bytes(const gsa_params_t& p, bool with_prepass) {
 // workspace of the backward call: [status][V' bf16][do bf16][lse2 fp32][delta fp32][key-range scratch][inverted index sets]
 struct BwdPlan {
     size_t vg_off, dos_off, lse_off, delta_off, range_off, inv_off, total;
+    bool masked;
 };
 static BwdPlan plan_bwd_ws(const gsa_params_t& p, int32_t rows_per_batch) {
     BwdPlan w;
@@ -270,7 +271,11 @@ static BwdPlan plan_bwd_ws(const gsa_params_t& p, int32_t rows_per_batch) {
     w.lse_off = off;   off += align_up((size_t)p.B * p.Lq * p.n_h * 4, 256);
     w.delta_off = off; off += align_up((size_t)p.B * p.Lq * p.n_h * 4, 256);
     w.range_off = off; off += attn_bwd_range_bytes(p);
-    w.inv_off = off;   off += attn_bwd_invert_bytes(p, rows_per_batch);
+    // (the inverted index sets, or the masks and what stands in for them where those are the cheaper path)
+    const RowRange rr{0, p.B, p.q_begin, rows_per_batch};
+    w.masked = masked_bwd_preferred(p, rr);
+    const size_t inv = attn_bwd_invert_bytes(p, rows_per_batch), msk = w.masked ? masked_bwd_bytes(p, rr) : 0;
+    w.inv_off = off;   off += inv > msk ? inv : msk;
     w.total = off;
     return w;
 }
@@ -311,9 +316,18 @@ int gsa_sparse_gated_attn_bwd(const gsa_params_t* p, const void* Q, const void* 
     t_dev_status = (int32_t*)ws;
     cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
     if (e == cudaSuccess)
-        e = launch_value_gate((const bf16*)V, (const bf16*)g2_logits, Vg, (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st);
+        e = launch_value_gate((const bf16*)V, (const bf16*)g2_logits, Vg, (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st,
+                              t_dev_status + kStatusGeneralWord);
     IdxLayout il{0, rr.q_begin, rr.R};
     if (e == cudaSuccess && pbar) e = cudaMemsetAsync(pbar, 0, (size_t)rr.rows() * p->k_max * 4, st);
+    if (wp.masked) {
+        if (e == cudaSuccess)
+            e = launch_masked_bwd(*p, rr, (const bf16*)Q, (const bf16*)K, (const bf16*)V, Vg, (const bf16*)g1_logits,
+                                  (const bf16*)g2_logits, (const bf16*)out, (const bf16*)dout, idx, kt, il, (bf16*)dQ, (bf16*)dK,
+                                  (bf16*)dV, (bf16*)dg1, (bf16*)dg2, dOs, lse2, delta, pbar, lse, wsb + wp.inv_off,
+                                  (int32_t*)ws, st);
+        return cuda_rc(e);
+    }
     if (e == cudaSuccess)
         e = launch_sparse_attn_bwd(*p, rr, (const bf16*)Q, (const bf16*)K, Vg, (const bf16*)g1_logits,
                                    (const bf16*)out, (const bf16*)dout, idx, kt, il, (bf16*)dQ, (bf16*)dg1,

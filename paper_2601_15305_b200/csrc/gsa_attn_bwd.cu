@@ -80,7 +80,8 @@ __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* 
                                                            const __nv_bfloat16* __restrict__ out,
                                                            const __nv_bfloat16* __restrict__ dout,
                                                            __nv_bfloat16* __restrict__ dOs, __nv_bfloat16* __restrict__ dg1,
-                                                           float* __restrict__ delta, RowRange rr, int32_t Lq, int32_t n_h) {
+                                                           float* __restrict__ delta, RowRange rr, int32_t Lq, int32_t n_h,
+                                                           int32_t* nonfinite /*nullable: raised if do or delta is*/) {
     constexpr int EPL = DH / 32;
     const int lane = threadIdx.x & 31;
     const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -88,19 +89,28 @@ __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* 
     const int lr = (int)(w / n_h), h = (int)(w % n_h);
     const int64_t qrow = (int64_t)(rr.b0 + lr / rr.R) * Lq + rr.q_begin + lr % rr.R;
     const int64_t at = (qrow * n_h + h) * DH + lane * EPL;
-    float part = 0.f;
+    struct __align__(EPL * 2) Vec { __nv_bfloat16 x[EPL]; };           // this lane's values: one load, one store
+    const Vec vdy = *reinterpret_cast<const Vec*>(dout + at), vy = *reinterpret_cast<const Vec*>(out + at),
+              vg = *reinterpret_cast<const Vec*>(g1 + at);
+    Vec vdo, vdg;
+    float part = 0.f, sum_do = 0.f;
 #pragma unroll
     for (int e = 0; e < EPL; ++e) {
-        const float dy = __bfloat162float(dout[at + e]);
-        const float y = __bfloat162float(out[at + e]);
-        const float sg = 1.0f / (1.0f + __expf(-__bfloat162float(g1[at + e])));
-        dOs[at + e] = __float2bfloat16(dy * sg);
-        dg1[at + e] = __float2bfloat16(dy * y * (1.0f - sg));
+        const float dy = __bfloat162float(vdy.x[e]);
+        const float y = __bfloat162float(vy.x[e]);
+        const float sg = 1.0f / (1.0f + __expf(-__bfloat162float(vg.x[e])));
+        vdo.x[e] = __float2bfloat16(dy * sg);
+        vdg.x[e] = __float2bfloat16(dy * y * (1.0f - sg));
+        sum_do += dy * sg;
         part = fmaf(dy, y, part);
     }
+    *reinterpret_cast<Vec*>(dOs + at) = vdo;
+    *reinterpret_cast<Vec*>(dg1 + at) = vdg;
+    const float watch = part + sum_do;                                 // (infinities and NaN spread into it)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
     if (lane == 0) delta[qrow * n_h + h] = part;
+    if (nonfinite && !(fabsf(watch) < INFINITY && fabsf(part) < INFINITY)) *nonfinite = 1;
 }
 
 // first position j of the ascending list S[0 .. n) with S[j] >= x; the whole warp calls it (32 probes a round)
@@ -477,14 +487,6 @@ cudaError_t launch_bwd_mode(const BwdArgs& a, cudaStream_t st) {
 
 template <int DH, int G>
 cudaError_t launch_bwd_t(const BwdArgs& a, cudaStream_t st) {
-    {
-        const int64_t warps = (int64_t)a.rr.rows() * a.n_h;
-        gsa_bwd_prep_kernel<DH><<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(a.g1, a.out, a.dout, a.dOs, a.dg1, a.delta,
-                                                                            a.rr, a.Lq, a.n_h);
-        ++g_launches;
-        cudaError_t e0 = cudaGetLastError();
-        if (e0 != cudaSuccess) return e0;
-    }
     if (a.n_ranges <= 1) return launch_bwd_mode<DH, G, 0>(a, st);
     gsa_bwd_range_cuts_kernel<<<(unsigned)((a.rr.rows() + 7) / 8), 256, 0, st>>>(a.idx, a.kt, const_cast<int32_t*>(a.cuts), a.rr,
                                                                                   a.il, a.Lq, a.k_max, a.n_ranges, a.range_keys);
@@ -522,6 +524,16 @@ size_t attn_bwd_range_bytes(const gsa_params_t& p) {
            (rows * (br.n_ranges + 1) * 4 + 255) / 256 * 256;
 }
 
+cudaError_t launch_bwd_prep(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* g1, const __nv_bfloat16* out,
+                            const __nv_bfloat16* dout, __nv_bfloat16* dOs, __nv_bfloat16* dg1, float* delta,
+                            int32_t* nonfinite, cudaStream_t st) {
+    const unsigned ctas = (unsigned)(((int64_t)rr.rows() * p.n_h + 7) / 8);
+    if (p.d_h == 128) gsa_bwd_prep_kernel<128><<<ctas, 256, 0, st>>>(g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, nonfinite);
+    else gsa_bwd_prep_kernel<64><<<ctas, 256, 0, st>>>(g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, nonfinite);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
 bool attn_bwd_supported(const gsa_params_t& p) {
     const int G = p.n_h / p.n_kv;
     return (p.d_h == 128 || p.d_h == 64) && (G == 1 || G == 2 || G == 4 || G == 8);
@@ -545,6 +557,8 @@ cudaError_t launch_sparse_attn_bwd(const gsa_params_t& p, RowRange rr, const __n
     a.dQ = dQ; a.dg1 = dg1; a.dOs = dOs; a.lse2 = lse2; a.delta = delta; a.pbar = pbar; a.rr = rr; a.il = il;
     a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv; a.k_max = p.k_max;
     a.scale = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
+    const cudaError_t e0 = launch_bwd_prep(p, rr, g1, out, dout, dOs, dg1, delta, nullptr, st);
+    if (e0 != cudaSuccess) return e0;
     const int G = p.n_h / p.n_kv;
 #define GSA_BWD_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_bwd_t<DH_, G_>(a, st)
     GSA_BWD_CASE(128, 1); GSA_BWD_CASE(128, 2); GSA_BWD_CASE(128, 4); GSA_BWD_CASE(128, 8);

@@ -74,6 +74,10 @@ cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, _
 // (gsa_attn_bwd_keys.cu), which inverts the index sets inside invert_ws (attn_bwd_invert_bytes) and writes
 // dK, dV, dg2 for every key.
 bool attn_bwd_supported(const gsa_params_t& p);
+// do = dout * sigmoid(g1), dg1 and delta = sum_d dout * out per (row, head); *nonfinite (nullable) is raised if one is not finite
+cudaError_t launch_bwd_prep(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* g1, const __nv_bfloat16* out,
+                            const __nv_bfloat16* dout, __nv_bfloat16* dOs, __nv_bfloat16* dg1, float* delta,
+                            int32_t* nonfinite, cudaStream_t st);
 cudaError_t launch_sparse_attn_bwd(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q,
                                    const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1,
                                    const __nv_bfloat16* out, const __nv_bfloat16* dout, const int32_t* idx,

@@ -53,11 +53,22 @@ cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, co
                                    __nv_bfloat16* out, float* lse, const int32_t* idx, const int32_t* kt, IdxLayout il,
                                    int32_t* dev_status, cudaStream_t st);
 
+// Backward (gsa_masked_bwd.cu): all gradients of the attention stage and the target of the indexer's loss (pbar, zeroed by
+// the caller; may be null).  V: as given, Vg: gated and scanned.  ws: masked_bwd_bytes(p, rr) bytes.
+bool masked_bwd_preferred(const gsa_params_t& p, const RowRange& rr);
+size_t masked_bwd_bytes(const gsa_params_t& p, const RowRange& rr);
+cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                              const __nv_bfloat16* V, const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const __nv_bfloat16* g2,
+                              const __nv_bfloat16* out, const __nv_bfloat16* dout, const int32_t* idx, const int32_t* kt,
+                              IdxLayout il, __nv_bfloat16* dQ, __nv_bfloat16* dK, __nv_bfloat16* dV, __nv_bfloat16* dg1,
+                              __nv_bfloat16* dg2, __nv_bfloat16* dOs, float* lse_ws, float* delta, float* pbar,
+                              const float* lse_in /*nullable*/, void* ws, int32_t* dev_status, cudaStream_t st);
+
 // ---- device helpers --------------------------------------------------------------------------------------
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
+__device__ __forceinline__ void tma_load_tile(uint32_t dst, const CUtensorMap* tm, int d, int head, int token, int b, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(dst), "l"(tm), "r"(x), "r"(y), "r"(z), "r"(bar)
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+        ::"r"(dst), "l"(tm), "r"(d), "r"(head), "r"(token), "r"(b), "r"(bar)
         : "memory");
 }
 
@@ -163,17 +174,17 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// tokens x heads x d_h bf16 (row-major); box = tokens_box x heads_box x 64 values (one 128-byte swizzle span).  Tokens
-// past the end read as zero.
-inline bool make_heads_tmap(CUtensorMap* tm, const void* base, uint64_t tokens, uint64_t heads, uint64_t d_h,
-                            uint32_t tokens_box, uint32_t heads_box) {
+// batch x tokens x heads x d_h bf16 (row-major, batch_stride tokens from one batch element to the next); box = tokens_box x
+// heads_box x 64 values (one 128-byte swizzle span).  Tokens past a batch element's last read as zero.
+inline bool make_heads_tmap(CUtensorMap* tm, const void* base, uint64_t batch, uint64_t batch_stride, uint64_t tokens,
+                            uint64_t heads, uint64_t d_h, uint32_t tokens_box, uint32_t heads_box) {
     auto fn = get_encode_fn();
     if (!fn) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)d_h, (cuuint64_t)heads, (cuuint64_t)tokens};
-    cuuint64_t strides[2] = {(cuuint64_t)d_h * 2, (cuuint64_t)(heads * d_h) * 2};
-    cuuint32_t box[3] = {64u, heads_box, tokens_box};
-    cuuint32_t estr[3] = {1, 1, 1};
-    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+    cuuint64_t dims[4] = {(cuuint64_t)d_h, (cuuint64_t)heads, (cuuint64_t)tokens, (cuuint64_t)batch};
+    cuuint64_t strides[3] = {(cuuint64_t)d_h * 2, (cuuint64_t)(heads * d_h) * 2, (cuuint64_t)(batch_stride * heads * d_h) * 2};
+    cuuint32_t box[4] = {64u, heads_box, tokens_box, 1u};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }

@@ -389,8 +389,7 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 for (int s = 0; s < 2; ++s) {
                     mbar_expect_tx(bar_q(s), P::TILE_BYTES);
                     for (int c = 0; c < CH; ++c)
-                        tma_load_3d(sbase + s * P::TILE_BYTES + c * P::CHUNK_BYTES, &tm_q, c * 64, g * G,
-                                    b * a.Lq + a.q0 + r0 + s * QT, bar_q(s));
+                        tma_load_tile(sbase + s * P::TILE_BYTES + c * P::CHUNK_BYTES, &tm_q, c * 64, g * G, r0 + s * QT, b, bar_q(s));
                     q_issued = s + 1;
                 }
                 bool ok = true;
@@ -399,8 +398,8 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     if (!mbar_wait(bar_empty(s), ((n / P::SLOTS) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
                     mbar_expect_tx(bar_full(s), P::TILE_BYTES);
                     for (int c = 0; c < CH; ++c)
-                        tma_load_3d(sbase + P::OFF_RING + s * P::TILE_BYTES + c * P::CHUNK_BYTES, (n & 1) ? &tm_v : &tm_k,
-                                    c * 64, g, b * a.Lk + (n >> 1) * kMaskTileKeys, bar_full(s));
+                        tma_load_tile(sbase + P::OFF_RING + s * P::TILE_BYTES + c * P::CHUNK_BYTES, (n & 1) ? &tm_v : &tm_k,
+                                      c * 64, g, (n >> 1) * kMaskTileKeys, b, bar_full(s));
                     copies_issued = n + 1;
                 }
                 if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
@@ -524,9 +523,9 @@ cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, co
                                    int32_t* dev_status, cudaStream_t st) {
     const int G = p.n_h / p.n_kv;
     CUtensorMap tq, tk, tv;
-    if (!make_heads_tmap(&tq, Q, (uint64_t)p.B * p.Lq, p.n_h, p.d_h, 128 / G, G)) return cudaErrorUnknown;
-    if (!make_heads_tmap(&tk, K, (uint64_t)p.B * p.Lk, p.n_kv, p.d_h, kMaskTileKeys, 1)) return cudaErrorUnknown;
-    if (!make_heads_tmap(&tv, Vg, (uint64_t)p.B * p.Lk, p.n_kv, p.d_h, kMaskTileKeys, 1)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&tq, Q + (size_t)mp.q0 * p.n_h * p.d_h, p.B, p.Lq, mp.rows, p.n_h, p.d_h, 128 / G, G)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&tk, K, p.B, p.Lk, p.Lk, p.n_kv, p.d_h, kMaskTileKeys, 1)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&tv, Vg, p.B, p.Lk, p.Lk, p.n_kv, p.d_h, kMaskTileKeys, 1)) return cudaErrorUnknown;
     MaskedFwdArgs a;
     a.mask = mask; a.g1 = g1; a.out = out; a.lse = lse; a.dev_status = dev_status; a.general = dev_status + kStatusGeneralWord;
     a.q0 = mp.q0; a.rows = mp.rows; a.row_pitch = mp.row_pitch; a.key_tiles = mp.key_tiles;

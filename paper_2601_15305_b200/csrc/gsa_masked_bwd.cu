@@ -1,0 +1,953 @@
+// Backward of sparse gated attention on masked dense tiles (see gsa_masked.cuh): the same derivatives as
+// gsa_attn_bwd.cu / gsa_attn_bwd_keys.cu, for index sets that hold more than a few per cent of the visible keys.
+//
+// With P = exp2(S - lse) on the set and 0 outside, dS = P (dP - delta), S = scale Q K^T, dP = do V'^T:
+//   keys kernel (one CTA = 128 keys of a KV head, all rows that see them):    dV' = P^T do,   dK = scale dS^T Q
+//   rows kernel (one CTA = 128 (query, head) rows of a KV head, all keys):    dQ = scale dS K
+//   target kernel (one CTA = 128 rows x 256 keys at a time, all heads):       pbar = mean over the heads of P
+// S and dP are computed in both of the first two: two products more than one fused kernel needs, but every sum stays in
+// TMEM from the first tile to the last -- no fp32 array that the row tiles' dQ meet in, no atomics, results that do not
+// depend on scheduling.  P and dS go back to TMEM as bf16 over the columns they came from and are the A operand of the
+// next product; Q, do, K, V' tiles lie in shared memory once and are read along rows (K-major) for S and dP and along
+// columns (MN-major) for the sums.
+//
+// Bound: the products and the elementwise work between them in turn.  Measured at L = 32K, 16 heads of 128 on 8 KV heads, mean
+// budget 2048: keys 6.3 ms (four products, 1.4 PFLOP/s), rows 5.3 ms (three, 1.24 PFLOP/s), target 4.9 ms (one, and all the
+// exponentials); the gather kernels took 92 ms for the same.
+//
+// Roles in all three: warps 0-7 the elementwise work (two warpgroups side by side), warp 8 copies, warp 9 MMA issue.
+#include "gsa_masked.cuh"
+
+namespace gsa {
+
+namespace {
+
+constexpr int kBwdThreads = 384;
+constexpr float kLog2e = 1.4426950408889634f;
+
+template <int DH>
+struct TileBytes {
+    static constexpr int CHUNKS = DH / 64;
+    static constexpr int CHUNK = 128 * 128;                        // 128 rows of 64 bf16
+    static constexpr int TILE = CHUNKS * CHUNK;
+};
+
+struct MaskedBwdArgs {
+    const uint4* mask;
+    const float* lse;              // [B, Lq, n_h], natural logarithm
+    const float* delta;            // [B, Lq, n_h]
+    const __nv_bfloat16* V;
+    const __nv_bfloat16* g2;
+    const int32_t* idx;
+    const int32_t* kt;
+    IdxLayout il;
+    __nv_bfloat16* dQ;
+    __nv_bfloat16* dK;
+    __nv_bfloat16* dV;
+    __nv_bfloat16* dg2;
+    float* pbar;
+    int32_t* dev_status;
+    const int32_t* general;
+    int32_t q0, rows, row_pitch, key_tiles;
+    int32_t B, Lq, Lk, n_h, n_kv, k_max;
+    int32_t row_blocks;            // of 128 / G queries
+    int32_t pairs_per_cta;         // target kernel: runs of 256 keys per CTA
+    float scale, scale_log2;
+    long long wait_cycles;
+};
+
+// 128-row K-major operand: k-step of 16 columns
+__device__ __forceinline__ uint64_t kmajor_step(int k) { return (uint64_t)((k >> 2) * (TileBytes<128>::CHUNK >> 4) + 2 * (k & 3)); }
+
+template <int DH>
+__device__ __forceinline__ void mma_kmajor(uint32_t d, uint32_t a_smem, uint32_t b_smem) {        // D = A B^T over DH columns
+    const uint64_t ad = make_kmajor_desc<128>(a_smem), bd = make_kmajor_desc<128>(b_smem);
+#pragma unroll
+    for (int k = 0; k < DH / 16; ++k)
+        tc_mma_bf16(d, ad + kmajor_step(k), bd + kmajor_step(k), make_idesc_bf16(128, 128), k > 0);
+}
+// D += A B with A (128 x 128, bf16) in TMEM in two halves of 64 contraction elements, 64 columns apart, and B the rows of a tile
+template <int DH>
+__device__ __forceinline__ void mma_tmem_rows(uint32_t d, uint32_t a_tmem, uint32_t b_smem, bool accumulate) {
+    const uint64_t bd = make_mnmajor_desc(b_smem, TileBytes<DH>::CHUNK);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        tc_mma_bf16_ts(d, a_tmem + (k >> 2) * 64 + (k & 3) * 8, bd + 128 * k, make_idesc_bf16(128, DH) | kIdescTransB,
+                       accumulate || k > 0);
+}
+
+#define GSA_TILE_PROLOGUE(PLAN)                                                                                          \
+    extern __shared__ unsigned char dyn_smem_raw[];                                                                     \
+    const uint32_t raw_u32 = smem_u32(dyn_smem_raw);                                                                    \
+    const uint32_t pad = (1024u - (raw_u32 & 1023u)) & 1023u;                                                           \
+    unsigned char* const smem = dyn_smem_raw + pad;                                                                     \
+    const uint32_t sbase = raw_u32 + pad;                                                                               \
+    uint32_t* const s_tmem = reinterpret_cast<uint32_t*>(smem + PLAN::OFF_TMEM);                                        \
+    volatile int* const s_abort = reinterpret_cast<volatile int*>(smem + PLAN::OFF_ABORT);                              \
+    const uint32_t bar0 = sbase + PLAN::OFF_BAR;                                                                        \
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+__device__ __forceinline__ uint32_t tile_start(int warp, uint32_t tmem_slot, const uint32_t* s_tmem, volatile int* s_abort) {
+    if (threadIdx.x == 0) {
+        *s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 9) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(tmem_slot) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    return *s_tmem;
+}
+
+// End of a kernel: on the give-up path what was issued completes first (each poll is bounded), then TMEM is released.
+// drain_copies / drain_commits poll the barriers of the issuing threads' own copies / commits.
+template <class FC, class FM>
+__device__ __forceinline__ void tile_end(int warp, int lane, uint32_t tmem, volatile int* s_abort, uint32_t bar_drain,
+                                         FC drain_copies, FM drain_commits) {
+    tc_fence_before();
+    __syncthreads();
+    if (*s_abort) {
+        if (warp == 8 && lane == 0) drain_copies();
+        if (warp == 9 && lane == 0) {
+            tc_commit(bar_drain);
+            mbar_drain(bar_drain, 0);
+            drain_commits();
+        }
+        tc_fence_before();
+        __syncthreads();
+    }
+    if (warp == 9) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+    }
+}
+
+// ---- keys: dK, dV, dg2 -----------------------------------------------------------------------------------------
+template <int DH, int G>
+struct KeysSmem {
+    using T = TileBytes<DH>;
+    static constexpr int QT = 128 / G;
+    static constexpr int STAGES = DH == 128 ? 2 : 4;               // (Q, do) tile pairs in flight
+    static constexpr int OFF_K = 0, OFF_V = T::TILE, OFF_RING = 2 * T::TILE;
+    static constexpr int OFF_STAT = OFF_RING + STAGES * 2 * T::TILE;
+    static constexpr int STAT_BYTES = 128 * 8 + QT * 16;           // lse2 and delta per row, four mask words per query
+    static constexpr int OFF_BAR = OFF_STAT + STAGES * STAT_BYTES;
+    static constexpr int N_BARS = 5 * STAGES + 8;
+    static constexpr int OFF_TMEM = OFF_BAR + N_BARS * 8;
+    static constexpr int OFF_ABORT = OFF_TMEM + 8;
+    static constexpr int ALLOC = OFF_ABORT + 8 + 1024;
+};
+
+template <int DH, int G>
+__global__ void __launch_bounds__(kBwdThreads, 1)
+gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
+                           const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+                           const MaskedBwdArgs a) {
+    using P = KeysSmem<DH, G>;
+    using T = TileBytes<DH>;
+    constexpr int QT = P::QT, ST = P::STAGES;
+    constexpr uint32_t kTmS = 0, kTmP = 128, kTmV = 256, kTmK = 384;
+    if (*a.general) return;
+    GSA_TILE_PROLOGUE(P)
+    auto bar_q = [&](int s) { return bar0 + 8u * s; };                       // Q tile landed
+    auto bar_d = [&](int s) { return bar0 + 8u * (ST + s); };                // do tile landed
+    auto bar_free = [&](int s) { return bar0 + 8u * (2 * ST + s); };         // both consumed
+    auto bar_stat = [&](int s) { return bar0 + 8u * (3 * ST + s); };         // row statistics and masks stored
+    auto bar_statfree = [&](int s) { return bar0 + 8u * (4 * ST + s); };
+    const uint32_t bar_kv = bar0 + 8u * (5 * ST), bar_s = bar_kv + 8, bar_dp = bar_kv + 16, bar_p = bar_kv + 24,
+                   bar_ds = bar_kv + 32, bar_done = bar_kv + 40, bar_drain = bar_kv + 48;
+
+    // early key tiles (the longest) first; (batch element, KV head) outermost
+    const int tile = blockIdx.x % a.key_tiles, bh = blockIdx.x / a.key_tiles;
+    const int g = bh % a.n_kv, b = bh / a.n_kv;
+    const int off = a.Lk - a.Lq;
+    const int r_first = max(0, tile * kMaskTileKeys - off - a.q0);           // first row that sees a key of the tile
+    const int i0 = r_first / QT;
+    const int n = r_first < a.rows ? a.row_blocks - i0 : 0;                  // (tiles that no row sees have no masks)
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < ST; ++s) {
+            mbar_init(bar_q(s), 1); mbar_init(bar_d(s), 1); mbar_init(bar_free(s), 1);
+            mbar_init(bar_stat(s), 64); mbar_init(bar_statfree(s), 8);
+        }
+        mbar_init(bar_kv, 1); mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_p, 8); mbar_init(bar_ds, 8);
+        mbar_init(bar_done, 1); mbar_init(bar_drain, 1);
+    }
+    const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
+    int copies = 0, kv_issued = 0, released = 0;
+
+    if (warp == 8) {
+        if (lane == 0 && n > 0) {
+            mbar_expect_tx(bar_kv, 2 * T::TILE);
+            for (int c = 0; c < T::CHUNKS; ++c) {
+                tma_load_tile(sbase + P::OFF_K + c * T::CHUNK, &tm_k, c * 64, g, tile * kMaskTileKeys, b, bar_kv);
+                tma_load_tile(sbase + P::OFF_V + c * T::CHUNK, &tm_v, c * 64, g, tile * kMaskTileKeys, b, bar_kv);
+            }
+            kv_issued = 1;
+            bool ok = true;
+            for (int i = 0; ok && i < n; ++i) {
+                const int s = i % ST;
+                if (!mbar_wait(bar_free(s), ((i / ST) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                const uint32_t dst = sbase + P::OFF_RING + s * 2 * T::TILE;
+                const int z = (i0 + i) * QT;
+                mbar_expect_tx(bar_q(s), T::TILE);
+                for (int c = 0; c < T::CHUNKS; ++c) tma_load_tile(dst + c * T::CHUNK, &tm_q, c * 64, g * G, z, b, bar_q(s));
+                mbar_expect_tx(bar_d(s), T::TILE);
+                for (int c = 0; c < T::CHUNKS; ++c)
+                    tma_load_tile(dst + T::TILE + c * T::CHUNK, &tm_do, c * 64, g * G, z, b, bar_d(s));
+                copies = i + 1;
+            }
+            if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
+        }
+    } else if (warp == 9) {
+        if (lane == 0 && n > 0) {
+            auto q_at = [&](int i) { return sbase + P::OFF_RING + (i % ST) * 2 * T::TILE; };
+            auto d_at = [&](int i) { return q_at(i) + T::TILE; };
+            auto wait = [&](uint32_t bar, uint32_t parity) {
+                const bool r = mbar_wait(bar, parity, s_abort, a.wait_cycles);
+                tc_fence_after();
+                return r;
+            };
+            auto issue_s = [&](int i) {                            // S^T = K Q^T
+                if (!wait(bar_q(i % ST), (i / ST) & 1)) return false;
+                mma_kmajor<DH>(tmem + kTmS, sbase + P::OFF_K, q_at(i));
+                tc_commit(bar_s);
+                return true;
+            };
+            auto issue_dp = [&](int i) {                           // dP^T = V' do^T
+                if (!wait(bar_d(i % ST), (i / ST) & 1)) return false;
+                mma_kmajor<DH>(tmem + kTmP, sbase + P::OFF_V, d_at(i));
+                tc_commit(bar_dp);
+                return true;
+            };
+            bool ok = wait(bar_kv, 0) && issue_s(0) && issue_dp(0);
+            for (int i = 0; ok && i < n; ++i) {
+                // every product is issued behind the one that reads what it overwrites
+                if (!(ok = wait(bar_p, i & 1))) break;
+                mma_tmem_rows<DH>(tmem + kTmV, tmem + kTmS, d_at(i), i > 0);       // dV' += P^T do
+                if (i + 1 < n && !(ok = issue_s(i + 1))) break;
+                if (!(ok = wait(bar_ds, i & 1))) break;
+                mma_tmem_rows<DH>(tmem + kTmK, tmem + kTmP, q_at(i), i > 0);       // dK += dS^T Q
+                tc_commit(bar_free(i % ST));
+                released = i + 1;
+                if (i + 1 < n) ok = issue_dp(i + 1);
+            }
+            if (ok) tc_commit(bar_done);
+            else atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
+        }
+    } else if (warp >= 10) {
+        // row statistics and masks of the next tiles: thread = two rows
+        const int j = threadIdx.x - 320;
+        bool ok = true;
+        for (int i = 0; ok && i < n; ++i) {
+            const int s = i % ST;
+            float l2[2], dl[2];
+            uint4 mk[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int m = j + 64 * u, r = (i0 + i) * QT + m / G;
+                l2[u] = dl[u] = 0.f;
+                if (r < a.rows) {
+                    const size_t at = ((size_t)b * a.Lq + a.q0 + r) * a.n_h + g * G + m % G;
+                    l2[u] = a.lse[at] * kLog2e;
+                    dl[u] = a.delta[at];
+                }
+                const int rq = (i0 + i) * QT + m;                  // (this thread's query for the masks)
+                mk[u] = make_uint4(0u, 0u, 0u, 0u);
+                if (m < QT && rq < a.rows) mk[u] = a.mask[((int64_t)b * a.key_tiles + tile) * a.row_pitch + rq];
+            }
+            if (!mbar_wait(bar_statfree(s), ((i / ST) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+            float* st = reinterpret_cast<float*>(smem + P::OFF_STAT + s * P::STAT_BYTES);
+            uint32_t* sm = reinterpret_cast<uint32_t*>(st + 256);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int m = j + 64 * u;
+                st[m] = l2[u];
+                st[128 + m] = dl[u];
+                if (m < QT) { sm[m] = mk[u].x; sm[QT + m] = mk[u].y; sm[2 * QT + m] = mk[u].z; sm[3 * QT + m] = mk[u].w; }
+            }
+            mbar_arrive(bar_stat(s));
+        }
+        if (!ok && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
+    } else {
+        // lane = key; this warpgroup's half of the 128 rows
+        const int half = warp >> 2, quad = warp & 3;
+        const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
+        const uint32_t ts = lane_base + kTmS + 64 * half, tp = lane_base + kTmP + 64 * half;
+        const uint32_t my_bit = 1u << lane;
+        bool ok = true;
+        for (int i = 0; i < n; ++i) {
+            const int s = i % ST;
+            const float* st = reinterpret_cast<const float*>(smem + P::OFF_STAT + s * P::STAT_BYTES) + 64 * half;
+            const uint32_t* sm = reinterpret_cast<const uint32_t*>(smem + P::OFF_STAT + s * P::STAT_BYTES + 1024) +
+                                 quad * QT + 64 / G * half;
+            if (!mbar_wait(bar_stat(s), (i / ST) & 1, s_abort, a.wait_cycles) ||
+                !mbar_wait(bar_s, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
+            tc_fence_after();
+            uint32_t v[2][32];
+            tc_ld32(ts, v[0]);
+            tc_ld32(ts + 32, v[1]);
+            tc_wait_ld32(v[0]);
+            tc_tie32(v[1]);
+            uint32_t pk[32];
+#pragma unroll
+            for (int c = 0; c < 64; c += 4) {
+                const float4 l2 = *reinterpret_cast<const float4*>(st + c);
+                const float lv[4] = {l2.x, l2.y, l2.z, l2.w};
+                float pv[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float x = ex2_approx(fmaf(__uint_as_float(v[c >> 5][(c & 31) + e]), a.scale_log2, -lv[e]));
+                    pv[e] = (sm[(c + e) / G] & my_bit) ? x : 0.f;
+                    v[c >> 5][(c & 31) + e] = __float_as_uint(pv[e]);
+                }
+                pk[c / 2] = pack_bf16(pv[0], pv[1]);
+                pk[c / 2 + 1] = pack_bf16(pv[2], pv[3]);
+            }
+            tc_st32(ts, pk);
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_p);
+
+            if (!mbar_wait(bar_dp, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
+            tc_fence_after();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t w[32];
+                tc_ld32(tp + 32 * h, w);
+                tc_wait_ld32(w);
+#pragma unroll
+                for (int c = 0; c < 32; c += 4) {
+                    const float4 dl = *reinterpret_cast<const float4*>(st + 128 + 32 * h + c);
+                    const float dv[4] = {dl.x, dl.y, dl.z, dl.w};
+                    float ds[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) ds[e] = __uint_as_float(v[h][c + e]) * (__uint_as_float(w[c + e]) - dv[e]);
+                    pk[16 * h + c / 2] = pack_bf16(ds[0], ds[1]);
+                    pk[16 * h + c / 2 + 1] = pack_bf16(ds[2], ds[3]);
+                }
+            }
+            tc_st32(tp, pk);
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) { mbar_arrive(bar_ds); mbar_arrive(bar_statfree(s)); }
+        }
+        if (ok && n > 0 && !mbar_wait(bar_done, 0, s_abort, a.wait_cycles)) ok = false;
+        if (!ok) {
+            if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
+        } else {
+            tc_fence_after();
+            const int key = tile * kMaskTileKeys + quad * 32 + lane;
+            const size_t at = (((size_t)b * a.Lk + min(key, a.Lk - 1)) * a.n_kv + g) * DH + half * (DH / 2);
+#pragma unroll
+            for (int c = 0; c < DH / 64; ++c) {
+                uint32_t dk[32], dv[32];
+                if (n > 0) {
+                    tc_ld32(lane_base + kTmK + half * (DH / 2) + 32 * c, dk);
+                    tc_ld32(lane_base + kTmV + half * (DH / 2) + 32 * c, dv);
+                    tc_wait_ld32(dk);
+                    tc_tie32(dv);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) dk[e] = dv[e] = 0u;
+                }
+                if (key >= a.Lk) continue;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const size_t p8 = at + 32 * c + 8 * q;
+                    const uint4 vv = *reinterpret_cast<const uint4*>(a.V + p8), gg = *reinterpret_cast<const uint4*>(a.g2 + p8);
+                    const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
+                    const __nv_bfloat162* gp = reinterpret_cast<const __nv_bfloat162*>(&gg);
+                    uint32_t ok_[4], ov[4], og[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 vf = __bfloat1622float2(vp[e]), gf = __bfloat1622float2(gp[e]);
+                        const float s0 = 1.0f / (1.0f + __expf(-gf.x)), s1 = 1.0f / (1.0f + __expf(-gf.y));
+                        const float d0 = __uint_as_float(dv[8 * q + 2 * e]), d1 = __uint_as_float(dv[8 * q + 2 * e + 1]);
+                        ok_[e] = pack_bf16(__uint_as_float(dk[8 * q + 2 * e]) * a.scale, __uint_as_float(dk[8 * q + 2 * e + 1]) * a.scale);
+                        ov[e] = pack_bf16(d0 * s0, d1 * s1);
+                        og[e] = pack_bf16(d0 * vf.x * s0 * (1.0f - s0), d1 * vf.y * s1 * (1.0f - s1));
+                    }
+                    *reinterpret_cast<uint4*>(a.dK + p8) = make_uint4(ok_[0], ok_[1], ok_[2], ok_[3]);
+                    *reinterpret_cast<uint4*>(a.dV + p8) = make_uint4(ov[0], ov[1], ov[2], ov[3]);
+                    *reinterpret_cast<uint4*>(a.dg2 + p8) = make_uint4(og[0], og[1], og[2], og[3]);
+                }
+            }
+        }
+    }
+    tile_end(warp, lane, tmem, s_abort, bar_drain,
+             [&] {
+                 if (kv_issued) mbar_drain(bar_kv, 0);
+                 for (int i = max(0, copies - ST); i < copies; ++i) {
+                     mbar_drain(bar_q(i % ST), (i / ST) & 1);
+                     mbar_drain(bar_d(i % ST), (i / ST) & 1);
+                 }
+             },
+             [&] { for (int i = max(0, released - ST); i < released; ++i) mbar_drain(bar_free(i % ST), (i / ST) & 1); });
+}
+
+// ---- rows: dQ --------------------------------------------------------------------------------------------------
+template <int DH>
+struct RowsSmem {
+    using T = TileBytes<DH>;
+    static constexpr int SLOTS = DH == 128 ? 5 : 8;                // K_0 V_0 K_1 V_1 ... in flight
+    static constexpr int OFF_Q = 0, OFF_D = T::TILE, OFF_RING = 2 * T::TILE;
+    static constexpr int OFF_BAR = OFF_RING + SLOTS * T::TILE;
+    static constexpr int N_BARS = 2 * SLOTS + 8;
+    static constexpr int OFF_TMEM = OFF_BAR + N_BARS * 8;
+    static constexpr int OFF_ABORT = OFF_TMEM + 8;
+    static constexpr int ALLOC = OFF_ABORT + 8 + 1024;
+};
+
+template <int DH, int G>
+__global__ void __launch_bounds__(kBwdThreads, 1)
+gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
+                           const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+                           const MaskedBwdArgs a) {
+    using P = RowsSmem<DH>;
+    using T = TileBytes<DH>;
+    constexpr int QT = 128 / G, SL = P::SLOTS;
+    constexpr uint32_t kTmS = 0, kTmP = 256, kTmQ = 384;           // S at kTmS + 128 (i & 1)
+    if (*a.general) return;
+    GSA_TILE_PROLOGUE(P)
+    auto bar_full = [&](int s) { return bar0 + 8u * s; };
+    auto bar_empty = [&](int s) { return bar0 + 8u * (SL + s); };
+    const uint32_t bar_qd = bar0 + 8u * (2 * SL), bar_s0 = bar_qd + 8, bar_dp = bar_qd + 24, bar_read = bar_qd + 32,
+                   bar_ds = bar_qd + 40, bar_done = bar_qd + 48, bar_drain = bar_qd + 56;
+    auto bar_s = [&](int i) { return bar_s0 + 8u * (i & 1); };     // (both buffers may be outstanding)
+
+    const int blk = a.row_blocks - 1 - (int)(blockIdx.x % a.row_blocks), bh = blockIdx.x / a.row_blocks;
+    const int g = bh % a.n_kv, b = bh / a.n_kv;
+    const int r0 = blk * QT, off = a.Lk - a.Lq;
+    const int n = min((off + a.q0 + min(r0 + QT, a.rows) + kMaskTileKeys - 1) / kMaskTileKeys, a.key_tiles);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < SL; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
+        mbar_init(bar_qd, 1); mbar_init(bar_s(0), 1); mbar_init(bar_s(1), 1); mbar_init(bar_dp, 1); mbar_init(bar_read, 8);
+        mbar_init(bar_ds, 8); mbar_init(bar_done, 1); mbar_init(bar_drain, 1);
+    }
+    const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
+    int copies = 0, qd_issued = 0, k_released = 0, v_released = 0;
+
+    if (warp == 8) {
+        if (lane == 0) {
+            mbar_expect_tx(bar_qd, 2 * T::TILE);
+            for (int c = 0; c < T::CHUNKS; ++c) {
+                tma_load_tile(sbase + P::OFF_Q + c * T::CHUNK, &tm_q, c * 64, g * G, r0, b, bar_qd);
+                tma_load_tile(sbase + P::OFF_D + c * T::CHUNK, &tm_do, c * 64, g * G, r0, b, bar_qd);
+            }
+            qd_issued = 1;
+            bool ok = true;
+            for (int e = 0; ok && e < 2 * n; ++e) {
+                const int s = e % SL;
+                if (!mbar_wait(bar_empty(s), ((e / SL) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                mbar_expect_tx(bar_full(s), T::TILE);
+                for (int c = 0; c < T::CHUNKS; ++c)
+                    tma_load_tile(sbase + P::OFF_RING + s * T::TILE + c * T::CHUNK, (e & 1) ? &tm_v : &tm_k, c * 64, g,
+                                  (e >> 1) * kMaskTileKeys, b, bar_full(s));
+                copies = e + 1;
+            }
+            if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
+        }
+    } else if (warp == 9) {
+        if (lane == 0) {
+            auto wait = [&](uint32_t bar, uint32_t parity) {
+                const bool r = mbar_wait(bar, parity, s_abort, a.wait_cycles);
+                tc_fence_after();
+                return r;
+            };
+            auto slot = [&](int e) { return sbase + P::OFF_RING + (e % SL) * T::TILE; };
+            auto landed = [&](int e) { return wait(bar_full(e % SL), (e / SL) & 1); };
+            auto issue_s = [&](int i) {                            // S = Q K^T
+                if (!landed(2 * i)) return false;
+                mma_kmajor<DH>(tmem + kTmS + 128 * (i & 1), sbase + P::OFF_Q, slot(2 * i));
+                tc_commit(bar_s(i));
+                return true;
+            };
+            auto issue_dp = [&](int i) {                           // dP = do V'^T
+                if (!landed(2 * i + 1)) return false;
+                mma_kmajor<DH>(tmem + kTmP, sbase + P::OFF_D, slot(2 * i + 1));
+                tc_commit(bar_dp);
+                tc_commit(bar_empty((2 * i + 1) % SL));
+                v_released = i + 1;
+                return true;
+            };
+            bool ok = wait(bar_qd, 0) && issue_s(0) && issue_dp(0) && (n < 2 || issue_s(1));
+            for (int i = 0; ok && i < n; ++i) {
+                if (i + 1 < n) ok = wait(bar_read, i & 1) && issue_dp(i + 1);      // the columns of dP(i) have been read
+                if (!ok || !(ok = wait(bar_ds, i & 1))) break;
+                mma_tmem_rows<DH>(tmem + kTmQ, tmem + kTmS + 128 * (i & 1), slot(2 * i), i > 0);      // dQ += dS K
+                tc_commit(bar_empty((2 * i) % SL));
+                k_released = i + 1;
+                if (i + 2 < n) ok = issue_s(i + 2);
+            }
+            if (ok) tc_commit(bar_done);
+            else atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
+        }
+    } else if (warp < 8) {
+        const int half = warp >> 2, quad = warp & 3;
+        const int m = quad * 32 + lane, r = r0 + m / G, h = g * G + m % G;
+        const bool live = r < a.rows;
+        const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
+        const uint2* __restrict__ mrow =
+            reinterpret_cast<const uint2*>(a.mask + (int64_t)b * a.key_tiles * a.row_pitch + (live ? r : 0)) + half;
+        float l2 = 0.f, dl = 0.f;
+        if (live) {
+            const size_t at = ((size_t)b * a.Lq + a.q0 + r) * a.n_h + h;
+            l2 = a.lse[at] * kLog2e;
+            dl = a.delta[at];
+        }
+        uint2 mk_next = live ? __ldg(mrow) : make_uint2(0u, 0u);
+        bool ok = true;
+        for (int i = 0; i < n; ++i) {
+            const uint2 mk = mk_next;
+            if (live && i + 1 < n) mk_next = __ldg(mrow + (int64_t)(i + 1) * a.row_pitch * 2);
+            const uint32_t ts = lane_base + kTmS + 128 * (i & 1) + 64 * half, tp = lane_base + kTmP + 64 * half;
+            if (!mbar_wait(bar_s(i), (i >> 1) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
+            tc_fence_after();
+            uint32_t v[2][32], w[2][32];
+            tc_ld32(ts, v[0]);
+            tc_ld32(ts + 32, v[1]);
+            tc_wait_ld32(v[0]);
+            tc_tie32(v[1]);
+            const uint32_t mw[2] = {mk.x, mk.y};
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float x = ex2_approx(fmaf(__uint_as_float(v[c][j]), a.scale_log2, -l2));
+                    v[c][j] = __float_as_uint((mw[c] >> j) & 1u ? x : 0.f);
+                }
+            if (!mbar_wait(bar_dp, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
+            tc_fence_after();
+            tc_ld32(tp, w[0]);
+            tc_ld32(tp + 32, w[1]);
+            tc_wait_ld32(w[0]);
+            tc_tie32(w[1]);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_read);
+            uint32_t pk[32];
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int j = 0; j < 32; j += 2)
+                    pk[16 * c + j / 2] = pack_bf16(__uint_as_float(v[c][j]) * (__uint_as_float(w[c][j]) - dl),
+                                                   __uint_as_float(v[c][j + 1]) * (__uint_as_float(w[c][j + 1]) - dl));
+            tc_st32(ts, pk);
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_ds);
+        }
+        if (ok && !mbar_wait(bar_done, 0, s_abort, a.wait_cycles)) ok = false;
+        if (!ok) {
+            if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
+        } else {
+            tc_fence_after();
+            __nv_bfloat16* dst = a.dQ + (((size_t)b * a.Lq + a.q0 + (live ? r : 0)) * a.n_h + h) * DH + half * (DH / 2);
+#pragma unroll
+            for (int c = 0; c < DH / 64; ++c) {
+                uint32_t o[32];
+                tc_ld32(lane_base + kTmQ + half * (DH / 2) + 32 * c, o);
+                tc_wait_ld32(o);
+                if (!live) continue;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t x[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        x[e] = pack_bf16(__uint_as_float(o[8 * q + 2 * e]) * a.scale, __uint_as_float(o[8 * q + 2 * e + 1]) * a.scale);
+                    *reinterpret_cast<uint4*>(dst + 32 * c + 8 * q) = make_uint4(x[0], x[1], x[2], x[3]);
+                }
+            }
+        }
+    }
+    tile_end(warp, lane, tmem, s_abort, bar_drain,
+             [&] {
+                 if (qd_issued) mbar_drain(bar_qd, 0);
+                 for (int e = max(0, copies - SL); e < copies; ++e) mbar_drain(bar_full(e % SL), (e / SL) & 1);
+             },
+             [&] {
+                 // (commits arrive in order: the last one of either kind covers the others)
+                 if (k_released) mbar_drain(bar_empty((2 * (k_released - 1)) % SL), ((2 * (k_released - 1)) / SL) & 1);
+                 if (v_released) mbar_drain(bar_empty((2 * v_released - 1) % SL), ((2 * v_released - 1) / SL) & 1);
+             });
+}
+
+// ---- target of the indexer's loss: pbar --------------------------------------------------------------------------
+template <int DH>
+struct TargetSmem {
+    using T = TileBytes<DH>;
+    static constexpr int STAGES = 2;                               // (Q tile, two K tiles) of a KV head
+    static constexpr int STAGE = 3 * T::TILE;
+    static constexpr int OFF_BAR = STAGES * STAGE;
+    static constexpr int N_BARS = 2 * STAGES + 4 + 4 + 1;
+    static constexpr int OFF_TMEM = OFF_BAR + N_BARS * 8;
+    static constexpr int OFF_ABORT = OFF_TMEM + 8;
+    static constexpr int OFF_RANK = OFF_ABORT + 8;                 // first position of the key run in every query's set
+    static constexpr int ALLOC = OFF_RANK + 128 * 4 + 1024;
+};
+
+template <int DH, int G>
+__global__ void __launch_bounds__(kBwdThreads, 1)
+gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const MaskedBwdArgs a) {
+    using P = TargetSmem<DH>;
+    using T = TileBytes<DH>;
+    constexpr int QT = 128 / G;
+    if (*a.general) return;
+    const int blk = a.row_blocks - 1 - (int)blockIdx.y, b = blockIdx.z;
+    const int r0 = blk * QT, off = a.Lk - a.Lq;
+    const int ntiles = min((off + a.q0 + min(r0 + QT, a.rows) + kMaskTileKeys - 1) / kMaskTileKeys, a.key_tiles);
+    const int pair0 = blockIdx.x * a.pairs_per_cta, pair1 = min(pair0 + a.pairs_per_cta, (ntiles + 1) / 2);
+    if (pair0 >= pair1) return;
+    const int n = (pair1 - pair0) * a.n_kv;                        // steps: (key pair, KV head)
+    GSA_TILE_PROLOGUE(P)
+    auto bar_full = [&](int s) { return bar0 + 8u * s; };
+    auto bar_empty = [&](int s) { return bar0 + 8u * (2 + s); };
+    auto bar_s = [&](int s, int w) { return bar0 + 8u * (4 + 2 * s + w); };
+    auto bar_sfree = [&](int s, int w) { return bar0 + 8u * (8 + 2 * s + w); };
+    const uint32_t bar_drain = bar0 + 8u * 12;
+    int* const s_rank = reinterpret_cast<int*>(smem + P::OFF_RANK);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1);
+            for (int w = 0; w < 2; ++w) { mbar_init(bar_s(s, w), 1); mbar_init(bar_sfree(s, w), 4); }
+        }
+        mbar_init(bar_drain, 1);
+    }
+    if (threadIdx.x >= 256) {
+        // where the CTA's run of keys starts in every query's set
+        const int q = threadIdx.x - 256, r = r0 + q;
+        if (q < QT) {
+            int lo = 0;
+            if (r < a.rows) {
+                const int64_t irow = a.il.row(b, a.q0 + r);
+                const int32_t* __restrict__ set = a.idx + irow * a.k_max;
+                int hi = clamp_budget(a.kt[irow], a.k_max);
+                const int first = pair0 * 2 * kMaskTileKeys;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (set[mid] < first) lo = mid + 1; else hi = mid;
+                }
+            }
+            s_rank[q] = lo;
+        }
+    }
+    const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
+    int copies = 0, released = 0;
+
+    if (warp < 8) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        const int w = warp >> 2, quad = warp & 3;                  // this warpgroup's key tile of the pair
+        const int m = quad * 32 + lane, q = m / G, r = r0 + q;
+        const bool live = r < a.rows;
+        const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
+        const float* __restrict__ lse = a.lse + ((size_t)b * a.Lq + a.q0 + (live ? r : 0)) * a.n_h + m % G;
+        float* __restrict__ dst = a.pbar + a.il.row(b, a.q0 + (live ? r : 0)) * a.k_max;
+        const float inv_heads = 1.0f / (float)a.n_h;
+        const uint64_t scale2 = pack_f32x2(a.scale_log2, a.scale_log2);
+        int rank = s_rank[q];
+        bool ok = true;
+        int it = 0;
+        for (int pair = pair0; ok && pair < pair1; ++pair) {
+            uint4 mk0 = make_uint4(0u, 0u, 0u, 0u), mk1 = mk0;     // masks of both tiles: the ranks run through both
+            if (live) {
+                mk0 = a.mask[((int64_t)b * a.key_tiles + 2 * pair) * a.row_pitch + r];
+                if (2 * pair + 1 < ntiles) mk1 = a.mask[((int64_t)b * a.key_tiles + 2 * pair + 1) * a.row_pitch + r];
+            }
+            uint64_t acc[64];
+#pragma unroll
+            for (int c = 0; c < 64; ++c) acc[c] = 0ull;
+            float l_next = live ? lse[0] : 0.f;
+            for (int g = 0; g < a.n_kv; ++g, ++it) {
+                const int s = it & 1;
+                const float neg = -l_next * kLog2e;
+                if (live && g + 1 < a.n_kv) l_next = lse[(g + 1) * G];
+                const uint64_t neg2 = pack_f32x2(neg, neg);
+                if (!mbar_wait(bar_s(s, w), (it >> 1) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t ts = lane_base + 256 * s + 128 * w;
+                uint32_t v[2][16];                                 // the next 16 columns arrive behind the current ones' arithmetic
+                tc_ld16(ts, v[0]);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    tc_wait_ld16(v[c & 1]);
+                    if (c < 7) tc_ld16(ts + 16 * (c + 1), v[(c + 1) & 1]);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        float x0, x1;
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[c & 1][2 * j]), __uint_as_float(v[c & 1][2 * j + 1])), scale2, neg2), x0, x1);
+                        acc[8 * c + j] = add_f32x2(acc[8 * c + j], pack_f32x2(ex2_approx(x0), ex2_approx(x1)));
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_sfree(s, w));
+            }
+            if (!ok) break;
+            // sum over the heads of the group (neighbouring lanes), then to the set's positions; the group's lanes share the columns
+            const uint4 mk = w ? mk1 : mk0;
+            const int n0 = __popc(mk0.x) + __popc(mk0.y) + __popc(mk0.z) + __popc(mk0.w);
+            const uint32_t words[4] = {mk.x, mk.y, mk.z, mk.w};
+            int at = rank + (w ? n0 : 0);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    float x0, x1;
+                    unpack_f32x2(acc[16 * c + j], x0, x1);
+#pragma unroll
+                    for (int e = 1; e < G; e <<= 1) {
+                        x0 += __shfl_xor_sync(0xFFFFFFFFu, x0, e);
+                        x1 += __shfl_xor_sync(0xFFFFFFFFu, x1, e);
+                    }
+                    const bool mine = (16 * c + j) % G == m % G;
+                    const int p0 = at + __popc(words[c] & ((1u << (2 * j)) - 1u)), p1 = p0 + ((words[c] >> (2 * j)) & 1u);
+                    if (mine && (words[c] >> (2 * j)) & 1u) dst[p0] = x0 * inv_heads;
+                    if (mine && (words[c] >> (2 * j + 1)) & 1u) dst[p1] = x1 * inv_heads;
+                }
+                at += __popc(words[c]);
+            }
+            rank += n0 + __popc(mk1.x) + __popc(mk1.y) + __popc(mk1.z) + __popc(mk1.w);
+        }
+        if (!ok && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        if (warp == 8) {
+            if (lane == 0) {
+                bool ok = true;
+                for (int it = 0; ok && it < n; ++it) {
+                    const int s = it & 1, g = it % a.n_kv, pair = pair0 + it / a.n_kv;
+                    if (!mbar_wait(bar_empty(s), ((it >> 1) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                    mbar_expect_tx(bar_full(s), P::STAGE);
+                    const uint32_t dst = sbase + s * P::STAGE;
+                    for (int c = 0; c < T::CHUNKS; ++c) {
+                        tma_load_tile(dst + c * T::CHUNK, &tm_q, c * 64, g * G, r0, b, bar_full(s));
+                        for (int w = 0; w < 2; ++w)
+                            tma_load_tile(dst + (1 + w) * T::TILE + c * T::CHUNK, &tm_k, c * 64, g, (2 * pair + w) * kMaskTileKeys, b,
+                                          bar_full(s));
+                    }
+                    copies = it + 1;
+                }
+                if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
+            }
+        } else if (warp == 9) {
+            if (lane == 0) {
+                bool ok = true;
+                for (int it = 0; ok && it < n; ++it) {
+                    const int s = it & 1;
+                    if (!mbar_wait(bar_full(s), (it >> 1) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                    for (int w = 0; ok && w < 2; ++w) {
+                        if (!mbar_wait(bar_sfree(s, w), ((it >> 1) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                        tc_fence_after();
+                        mma_kmajor<DH>(tmem + 256 * s + 128 * w, sbase + s * P::STAGE, sbase + s * P::STAGE + (1 + w) * T::TILE);
+                        tc_commit(bar_s(s, w));
+                    }
+                    if (!ok) break;
+                    tc_commit(bar_empty(s));
+                    released = it + 1;
+                }
+                if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
+            }
+        }
+    }
+    tile_end(warp, lane, tmem, s_abort, bar_drain,
+             [&] { for (int i = max(0, copies - 2); i < copies; ++i) mbar_drain(bar_full(i & 1), (i >> 1) & 1); },
+             [&] { for (int i = max(0, released - 2); i < released; ++i) mbar_drain(bar_empty(i & 1), (i >> 1) & 1); });
+}
+
+// ---- what the tiles cannot take (see gsa_general_attn_kernel) -------------------------------------------------------
+// Only when `general` is raised: fp32 sums of dK, dV' by atomics, one warp per (row, KV head), the set entry by entry.
+__global__ void __launch_bounds__(256) gsa_general_bwd_zero_kernel(const int32_t* __restrict__ general, float4* x, int64_t n) {
+    if (*general == 0) return;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+template <int DH, int G>
+__global__ void __launch_bounds__(256)
+gsa_general_bwd_rows_kernel(const MaskedBwdArgs a, const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K,
+                            const __nv_bfloat16* __restrict__ Vg, const __nv_bfloat16* __restrict__ dOs,
+                            float* __restrict__ dK32, float* __restrict__ dV32) {
+    if (*a.general == 0) return;
+    constexpr int NV = DH / 32;
+    const int lane = threadIdx.x & 31;
+    auto load = [&](const __nv_bfloat16* p, float (&f)[NV]) {
+#pragma unroll
+        for (int c = 0; c < NV; ++c) f[c] = __bfloat162float(p[lane * NV + c]);
+    };
+    auto dot = [&](const float (&x)[NV], const float (&y)[NV]) {
+        float z = 0.f;
+#pragma unroll
+        for (int c = 0; c < NV; ++c) z = fmaf(x[c], y[c], z);
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, d);
+        return z;
+    };
+    const int64_t items = (int64_t)a.B * a.rows * a.n_kv;
+    for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < items; item += (int64_t)gridDim.x * 8) {
+        const int g = (int)(item % a.n_kv), b = (int)(item / a.n_kv / a.rows), t = a.q0 + (int)(item / a.n_kv % a.rows);
+        const int64_t irow = a.il.row(b, t);
+        const int k = checked_budget(a.kt[irow], a.k_max, a.dev_status);
+        float q[G][NV], d[G][NV], dq[G][NV], l2[G], dl[G];
+#pragma unroll
+        for (int e = 0; e < G; ++e) {
+            const size_t h = ((size_t)b * a.Lq + t) * a.n_h + g * G + e;
+            load(Q + h * DH, q[e]);
+            load(dOs + h * DH, d[e]);
+            l2[e] = a.lse[h] * kLog2e; dl[e] = a.delta[h];
+#pragma unroll
+            for (int c = 0; c < NV; ++c) dq[e][c] = 0.f;
+        }
+        for (int j = 0; j < k; ++j) {
+            const int s = checked_pos(a.idx[irow * a.k_max + j], a.Lk, a.dev_status);
+            const size_t at = (((size_t)b * a.Lk + s) * a.n_kv + g) * DH;
+            float kr[NV], vr[NV], dk[NV], dv[NV], psum = 0.f;
+            load(K + at, kr);
+            load(Vg + at, vr);
+#pragma unroll
+            for (int c = 0; c < NV; ++c) dk[c] = dv[c] = 0.f;
+#pragma unroll
+            for (int e = 0; e < G; ++e) {
+                const float pz = exp2f(fmaf(dot(q[e], kr), a.scale_log2, -l2[e]));
+                const float ds = pz * (dot(d[e], vr) - dl[e]);
+                psum += pz;
+#pragma unroll
+                for (int c = 0; c < NV; ++c) {
+                    dq[e][c] = fmaf(ds, kr[c], dq[e][c]);
+                    dk[c] = fmaf(ds, q[e][c], dk[c]);
+                    dv[c] = fmaf(pz, d[e][c], dv[c]);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < NV; ++c) {
+                atomicAdd(dK32 + at + lane * NV + c, dk[c]);
+                atomicAdd(dV32 + at + lane * NV + c, dv[c]);
+            }
+            if (a.pbar && lane == 0) atomicAdd(a.pbar + irow * a.k_max + j, psum / (float)a.n_h);      // (zeroed by the caller)
+        }
+#pragma unroll
+        for (int e = 0; e < G; ++e)
+#pragma unroll
+            for (int c = 0; c < NV; ++c)
+                a.dQ[(((size_t)b * a.Lq + t) * a.n_h + g * G + e) * DH + lane * NV + c] = __float2bfloat16_rn(dq[e][c] * a.scale);
+    }
+}
+
+__global__ void __launch_bounds__(256) gsa_general_bwd_finish_kernel(const MaskedBwdArgs a, const float* __restrict__ dK32,
+                                                                     const float* __restrict__ dV32, int64_t n) {
+    if (*a.general == 0) return;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const float sg = 1.0f / (1.0f + __expf(-__bfloat162float(a.g2[i])));
+        a.dK[i] = __float2bfloat16_rn(dK32[i] * a.scale);
+        a.dV[i] = __float2bfloat16_rn(dV32[i] * sg);
+        a.dg2[i] = __float2bfloat16_rn(dV32[i] * __bfloat162float(a.V[i]) * sg * (1.0f - sg));
+    }
+}
+
+template <int DH, int G>
+cudaError_t launch_bwd_t(const MaskedBwdArgs& a, const gsa_params_t& p, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                         const __nv_bfloat16* Vg, const __nv_bfloat16* dOs, float* dKV32, cudaStream_t st) {
+    CUtensorMap tq, td, tk, tv;
+    if (!make_heads_tmap(&tq, Q + (size_t)a.q0 * p.n_h * DH, p.B, p.Lq, a.rows, p.n_h, DH, 128 / G, G)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&td, dOs + (size_t)a.q0 * p.n_h * DH, p.B, p.Lq, a.rows, p.n_h, DH, 128 / G, G)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&tk, K, p.B, p.Lk, p.Lk, p.n_kv, DH, kMaskTileKeys, 1)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&tv, Vg, p.B, p.Lk, p.Lk, p.n_kv, DH, kMaskTileKeys, 1)) return cudaErrorUnknown;
+    auto set_smem = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+    constexpr int kSmemK = KeysSmem<DH, G>::ALLOC, kSmemR = RowsSmem<DH>::ALLOC, kSmemT = TargetSmem<DH>::ALLOC;
+    static_assert(kSmemK <= 232448 && kSmemR <= 232448 && kSmemT <= 232448, "shared memory of one CTA");
+    cudaError_t e = set_smem(gsa_masked_bwd_keys_kernel<DH, G>, kSmemK);
+    if (e == cudaSuccess) e = set_smem(gsa_masked_bwd_rows_kernel<DH, G>, kSmemR);
+    if (e == cudaSuccess) e = set_smem(gsa_masked_target_kernel<DH, G>, kSmemT);
+    if (e != cudaSuccess) return e;
+    gsa_masked_bwd_keys_kernel<DH, G><<<(unsigned)(a.key_tiles * p.n_kv * p.B), kBwdThreads, kSmemK, st>>>(tq, td, tk, tv, a);
+    gsa_masked_bwd_rows_kernel<DH, G><<<(unsigned)(a.row_blocks * p.n_kv * p.B), kBwdThreads, kSmemR, st>>>(tq, td, tk, tv, a);
+    g_launches += 2;
+    if (a.pbar) {
+        const int pairs = (a.key_tiles + 1) / 2;
+        const dim3 grid((unsigned)((pairs + a.pairs_per_cta - 1) / a.pairs_per_cta), (unsigned)a.row_blocks, (unsigned)p.B);
+        gsa_masked_target_kernel<DH, G><<<grid, kBwdThreads, kSmemT, st>>>(tq, tk, a);
+        ++g_launches;
+    }
+    const int64_t n = (int64_t)p.B * p.Lk * p.n_kv * DH;
+    const int ctas = sm_count() * 4;
+    gsa_general_bwd_zero_kernel<<<ctas, 256, 0, st>>>(a.general, reinterpret_cast<float4*>(dKV32), n / 2);
+    gsa_general_bwd_rows_kernel<DH, G><<<ctas, 256, 0, st>>>(a, Q, K, Vg, dOs, dKV32, dKV32 + n);
+    gsa_general_bwd_finish_kernel<<<ctas, 256, 0, st>>>(a, dKV32, dKV32 + n, n);
+    g_launches += 3;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t masked_bwd_bytes(const gsa_params_t& p, const RowRange& rr) {
+    const size_t masks = mask_plan(p, rr.q_begin, rr.R).bytes(p.B);
+    const size_t sums = (size_t)p.B * p.Lk * p.n_kv * p.d_h * 8;
+    return ((masks > sums ? masks : sums) + 255) / 256 * 256;
+}
+
+// A gathered pair of the backward costs 1.4 ns at 16 heads of 128 on 8 KV heads (12 KB of rows; L = 32K: 92 ms with the loss
+// target), a visible pair of the tiles 31 ps (16.5 ms): the line is drawn at a mean share of 1 / 50, where both take about as
+// long; as in the forward (masked_rows_end) it moves with the heads per KV head, which a gathered row serves together.
+bool masked_bwd_preferred(const gsa_params_t& p, const RowRange& rr) {
+    const int G = p.n_h / p.n_kv;
+    const int64_t block = masked_block_rows(p);
+    if (((int64_t)rr.R + block - 1) / block * p.n_kv * rr.nb * 3 < 2 * sm_count()) return false;
+    if (p.k_mode == 3) return true;
+    const int64_t k = p.k_base < p.k_min ? p.k_min : (p.k_base > p.k_max ? p.k_max : p.k_base);
+    const int64_t mean_visible = p.Lk - p.Lq + rr.q_begin + rr.R / 2;
+    return mean_visible * G < k * (p.d_h == 128 ? 100 : 80);
+}
+
+cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                              const __nv_bfloat16* V, const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const __nv_bfloat16* g2,
+                              const __nv_bfloat16* out, const __nv_bfloat16* dout, const int32_t* idx, const int32_t* kt,
+                              IdxLayout il, __nv_bfloat16* dQ, __nv_bfloat16* dK, __nv_bfloat16* dV, __nv_bfloat16* dg1,
+                              __nv_bfloat16* dg2, __nv_bfloat16* dOs, float* lse_ws, float* delta, float* pbar,
+                              const float* lse_in, void* ws, int32_t* dev_status, cudaStream_t st) {
+    int32_t* general = dev_status + kStatusGeneralWord;
+    cudaError_t e = launch_bwd_prep(p, rr, g1, out, dout, dOs, dg1, delta, general, st);
+    // (outside the sets the tiles multiply by zero: everything they read has to be finite.  V' and dOs are watched where they
+    // are written; rows of dOs past the range read as zero)
+    if (e == cudaSuccess) e = launch_check_finite(Q, (int64_t)p.B * p.Lq * p.n_h * p.d_h, general, st);
+    if (e == cudaSuccess) e = launch_check_finite(K, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, general, st);
+    const MaskPlan mp = mask_plan(p, rr.q_begin, rr.R);
+    uint4* mask = (uint4*)ws;
+    if (e == cudaSuccess) e = launch_build_masks(p, mp, masked_block_rows(p), idx, kt, il, mask, general, st);
+    if (e == cudaSuccess && !lse_in) {
+        // the statistics were not saved: the forward's tiles once more (their output goes where dQ is written afterwards)
+        e = launch_masked_attn_fwd(p, mp, mask, Q, K, Vg, g1, dQ, lse_ws, idx, kt, il, dev_status, st);
+        lse_in = lse_ws;
+    }
+    if (e != cudaSuccess) return e;
+    MaskedBwdArgs a;
+    a.mask = mask; a.lse = lse_in; a.delta = delta; a.V = V; a.g2 = g2; a.idx = idx; a.kt = kt; a.il = il;
+    a.dQ = dQ; a.dK = dK; a.dV = dV; a.dg2 = dg2; a.pbar = pbar; a.dev_status = dev_status; a.general = general;
+    a.q0 = mp.q0; a.rows = mp.rows; a.row_pitch = mp.row_pitch; a.key_tiles = mp.key_tiles;
+    a.B = p.B; a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv; a.k_max = p.k_max;
+    const int G = p.n_h / p.n_kv;
+    a.row_blocks = (mp.rows + 128 / G - 1) / (128 / G);
+    // target kernel: runs of key pairs long enough to pay for a CTA's start, short enough for four CTAs per SM (visible pairs
+    // only: half of them in a square range)
+    const int64_t pairs = (int64_t)((a.key_tiles + 1) / 2) * a.row_blocks * p.B;
+    a.pairs_per_cta = (int)(pairs / 2 / (4 * sm_count()));
+    a.pairs_per_cta = a.pairs_per_cta < 1 ? 1 : (a.pairs_per_cta > 8 ? 8 : a.pairs_per_cta);
+    a.scale = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
+    a.scale_log2 = a.scale * kLog2e;
+    a.wait_cycles = wait_limit_cycles();
+#define GSA_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_bwd_t<DH_, G_>(a, p, Q, K, Vg, dOs, (float*)ws, st)
+    GSA_CASE(128, 1); GSA_CASE(128, 2); GSA_CASE(128, 4); GSA_CASE(128, 8);
+    GSA_CASE(64, 1); GSA_CASE(64, 2); GSA_CASE(64, 4); GSA_CASE(64, 8);
+#undef GSA_CASE
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace gsa

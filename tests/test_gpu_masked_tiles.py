@@ -60,7 +60,7 @@ def _check(cfg, x, out, lse, idx, kt, rows):
     (1, 1664, 1664, 16, 8, 128),      # whole tiles
     (2, 1025, 1793, 16, 8, 128),      # one row and one key past a tile
     (1, 3327, 3327, 8, 8, 128),       # one row and one key short of a tile, no head sharing
-    (1, 1665, 1801, 16, 2, 128),      # eight heads per KV head
+    (1, 2401, 2500, 16, 2, 128),      # eight heads per KV head
     (2, 865, 1153, 32, 8, 64),        # d_h = 64, four heads
     (1, 707, 900, 64, 8, 64),
     (5, 2561, 2561, 2, 2, 64),
@@ -111,3 +111,81 @@ def test_inputs_that_a_mask_cannot_stand_for(what):
     rows = _rows(cfg)
     keep = rows[~hit[:, rows].any(0).numpy()]
     _check(cfg, x, out, lse, idx, kt, np.unique(np.concatenate([keep, [500]])) if not hit[:, 500].any() else keep)
+
+
+# ---- backward ------------------------------------------------------------------------------------------------------
+def _run_bwd(cfg, d, idx, kt, q0, q1, saved_lse):
+    p = gsa.make_params(cfg, q_begin=q0, q_end=q1)
+    nan = float("nan")
+    out, lse = torch.full_like(d["Q"], nan), torch.full((cfg.B, cfg.Lq, cfg.n_h), nan, dtype=torch.float32, device="cuda")
+    ws = torch.empty(max(gsa.gsa_attn_workspace_bytes(p, True), gsa.gsa_attn_bwd_workspace_bytes(p)), dtype=torch.uint8, device="cuda").fill_(0xFF)
+    i, k = idx[:, q0:q1].contiguous().cuda(), kt[:, q0:q1].contiguous().cuda()
+    gsa.gsa_sparse_gated_attn_fwd_lse(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], i, k, out, lse, ws)
+    got = {n: torch.full_like(d["Q" if n in ("dQ", "dg1") else "K"], nan) for n in ("dQ", "dg1", "dK", "dV", "dg2")}
+    got["pbar"] = torch.full((cfg.B, q1 - q0, cfg.k_max), nan, dtype=torch.float32, device="cuda")
+    ws.fill_(0xFF)
+    n0 = gsa.gsa_launch_count()
+    gsa.gsa_sparse_gated_attn_bwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], i, k, out, d["dout"], got["dQ"], got["dK"], got["dV"],
+                                  got["dg1"], got["dg2"], ws, pbar=got["pbar"], lse=lse if saved_lse else None)
+    # gate, preparation, two scans, masks, keys, rows, target, three of the plain path (and the statistics' two)
+    assert gsa.gsa_launch_count() - n0 == (11 if saved_lse else 13)
+    return got, gsa.gsa_device_status(ws)
+
+
+@pytest.mark.parametrize("B,Lq,Lk,n_h,n_kv,d_h,q0,q1,saved_lse", [
+    (1, 1664, 1664, 16, 8, 128, 0, 1664, True),       # whole tiles
+    (2, 901, 1153, 16, 8, 128, 5, 898, False),        # a row range off the tiles, one key past a tile, statistics recomputed
+    (1, 3327, 3327, 8, 8, 128, 0, 3327, True),        # no head sharing, one short of a tile
+    (1, 1601, 1700, 16, 2, 128, 0, 1601, True),         # eight heads per KV head
+    (2, 865, 1025, 32, 8, 64, 0, 865, True),          # d_h = 64, four heads
+    (1, 451, 577, 64, 8, 64, 0, 451, False),
+])
+def test_masked_backward_matches_the_oracle(B, Lq, Lk, n_h, n_kv, d_h, q0, q1, saved_lse):
+    from test_gpu_backward import _compare
+    cfg = CONFIGS["tiny"].with_(name="masked_bwd", B=B, Lq=Lq, Lk=Lk, n_h=n_h, n_kv=n_kv, d_h=d_h, k_base=150, k_min=1, k_max=209,
+                                seed=230 + Lq)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 231, empty=[(0, q0 + 3), (B - 1, q1 - 1)])
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(232)) * 0.25).to(torch.bfloat16)
+    d = U.to_dev({**x, "dout": dout})
+    got, status = _run_bwd(cfg, d, idx, kt, q0, q1, saved_lse)
+    assert status == 0
+    _compare(cfg, x, got, idx[:, q0:q1].contiguous(), kt[:, q0:q1].contiguous(), dout, q0, q1)
+
+
+@pytest.mark.parametrize("what", ["unsorted", "duplicate", "inf_value", "nan_dout"])
+def test_masked_backward_leaves_other_inputs_to_the_plain_path(what):
+    from test_gpu_backward import _compare
+    cfg = CONFIGS["tiny"].with_(name="general_bwd", B=2, Lq=900, Lk=1000, n_h=16, n_kv=8, d_h=128, k_base=150, k_min=1, k_max=209, seed=240)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 241)
+    kt[1, 500] = 7
+    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, 700, 800], dtype=torch.int32)
+    idx[1, 500, 7:] = -1
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(242)) * 0.25).to(torch.bfloat16)
+    if what == "unsorted":
+        idx[1, 500, :7] = idx[1, 500, :7].flip(0)
+    elif what == "duplicate":
+        idx[1, 500, 4] = 400
+    elif what == "inf_value":
+        x["V"][0, 700, 3, 5] = float("inf")
+    else:
+        dout[0, 600, 3, 5] = float("nan")
+    d = U.to_dev({**x, "dout": dout})
+    got, status = _run_bwd(cfg, d, idx, kt, 0, cfg.Lq, True)
+    assert status == 0
+    if what in ("unsorted", "duplicate"):
+        _compare(cfg, x, got, idx, kt, dout, 0, cfg.Lq)
+        return
+    # the value reaches the rows that select its key (the keys that its row selects) and no others
+    bad_rows = ~torch.isfinite(got["dQ"].float().cpu()).all(-1).all(-1)
+    bad_keys = ~torch.isfinite(got["dV"].float().cpu()).all(-1).all(-1)
+    rows = ((idx == 700) & (torch.arange(cfg.k_max) < kt[..., None])).any(-1)
+    rows[1] = False
+    if what == "nan_dout":
+        rows[:] = False
+        rows[0, 600] = True
+        keys = torch.zeros(cfg.B, cfg.Lk, dtype=torch.bool)
+        keys[0, idx[0, 600, :int(kt[0, 600])].long()] = True
+        assert bad_keys.any() and not (bad_keys & ~keys).any()
+    assert bad_rows.any() and not (bad_rows & ~rows).any()
