@@ -290,46 +290,16 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             if (live && i + 1 < ntiles) mk_next = __ldg(mrow + (int64_t)(i + 1) * a.row_pitch);
             if (!mbar_wait(bar_s(s), i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
             tc_fence_after();
-            uint32_t v[4][32];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) tc_ld32(ts + 32 * c, v[c]);
-            tc_wait_ld32(v[0]);
-            tc_tie32(v[1]); tc_tie32(v[2]); tc_tie32(v[3]);
+            // The reference of the tiles before nearly always still serves, so the numerators are taken against it at once,
+            // 32 columns at a time with the next 32 on their way; only if a selected score then turns out to exceed it
+            // by more than 2^8 (a row's first tiles) is the tile's work done again from the scores, still in registers.
             const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
+            uint32_t v[4][32];
             float mx[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                mx[c] = -INFINITY;
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float x = (mw[c] >> j) & 1u ? __uint_as_float(v[c][j]) : -INFINITY;
-                    v[c][j] = __float_as_uint(x);
-                    mx[c] = fmaxf(mx[c], x);
-                }
-            }
-            const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * a.scale_log2;
-            if (__any_sync(0xFFFFFFFFu, top > m_ref + 8.0f)) {
-                const float m_new = fmaxf(m_ref, top);
-                const float alpha = m_ref == -INFINITY ? 0.f : ex2_approx(m_ref - m_new);
-                m_ref = m_new;
-                const uint64_t al2 = pack_f32x2(alpha, alpha);
-                l2[0] = mul_f32x2(l2[0], al2); l2[1] = mul_f32x2(l2[1], al2);
-                if (i > 0) {                                       // every product into O so far has completed (bar_s)
-                    uint32_t o[32];
-#pragma unroll
-                    for (int c = 0; c < DH / 32; ++c) {
-                        tc_ld32(to + 32 * c, o);
-                        tc_wait_ld32(o);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
-                        tc_st32(to + 32 * c, o);
-                    }
-                }
-            }
-            const float neg = m_ref == -INFINITY ? 0.f : -m_ref;
-            const uint64_t neg2 = pack_f32x2(neg, neg);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            uint64_t sum[2] = {0ull, 0ull};
+            const float neg0 = m_ref == -INFINITY ? 0.f : -m_ref;
+            uint64_t neg2 = pack_f32x2(neg0, neg0);
+            auto numerators = [&](int c) {
                 uint32_t pk[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
@@ -337,11 +307,52 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     float x0, x1;
                     unpack_f32x2(x, x0, x1);
                     x0 = ex2_approx(x0); x1 = ex2_approx(x1);
-                    l2[j & 1] = add_f32x2(l2[j & 1], pack_f32x2(x0, x1));
+                    sum[j & 1] = add_f32x2(sum[j & 1], pack_f32x2(x0, x1));
                     pk[j] = pack_bf16(x0, x1);
                 }
                 tc_st16(ts + 16 * c, pk);
+            };
+            tc_ld32(ts, v[0]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                tc_wait_ld32(v[c]);
+                if (c < 3) tc_ld32(ts + 32 * (c + 1), v[c + 1]);
+                mx[c] = -INFINITY;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float x = (mw[c] >> j) & 1u ? __uint_as_float(v[c][j]) : -INFINITY;
+                    v[c][j] = __float_as_uint(x);
+                    mx[c] = fmaxf(mx[c], x);
+                }
+                // (the numerators of these columns go over columns 16 c .. 16 c + 15, which have been read)
+                numerators(c);
             }
+            const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * a.scale_log2;
+            if (__any_sync(0xFFFFFFFFu, top > m_ref + 8.0f)) {
+                const float m_new = fmaxf(m_ref, top);
+                const float alpha = m_ref == -INFINITY ? 0.f : ex2_approx(m_ref - m_new);
+                m_ref = m_new;
+                const float neg1 = m_ref == -INFINITY ? 0.f : -m_ref;
+                neg2 = pack_f32x2(neg1, neg1);
+                const uint64_t al2 = pack_f32x2(alpha, alpha);
+                l2[0] = mul_f32x2(l2[0], al2); l2[1] = mul_f32x2(l2[1], al2);
+                sum[0] = sum[1] = 0ull;
+                tc_wait_st();                                      // (the columns are written a second time)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) numerators(c);
+                if (i > 0) {                                       // every product into O so far has completed (bar_s)
+                    uint32_t o[16];
+#pragma unroll
+                    for (int c = 0; c < DH / 16; ++c) {
+                        tc_ld16(to + 16 * c, o);
+                        tc_wait_ld16(o);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
+                        tc_st16(to + 16 * c, o);
+                    }
+                }
+            }
+            l2[0] = add_f32x2(l2[0], sum[0]); l2[1] = add_f32x2(l2[1], sum[1]);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
@@ -405,60 +416,54 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
             }
         } else if (warp == 9) {
-            // ================= MMA issuer ===============================================================
-            if (lane == 0) {
-                bool ok = true;
-                auto wait_slot = [&](int n) {                          // ring entry n has landed
-                    ok = ok && mbar_wait(bar_full(n % P::SLOTS), (n / P::SLOTS) & 1, s_abort, a.wait_cycles);
-                    tc_fence_after();
-                };
-                auto slot_addr = [&](int n) { return sbase + P::OFF_RING + (n % P::SLOTS) * P::TILE_BYTES; };
-                auto issue_s = [&](int s, int i) {                     // S_s = Q_s K_i^T
-                    const uint64_t qd = make_kmajor_desc<128>(sbase + s * P::TILE_BYTES);
-                    const uint64_t kd = make_kmajor_desc<128>(slot_addr(2 * i));
-    #pragma unroll
-                    for (int k = 0; k < DH / 16; ++k) {
-                        const uint64_t step = (uint64_t)((k >> 2) * (P::CHUNK_BYTES >> 4) + 2 * (k & 3));
-                        tc_mma_bf16(tmem + kTmS + 128 * s, qd + step, kd + step, kIdescS, k > 0);
-                    }
-                };
-                auto issue_o = [&](int s, int i) {                     // O_s += P_s V'_i
-                    const uint64_t vd = make_mnmajor_desc(slot_addr(2 * i + 1), P::CHUNK_BYTES);
-    #pragma unroll
-                    for (int k = 0; k < kMaskTileKeys / 16; ++k)       // 16 keys = 2048 bytes of the V' tile, 8 columns of P
-                        tc_mma_bf16_ts(tmem + kTmO + 128 * s, tmem + kTmS + 128 * s + 8 * k, vd + 128 * k, kIdescO, (i | k) != 0);
-                };
-                auto release = [&](int n) { tc_commit(bar_empty(n % P::SLOTS)); slots_released = n + 1; };
-                wait_slot(0);
-                for (int s = 0; ok && s < 2; ++s) {
-                    ok = mbar_wait(bar_q(s), 0, s_abort, a.wait_cycles);
-                    tc_fence_after();
-                    if (ok) { issue_s(s, 0); tc_commit(bar_s(s)); }
+            // ================= MMA issue (converged warp) ================================================
+            const uint32_t el = elect_lane();
+            bool ok = true;
+            auto wait = [&](uint32_t bar, uint32_t parity) { return warp_wait(bar, parity, s_abort, a.wait_cycles); };
+            auto wait_slot = [&](int n) { return wait(bar_full(n % P::SLOTS), (n / P::SLOTS) & 1); };      // ring entry n has landed
+            auto slot_addr = [&](int n) { return sbase + P::OFF_RING + (n % P::SLOTS) * P::TILE_BYTES; };
+            auto issue_s = [&](int s, int i) {                     // S_s = Q_s K_i^T
+                const uint64_t qd = make_kmajor_desc<128>(sbase + s * P::TILE_BYTES);
+                const uint64_t kd = make_kmajor_desc<128>(slot_addr(2 * i));
+#pragma unroll
+                for (int k = 0; k < DH / 16; ++k) {
+                    const uint64_t step = (uint64_t)((k >> 2) * (P::CHUNK_BYTES >> 4) + 2 * (k & 3));
+                    warp_mma_ss(el, tmem + kTmS + 128 * s, qd + step, kd + step, kIdescS, k > 0);
                 }
-                if (ok) release(0);
-                for (int i = 0; ok && i < ntiles; ++i) {
-                    wait_slot(2 * i + 1);
-                    for (int s = 0; ok && s < 2; ++s) {
-                        ok = mbar_wait(bar_p(s), i & 1, s_abort, a.wait_cycles);
-                        tc_fence_after();
-                        if (!ok) break;
-                        issue_o(s, i);
-                        if (i + 1 < ntiles) {
-                            if (s == 0) wait_slot(2 * i + 2);
-                            if (!ok) break;
-                            // (in order behind the product that reads P from these columns)
-                            issue_s(s, i + 1);
-                            tc_commit(bar_s(s));
-                        } else {
-                            tc_commit(bar_o(s));
-                        }
-                    }
-                    if (!ok) break;
-                    release(2 * i + 1);
-                    if (i + 1 < ntiles) release(2 * i + 2);
-                }
-                if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
+            };
+            auto issue_o = [&](int s, int i) {                     // O_s += P_s V'_i
+                const uint64_t vd = make_mnmajor_desc(slot_addr(2 * i + 1), P::CHUNK_BYTES);
+#pragma unroll
+                for (int k = 0; k < kMaskTileKeys / 16; ++k)       // 16 keys = 2048 bytes of the V' tile, 8 columns of P
+                    warp_mma_ts(el, tmem + kTmO + 128 * s, tmem + kTmS + 128 * s + 8 * k, vd + 128 * k, kIdescO, (i | k) != 0);
+            };
+            auto release = [&](int n) { warp_commit(el, bar_empty(n % P::SLOTS)); slots_released = n + 1; };
+            ok = wait_slot(0);
+            for (int s = 0; ok && s < 2; ++s) {
+                ok = wait(bar_q(s), 0);
+                if (ok) { issue_s(s, 0); warp_commit(el, bar_s(s)); }
             }
+            if (ok) release(0);
+            for (int i = 0; ok && i < ntiles; ++i) {
+                ok = wait_slot(2 * i + 1);
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    if (!ok || !(ok = wait(bar_p(s), i & 1))) break;
+                    issue_o(s, i);
+                    if (i + 1 < ntiles) {
+                        if (s == 0 && !(ok = wait_slot(2 * i + 2))) break;
+                        // (in order behind the product that reads P from these columns)
+                        issue_s(s, i + 1);
+                        warp_commit(el, bar_s(s));
+                    } else {
+                        warp_commit(el, bar_o(s));
+                    }
+                }
+                if (!ok) break;
+                release(2 * i + 1);
+                if (i + 1 < ntiles) release(2 * i + 2);
+            }
+            if (!ok && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
         }
     }
 
@@ -471,8 +476,8 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             for (int n = max(0, copies_issued - P::SLOTS); n < copies_issued; ++n)
                 mbar_drain(bar_full(n % P::SLOTS), (n / P::SLOTS) & 1);
         }
-        if (warp == 9 && lane == 0) {
-            tc_commit(bar_drain);
+        if (warp == 9) {
+            warp_commit(elect_lane(), bar_drain);
             mbar_drain(bar_drain, 0);
             for (int n = max(0, slots_released - P::SLOTS); n < slots_released; ++n)
                 mbar_drain(bar_empty(n % P::SLOTS), (n / P::SLOTS) & 1);

@@ -15,14 +15,16 @@
 // budget 2048: keys 6.3 ms (four products, 1.4 PFLOP/s), rows 5.3 ms (three, 1.24 PFLOP/s), target 4.9 ms (one, and all the
 // exponentials); the gather kernels took 92 ms for the same.
 //
-// Roles in all three: warps 0-7 the elementwise work (two warpgroups side by side), warp 8 copies, warp 9 MMA issue.
+// Roles in all three: warps 0-15 the elementwise work (four warpgroups side by side, 32 columns of a tile each: with two of
+// them the products waited for it), warp 16 copies, warp 17 MMA issue, 18 and 19 small loads.
 #include "gsa_masked.cuh"
 
 namespace gsa {
 
 namespace {
 
-constexpr int kBwdThreads = 384;
+constexpr int kBwdThreads = 640;
+constexpr int kCopyWarp = 16, kMmaWarp = 17;
 constexpr float kLog2e = 1.4426950408889634f;
 
 template <int DH>
@@ -60,19 +62,19 @@ struct MaskedBwdArgs {
 __device__ __forceinline__ uint64_t kmajor_step(int k) { return (uint64_t)((k >> 2) * (TileBytes<128>::CHUNK >> 4) + 2 * (k & 3)); }
 
 template <int DH>
-__device__ __forceinline__ void mma_kmajor(uint32_t d, uint32_t a_smem, uint32_t b_smem) {        // D = A B^T over DH columns
+__device__ __forceinline__ void mma_kmajor(uint32_t el, uint32_t d, uint32_t a_smem, uint32_t b_smem) {        // D = A B^T over DH columns
     const uint64_t ad = make_kmajor_desc<128>(a_smem), bd = make_kmajor_desc<128>(b_smem);
 #pragma unroll
     for (int k = 0; k < DH / 16; ++k)
-        tc_mma_bf16(d, ad + kmajor_step(k), bd + kmajor_step(k), make_idesc_bf16(128, 128), k > 0);
+        warp_mma_ss(el, d, ad + kmajor_step(k), bd + kmajor_step(k), make_idesc_bf16(128, 128), k > 0);
 }
-// D += A B with A (128 x 128, bf16) in TMEM in two halves of 64 contraction elements, 64 columns apart, and B the rows of a tile
+// D += A B with A (128 x 128, bf16) in TMEM in four parts of 32 contraction elements, 32 columns apart, and B the rows of a tile
 template <int DH>
-__device__ __forceinline__ void mma_tmem_rows(uint32_t d, uint32_t a_tmem, uint32_t b_smem, bool accumulate) {
+__device__ __forceinline__ void mma_tmem_rows(uint32_t el, uint32_t d, uint32_t a_tmem, uint32_t b_smem, bool accumulate) {
     const uint64_t bd = make_mnmajor_desc(b_smem, TileBytes<DH>::CHUNK);
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-        tc_mma_bf16_ts(d, a_tmem + (k >> 2) * 64 + (k & 3) * 8, bd + 128 * k, make_idesc_bf16(128, DH) | kIdescTransB,
+        warp_mma_ts(el, d, a_tmem + (k >> 1) * 32 + (k & 1) * 8, bd + 128 * k, make_idesc_bf16(128, DH) | kIdescTransB,
                        accumulate || k > 0);
 }
 
@@ -93,7 +95,7 @@ __device__ __forceinline__ uint32_t tile_start(int warp, uint32_t tmem_slot, con
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 9) {
+    if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(tmem_slot) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -111,16 +113,16 @@ __device__ __forceinline__ void tile_end(int warp, int lane, uint32_t tmem, vola
     tc_fence_before();
     __syncthreads();
     if (*s_abort) {
-        if (warp == 8 && lane == 0) drain_copies();
-        if (warp == 9 && lane == 0) {
-            tc_commit(bar_drain);
+        if (warp == kCopyWarp && lane == 0) drain_copies();
+        if (warp == kMmaWarp) {
+            warp_commit(elect_lane(), bar_drain);
             mbar_drain(bar_drain, 0);
             drain_commits();
         }
         tc_fence_before();
         __syncthreads();
     }
-    if (warp == 9) {
+    if (warp == kMmaWarp) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     }
@@ -172,15 +174,15 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     if (threadIdx.x == 0) {
         for (int s = 0; s < ST; ++s) {
             mbar_init(bar_q(s), 1); mbar_init(bar_d(s), 1); mbar_init(bar_free(s), 1);
-            mbar_init(bar_stat(s), 64); mbar_init(bar_statfree(s), 8);
+            mbar_init(bar_stat(s), 64); mbar_init(bar_statfree(s), 16);
         }
-        mbar_init(bar_kv, 1); mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_p, 8); mbar_init(bar_ds, 8);
+        mbar_init(bar_kv, 1); mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_p, 16); mbar_init(bar_ds, 16);
         mbar_init(bar_done, 1); mbar_init(bar_drain, 1);
     }
     const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
     int copies = 0, kv_issued = 0, released = 0;
 
-    if (warp == 8) {
+    if (warp == kCopyWarp) {
         if (lane == 0 && n > 0) {
             mbar_expect_tx(bar_kv, 2 * T::TILE);
             for (int c = 0; c < T::CHUNKS; ++c) {
@@ -203,45 +205,42 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             }
             if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
         }
-    } else if (warp == 9) {
-        if (lane == 0 && n > 0) {
+    } else if (warp == kMmaWarp) {
+        if (n > 0) {                                               // (converged warp)
+            const uint32_t el = elect_lane();
             auto q_at = [&](int i) { return sbase + P::OFF_RING + (i % ST) * 2 * T::TILE; };
             auto d_at = [&](int i) { return q_at(i) + T::TILE; };
-            auto wait = [&](uint32_t bar, uint32_t parity) {
-                const bool r = mbar_wait(bar, parity, s_abort, a.wait_cycles);
-                tc_fence_after();
-                return r;
-            };
+            auto wait = [&](uint32_t bar, uint32_t parity) { return warp_wait(bar, parity, s_abort, a.wait_cycles); };
             auto issue_s = [&](int i) {                            // S^T = K Q^T
                 if (!wait(bar_q(i % ST), (i / ST) & 1)) return false;
-                mma_kmajor<DH>(tmem + kTmS, sbase + P::OFF_K, q_at(i));
-                tc_commit(bar_s);
+                mma_kmajor<DH>(el, tmem + kTmS, sbase + P::OFF_K, q_at(i));
+                warp_commit(el, bar_s);
                 return true;
             };
             auto issue_dp = [&](int i) {                           // dP^T = V' do^T
                 if (!wait(bar_d(i % ST), (i / ST) & 1)) return false;
-                mma_kmajor<DH>(tmem + kTmP, sbase + P::OFF_V, d_at(i));
-                tc_commit(bar_dp);
+                mma_kmajor<DH>(el, tmem + kTmP, sbase + P::OFF_V, d_at(i));
+                warp_commit(el, bar_dp);
                 return true;
             };
             bool ok = wait(bar_kv, 0) && issue_s(0) && issue_dp(0);
             for (int i = 0; ok && i < n; ++i) {
                 // every product is issued behind the one that reads what it overwrites
                 if (!(ok = wait(bar_p, i & 1))) break;
-                mma_tmem_rows<DH>(tmem + kTmV, tmem + kTmS, d_at(i), i > 0);       // dV' += P^T do
+                mma_tmem_rows<DH>(el, tmem + kTmV, tmem + kTmS, d_at(i), i > 0);       // dV' += P^T do
                 if (i + 1 < n && !(ok = issue_s(i + 1))) break;
                 if (!(ok = wait(bar_ds, i & 1))) break;
-                mma_tmem_rows<DH>(tmem + kTmK, tmem + kTmP, q_at(i), i > 0);       // dK += dS^T Q
-                tc_commit(bar_free(i % ST));
+                mma_tmem_rows<DH>(el, tmem + kTmK, tmem + kTmP, q_at(i), i > 0);       // dK += dS^T Q
+                warp_commit(el, bar_free(i % ST));
                 released = i + 1;
                 if (i + 1 < n) ok = issue_dp(i + 1);
             }
-            if (ok) tc_commit(bar_done);
-            else atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
+            if (ok) warp_commit(el, bar_done);
+            else if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
         }
-    } else if (warp >= 10) {
+    } else if (warp > kMmaWarp) {
         // row statistics and masks of the next tiles: thread = two rows
-        const int j = threadIdx.x - 320;
+        const int j = threadIdx.x - (kMmaWarp + 1) * 32;
         bool ok = true;
         for (int i = 0; ok && i < n; ++i) {
             const int s = i % ST;
@@ -274,41 +273,38 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         }
         if (!ok && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
     } else {
-        // lane = key; this warpgroup's half of the 128 rows
-        const int half = warp >> 2, quad = warp & 3;
+        // lane = key; this warpgroup's quarter of the 128 rows
+        const int part = warp >> 2, quad = warp & 3;
         const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
-        const uint32_t ts = lane_base + kTmS + 64 * half, tp = lane_base + kTmP + 64 * half;
+        const uint32_t ts = lane_base + kTmS + 32 * part, tp = lane_base + kTmP + 32 * part;
         const uint32_t my_bit = 1u << lane;
         bool ok = true;
         for (int i = 0; i < n; ++i) {
             const int s = i % ST;
-            const float* st = reinterpret_cast<const float*>(smem + P::OFF_STAT + s * P::STAT_BYTES) + 64 * half;
+            const float* st = reinterpret_cast<const float*>(smem + P::OFF_STAT + s * P::STAT_BYTES) + 32 * part;
             const uint32_t* sm = reinterpret_cast<const uint32_t*>(smem + P::OFF_STAT + s * P::STAT_BYTES + 1024) +
-                                 quad * QT + 64 / G * half;
+                                 quad * QT + 32 / G * part;
             if (!mbar_wait(bar_stat(s), (i / ST) & 1, s_abort, a.wait_cycles) ||
                 !mbar_wait(bar_s, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
             tc_fence_after();
-            uint32_t v[2][32];
-            tc_ld32(ts, v[0]);
-            tc_ld32(ts + 32, v[1]);
-            tc_wait_ld32(v[0]);
-            tc_tie32(v[1]);
-            uint32_t pk[32];
+            uint32_t v[32], pk[16];
+            tc_ld32(ts, v);
+            tc_wait_ld32(v);
 #pragma unroll
-            for (int c = 0; c < 64; c += 4) {
+            for (int c = 0; c < 32; c += 4) {
                 const float4 l2 = *reinterpret_cast<const float4*>(st + c);
                 const float lv[4] = {l2.x, l2.y, l2.z, l2.w};
                 float pv[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float x = ex2_approx(fmaf(__uint_as_float(v[c >> 5][(c & 31) + e]), a.scale_log2, -lv[e]));
+                    const float x = ex2_approx(fmaf(__uint_as_float(v[c + e]), a.scale_log2, -lv[e]));
                     pv[e] = (sm[(c + e) / G] & my_bit) ? x : 0.f;
-                    v[c >> 5][(c & 31) + e] = __float_as_uint(pv[e]);
+                    v[c + e] = __float_as_uint(pv[e]);
                 }
                 pk[c / 2] = pack_bf16(pv[0], pv[1]);
                 pk[c / 2 + 1] = pack_bf16(pv[2], pv[3]);
             }
-            tc_st32(ts, pk);
+            tc_st16(ts, pk);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
@@ -316,23 +312,20 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
 
             if (!mbar_wait(bar_dp, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
             tc_fence_after();
+            uint32_t w[32];
+            tc_ld32(tp, w);
+            tc_wait_ld32(w);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint32_t w[32];
-                tc_ld32(tp + 32 * h, w);
-                tc_wait_ld32(w);
+            for (int c = 0; c < 32; c += 4) {
+                const float4 dl = *reinterpret_cast<const float4*>(st + 128 + c);
+                const float dv[4] = {dl.x, dl.y, dl.z, dl.w};
+                float ds[4];
 #pragma unroll
-                for (int c = 0; c < 32; c += 4) {
-                    const float4 dl = *reinterpret_cast<const float4*>(st + 128 + 32 * h + c);
-                    const float dv[4] = {dl.x, dl.y, dl.z, dl.w};
-                    float ds[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) ds[e] = __uint_as_float(v[h][c + e]) * (__uint_as_float(w[c + e]) - dv[e]);
-                    pk[16 * h + c / 2] = pack_bf16(ds[0], ds[1]);
-                    pk[16 * h + c / 2 + 1] = pack_bf16(ds[2], ds[3]);
-                }
+                for (int e = 0; e < 4; ++e) ds[e] = __uint_as_float(v[c + e]) * (__uint_as_float(w[c + e]) - dv[e]);
+                pk[c / 2] = pack_bf16(ds[0], ds[1]);
+                pk[c / 2 + 1] = pack_bf16(ds[2], ds[3]);
             }
-            tc_st32(tp, pk);
+            tc_st16(tp, pk);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
@@ -344,23 +337,23 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         } else {
             tc_fence_after();
             const int key = tile * kMaskTileKeys + quad * 32 + lane;
-            const size_t at = (((size_t)b * a.Lk + min(key, a.Lk - 1)) * a.n_kv + g) * DH + half * (DH / 2);
+            const size_t at = (((size_t)b * a.Lk + min(key, a.Lk - 1)) * a.n_kv + g) * DH + part * (DH / 4);
 #pragma unroll
             for (int c = 0; c < DH / 64; ++c) {
-                uint32_t dk[32], dv[32];
+                uint32_t dk[16], dv[16];
                 if (n > 0) {
-                    tc_ld32(lane_base + kTmK + half * (DH / 2) + 32 * c, dk);
-                    tc_ld32(lane_base + kTmV + half * (DH / 2) + 32 * c, dv);
-                    tc_wait_ld32(dk);
-                    tc_tie32(dv);
+                    tc_ld16(lane_base + kTmK + part * (DH / 4) + 16 * c, dk);
+                    tc_wait_ld16(dk);
+                    tc_ld16(lane_base + kTmV + part * (DH / 4) + 16 * c, dv);
+                    tc_wait_ld16(dv);
                 } else {
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) dk[e] = dv[e] = 0u;
+                    for (int e = 0; e < 16; ++e) dk[e] = dv[e] = 0u;
                 }
                 if (key >= a.Lk) continue;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const size_t p8 = at + 32 * c + 8 * q;
+                for (int q = 0; q < 2; ++q) {
+                    const size_t p8 = at + 16 * c + 8 * q;
                     const uint4 vv = *reinterpret_cast<const uint4*>(a.V + p8), gg = *reinterpret_cast<const uint4*>(a.g2 + p8);
                     const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
                     const __nv_bfloat162* gp = reinterpret_cast<const __nv_bfloat162*>(&gg);
@@ -429,13 +422,13 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < SL; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-        mbar_init(bar_qd, 1); mbar_init(bar_s(0), 1); mbar_init(bar_s(1), 1); mbar_init(bar_dp, 1); mbar_init(bar_read, 8);
-        mbar_init(bar_ds, 8); mbar_init(bar_done, 1); mbar_init(bar_drain, 1);
+        mbar_init(bar_qd, 1); mbar_init(bar_s(0), 1); mbar_init(bar_s(1), 1); mbar_init(bar_dp, 1); mbar_init(bar_read, 16);
+        mbar_init(bar_ds, 16); mbar_init(bar_done, 1); mbar_init(bar_drain, 1);
     }
     const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
     int copies = 0, qd_issued = 0, k_released = 0, v_released = 0;
 
-    if (warp == 8) {
+    if (warp == kCopyWarp) {
         if (lane == 0) {
             mbar_expect_tx(bar_qd, 2 * T::TILE);
             for (int c = 0; c < T::CHUNKS; ++c) {
@@ -455,26 +448,23 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             }
             if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
         }
-    } else if (warp == 9) {
-        if (lane == 0) {
-            auto wait = [&](uint32_t bar, uint32_t parity) {
-                const bool r = mbar_wait(bar, parity, s_abort, a.wait_cycles);
-                tc_fence_after();
-                return r;
-            };
+    } else if (warp == kMmaWarp) {
+        {
+            const uint32_t el = elect_lane();
+            auto wait = [&](uint32_t bar, uint32_t parity) { return warp_wait(bar, parity, s_abort, a.wait_cycles); };
             auto slot = [&](int e) { return sbase + P::OFF_RING + (e % SL) * T::TILE; };
             auto landed = [&](int e) { return wait(bar_full(e % SL), (e / SL) & 1); };
             auto issue_s = [&](int i) {                            // S = Q K^T
                 if (!landed(2 * i)) return false;
-                mma_kmajor<DH>(tmem + kTmS + 128 * (i & 1), sbase + P::OFF_Q, slot(2 * i));
-                tc_commit(bar_s(i));
+                mma_kmajor<DH>(el, tmem + kTmS + 128 * (i & 1), sbase + P::OFF_Q, slot(2 * i));
+                warp_commit(el, bar_s(i));
                 return true;
             };
             auto issue_dp = [&](int i) {                           // dP = do V'^T
                 if (!landed(2 * i + 1)) return false;
-                mma_kmajor<DH>(tmem + kTmP, sbase + P::OFF_D, slot(2 * i + 1));
-                tc_commit(bar_dp);
-                tc_commit(bar_empty((2 * i + 1) % SL));
+                mma_kmajor<DH>(el, tmem + kTmP, sbase + P::OFF_D, slot(2 * i + 1));
+                warp_commit(el, bar_dp);
+                warp_commit(el, bar_empty((2 * i + 1) % SL));
                 v_released = i + 1;
                 return true;
             };
@@ -482,65 +472,55 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             for (int i = 0; ok && i < n; ++i) {
                 if (i + 1 < n) ok = wait(bar_read, i & 1) && issue_dp(i + 1);      // the columns of dP(i) have been read
                 if (!ok || !(ok = wait(bar_ds, i & 1))) break;
-                mma_tmem_rows<DH>(tmem + kTmQ, tmem + kTmS + 128 * (i & 1), slot(2 * i), i > 0);      // dQ += dS K
-                tc_commit(bar_empty((2 * i) % SL));
+                mma_tmem_rows<DH>(el, tmem + kTmQ, tmem + kTmS + 128 * (i & 1), slot(2 * i), i > 0);      // dQ += dS K
+                warp_commit(el, bar_empty((2 * i) % SL));
                 k_released = i + 1;
                 if (i + 2 < n) ok = issue_s(i + 2);
             }
-            if (ok) tc_commit(bar_done);
-            else atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
+            if (ok) warp_commit(el, bar_done);
+            else if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
         }
-    } else if (warp < 8) {
-        const int half = warp >> 2, quad = warp & 3;
+    } else if (warp < 16) {
+        const int part = warp >> 2, quad = warp & 3;
         const int m = quad * 32 + lane, r = r0 + m / G, h = g * G + m % G;
         const bool live = r < a.rows;
         const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
-        const uint2* __restrict__ mrow =
-            reinterpret_cast<const uint2*>(a.mask + (int64_t)b * a.key_tiles * a.row_pitch + (live ? r : 0)) + half;
+        const uint32_t* __restrict__ mrow =
+            reinterpret_cast<const uint32_t*>(a.mask + (int64_t)b * a.key_tiles * a.row_pitch + (live ? r : 0)) + part;
         float l2 = 0.f, dl = 0.f;
         if (live) {
             const size_t at = ((size_t)b * a.Lq + a.q0 + r) * a.n_h + h;
             l2 = a.lse[at] * kLog2e;
             dl = a.delta[at];
         }
-        uint2 mk_next = live ? __ldg(mrow) : make_uint2(0u, 0u);
+        uint32_t mk_next = live ? __ldg(mrow) : 0u;
         bool ok = true;
         for (int i = 0; i < n; ++i) {
-            const uint2 mk = mk_next;
-            if (live && i + 1 < n) mk_next = __ldg(mrow + (int64_t)(i + 1) * a.row_pitch * 2);
-            const uint32_t ts = lane_base + kTmS + 128 * (i & 1) + 64 * half, tp = lane_base + kTmP + 64 * half;
+            const uint32_t mk = mk_next;
+            if (live && i + 1 < n) mk_next = __ldg(mrow + (int64_t)(i + 1) * a.row_pitch * 4);
+            const uint32_t ts = lane_base + kTmS + 128 * (i & 1) + 32 * part, tp = lane_base + kTmP + 32 * part;
             if (!mbar_wait(bar_s(i), (i >> 1) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
             tc_fence_after();
-            uint32_t v[2][32], w[2][32];
-            tc_ld32(ts, v[0]);
-            tc_ld32(ts + 32, v[1]);
-            tc_wait_ld32(v[0]);
-            tc_tie32(v[1]);
-            const uint32_t mw[2] = {mk.x, mk.y};
+            uint32_t v[32], w[32], pk[16];
+            tc_ld32(ts, v);
+            tc_wait_ld32(v);
 #pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float x = ex2_approx(fmaf(__uint_as_float(v[c][j]), a.scale_log2, -l2));
-                    v[c][j] = __float_as_uint((mw[c] >> j) & 1u ? x : 0.f);
-                }
+            for (int j = 0; j < 32; ++j) {
+                const float x = ex2_approx(fmaf(__uint_as_float(v[j]), a.scale_log2, -l2));
+                v[j] = __float_as_uint((mk >> j) & 1u ? x : 0.f);
+            }
             if (!mbar_wait(bar_dp, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
             tc_fence_after();
-            tc_ld32(tp, w[0]);
-            tc_ld32(tp + 32, w[1]);
-            tc_wait_ld32(w[0]);
-            tc_tie32(w[1]);
+            tc_ld32(tp, w);
+            tc_wait_ld32(w);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_read);
-            uint32_t pk[32];
 #pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int j = 0; j < 32; j += 2)
-                    pk[16 * c + j / 2] = pack_bf16(__uint_as_float(v[c][j]) * (__uint_as_float(w[c][j]) - dl),
-                                                   __uint_as_float(v[c][j + 1]) * (__uint_as_float(w[c][j + 1]) - dl));
-            tc_st32(ts, pk);
+            for (int j = 0; j < 32; j += 2)
+                pk[j / 2] = pack_bf16(__uint_as_float(v[j]) * (__uint_as_float(w[j]) - dl),
+                                      __uint_as_float(v[j + 1]) * (__uint_as_float(w[j + 1]) - dl));
+            tc_st16(ts, pk);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
@@ -551,20 +531,20 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
         } else {
             tc_fence_after();
-            __nv_bfloat16* dst = a.dQ + (((size_t)b * a.Lq + a.q0 + (live ? r : 0)) * a.n_h + h) * DH + half * (DH / 2);
+            __nv_bfloat16* dst = a.dQ + (((size_t)b * a.Lq + a.q0 + (live ? r : 0)) * a.n_h + h) * DH + part * (DH / 4);
 #pragma unroll
             for (int c = 0; c < DH / 64; ++c) {
-                uint32_t o[32];
-                tc_ld32(lane_base + kTmQ + half * (DH / 2) + 32 * c, o);
-                tc_wait_ld32(o);
+                uint32_t o[16];
+                tc_ld16(lane_base + kTmQ + part * (DH / 4) + 16 * c, o);
+                tc_wait_ld16(o);
                 if (!live) continue;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < 2; ++q) {
                     uint32_t x[4];
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                         x[e] = pack_bf16(__uint_as_float(o[8 * q + 2 * e]) * a.scale, __uint_as_float(o[8 * q + 2 * e + 1]) * a.scale);
-                    *reinterpret_cast<uint4*>(dst + 32 * c + 8 * q) = make_uint4(x[0], x[1], x[2], x[3]);
+                    *reinterpret_cast<uint4*>(dst + 16 * c + 8 * q) = make_uint4(x[0], x[1], x[2], x[3]);
                 }
             }
         }
@@ -619,13 +599,13 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
             mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1);
-            for (int w = 0; w < 2; ++w) { mbar_init(bar_s(s, w), 1); mbar_init(bar_sfree(s, w), 4); }
+            for (int w = 0; w < 2; ++w) { mbar_init(bar_s(s, w), 1); mbar_init(bar_sfree(s, w), 8); }
         }
         mbar_init(bar_drain, 1);
     }
-    if (threadIdx.x >= 256) {
+    if (threadIdx.x >= 512) {
         // where the CTA's run of keys starts in every query's set
-        const int q = threadIdx.x - 256, r = r0 + q;
+        const int q = threadIdx.x - 512, r = r0 + q;
         if (q < QT) {
             int lo = 0;
             if (r < a.rows) {
@@ -644,9 +624,10 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
     int copies = 0, released = 0;
 
-    if (warp < 8) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
-        const int w = warp >> 2, quad = warp & 3;                  // this warpgroup's key tile of the pair
+    // 640 threads launched at 96 registers: 512 * 104 + 128 * 64 = 61440
+    if (warp < 16) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+        const int w = warp >> 3, half = (warp >> 2) & 1, quad = warp & 3;      // half of a key tile of the pair
         const int m = quad * 32 + lane, q = m / G, r = r0 + q;
         const bool live = r < a.rows;
         const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
@@ -658,14 +639,9 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         bool ok = true;
         int it = 0;
         for (int pair = pair0; ok && pair < pair1; ++pair) {
-            uint4 mk0 = make_uint4(0u, 0u, 0u, 0u), mk1 = mk0;     // masks of both tiles: the ranks run through both
-            if (live) {
-                mk0 = a.mask[((int64_t)b * a.key_tiles + 2 * pair) * a.row_pitch + r];
-                if (2 * pair + 1 < ntiles) mk1 = a.mask[((int64_t)b * a.key_tiles + 2 * pair + 1) * a.row_pitch + r];
-            }
-            uint64_t acc[64];
+            uint64_t acc[32];
 #pragma unroll
-            for (int c = 0; c < 64; ++c) acc[c] = 0ull;
+            for (int c = 0; c < 32; ++c) acc[c] = 0ull;
             float l_next = live ? lse[0] : 0.f;
             for (int g = 0; g < a.n_kv; ++g, ++it) {
                 const int s = it & 1;
@@ -674,17 +650,16 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                 const uint64_t neg2 = pack_f32x2(neg, neg);
                 if (!mbar_wait(bar_s(s, w), (it >> 1) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t ts = lane_base + 256 * s + 128 * w;
-                uint32_t v[2][16];                                 // the next 16 columns arrive behind the current ones' arithmetic
-                tc_ld16(ts, v[0]);
+                const uint32_t ts = lane_base + 256 * s + 128 * w + 64 * half;
+                uint32_t v[16];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    tc_wait_ld16(v[c & 1]);
-                    if (c < 7) tc_ld16(ts + 16 * (c + 1), v[(c + 1) & 1]);
+                for (int c = 0; c < 4; ++c) {
+                    tc_ld16(ts + 16 * c, v);
+                    tc_wait_ld16(v);
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         float x0, x1;
-                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[c & 1][2 * j]), __uint_as_float(v[c & 1][2 * j + 1])), scale2, neg2), x0, x1);
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), scale2, neg2), x0, x1);
                         acc[8 * c + j] = add_f32x2(acc[8 * c + j], pack_f32x2(ex2_approx(x0), ex2_approx(x1)));
                     }
                 }
@@ -693,13 +668,21 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                 if (lane == 0) mbar_arrive(bar_sfree(s, w));
             }
             if (!ok) break;
-            // sum over the heads of the group (neighbouring lanes), then to the set's positions; the group's lanes share the columns
+            // sum over the heads of the group (neighbouring lanes), then to the set's positions; the group's lanes share the
+            // columns.  The ranks run through both tiles of the pair.
+            uint4 mk0 = make_uint4(0u, 0u, 0u, 0u), mk1 = mk0;
+            if (live) {
+                mk0 = a.mask[((int64_t)b * a.key_tiles + 2 * pair) * a.row_pitch + r];
+                if (2 * pair + 1 < ntiles) mk1 = a.mask[((int64_t)b * a.key_tiles + 2 * pair + 1) * a.row_pitch + r];
+            }
+            const int n0 = __popc(mk0.x) + __popc(mk0.y), n1 = n0 + __popc(mk0.z) + __popc(mk0.w),
+                      n2 = n1 + __popc(mk1.x) + __popc(mk1.y);
+            int at = rank + (w ? (half ? n2 : n1) : (half ? n0 : 0));
             const uint4 mk = w ? mk1 : mk0;
-            const int n0 = __popc(mk0.x) + __popc(mk0.y) + __popc(mk0.z) + __popc(mk0.w);
-            const uint32_t words[4] = {mk.x, mk.y, mk.z, mk.w};
-            int at = rank + (w ? n0 : 0);
+            const uint32_t words[2] = {half ? mk.z : mk.x, half ? mk.w : mk.y};
+            rank += n2 + __popc(mk1.z) + __popc(mk1.w);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < 2; ++c) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     float x0, x1;
@@ -716,12 +699,11 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                 }
                 at += __popc(words[c]);
             }
-            rank += n0 + __popc(mk1.x) + __popc(mk1.y) + __popc(mk1.z) + __popc(mk1.w);
         }
         if (!ok && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
     } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-        if (warp == 8) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        if (warp == kCopyWarp) {
             if (lane == 0) {
                 bool ok = true;
                 for (int it = 0; ok && it < n; ++it) {
@@ -739,24 +721,23 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                 }
                 if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
             }
-        } else if (warp == 9) {
-            if (lane == 0) {
-                bool ok = true;
-                for (int it = 0; ok && it < n; ++it) {
-                    const int s = it & 1;
-                    if (!mbar_wait(bar_full(s), (it >> 1) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
-                    for (int w = 0; ok && w < 2; ++w) {
-                        if (!mbar_wait(bar_sfree(s, w), ((it >> 1) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
-                        tc_fence_after();
-                        mma_kmajor<DH>(tmem + 256 * s + 128 * w, sbase + s * P::STAGE, sbase + s * P::STAGE + (1 + w) * T::TILE);
-                        tc_commit(bar_s(s, w));
-                    }
-                    if (!ok) break;
-                    tc_commit(bar_empty(s));
-                    released = it + 1;
+        } else if (warp == kMmaWarp) {
+            const uint32_t el = elect_lane();                      // (converged warp)
+            bool ok = true;
+            for (int it = 0; ok && it < n; ++it) {
+                const int s = it & 1;
+                if (!(ok = warp_wait(bar_full(s), (it >> 1) & 1, s_abort, a.wait_cycles))) break;
+#pragma unroll
+                for (int w = 0; w < 2; ++w) {
+                    if (!(ok = warp_wait(bar_sfree(s, w), ((it >> 1) & 1) ^ 1, s_abort, a.wait_cycles))) break;
+                    mma_kmajor<DH>(el, tmem + 256 * s + 128 * w, sbase + s * P::STAGE, sbase + s * P::STAGE + (1 + w) * T::TILE);
+                    warp_commit(el, bar_s(s, w));
                 }
-                if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
+                if (!ok) break;
+                warp_commit(el, bar_empty(s));
+                released = it + 1;
             }
+            if (!ok && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
         }
     }
     tile_end(warp, lane, tmem, s_abort, bar_drain,
