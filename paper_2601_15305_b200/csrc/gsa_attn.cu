@@ -113,6 +113,7 @@ __host__ __device__ __forceinline__ int parts_of(int k_eff, int max_parts) {
 template <int DH, int G, bool FUSE_G2>
 __global__ void __launch_bounds__((FUSE_G2 ? kWarpsFused : kWarpsPrefill) * 32, 1)
 gsa_sparse_attn_kernel(const AttnArgs a) {
+    chain_wait();
     constexpr int kWarpsPerCta = FUSE_G2 ? kWarpsFused : kWarpsPrefill;
     constexpr int HEAD_BYTES = DH * 2;
     constexpr int NC = DH / 32;                         // 32-d chunks of a head row (one uint4 per thread each)
@@ -395,6 +396,7 @@ gsa_sparse_attn_kernel(const AttnArgs a) {
 __global__ void __launch_bounds__(256) gsa_range_cuts_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ kt,
                                                              int32_t* __restrict__ cuts, RowRange rr, IdxLayout il,
                                                              int k_max, int n_cuts, int range_keys) {
+    chain_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)rr.rows() * n_cuts) return;
     const int c = (int)(i % n_cuts);
@@ -421,6 +423,7 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
                                                                 RowRange rr, IdxLayout il, int64_t idx_rows, int Lq, int n_h,
                                                                 int n_kv, int k_max, int mode, int max_parts,
                                                                 float* __restrict__ lse) {
+    chain_wait();
     constexpr int STATE_F = G * (DH + 2);
     const int rows = rr.rows();
     // range mode: kFinRows rows per CTA, all (KV head, d) pairs; parts mode (few rows, several state slots to
@@ -526,6 +529,7 @@ __global__ void __launch_bounds__(256) gsa_value_gate_kernel(const uint4* __rest
                                                              const uint4* __restrict__ g2,
                                                              uint4* __restrict__ Vg, int64_t n_vec,
                                                              int32_t* nonfinite) {
+    chain_wait();
     uint32_t bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -593,7 +597,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
 
     if (pl.mode == 0 && pl.n_ranges > 1) {
         const int64_t n = (int64_t)rr_all.rows() * pl.n_ranges;
-        gsa_range_cuts_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a.idx, a.kt, cuts, rr_all, a.il, a.k_max,
+        launch_chained(gsa_range_cuts_kernel, (unsigned)((n + 255) / 256), 256, 0, st, a.idx, a.kt, cuts, rr_all, a.il, a.k_max,
                                                                           pl.n_ranges, g_range_keys);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -611,7 +615,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
         fr.q_begin = t_lo; fr.R = t_hi - t_lo;
         const dim3 fin_grid = pl.mode == 0 ? dim3((unsigned)((fr.rows() + kFinRows - 1) / kFinRows), 1)
                                            : dim3((unsigned)fr.rows(), (unsigned)a.n_kv);
-        gsa_attn_finalize_kernel<DH, G><<<fin_grid, pl.mode == 0 ? fin_threads : DH, 0, st>>>(
+        launch_chained(gsa_attn_finalize_kernel<DH, G>, fin_grid, pl.mode == 0 ? fin_threads : DH, 0, st,
             a.state, a.kt, g1, out, fr, a.il, a.idx_rows, p.Lq, p.n_h, p.n_kv, p.k_max, pl.mode, pl.slots, a.lse);
         ++g_launches;
         cudaError_t fe = cudaGetLastError();
@@ -636,7 +640,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
         const int64_t items = (int64_t)ar.rr.rows() * a.n_kv * (pl.mode == 1 ? pl.slots : 1);
         const int64_t want = (items + kWarpsPerCta - 1) / kWarpsPerCta;
         const int ctas = (int)(want < cap ? want : cap);
-        kern<<<ctas, kWarpsPerCta * 32, smem, st>>>(ar);
+        launch_chained(kern, ctas, kWarpsPerCta * 32, smem, st, ar);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         timeline_mark(kStageAttn, st);
@@ -723,7 +727,7 @@ cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, _
     const int64_t n_vec = n_elems / 8;
     if (n_vec <= 0) return cudaSuccess;
     const int blocks = (int)((n_vec + 255) / 256 < sm_count() * 16 ? (n_vec + 255) / 256 : sm_count() * 16);
-    gsa_value_gate_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const uint4*>(V),
+    launch_chained(gsa_value_gate_kernel, blocks, 256, 0, st, reinterpret_cast<const uint4*>(V),
                                                   reinterpret_cast<const uint4*>(g2),
                                                   reinterpret_cast<uint4*>(Vg), n_vec, nonfinite);
     ++g_launches;

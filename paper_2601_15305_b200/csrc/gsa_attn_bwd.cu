@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* 
                                                            __nv_bfloat16* __restrict__ dOs, __nv_bfloat16* __restrict__ dg1,
                                                            float* __restrict__ delta, RowRange rr, int32_t Lq, int32_t n_h,
                                                            int32_t* nonfinite /*nullable: raised if do or delta is*/) {
+    chain_wait();
     constexpr int EPL = DH / 32;
     const int lane = threadIdx.x & 31;
     const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -133,6 +134,7 @@ __device__ __forceinline__ int warp_lower_bound(const int32_t* __restrict__ S, i
 __global__ void __launch_bounds__(256) gsa_bwd_range_cuts_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ kt,
                                                                  int32_t* __restrict__ cuts, RowRange rr, IdxLayout il,
                                                                  int32_t Lq, int32_t k_max, int32_t n_ranges, int32_t range_keys) {
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int64_t lr = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (lr >= rr.rows()) return;
@@ -153,6 +155,7 @@ __global__ void __launch_bounds__(256) gsa_bwd_range_cuts_kernel(const int32_t* 
 //         range's part, dQ added into dq32; the items of range 0 also write dg1, do, delta and lse2.
 template <int DH, int G, int MODE>
 __global__ void __launch_bounds__(kBwdWarps * 32, 4) gsa_sparse_attn_bwd_kernel(const BwdArgs a) {
+    chain_wait();
     constexpr int ROW = (DH + 8) * 2;                  // bytes of a padded tile row (odd multiple of 16)
     constexpr int KTILE = 16 * ROW, QTILE = 8 * ROW;
     constexpr int STAGE = KTILE;                       // a K tile (V' rows go straight into MMA fragments)
@@ -459,6 +462,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 4) gsa_sparse_attn_bwd_kernel(
 __global__ void __launch_bounds__(256) gsa_bwd_dq_finish_kernel(const float* __restrict__ dq32,
                                                                 __nv_bfloat16* __restrict__ dQ, RowRange rr,
                                                                 int32_t Lq, int64_t row_elems) {
+    chain_wait();
     const int lr = blockIdx.x;
     const int64_t qrow = (int64_t)(rr.b0 + lr / rr.R) * Lq + rr.q_begin + lr % rr.R;
     for (int64_t i = threadIdx.x * 4; i < row_elems; i += blockDim.x * 4) {
@@ -480,7 +484,7 @@ cudaError_t launch_bwd_mode(const BwdArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const int64_t items = (int64_t)a.rr.rows() * a.n_kv * (MODE == 0 ? 1 : a.n_ranges);
     const int64_t ctas = (items + kBwdWarps - 1) / kBwdWarps;
-    kern<<<(unsigned)ctas, kBwdWarps * 32, smem, st>>>(a);
+    launch_chained(kern, (unsigned)ctas, kBwdWarps * 32, smem, st, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -488,7 +492,7 @@ cudaError_t launch_bwd_mode(const BwdArgs& a, cudaStream_t st) {
 template <int DH, int G>
 cudaError_t launch_bwd_t(const BwdArgs& a, cudaStream_t st) {
     if (a.n_ranges <= 1) return launch_bwd_mode<DH, G, 0>(a, st);
-    gsa_bwd_range_cuts_kernel<<<(unsigned)((a.rr.rows() + 7) / 8), 256, 0, st>>>(a.idx, a.kt, const_cast<int32_t*>(a.cuts), a.rr,
+    launch_chained(gsa_bwd_range_cuts_kernel, (unsigned)((a.rr.rows() + 7) / 8), 256, 0, st, a.idx, a.kt, const_cast<int32_t*>(a.cuts), a.rr,
                                                                                   a.il, a.Lq, a.k_max, a.n_ranges, a.range_keys);
     ++g_launches;
     cudaError_t e = cudaGetLastError();
@@ -496,7 +500,7 @@ cudaError_t launch_bwd_t(const BwdArgs& a, cudaStream_t st) {
     if (e == cudaSuccess && !a.lse_in) e = launch_bwd_mode<DH, G, 1>(a, st);
     if (e == cudaSuccess) e = launch_bwd_mode<DH, G, 2>(a, st);
     if (e != cudaSuccess) return e;
-    gsa_bwd_dq_finish_kernel<<<a.rr.rows(), 256, 0, st>>>(a.dq32, a.dQ, a.rr, a.Lq, (int64_t)a.n_h * DH);
+    launch_chained(gsa_bwd_dq_finish_kernel, a.rr.rows(), 256, 0, st, a.dq32, a.dQ, a.rr, a.Lq, (int64_t)a.n_h * DH);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -528,8 +532,8 @@ cudaError_t launch_bwd_prep(const gsa_params_t& p, RowRange rr, const __nv_bfloa
                             const __nv_bfloat16* dout, __nv_bfloat16* dOs, __nv_bfloat16* dg1, float* delta,
                             int32_t* nonfinite, cudaStream_t st) {
     const unsigned ctas = (unsigned)(((int64_t)rr.rows() * p.n_h + 7) / 8);
-    if (p.d_h == 128) gsa_bwd_prep_kernel<128><<<ctas, 256, 0, st>>>(g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, nonfinite);
-    else gsa_bwd_prep_kernel<64><<<ctas, 256, 0, st>>>(g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, nonfinite);
+    if (p.d_h == 128) launch_chained(gsa_bwd_prep_kernel<128>, ctas, 256, 0, st, g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, nonfinite);
+    else launch_chained(gsa_bwd_prep_kernel<64>, ctas, 256, 0, st, g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, nonfinite);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -47,6 +47,19 @@ bool withhold_first_copy();
 
 extern std::atomic<int64_t> g_launches;   // host-side launch counter (any host thread may launch)
 
+// Launch behind the stream's previous kernel such that this one's start-up (and the launch itself) overlaps the other's end:
+// the kernel begins with chain_wait(), which returns once everything before it on the stream is complete and visible.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // multiprocessors of the current device (cached per device; 148 if the query fails)
 int sm_count();
 
@@ -148,6 +161,13 @@ cudaError_t launch_project(const gsa_params_t& p, int d_model, const __nv_bfloat
 
 cudaError_t launch_gemm_bf16(int M, int K, int N, const __nv_bfloat16* A, const __nv_bfloat16* Bt, __nv_bfloat16* C,
                              int32_t* dev_status, cudaStream_t st);
+
+// First statement of every kernel that launch_chained starts: nothing before it may touch memory.  The next kernel may be
+// brought up from here on.
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // ---- device helpers ------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

@@ -63,6 +63,7 @@ struct ProbsArgs {
 
 template <int DH, int G>
 __global__ void __launch_bounds__(kLossWarps * 32) gsa_attn_probs_mean_kernel(const ProbsArgs a) {
+    chain_wait();
     constexpr int ROW = (DH + 8) * 2;
     constexpr int KTILE = 16 * ROW, QTILE = 8 * ROW;
     constexpr int WARP_SMEM = 2 * KTILE;               // two stages; the Q tile borrows stage 1 first
@@ -216,6 +217,7 @@ struct KlArgs {
 
 template <int DI, int HI>
 __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const KlArgs a) {
+    chain_wait();
     constexpr int ROW = (DI + 8) * 2;                  // bytes of a padded tile row (odd multiple of 16)
     constexpr int KTILE = 16 * ROW, QTILE = 8 * ROW;
     constexpr int WARP_SMEM = 2 * KTILE + QTILE;       // two k^I stages and the row's q^I tile
@@ -427,6 +429,7 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
 
 __global__ void __launch_bounds__(256) gsa_f32_to_bf16_kernel(const float* __restrict__ src,
                                                               __nv_bfloat16* __restrict__ dst, int64_t n) {
+    chain_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += stride) {
         const float4 v = *reinterpret_cast<const float4*>(src + i);
@@ -443,7 +446,7 @@ cudaError_t launch_probs_t(const ProbsArgs& a, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const int64_t items = (int64_t)a.rr.rows() * a.n_kv;
-    kern<<<(unsigned)((items + kLossWarps - 1) / kLossWarps), kLossWarps * 32, smem, st>>>(a);
+    launch_chained(kern, (unsigned)((items + kLossWarps - 1) / kLossWarps), kLossWarps * 32, smem, st, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -453,7 +456,7 @@ cudaError_t launch_kl_t(const KlArgs& a, cudaStream_t st) {
     constexpr int smem = kLossWarps * (2 * 16 + 8) * (DI + 8) * 2;
     auto kern = gsa_indexer_kl_kernel<DI, HI>;
     const int64_t items = a.rr.rows();
-    kern<<<(unsigned)((items + kLossWarps - 1) / kLossWarps), kLossWarps * 32, smem, st>>>(a);
+    launch_chained(kern, (unsigned)((items + kLossWarps - 1) / kLossWarps), kLossWarps * 32, smem, st, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -500,7 +503,7 @@ cudaError_t launch_indexer_kl(const gsa_params_t& p, RowRange rr, const __nv_bfl
         if (e != cudaSuccess) return e;
     }
     const int64_t want = (n_k / 4 + 255) / 256;
-    gsa_f32_to_bf16_kernel<<<(int)(want < sm_count() * 16 ? (want > 0 ? want : 1) : sm_count() * 16), 256, 0, st>>>(dkI32, dkI, n_k);
+    launch_chained(gsa_f32_to_bf16_kernel, (int)(want < sm_count() * 16 ? (want > 0 ? want : 1) : sm_count() * 16), 256, 0, st, dkI32, dkI, n_k);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -38,6 +38,7 @@ __device__ __forceinline__ void ldg32(const void* p, uint4& lo, uint4& hi) {
 
 template <int DI, int HI>
 __global__ void __launch_bounds__(kRowsWarps * 32) gsa_indexer_rows_kernel(const RowsIdxArgs a) {
+    chain_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gid = lane >> 2, tig = lane & 3;
     const int lr = blockIdx.y;
@@ -135,7 +136,7 @@ cudaError_t launch_rows_t(const gsa_params_t& p, RowRange rr, const RowsIdxArgs&
     if (per < step) per = step;
     a.keys_per_cta = (int32_t)per;
     dim3 grid((unsigned)((n_max + per - 1) / per), (unsigned)rr.rows());
-    gsa_indexer_rows_kernel<DI, HI><<<grid, kRowsWarps * 32, 0, st>>>(a);
+    launch_chained(gsa_indexer_rows_kernel<DI, HI>, grid, kRowsWarps * 32, 0, st, a);
     ++g_launches;
     return cudaGetLastError();
 }

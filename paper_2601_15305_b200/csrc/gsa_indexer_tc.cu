@@ -147,6 +147,7 @@ template <int DI, int HI, bool RELU>
 __global__ void __launch_bounds__(kThreads, 1)
 gsa_indexer_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_q,
                       const TcArgs a) {
+    chain_wait();
     using P = SmemPlan<DI>;
     constexpr int NQ = kNCols / HI;             // queries per group
     constexpr int KSTEPS = DI / 16;
@@ -381,7 +382,7 @@ cudaError_t launch_t(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* qI
     auto kern = gsa_indexer_tc_kernel<DI, HI, RELU>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, kSmem, st>>>(tm_k, tm_q, a);
+    launch_chained(kern, grid, kThreads, kSmem, st, tm_k, tm_q, a);
     ++g_launches;
     return cudaGetLastError();
 }

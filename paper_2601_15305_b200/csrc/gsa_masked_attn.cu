@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(kMaskRowAlign * 32)
 gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ kt, uint4* __restrict__ mask,
                        IdxLayout il, int q0, int rows, int row_pitch, int key_tiles, int block_rows, int k_max, int off,
                        int32_t* __restrict__ general) {
+    chain_wait();
     __shared__ __align__(16) uint32_t s_bits[kMaskRowAlign * kMaskRowWords];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y, r0 = blockIdx.x * kMaskRowAlign, r = r0 + warp;
@@ -114,6 +115,7 @@ gsa_general_attn_kernel(const int32_t* __restrict__ general, const __nv_bfloat16
                         const int32_t* __restrict__ kt, IdxLayout il, __nv_bfloat16* __restrict__ out,
                         float* __restrict__ lse, int32_t* dev_status, int q0, int rows, int B, int Lq, int Lk, int n_kv,
                         int k_max, float scale_log2) {
+    chain_wait();
     if (*general == 0) return;
     constexpr int NV = DH / 32;
     const int lane = threadIdx.x & 31, n_h = n_kv * G;
@@ -175,6 +177,7 @@ gsa_general_attn_kernel(const int32_t* __restrict__ general, const __nv_bfloat16
 
 // raises `general` if a bf16 value is infinite or NaN
 __global__ void __launch_bounds__(256) gsa_check_finite_kernel(const uint4* __restrict__ x, int64_t n_vec, int32_t* general) {
+    chain_wait();
     uint32_t bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * blockDim.x)
         bad |= nonfinite_bf16x8(__ldg(x + i));
@@ -217,6 +220,7 @@ template <int DH, int G>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                            const __grid_constant__ CUtensorMap tm_v, const MaskedFwdArgs a) {
+    chain_wait();
     using P = FwdSmem<DH>;
     constexpr int QT = 128 / G;                                    // queries per M tile
     constexpr int CH = P::CHUNKS;
@@ -498,7 +502,7 @@ cudaError_t launch_fwd_t(const MaskedFwdArgs& a, const gsa_params_t& p, const CU
     auto kern = gsa_masked_attn_fwd_kernel<DH, G>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)(a.row_blocks * p.n_kv * p.B), kFwdThreads, kSmem, st>>>(tq, tk, tv, a);
+    launch_chained(kern, (unsigned)(a.row_blocks * p.n_kv * p.B), kFwdThreads, kSmem, st, tq, tk, tv, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -508,7 +512,7 @@ cudaError_t launch_fwd_t(const MaskedFwdArgs& a, const gsa_params_t& p, const CU
 cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int block_rows, const int32_t* idx,
                                const int32_t* kt, IdxLayout il, uint4* mask, int32_t* general, cudaStream_t st) {
     const dim3 grid((unsigned)(mp.row_pitch / kMaskRowAlign), (unsigned)p.B);
-    gsa_build_masks_kernel<<<grid, kMaskRowAlign * 32, 0, st>>>(idx, kt, mask, il, mp.q0, mp.rows, mp.row_pitch, mp.key_tiles,
+    launch_chained(gsa_build_masks_kernel, grid, kMaskRowAlign * 32, 0, st, idx, kt, mask, il, mp.q0, mp.rows, mp.row_pitch, mp.key_tiles,
                                                                block_rows, p.k_max, p.Lk - p.Lq, general);
     ++g_launches;
     return cudaGetLastError();
@@ -517,7 +521,7 @@ cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int bl
 cudaError_t launch_check_finite(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st) {
     const int64_t n_vec = n_elems / 8;
     const int64_t want = (n_vec + 255) / 256, cap = (int64_t)sm_count() * 8;
-    gsa_check_finite_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, st>>>(reinterpret_cast<const uint4*>(x), n_vec, general);
+    launch_chained(gsa_check_finite_kernel, (unsigned)(want < cap ? want : cap), 256, 0, st, reinterpret_cast<const uint4*>(x), n_vec, general);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -544,7 +548,7 @@ cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, co
     if (p.d_h == DH_ && G == G_) {                                                                                     \
         cudaError_t e = launch_fwd_t<DH_, G_>(a, p, tq, tk, tv, st);                                                   \
         if (e != cudaSuccess) return e;                                                                                \
-        gsa_general_attn_kernel<DH_, G_><<<ctas, 256, 0, st>>>(a.general, Q, K, Vg, g1, idx, kt, il, out, lse,         \
+        launch_chained(gsa_general_attn_kernel<DH_, G_>, ctas, 256, 0, st, a.general, Q, K, Vg, g1, idx, kt, il, out, lse,         \
                                                                dev_status, mp.q0, mp.rows, p.B, p.Lq, p.Lk, p.n_kv,   \
                                                                p.k_max, a.scale_log2);                                \
         ++g_launches;                                                                                                  \

@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
 gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
                            const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                            const MaskedBwdArgs a) {
+    chain_wait();
     using P = KeysSmem<DH, G>;
     using T = TileBytes<DH>;
     constexpr int QT = P::QT, ST = P::STAGES;
@@ -403,6 +404,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1)
 gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
                            const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                            const MaskedBwdArgs a) {
+    chain_wait();
     using P = RowsSmem<DH>;
     using T = TileBytes<DH>;
     constexpr int QT = 128 / G, SL = P::SLOTS;
@@ -578,6 +580,7 @@ struct TargetSmem {
 template <int DH, int G>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const MaskedBwdArgs a) {
+    chain_wait();
     using P = TargetSmem<DH>;
     using T = TileBytes<DH>;
     constexpr int QT = 128 / G;
@@ -748,6 +751,7 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
 // ---- what the tiles cannot take (see gsa_general_attn_kernel) -------------------------------------------------------
 // Only when `general` is raised: fp32 sums of dK, dV' by atomics, one warp per (row, KV head), the set entry by entry.
 __global__ void __launch_bounds__(256) gsa_general_bwd_zero_kernel(const int32_t* __restrict__ general, float4* x, int64_t n) {
+    chain_wait();
     if (*general == 0) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -758,6 +762,7 @@ __global__ void __launch_bounds__(256)
 gsa_general_bwd_rows_kernel(const MaskedBwdArgs a, const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K,
                             const __nv_bfloat16* __restrict__ Vg, const __nv_bfloat16* __restrict__ dOs,
                             float* __restrict__ dK32, float* __restrict__ dV32) {
+    chain_wait();
     if (*a.general == 0) return;
     constexpr int NV = DH / 32;
     const int lane = threadIdx.x & 31;
@@ -825,6 +830,7 @@ gsa_general_bwd_rows_kernel(const MaskedBwdArgs a, const __nv_bfloat16* __restri
 
 __global__ void __launch_bounds__(256) gsa_general_bwd_finish_kernel(const MaskedBwdArgs a, const float* __restrict__ dK32,
                                                                      const float* __restrict__ dV32, int64_t n) {
+    chain_wait();
     if (*a.general == 0) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float sg = 1.0f / (1.0f + __expf(-__bfloat162float(a.g2[i])));
@@ -849,20 +855,20 @@ cudaError_t launch_bwd_t(const MaskedBwdArgs& a, const gsa_params_t& p, const __
     if (e == cudaSuccess) e = set_smem(gsa_masked_bwd_rows_kernel<DH, G>, kSmemR);
     if (e == cudaSuccess) e = set_smem(gsa_masked_target_kernel<DH, G>, kSmemT);
     if (e != cudaSuccess) return e;
-    gsa_masked_bwd_keys_kernel<DH, G><<<(unsigned)(a.key_tiles * p.n_kv * p.B), kBwdThreads, kSmemK, st>>>(tq, td, tk, tv, a);
-    gsa_masked_bwd_rows_kernel<DH, G><<<(unsigned)(a.row_blocks * p.n_kv * p.B), kBwdThreads, kSmemR, st>>>(tq, td, tk, tv, a);
+    launch_chained(gsa_masked_bwd_keys_kernel<DH, G>, (unsigned)(a.key_tiles * p.n_kv * p.B), kBwdThreads, kSmemK, st, tq, td, tk, tv, a);
+    launch_chained(gsa_masked_bwd_rows_kernel<DH, G>, (unsigned)(a.row_blocks * p.n_kv * p.B), kBwdThreads, kSmemR, st, tq, td, tk, tv, a);
     g_launches += 2;
     if (a.pbar) {
         const int pairs = (a.key_tiles + 1) / 2;
         const dim3 grid((unsigned)((pairs + a.pairs_per_cta - 1) / a.pairs_per_cta), (unsigned)a.row_blocks, (unsigned)p.B);
-        gsa_masked_target_kernel<DH, G><<<grid, kBwdThreads, kSmemT, st>>>(tq, tk, a);
+        launch_chained(gsa_masked_target_kernel<DH, G>, grid, kBwdThreads, kSmemT, st, tq, tk, a);
         ++g_launches;
     }
     const int64_t n = (int64_t)p.B * p.Lk * p.n_kv * DH;
     const int ctas = sm_count() * 4;
-    gsa_general_bwd_zero_kernel<<<ctas, 256, 0, st>>>(a.general, reinterpret_cast<float4*>(dKV32), n / 2);
-    gsa_general_bwd_rows_kernel<DH, G><<<ctas, 256, 0, st>>>(a, Q, K, Vg, dOs, dKV32, dKV32 + n);
-    gsa_general_bwd_finish_kernel<<<ctas, 256, 0, st>>>(a, dKV32, dKV32 + n, n);
+    launch_chained(gsa_general_bwd_zero_kernel, ctas, 256, 0, st, a.general, reinterpret_cast<float4*>(dKV32), n / 2);
+    launch_chained(gsa_general_bwd_rows_kernel<DH, G>, ctas, 256, 0, st, a, Q, K, Vg, dOs, dKV32, dKV32 + n);
+    launch_chained(gsa_general_bwd_finish_kernel, ctas, 256, 0, st, a, dKV32, dKV32 + n, n);
     g_launches += 3;
     return cudaGetLastError();
 }

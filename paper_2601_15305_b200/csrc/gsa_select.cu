@@ -212,6 +212,7 @@ __device__ __forceinline__ int budget_from_var(const SelectArgs& a, double var, 
 }
 
 __global__ void __launch_bounds__(kSelThreads, 2) gsa_select_kernel(const SelectArgs a, int q_first, int q_rows) {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     SelShared& sh = *reinterpret_cast<SelShared*>(dyn_smem);
 
@@ -593,6 +594,7 @@ struct ShortShared {
 
 template <int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const SelectArgs a, int q_first, int q_rows) {
+    chain_wait();
     constexpr int NW = NT / 32, BPT = kShortBins / NT;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     ShortShared<NT>& sh = *reinterpret_cast<ShortShared<NT>*>(dyn_smem);
@@ -794,6 +796,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
 __global__ void __launch_bounds__(256) gsa_all_visible_kernel(RowRange rr, IdxLayout il, int32_t Lq, int32_t Lk,
                                                               int32_t k_max, int32_t* __restrict__ idx,
                                                               int32_t* __restrict__ kt, float* __restrict__ var) {
+    chain_wait();
     const int lr = blockIdx.x;
     const int b = rr.b0 + lr / rr.R, t = rr.q_begin + lr % rr.R;
     const int n = Lk - Lq + t + 1;
@@ -810,7 +813,7 @@ cudaError_t launch_short(const SelectArgs& a, int q_first, int q_rows, cudaStrea
     constexpr int smem = (int)sizeof(ShortShared<NT>);
     cudaError_t e = cudaFuncSetAttribute(gsa_select_short_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    gsa_select_short_kernel<NT><<<(unsigned)(a.rr.nb * q_rows), NT, smem, st>>>(a, q_first, q_rows);
+    launch_chained(gsa_select_short_kernel<NT>, (unsigned)(a.rr.nb * q_rows), NT, smem, st, a, q_first, q_rows);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -820,7 +823,7 @@ cudaError_t launch_short(const SelectArgs& a, int q_first, int q_rows, cudaStrea
 cudaError_t launch_all_visible(const gsa_params_t& p, RowRange rr, int32_t* idx, int32_t* kt, float* var,
                                IdxLayout il, cudaStream_t st) {
     if (rr.rows() <= 0) return cudaSuccess;
-    gsa_all_visible_kernel<<<rr.rows(), 256, 0, st>>>(rr, il, p.Lq, p.Lk, p.k_max, idx, kt, var);
+    launch_chained(gsa_all_visible_kernel, rr.rows(), 256, 0, st, rr, il, p.Lq, p.Lk, p.k_max, idx, kt, var);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -850,7 +853,7 @@ cudaError_t launch_select(const gsa_params_t& p, RowRange rr, const float* score
     // (set on every call: the attribute belongs to the current device)
     e = cudaFuncSetAttribute(gsa_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    gsa_select_kernel<<<rr.nb * (t_end - t16), kSelThreads, smem, st>>>(a, t16, t_end - t16);
+    launch_chained(gsa_select_kernel, rr.nb * (t_end - t16), kSelThreads, smem, st, a, t16, t_end - t16);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -15,6 +15,7 @@ constexpr int kVbarThreads = 1024;
 __global__ void __launch_bounds__(kVbarThreads) gsa_vbar_update_kernel(const float* __restrict__ var, int64_t n,
                                                                        float momentum, float* v_bar,
                                                                        float* mean_var) {
+    chain_wait();
     __shared__ double part[kVbarThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     double s = 0.0;
@@ -36,7 +37,7 @@ __global__ void __launch_bounds__(kVbarThreads) gsa_vbar_update_kernel(const flo
 
 cudaError_t launch_vbar_update(const float* var, int64_t n, float momentum, float* v_bar, float* mean_var,
                                cudaStream_t st) {
-    gsa_vbar_update_kernel<<<1, kVbarThreads, 0, st>>>(var, n, momentum, v_bar, mean_var);
+    launch_chained(gsa_vbar_update_kernel, 1, kVbarThreads, 0, st, var, n, momentum, v_bar, mean_var);
     ++g_launches;
     return cudaGetLastError();
 }
