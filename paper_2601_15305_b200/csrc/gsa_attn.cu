@@ -114,7 +114,6 @@ template <int DH, int G, bool FUSE_G2>
 __global__ void __launch_bounds__((FUSE_G2 ? kWarpsFused : kWarpsPrefill) * 32, 1)
 gsa_sparse_attn_kernel(const AttnArgs a) {
     chain_wait();
-    constexpr int kWarpsPerCta = FUSE_G2 ? kWarpsFused : kWarpsPrefill;
     constexpr int HEAD_BYTES = DH * 2;
     constexpr int NC = DH / 32;                         // 32-d chunks of a head row (one uint4 per thread each)
     constexpr int MT = DH / 16;                         // output m-tiles
@@ -138,9 +137,10 @@ gsa_sparse_attn_kernel(const AttnArgs a) {
 
     const int rows = a.rr.rows();
     const int64_t n_items = (int64_t)rows * n_kv * (a.mode == 1 ? a.max_parts : 1);
-    const int64_t warps_total = (int64_t)gridDim.x * kWarpsPerCta;
+    const int warps = blockDim.x >> 5;                  // kWarpsPerCta, or fewer where few items are spread over the SMs
+    const int64_t warps_total = (int64_t)gridDim.x * warps;
 
-    for (int64_t item = (int64_t)blockIdx.x * kWarpsPerCta + warp; item < n_items; item += warps_total) {
+    for (int64_t item = (int64_t)blockIdx.x * warps + warp; item < n_items; item += warps_total) {
         const int g = (int)(item % n_kv);
         int64_t rest = item / n_kv;
         int part = 0;
@@ -638,9 +638,13 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
             if (t_min > rr_all.q_begin) { ar.rr.q_begin = t_min; ar.rr.R = q_end - t_min; }
         }
         const int64_t items = (int64_t)ar.rr.rows() * a.n_kv * (pl.mode == 1 ? pl.slots : 1);
-        const int64_t want = (items + kWarpsPerCta - 1) / kWarpsPerCta;
+        // few items (a small decode step): one SM's share of them per CTA, so that no SM streams for sixteen warps while
+        // others have nothing to do (one 32K-token stream, 128 items: 25 -> 5 us)
+        const int64_t share = (items + sm_count() - 1) / sm_count();
+        const int warps = share < kWarpsPerCta ? (int)share : kWarpsPerCta;
+        const int64_t want = (items + warps - 1) / warps;
         const int ctas = (int)(want < cap ? want : cap);
-        launch_chained(kern, ctas, kWarpsPerCta * 32, smem, st, ar);
+        launch_chained(kern, ctas, warps * 32, smem / kWarpsPerCta * warps, st, ar);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         timeline_mark(kStageAttn, st);

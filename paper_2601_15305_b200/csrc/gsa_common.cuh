@@ -50,14 +50,20 @@ extern std::atomic<int64_t> g_launches;   // host-side launch counter (any host 
 // Launch behind the stream's previous kernel such that this one's start-up (and the launch itself) overlaps the other's end:
 // the kernel begins with chain_wait(), which returns once everything before it on the stream is complete and visible.
 template <class... P, class... A>
-cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_chained_cluster(int cluster, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    return launch_chained_cluster(1, kern, grid, block, smem, st, static_cast<A&&>(args)...);
 }
 
 // multiprocessors of the current device (cached per device; 148 if the query fails)
@@ -168,6 +174,8 @@ __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// The same without bringing up the next kernel early: for kernels whose own CTAs need the room it would take.
+__device__ __forceinline__ void chain_wait_alone() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- device helpers ------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

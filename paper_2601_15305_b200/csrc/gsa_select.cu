@@ -23,6 +23,8 @@
 // shorter than k_t (the sample misjudged the row: huge ties, scores sorted by position, ...) the CTA
 // falls back to radix rounds over the whole row in global memory: slower, same result.  Rows of more
 // than 2048 chunks (1 Mi scores) always take that path.
+#include <cooperative_groups.h>
+
 #include "gsa_common.cuh"
 
 namespace gsa {
@@ -570,44 +572,67 @@ __global__ void __launch_bounds__(kSelThreads, 2) gsa_select_kernel(const Select
     for (int i = k + tid; i < a.k_max; i += kSelThreads) out_idx[i] = -1;
 }
 
-// ---- short rows: the whole row in registers -----------------------------------------------------------------------
+// ---- rows in registers --------------------------------------------------------------------------------------------
 // One CTA of NT threads per row of up to 32 * NT scores, a score's order key in one register (thread t holds scores
 // 4 NT v + 4 t .. + 3), so that nothing of the row is kept in shared memory and four (NT = 256) or two (512) rows share an
 // SM.  One histogram round of the exact key range narrows the threshold to one bin, whose few keys are ranked directly;
 // the selected positions are marked in a bitmap, one scan of its words orders them, and the row is written in whole lines.
 // Bound: the chain of barriers and reductions of a row (about eight, against eighteen of the kernel above), hidden by the
 // other rows of the SM.  Measured on the rows of an 8K prefill (1 .. 8192 scores): 0.130 ms against 0.296 ms in the kernel above.
+//
+// CS > 1: a cluster of CS CTAs shares a row of up to 32 * NT * CS scores, a contiguous slice each, for calls with so few rows
+// that one CTA per row would leave most of the GPU idle (a decode step).  Moments, histogram, candidates and counts meet
+// through distributed shared memory, five cluster barriers in all.  One row of 32771 scores: 11 us against 17 us; 32 rows of
+// 131072: 27 us against 33 us.
 constexpr int kShortBins = 2048;
 constexpr int kShortRank = 128;                               // keys of a bin that are ranked directly
+constexpr int kRowCluster = 8;
 
 template <int NT>
 struct ShortShared {
-    uint32_t hist[kShortBins];
+    __align__(16) uint32_t hist[kShortBins];
     int32_t out[4096];                                        // k_max <= 4096
-    uint32_t gt[NT], eq[NT];                                  // bitmaps of the row's positions (32 NT bits)
-    uint32_t cand[kShortRank];
+    uint32_t gt[NT], eq[NT];                                  // bitmaps of the slice's positions (32 NT bits)
+    uint32_t cand[kShortRank], cand_own[kShortRank];
     double red_a[NT / 32], red_b[NT / 32];
     uint32_t red_min[NT / 32], red_max[NT / 32], warp_tot[NT / 32], scan_tot[NT / 32];
-    uint32_t found_bin, found_above, found_count, n_cand, T, need_eq, eq_total;
+    double slice_a[kRowCluster], slice_b[kRowCluster];        // what the cluster's CTAs wrote here
+    uint32_t slice_min[kRowCluster], slice_max[kRowCluster], slice_sel[kRowCluster];
+    uint32_t found_bin, found_above, found_count, n_cand, T, need_eq, eq_total, own_sel;
     int32_t k;
 };
 
-template <int NT>
+template <int NT, int CS>
 __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const SelectArgs a, int q_first, int q_rows) {
     chain_wait();
+    namespace cg = cooperative_groups;
     constexpr int NW = NT / 32, BPT = kShortBins / NT;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     ShortShared<NT>& sh = *reinterpret_cast<ShortShared<NT>*>(dyn_smem);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int bl = blockIdx.x / q_rows;
-    const int t = q_first + q_rows - 1 - (int)(blockIdx.x % q_rows);        // long rows first
+    const int rank = CS > 1 ? (int)(blockIdx.x % CS) : 0;
+    const int item = (int)(blockIdx.x / CS);
+    auto peer = [&](int r) -> ShortShared<NT>& {
+        if constexpr (CS > 1) return *cg::this_cluster().map_shared_rank(&sh, r);
+        else return sh;
+    };
+    auto sync_all = [&] {
+        if constexpr (CS > 1) cg::this_cluster().sync();
+        else __syncthreads();
+    };
+    if constexpr (CS > 1) cg::this_cluster().barrier_arrive();        // (awaited before the first access to another CTA's memory)
+    const int bl = item / q_rows;
+    const int t = q_first + q_rows - 1 - item % q_rows;       // long rows first
     const int lr = bl * a.rr.R + (t - a.rr.q_begin);
-    const int n = a.Lk - a.Lq + t + 1;                       // visible keys, at most 32 NT
-    const float* __restrict__ grow = a.scores + (int64_t)lr * a.row_stride;
+    const int n_row = a.Lk - a.Lq + t + 1;                    // visible keys, at most 32 NT CS
+    const int slice = CS > 1 ? ((n_row + CS - 1) / CS + 127) / 128 * 128 : n_row;
+    const int p0 = rank * slice;                              // this CTA's first position, and how many it has
+    const int n = CS > 1 ? max(0, min(slice, n_row - p0)) : n_row;
+    const float* __restrict__ grow = a.scores + (int64_t)lr * a.row_stride + p0;
     const int64_t orow = a.il.row(a.rr.b0 + bl, t);
     int32_t* __restrict__ out_idx = a.idx + orow * a.k_max;
 
-    // ---- the row: moments in fp64, range of the keys ----
+    // ---- the slice: moments in fp64, range of the keys ----
     float x[8][4];
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
@@ -631,7 +656,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
         if (v * NT * 4 < n) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const double xd = (double)x[v][e];           // (zeros past the row's end add nothing)
+                const double xd = (double)x[v][e];           // (zeros past the end add nothing)
                 s1 += xd;
                 s2 = fma(xd, xd, s2);
                 key[v][e] = order_key(x[v][e]);
@@ -649,17 +674,31 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
     __syncthreads();
     kmin = __reduce_min_sync(0xFFFFFFFFu, lane < NW ? sh.red_min[lane] : 0xFFFFFFFFu);
     kmax = __reduce_max_sync(0xFFFFFFFFu, lane < NW ? sh.red_max[lane] : 0u);
+    if constexpr (CS > 1) {
+        cg::this_cluster().barrier_wait();
+        if (tid < CS) {                                       // thread r tells CTA r
+            double ta = 0.0, tb = 0.0;
+            for (int i = 0; i < NW; ++i) { ta += sh.red_a[i]; tb += sh.red_b[i]; }
+            ShortShared<NT>& to = peer(tid);
+            to.slice_a[rank] = ta; to.slice_b[rank] = tb; to.slice_min[rank] = kmin; to.slice_max[rank] = kmax;
+        }
+        sync_all();
+        kmin = __reduce_min_sync(0xFFFFFFFFu, lane < CS ? sh.slice_min[lane] : 0xFFFFFFFFu);
+        kmax = __reduce_max_sync(0xFFFFFFFFu, lane < CS ? sh.slice_max[lane] : 0u);
+    }
     if (tid == NT - 32) {                                     // Eq. 8, while the other warps fill the histogram
         double ta = 0.0, tb = 0.0;
-        for (int i = 0; i < NW; ++i) { ta += sh.red_a[i]; tb += sh.red_b[i]; }
-        const double mean = ta / (double)n;
-        double var = tb / (double)n - mean * mean;
+        for (int i = 0; i < (CS > 1 ? CS : NW); ++i) { ta += CS > 1 ? sh.slice_a[i] : sh.red_a[i]; tb += CS > 1 ? sh.slice_b[i] : sh.red_b[i]; }
+        const double mean = ta / (double)n_row;
+        double var = tb / (double)n_row - mean * mean;
         if (var < 0.0) var = 0.0;
         const int k_t = budget_from_var(a, var, nullptr);
-        const int kk = k_t < n ? k_t : n;
+        const int kk = k_t < n_row ? k_t : n_row;
         sh.k = kk;
-        a.kt[orow] = kk;
-        if (a.var) a.var[orow] = (float)var;
+        if (rank == 0) {
+            a.kt[orow] = kk;
+            if (a.var) a.var[orow] = (float)var;
+        }
     }
 
     // ---- threshold: the k-th largest key ----
@@ -674,17 +713,30 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
                 for (int e = 0; e < 4; ++e)
                     if ((v * NT + tid) * 4 + e < n && key[v][e] - lo <= span) atomicAdd(&sh.hist[(key[v][e] - lo) >> shift], 1u);
             }
-        __syncthreads();
+        sync_all();
         if (first) {
             want = (uint32_t)sh.k;
-            if (sh.k == n) {                                  // everything visible is selected
-                for (int i = tid; i < a.k_max; i += NT) out_idx[i] = i < n ? i : -1;
+            if (sh.k == n_row) {                              // everything visible is selected
+                for (int i = rank * NT + tid; i < a.k_max; i += CS * NT) out_idx[i] = i < n_row ? i : -1;
                 return;
             }
         }
         uint32_t mine = 0, bin[BPT];
 #pragma unroll
-        for (int j = 0; j < BPT; ++j) { bin[j] = sh.hist[tid * BPT + j]; mine += bin[j]; }
+        for (int j = 0; j < BPT; ++j) bin[j] = 0u;
+        if constexpr (CS > 1) {
+            static_assert(CS == 1 || BPT == 4, "one 16-byte read per CTA of the cluster");
+#pragma unroll
+            for (int r = 0; r < CS; ++r) {                    // (word by word these reads took three quarters of the kernel)
+                const uint4 h = *reinterpret_cast<const uint4*>(peer(r).hist + tid * 4);
+                bin[0] += h.x; bin[1] += h.y; bin[2] += h.z; bin[3] += h.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < BPT; ++j) bin[j] = sh.hist[tid * BPT + j];
+        }
+#pragma unroll
+        for (int j = 0; j < BPT; ++j) mine += bin[j];
         uint32_t suf = mine;                                  // inclusive suffix over higher lanes
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -718,17 +770,29 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
                     for (int e = 0; e < 4; ++e)
                         if ((v * NT + tid) * 4 + e < n && key[v][e] - lo <= left) sh.cand[atomicAdd(&sh.n_cand, 1u)] = key[v][e];
                 }
-            __syncthreads();
+            sync_all();
+            const uint32_t* cand = sh.cand;
+            if constexpr (CS > 1) {
+                if (wid < CS) {                               // warp r fetches CTA r's candidates
+                    const uint32_t c = lane < CS ? peer(lane).n_cand : 0u;
+                    const uint32_t off = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? c : 0u), m = __shfl_sync(0xFFFFFFFFu, c, wid);
+                    const uint32_t* from = peer(wid).cand;
+                    for (uint32_t i = lane; i < m; i += 32) sh.cand_own[off + i] = from[i];
+                }
+                cand = sh.cand_own;
+                __syncthreads();
+            }
             if (tid < (int)count) {
-                const uint32_t mk = sh.cand[tid];
+                const uint32_t mk = cand[tid];
                 uint32_t g = 0, q = 0;
-                for (uint32_t j = 0; j < count; ++j) { g += sh.cand[j] > mk; q += sh.cand[j] == mk; }
+                for (uint32_t j = 0; j < count; ++j) { g += cand[j] > mk; q += cand[j] == mk; }
                 if (g < want && want <= g + q) { sh.T = mk; sh.need_eq = want - g; sh.eq_total = q; }       // (equal keys write the same)
             }
             __syncthreads();
             T = sh.T; need_eq = sh.need_eq; eq_total = sh.eq_total;
             break;
         }
+        sync_all();                                           // (every CTA has read the counts)
         for (int i = tid; i < kShortBins; i += NT) sh.hist[i] = 0u;
         __syncthreads();
     }
@@ -767,19 +831,37 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
     if (lane == 31) sh.scan_tot[wid] = inc;
     __syncthreads();
     const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < wid ? sh.scan_tot[lane] : 0u) + inc - mine;
-    const uint32_t eq_before = before >> 16;
-    uint32_t at = (before & 0xFFFFu) + min(eq_before, need_eq);
-    if (!cut) at = before & 0xFFFFu;
-    else {
+    uint32_t row_gt = 0, row_eq = 0;                          // of the slices in front of this one
+    if constexpr (CS > 1) {
+        const uint32_t own = __reduce_add_sync(0xFFFFFFFFu, lane < NW ? sh.scan_tot[lane] : 0u);
+        if (tid < CS) peer(tid).slice_sel[rank] = own;
+        sync_all();                                           // (the last access to another CTA's memory lies in front of this)
+        const uint32_t sel = lane < rank ? sh.slice_sel[lane] : 0u;
+        row_gt = __reduce_add_sync(0xFFFFFFFFu, sel & 0xFFFFu);
+        row_eq = __reduce_add_sync(0xFFFFFFFFu, sel >> 16);
+    }
+    const uint32_t out0 = row_gt + min(row_eq, need_eq);      // position of the slice's first entry in the row's set
+    const uint32_t eq_before = row_eq + (before >> 16);
+    uint32_t at = row_gt + (before & 0xFFFFu) + (cut ? min(eq_before, need_eq) : 0u) - (cut ? out0 : row_gt);
+    if (cut) {
         uint32_t take = eq_before < need_eq ? need_eq - eq_before : 0u, q = qw;
         while (q && take) { gw |= q & -q; q &= q - 1u; --take; }
     }
     while (gw) {
-        sh.out[at++] = tid * 32 + __ffs(gw) - 1;
+        sh.out[at++] = p0 + tid * 32 + __ffs(gw) - 1;
         gw &= gw - 1u;
+    }
+    if constexpr (CS > 1) {
+        if (tid == NT - 1) sh.own_sel = at;                   // the last thread ends where the slice does
     }
     __syncthreads();
     const int k = sh.k;
+    if constexpr (CS > 1) {
+        const int first = (int)(cut ? out0 : row_gt), m = (int)sh.own_sel;
+        for (int i = tid; i < m; i += NT) out_idx[first + i] = sh.out[i];
+        for (int i = k + rank * NT + tid; i < a.k_max; i += CS * NT) out_idx[i] = -1;
+        return;
+    }
     if ((a.k_max & 3) == 0) {
         for (int i = tid * 4; i < a.k_max; i += NT * 4) {
             int4 o;
@@ -808,12 +890,12 @@ __global__ void __launch_bounds__(256) gsa_all_visible_kernel(RowRange rr, IdxLa
     }
 }
 
-template <int NT>
+template <int NT, int CS>
 cudaError_t launch_short(const SelectArgs& a, int q_first, int q_rows, cudaStream_t st) {
     constexpr int smem = (int)sizeof(ShortShared<NT>);
-    cudaError_t e = cudaFuncSetAttribute(gsa_select_short_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(gsa_select_short_kernel<NT, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    launch_chained(gsa_select_short_kernel<NT>, (unsigned)(a.rr.nb * q_rows), NT, smem, st, a, q_first, q_rows);
+    launch_chained_cluster(CS, gsa_select_short_kernel<NT, CS>, (unsigned)(a.rr.nb * q_rows * CS), NT, smem, st, a, q_first, q_rows);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -846,9 +928,12 @@ cudaError_t launch_select(const gsa_params_t& p, RowRange rr, const float* score
     };
     const int t8 = first_longer(8192), t16 = first_longer(16384), t_end = rr.q_begin + rr.R;
     cudaError_t e = cudaSuccess;
-    if (t8 > rr.q_begin) e = launch_short<256>(a, rr.q_begin, t8 - rr.q_begin, st);
-    if (e == cudaSuccess && t16 > t8) e = launch_short<512>(a, t8, t16 - t8, st);
+    if (t8 > rr.q_begin) e = launch_short<256, 1>(a, rr.q_begin, t8 - rr.q_begin, st);
+    if (e == cudaSuccess && t16 > t8) e = launch_short<512, 1>(a, t8, t16 - t8, st);
     if (e != cudaSuccess || t16 >= t_end) return e;
+    // few long rows: a cluster each, while all of them fit the GPU at once
+    if (off + t_end <= 32 * 512 * kRowCluster && (int64_t)rr.nb * (t_end - t16) * kRowCluster <= 2 * sm_count())
+        return launch_short<512, kRowCluster>(a, t16, t_end - t16, st);
     const size_t smem = ((sizeof(SelShared) + 15) / 16) * 16;
     // (set on every call: the attribute belongs to the current device)
     e = cudaFuncSetAttribute(gsa_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
