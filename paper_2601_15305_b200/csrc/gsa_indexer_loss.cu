@@ -262,9 +262,10 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
     }
 
     const __nv_bfloat16* const kbase = a.kI + (size_t)b * a.Lk * DI;
-    auto fetch = [&](int j, int stage) {
+    // positions are read a tile ahead of the copies they address: a tile then waits for one memory latency, not for two
+    auto positions = [&](int j) -> int32_t { return j < ke ? checked_pos(S[min(j + (lane & 15), ke - 1)], a.Lk, a.dev_status) : 0; };
+    auto fetch = [&](int j, int stage, int32_t pos16) {
         if (j < ke) {
-            const int32_t pos16 = checked_pos(S[min(j + (lane & 15), ke - 1)], a.Lk, a.dev_status);
 #pragma unroll
             for (int i = 0; i < 16 * CPR / 32; ++i) {
                 const int chunk = i * 32 + lane;
@@ -304,9 +305,11 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
 
     // ---- sweep 1: log-sum-exp of the scores, sum pbar, sum pbar I, sum pbar log pbar ------------------
     float m_run = -INFINITY, l_run = 0.f, s_p = 0.f, s_pi = 0.f, s_plp = 0.f;
-    fetch(0, 0);
+    int32_t pos_next = positions(16);
+    fetch(0, 0, positions(0));
     for (int j0 = 0, stage = 0; j0 < ke; j0 += 16, stage ^= 1) {
-        fetch(j0 + 16, stage ^ 1);
+        fetch(j0 + 16, stage ^ 1, pos_next);
+        pos_next = positions(j0 + 32);
         const bool v0 = j0 + gid < ke, v1 = j0 + gid + 8 < ke;
         const float p0 = v0 ? prow[j0 + gid] : 0.f, p1 = v1 ? prow[j0 + gid + 8] : 0.f;
         cp_async_wait<1>();
@@ -346,10 +349,14 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
 #pragma unroll
     for (int mt = 0; mt < KS; ++mt) dq[mt][0] = dq[mt][1] = dq[mt][2] = dq[mt][3] = 0.f;
     float dw_acc[2] = {0.f, 0.f}, db_acc[2] = {0.f, 0.f};
-    fetch(0, 0);
+    int32_t pos_cur = positions(0);
+    pos_next = positions(16);
+    fetch(0, 0, pos_cur);
     for (int j0 = 0, stage = 0; j0 < ke; j0 += 16, stage ^= 1) {
-        const int32_t pos16 = checked_pos(S[min(j0 + (lane & 15), ke - 1)], a.Lk, a.dev_status);
-        fetch(j0 + 16, stage ^ 1);
+        const int32_t pos16 = pos_cur;
+        fetch(j0 + 16, stage ^ 1, pos_next);
+        pos_cur = pos_next;
+        pos_next = positions(j0 + 32);
         const bool v0 = j0 + gid < ke, v1 = j0 + gid + 8 < ke;
         const float p0 = v0 ? prow[j0 + gid] : 0.f, p1 = v1 ? prow[j0 + gid + 8] : 0.f;
         cp_async_wait<1>();

@@ -17,6 +17,8 @@
 //
 // Roles in all three: warps 0-15 the elementwise work (four warpgroups side by side, 32 columns of a tile each: with two of
 // them the products waited for it), warp 16 copies, warp 17 MMA issue, 18 and 19 small loads.
+#include <cooperative_groups.h>
+
 #include "gsa_masked.cuh"
 
 namespace gsa {
@@ -144,7 +146,7 @@ struct KeysSmem {
     static constexpr int ALLOC = OFF_ABORT + 8 + 1024;
 };
 
-template <int DH, int G>
+template <int DH, int G, int SPLIT>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
                            const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -164,13 +166,18 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     const uint32_t bar_kv = bar0 + 8u * (5 * ST), bar_s = bar_kv + 8, bar_dp = bar_kv + 16, bar_p = bar_kv + 24,
                    bar_ds = bar_kv + 32, bar_done = bar_kv + 40, bar_drain = bar_kv + 48;
 
-    // early key tiles (the longest) first; (batch element, KV head) outermost
-    const int tile = blockIdx.x % a.key_tiles, bh = blockIdx.x / a.key_tiles;
+    // early key tiles (the longest) first; (batch element, KV head) outermost.  SPLIT = 2: a cluster of two CTAs shares a tile's
+    // rows, every other row tile each, for calls whose key tiles leave half of the SMs without work; the second CTA's
+    // sums go to the first through distributed shared memory at the end.
+    const int part_of = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) : 0;
+    const int item = (int)(blockIdx.x / SPLIT);
+    const int tile = item % a.key_tiles, bh = item / a.key_tiles;
     const int g = bh % a.n_kv, b = bh / a.n_kv;
     const int off = a.Lk - a.Lq;
     const int r_first = max(0, tile * kMaskTileKeys - off - a.q0);           // first row that sees a key of the tile
-    const int i0 = r_first / QT;
-    const int n = r_first < a.rows ? a.row_blocks - i0 : 0;                  // (tiles that no row sees have no masks)
+    const int i0 = r_first / QT + part_of;
+    // (tiles that no row sees have no masks)
+    const int n = r_first < a.rows && i0 < a.row_blocks ? (a.row_blocks - i0 + SPLIT - 1) / SPLIT : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < ST; ++s) {
@@ -182,6 +189,7 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     }
     const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
     int copies = 0, kv_issued = 0, released = 0;
+    bool done = false;
 
     if (warp == kCopyWarp) {
         if (lane == 0 && n > 0) {
@@ -196,7 +204,7 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 const int s = i % ST;
                 if (!mbar_wait(bar_free(s), ((i / ST) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
                 const uint32_t dst = sbase + P::OFF_RING + s * 2 * T::TILE;
-                const int z = (i0 + i) * QT;
+                const int z = (i0 + i * SPLIT) * QT;
                 mbar_expect_tx(bar_q(s), T::TILE);
                 for (int c = 0; c < T::CHUNKS; ++c) tma_load_tile(dst + c * T::CHUNK, &tm_q, c * 64, g * G, z, b, bar_q(s));
                 mbar_expect_tx(bar_d(s), T::TILE);
@@ -249,14 +257,14 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             uint4 mk[2];
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const int m = j + 64 * u, r = (i0 + i) * QT + m / G;
+                const int m = j + 64 * u, r = (i0 + i * SPLIT) * QT + m / G;
                 l2[u] = dl[u] = 0.f;
                 if (r < a.rows) {
                     const size_t at = ((size_t)b * a.Lq + a.q0 + r) * a.n_h + g * G + m % G;
                     l2[u] = a.lse[at] * kLog2e;
                     dl[u] = a.delta[at];
                 }
-                const int rq = (i0 + i) * QT + m;                  // (this thread's query for the masks)
+                const int rq = (i0 + i * SPLIT) * QT + m;                  // (this thread's query for the masks)
                 mk[u] = make_uint4(0u, 0u, 0u, 0u);
                 if (m < QT && rq < a.rows) mk[u] = a.mask[((int64_t)b * a.key_tiles + tile) * a.row_pitch + rq];
             }
@@ -332,24 +340,59 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             __syncwarp();
             if (lane == 0) { mbar_arrive(bar_ds); mbar_arrive(bar_statfree(s)); }
         }
-        if (ok && n > 0 && !mbar_wait(bar_done, 0, s_abort, a.wait_cycles)) ok = false;
-        if (!ok) {
-            if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
+        done = ok && (n == 0 || mbar_wait(bar_done, 0, s_abort, a.wait_cycles));
+        if (!done && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
+        tc_fence_after();
+    }
+    // ---- sums: dK and dV' of key (quad, lane), columns part * DH / 4 .. of the head ----
+    const int part = (warp & 15) >> 2, quad = warp & 3;
+    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
+    auto sums = [&](int c, uint32_t (&dk)[16], uint32_t (&dv)[16]) {       // 16 columns
+        if (n > 0) {
+            tc_ld16(lane_base + kTmK + part * (DH / 4) + 16 * c, dk);
+            tc_wait_ld16(dk);
+            tc_ld16(lane_base + kTmV + part * (DH / 4) + 16 * c, dv);
+            tc_wait_ld16(dv);
         } else {
-            tc_fence_after();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) dk[e] = dv[e] = 0u;
+        }
+    };
+    // (the ring of the first CTA is free once both have come here; one float per column and key, lanes side by side)
+    float* const other = reinterpret_cast<float*>(smem + P::OFF_RING) + part * (DH / 4) * 128 + quad * 32 + lane;
+    if constexpr (SPLIT > 1) {
+        namespace cg = cooperative_groups;
+        static_assert(P::STAGES * 2 * T::TILE >= 2 * DH * 128 * 4, "the second CTA's sums fit the ring");
+        cg::this_cluster().sync();
+        if (part_of == 1 && warp < 16 && done) {
+            float* const to = cg::this_cluster().map_shared_rank(other, 0);
+#pragma unroll
+            for (int c = 0; c < DH / 64; ++c) {
+                uint32_t dk[16], dv[16];
+                sums(c, dk, dv);
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    to[(16 * c + e) * 128] = __uint_as_float(dk[e]);
+                    to[(DH + 16 * c + e) * 128] = __uint_as_float(dv[e]);
+                }
+            }
+        }
+        cg::this_cluster().sync();
+    }
+    if (warp < 16 && part_of == 0 && done) {
+        {
             const int key = tile * kMaskTileKeys + quad * 32 + lane;
             const size_t at = (((size_t)b * a.Lk + min(key, a.Lk - 1)) * a.n_kv + g) * DH + part * (DH / 4);
 #pragma unroll
             for (int c = 0; c < DH / 64; ++c) {
                 uint32_t dk[16], dv[16];
-                if (n > 0) {
-                    tc_ld16(lane_base + kTmK + part * (DH / 4) + 16 * c, dk);
-                    tc_wait_ld16(dk);
-                    tc_ld16(lane_base + kTmV + part * (DH / 4) + 16 * c, dv);
-                    tc_wait_ld16(dv);
-                } else {
+                sums(c, dk, dv);
+                if constexpr (SPLIT > 1) {
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) dk[e] = dv[e] = 0u;
+                    for (int e = 0; e < 16; ++e) {
+                        dk[e] = __float_as_uint(__uint_as_float(dk[e]) + other[(16 * c + e) * 128]);
+                        dv[e] = __float_as_uint(__uint_as_float(dv[e]) + other[(DH + 16 * c + e) * 128]);
+                    }
                 }
                 if (key >= a.Lk) continue;
 #pragma unroll
@@ -851,11 +894,16 @@ cudaError_t launch_bwd_t(const MaskedBwdArgs& a, const gsa_params_t& p, const __
     auto set_smem = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
     constexpr int kSmemK = KeysSmem<DH, G>::ALLOC, kSmemR = RowsSmem<DH>::ALLOC, kSmemT = TargetSmem<DH>::ALLOC;
     static_assert(kSmemK <= 232448 && kSmemR <= 232448 && kSmemT <= 232448, "shared memory of one CTA");
-    cudaError_t e = set_smem(gsa_masked_bwd_keys_kernel<DH, G>, kSmemK);
+    // one wave of key tiles at most: two CTAs per tile (2 x 2051 keys, two KV heads: 68 tiles, 103 -> 65 us)
+    const int key_ctas = a.key_tiles * p.n_kv * p.B, split = key_ctas <= sm_count() && a.row_blocks > 1 ? 2 : 1;
+    cudaError_t e = split == 2 ? set_smem(gsa_masked_bwd_keys_kernel<DH, G, 2>, kSmemK) : set_smem(gsa_masked_bwd_keys_kernel<DH, G, 1>, kSmemK);
     if (e == cudaSuccess) e = set_smem(gsa_masked_bwd_rows_kernel<DH, G>, kSmemR);
     if (e == cudaSuccess) e = set_smem(gsa_masked_target_kernel<DH, G>, kSmemT);
     if (e != cudaSuccess) return e;
-    launch_chained(gsa_masked_bwd_keys_kernel<DH, G>, (unsigned)(a.key_tiles * p.n_kv * p.B), kBwdThreads, kSmemK, st, tq, td, tk, tv, a);
+    if (split == 2)
+        launch_chained_cluster(2, gsa_masked_bwd_keys_kernel<DH, G, 2>, (unsigned)(key_ctas * 2), kBwdThreads, kSmemK, st, tq, td, tk, tv, a);
+    else
+        launch_chained(gsa_masked_bwd_keys_kernel<DH, G, 1>, (unsigned)key_ctas, kBwdThreads, kSmemK, st, tq, td, tk, tv, a);
     launch_chained(gsa_masked_bwd_rows_kernel<DH, G>, (unsigned)(a.row_blocks * p.n_kv * p.B), kBwdThreads, kSmemR, st, tq, td, tk, tv, a);
     g_launches += 2;
     if (a.pbar) {
