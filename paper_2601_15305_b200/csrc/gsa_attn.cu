@@ -659,24 +659,49 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
     return finalize(finalized_to, q_end);
 }
 
-// First row from which the gather is the cheaper path (rr.q_begin: all of them; its end: none).
-// A gathered pair costs 36 ps per KV head at d_h = 128 and 24 ps at 64 (L2 rate, measured at L = 16K for 1, 2, 4 and 8
-// query heads per KV head), a visible pair of a masked tile 0.53 / 0.43 ps per query head: the tiles win while a row sees
-// fewer than 68 / G (56 / G) times the keys it selects.  The sets' sizes are on the device; the budget they centre on
-// stands for them.  Fewer CTAs than two thirds of the SMs leave too much of the GPU idle.
-int masked_rows_end(const gsa_params_t& p, const RowRange& rr) {
-    const int G = p.n_h / p.n_kv, q_end = rr.q_begin + rr.R;
-    int64_t t_end = q_end;
-    if (p.k_mode != 3) {
-        const int64_t k = p.k_base < p.k_min ? p.k_min : (p.k_base > p.k_max ? p.k_max : p.k_base);
-        t_end = k * (p.d_h == 128 ? 68 : 56) / G - (p.Lk - p.Lq);
+// First row from which the gather is the cheaper path (rr.q_begin: all of them; its end: none), from two models in
+// microseconds.  Tiles: a CTA takes 2.1 (d_h = 64: 1.9) per key tile of its 256 (row, head) rows and the GPU one CTA per SM,
+// plus 10 for the masks, the start and the plain kernel's launch (measured at L = 32K and 16K).  Gather: 36 ps (24) per pair
+// and KV head, 41 (27) out of several key ranges (measured at L = 16K and 128K for 1, 2, 4 and 8 query heads per KV head),
+// and a warp's own chain of 16-key steps where a call has few rows.
+struct ForwardCosts {
+    double tile_us, pair_us;
+    int block;
+    double tiles(const gsa_params_t& p, int nb, int q0, int rows, int64_t rows_per_chunk) const {
+        if (rows <= 0) return 0.0;
+        const RowsWork w = rows_work(p, nb, q0, rows, block);
+        const double chunks = (double)((rows + rows_per_chunk - 1) / rows_per_chunk);
+        const double all = w.key_tiles * p.n_kv / sm_count(), longest = w.chain * chunks;
+        return (all > longest ? all : longest) * tile_us + 10.0;
     }
-    const int block = masked_block_rows(p);
-    if (t_end <= rr.q_begin) return rr.q_begin;
-    if (t_end + 4 * block >= q_end) t_end = q_end;                 // (a short rest is not worth the gather's launches)
-    else t_end = rr.q_begin + (t_end - rr.q_begin) / block * block;
-    const int64_t ctas = (t_end - rr.q_begin + block - 1) / block * p.n_kv * rr.nb;
-    return ctas * 3 >= 2 * sm_count() ? (int)t_end : rr.q_begin;
+    double gather(const gsa_params_t& p, const AttnPlan& pl, int nb, int q0, int rows) const {
+        if (rows <= 0) return 0.0;
+        const RowsWork w = rows_work(p, nb, q0, rows, block);
+        const double all = w.selected * p.n_kv * pair_us;
+        const double longest = w.selected / ((double)nb * rows) / kTileKeys / (pl.mode == 1 ? pl.slots : 1) * 0.45;
+        return (all > longest ? all : longest) + 5.0 + 2.0 * pl.n_ranges;
+    }
+};
+
+int masked_rows_end(const gsa_params_t& p, const AttnPlan& pl, const RowRange& rr, size_t scratch_bytes) {
+    const int q_end = rr.q_begin + rr.R;
+    ForwardCosts c;
+    c.block = masked_block_rows(p);
+    c.tile_us = p.d_h == 128 ? 2.1 : 1.9;
+    c.pair_us = (p.d_h == 128 ? 36e-6 : 24e-6) * (pl.n_ranges > 1 ? 41.0 / 36.0 : 1.0);
+    const int64_t per = (int64_t)(scratch_bytes / (mask_plan(p, 0, kMaskRowAlign).bytes(p.B) / kMaskRowAlign)) / c.block * c.block;
+    if (per < c.block) return rr.q_begin;                          // (no room for the masks of one block of rows)
+    // the row that sees so many keys that its share of a block's tiles costs what gathering its set does
+    const int64_t k = p.k_mode == 3 ? p.Lk : (p.k_base < p.k_min ? p.k_min : (p.k_base > p.k_max ? p.k_max : p.k_base));
+    const double even = (double)k * c.pair_us * sm_count() * kMaskTileKeys * c.block / c.tile_us - (p.Lk - p.Lq);
+    int cut = even >= q_end ? q_end : (even <= rr.q_begin ? rr.q_begin : rr.q_begin + ((int)even - rr.q_begin) / c.block * c.block);
+    double best = c.gather(p, pl, rr.nb, rr.q_begin, rr.R);
+    int t_end = rr.q_begin;
+    for (const int t : {cut, q_end}) {
+        const double us = c.tiles(p, rr.nb, rr.q_begin, t - rr.q_begin, per) + c.gather(p, pl, rr.nb, t, q_end - t);
+        if (us < best) { best = us; t_end = t; }
+    }
+    return t_end;
 }
 
 cudaError_t launch_masked_rows(const gsa_params_t& p, const RowRange& rr, int t_end, const __nv_bfloat16* Q,
@@ -745,16 +770,17 @@ cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bf
                                cudaStream_t st, AttnProgress* progress, float* lse, bool values_scanned) {
     if (rr.rows() <= 0) return cudaSuccess;
     const AttnPlan pl = plan_attn(p);
-    if (!g2 && pl.mode == 0 && t_dev_status) {
+    const size_t scratch_bytes = (pl.state_bytes + 255) / 256 * 256 + pl.cuts_bytes;
+    if (!g2 && t_dev_status) {
         // rows whose sets hold a large enough share of what they see: masked tiles, in chunks whose masks fit the scratch
-        const int t_end = masked_rows_end(p, rr);
+        const int t_end = masked_rows_end(p, pl, rr, scratch_bytes);
         if (t_end > rr.q_begin) {
             cudaError_t e = cudaSuccess;
             if (!values_scanned)
                 e = launch_check_finite(V, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, t_dev_status + kStatusGeneralWord, st);
             if (e != cudaSuccess) return e;
-            e = launch_masked_rows(p, rr, t_end, Q, K, V, g1, idx, kt, il, out, scratch,
-                                               (pl.state_bytes + 255) / 256 * 256 + pl.cuts_bytes, st, progress, lse);
+            e = launch_masked_rows(p, rr, t_end, Q, K, V, g1, idx, kt, il, out, scratch, scratch_bytes, st,
+                                   progress, lse);
             if (e != cudaSuccess || t_end >= rr.q_begin + rr.R) return e;
             rr.R = rr.q_begin + rr.R - t_end;
             rr.q_begin = t_end;

@@ -42,6 +42,27 @@ cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int bl
 // Raises *general if one of n_elems (a multiple of 8) values is infinite or NaN.
 cudaError_t launch_check_finite(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st);
 
+// What a range of rows sees and selects, per KV head: for the choice between the tiles and the gather.  The sets' sizes are on
+// the device; the budget that they centre on stands for them.
+struct RowsWork {
+    double key_tiles;          // key tiles of the blocks of `block` rows, all batch elements
+    double chain;              // ... of the last block
+    double selected;           // selected (row, key) pairs, all batch elements
+};
+inline RowsWork rows_work(const gsa_params_t& p, int nb, int q0, int rows, int block) {
+    const double first = (double)p.Lk - p.Lq + q0 + 1, last = first + rows - 1;        // keys the first and the last row see
+    const int64_t k64 = p.k_mode == 3 ? p.Lk : (p.k_base < p.k_min ? p.k_min : (p.k_base > p.k_max ? p.k_max : p.k_base));
+    const double k = (double)k64;
+    RowsWork w;
+    const double blocks = (double)((rows + block - 1) / block);
+    w.chain = last / kMaskTileKeys + 1.0;
+    w.key_tiles = nb * blocks * (0.5 * (first + last) / kMaskTileKeys + 0.5 * block / kMaskTileKeys + 0.5);
+    if (w.key_tiles > nb * blocks * w.chain) w.key_tiles = nb * blocks * w.chain;
+    const double short_rows = k <= first ? 0.0 : (k >= last ? rows : k - first);      // rows that see fewer keys than the budget
+    w.selected = nb * (short_rows * (first + 0.5 * short_rows) + (rows - short_rows) * k);
+    return w;
+}
+
 // query rows of a forward CTA (two M = 128 tiles of (query, head of the group) rows)
 inline int masked_block_rows(const gsa_params_t& p) { return 256 / (p.n_h / p.n_kv); }
 

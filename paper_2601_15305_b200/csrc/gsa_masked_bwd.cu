@@ -929,17 +929,23 @@ size_t masked_bwd_bytes(const gsa_params_t& p, const RowRange& rr) {
     return ((masks > sums ? masks : sums) + 255) / 256 * 256;
 }
 
-// A gathered pair of the backward costs 1.4 ns at 16 heads of 128 on 8 KV heads (12 KB of rows; L = 32K: 92 ms with the loss
-// target), a visible pair of the tiles 31 ps (16.5 ms): the line is drawn at a mean share of 1 / 50, where both take about as
-// long; as in the forward (masked_rows_end) it moves with the heads per KV head, which a gathered row serves together.
+// Two models in microseconds, as in the forward (masked_rows_end).  Tiles: 1.7 + 1.45 + 1.05 (d_h = 64: 1.3 + 1.1 + 0.9) per
+// 128 x 128 tile in the keys, rows and target kernels, one CTA per SM, 40 for the launches around them (the target is charged
+// whether it is asked for or not).  Gather: 0.115 ps per byte of the K, V', Q and do rows that a pair moves (1.41 ns at 16
+// heads of 128 on 8 KV heads, measured at L = 32K), 20 for its launches.  Fewer row tiles than half of the SMs: the gather.
 bool masked_bwd_preferred(const gsa_params_t& p, const RowRange& rr) {
-    const int G = p.n_h / p.n_kv;
-    const int64_t block = masked_block_rows(p);
-    if (((int64_t)rr.R + block - 1) / block * p.n_kv * rr.nb * 3 < 2 * sm_count()) return false;
-    if (p.k_mode == 3) return true;
-    const int64_t k = p.k_base < p.k_min ? p.k_min : (p.k_base > p.k_max ? p.k_max : p.k_base);
-    const int64_t mean_visible = p.Lk - p.Lq + rr.q_begin + rr.R / 2;
-    return mean_visible * G < k * (p.d_h == 128 ? 100 : 80);
+    const int G = p.n_h / p.n_kv, block = 128 / G;
+    const double ctas = (double)((rr.R + block - 1) / block) * p.n_kv * rr.nb, sms = sm_count();
+    if (2.0 * ctas < sms) return false;
+    const RowsWork w = rows_work(p, rr.nb, rr.q_begin, rr.R, block);
+    const double all = w.key_tiles * p.n_kv / sms, row_tiles = (double)((rr.R + block - 1) / block);
+    const double key_ctas = (double)((p.Lk + kMaskTileKeys - 1) / kMaskTileKeys) * p.n_kv * rr.nb;
+    const double keys_chain = key_ctas <= sms ? 0.5 * row_tiles : row_tiles;
+    const bool wide = p.d_h == 128;
+    const double tiles = (all > keys_chain ? all : keys_chain) * (wide ? 1.7 : 1.3) + (all > w.chain ? all : w.chain) * (wide ? 1.45 : 1.1) +
+                         all * (wide ? 1.05 : 0.9) + 40.0;
+    const double gather = w.selected * 4.0 * (p.n_kv + p.n_h) * p.d_h * 0.115e-6 + 20.0;
+    return tiles < gather;
 }
 
 cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,

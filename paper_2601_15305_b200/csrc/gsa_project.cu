@@ -54,7 +54,6 @@ struct ProjArgs {
 __global__ void __launch_bounds__(kPThreads, 1)
 gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
                    const ProjArgs a) {
-    chain_wait();
     {   // an earlier CTA or launch gave up: leave, all threads together (one thread reads the word)
         __shared__ int s_go;
         if (threadIdx.x == 0) s_go = *reinterpret_cast<volatile int32_t*>(a.dev_status) == kDevOk;
@@ -267,7 +266,7 @@ cudaError_t launch_project(const gsa_params_t& p, int d_model, const __nv_bfloat
     if (e != cudaSuccess) return e;
     const int sms = sm_count();
     const int tiles = a.m_tiles * a.n_tiles;
-    launch_chained(gsa_project_kernel, tiles < sms ? tiles : sms, kPThreads, kSmemTotal, st, tm_h, tm_w, a);
+    gsa_project_kernel<<<tiles < sms ? tiles : sms, kPThreads, kSmemTotal, st>>>(tm_h, tm_w, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -292,7 +291,7 @@ cudaError_t launch_gemm_bf16(int M, int K, int N, const __nv_bfloat16* A, const 
     if (e != cudaSuccess) return e;
     const int sms = sm_count();
     const int tiles = a.m_tiles * a.n_tiles;
-    launch_chained(gsa_project_kernel, tiles < sms ? tiles : sms, kPThreads, kSmemTotal, st, tm_a, tm_b, a);
+    gsa_project_kernel<<<tiles < sms ? tiles : sms, kPThreads, kSmemTotal, st>>>(tm_a, tm_b, a);
     ++g_launches;
     return cudaGetLastError();
 }
