@@ -584,13 +584,14 @@ __global__ void __launch_bounds__(kSelThreads, 2) gsa_select_kernel(const Select
 // that one CTA per row would leave most of the GPU idle (a decode step).  Moments, histogram, candidates and counts meet
 // through distributed shared memory, five cluster barriers in all.  One row of 32771 scores: 11 us against 17 us; 32 rows of
 // 131072: 27 us against 33 us.
-constexpr int kShortBins = 2048;
+constexpr int short_bins(int NT) { return NT == 128 ? 1024 : 2048; }
+constexpr int short_bins_log2(int NT) { return NT == 128 ? 10 : 11; }
 constexpr int kShortRank = 128;                               // keys of a bin that are ranked directly
 constexpr int kRowCluster = 8;
 
 template <int NT>
 struct ShortShared {
-    __align__(16) uint32_t hist[kShortBins];
+    __align__(16) uint32_t hist[short_bins(NT)];
     int32_t out[4096];                                        // k_max <= 4096
     uint32_t gt[NT], eq[NT];                                  // bitmaps of the slice's positions (32 NT bits)
     uint32_t cand[kShortRank], cand_own[kShortRank];
@@ -606,7 +607,7 @@ template <int NT, int CS>
 __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const SelectArgs a, int q_first, int q_rows) {
     chain_wait();
     namespace cg = cooperative_groups;
-    constexpr int NW = NT / 32, BPT = kShortBins / NT;
+    constexpr int NW = NT / 32, BINS = short_bins(NT), BPT = BINS / NT;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     ShortShared<NT>& sh = *reinterpret_cast<ShortShared<NT>*>(dyn_smem);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -633,34 +634,41 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
     int32_t* __restrict__ out_idx = a.idx + orow * a.k_max;
 
     // ---- the slice: moments in fp64, range of the keys ----
+    // (a score past the end is 0 in the moments and has key 0, which no score has: below every threshold and outside every
+    // range of keys, so that nothing after this asks for positions)
     float x[8][4];
+    uint32_t key[8][4];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        const int i = (v * NT + tid) * 4;
-        if (i + 4 <= n) {
-            const float4 f = __ldg(reinterpret_cast<const float4*>(grow + i));
-            x[v][0] = f.x; x[v][1] = f.y; x[v][2] = f.z; x[v][3] = f.w;
-        } else {
+    for (int v = 0; v < 8; ++v)
+        if (v * NT * 4 < n) {
+            const int i = (v * NT + tid) * 4;
+            if (i + 4 <= n) {
+                const float4 f = __ldg(reinterpret_cast<const float4*>(grow + i));
+                x[v][0] = f.x; x[v][1] = f.y; x[v][2] = f.z; x[v][3] = f.w;
+            } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) x[v][e] = i + e < n ? __ldg(grow + i + e) : 0.f;
+                for (int e = 0; e < 4; ++e) x[v][e] = i + e < n ? __ldg(grow + i + e) : __uint_as_float(0xFFFFFFFFu);
+            }
         }
-    }
-    for (int i = tid; i < kShortBins; i += NT) sh.hist[i] = 0u;
+    for (int i = tid; i < BINS / 4; i += NT) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     sh.gt[tid] = 0u;
     sh.eq[tid] = 0u;
     if (tid == 0) sh.n_cand = 0u;
     double s1 = 0.0, s2 = 0.0;
-    uint32_t key[8][4], kmin = 0xFFFFFFFFu, kmax = 0u;
+    uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;                   // (kmin of key - 1: key 0 goes to the top)
 #pragma unroll
     for (int v = 0; v < 8; ++v)
         if (v * NT * 4 < n) {
+            const bool whole = (v + 1) * NT * 4 <= n;         // (uniform)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const double xd = (double)x[v][e];           // (zeros past the end add nothing)
+                const bool in = whole || (v * NT + tid) * 4 + e < n;
+                const double xd = in ? (double)x[v][e] : 0.0;
                 s1 += xd;
                 s2 = fma(xd, xd, s2);
-                key[v][e] = order_key(x[v][e]);
-                if ((v * NT + tid) * 4 + e < n) { kmin = min(kmin, key[v][e]); kmax = max(kmax, key[v][e]); }
+                key[v][e] = in ? order_key(x[v][e]) : 0u;
+                kmin = min(kmin, key[v][e] - 1u);
+                kmax = max(kmax, key[v][e]);
             }
         }
 #pragma unroll
@@ -674,6 +682,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
     __syncthreads();
     kmin = __reduce_min_sync(0xFFFFFFFFu, lane < NW ? sh.red_min[lane] : 0xFFFFFFFFu);
     kmax = __reduce_max_sync(0xFFFFFFFFu, lane < NW ? sh.red_max[lane] : 0u);
+    if constexpr (CS == 1) kmin += 1u;
     if constexpr (CS > 1) {
         cg::this_cluster().barrier_wait();
         if (tid < CS) {                                       // thread r tells CTA r
@@ -683,7 +692,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
             to.slice_a[rank] = ta; to.slice_b[rank] = tb; to.slice_min[rank] = kmin; to.slice_max[rank] = kmax;
         }
         sync_all();
-        kmin = __reduce_min_sync(0xFFFFFFFFu, lane < CS ? sh.slice_min[lane] : 0xFFFFFFFFu);
+        kmin = __reduce_min_sync(0xFFFFFFFFu, lane < CS ? sh.slice_min[lane] : 0xFFFFFFFFu) + 1u;
         kmax = __reduce_max_sync(0xFFFFFFFFu, lane < CS ? sh.slice_max[lane] : 0u);
     }
     if (tid == NT - 32) {                                     // Eq. 8, while the other warps fill the histogram
@@ -705,13 +714,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
     uint32_t lo = kmin, hi = kmax, want = 0, T, need_eq, eq_total;
     for (bool first = true;; first = false) {
         const uint32_t span = hi - lo;
-        const int bits = 32 - __clz(span), shift = bits > 11 ? bits - 11 : 0;       // (span >> shift) < kShortBins
+        const int bits = 32 - __clz(span), shift = bits > short_bins_log2(NT) ? bits - short_bins_log2(NT) : 0;       // (span >> shift) < BINS
 #pragma unroll
         for (int v = 0; v < 8; ++v)
             if (v * NT * 4 < n) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if ((v * NT + tid) * 4 + e < n && key[v][e] - lo <= span) atomicAdd(&sh.hist[(key[v][e] - lo) >> shift], 1u);
+                    if (key[v][e] - lo <= span) atomicAdd(&sh.hist[(key[v][e] - lo) >> shift], 1u);
             }
         sync_all();
         if (first) {
@@ -768,7 +777,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
                 if (v * NT * 4 < n) {
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
-                        if ((v * NT + tid) * 4 + e < n && key[v][e] - lo <= left) sh.cand[atomicAdd(&sh.n_cand, 1u)] = key[v][e];
+                        if (key[v][e] - lo <= left) sh.cand[atomicAdd(&sh.n_cand, 1u)] = key[v][e];
                 }
             sync_all();
             const uint32_t* cand = sh.cand;
@@ -793,12 +802,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
             break;
         }
         sync_all();                                           // (every CTA has read the counts)
-        for (int i = tid; i < kShortBins; i += NT) sh.hist[i] = 0u;
+        for (int i = tid; i < BINS / 4; i += NT) reinterpret_cast<uint4*>(sh.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
     }
 
     // ---- emission: bitmaps, one scan, ascending positions ----
     const bool cut = eq_total != need_eq;                     // a group of equal keys is cut: lower positions win
+    const uint32_t from = cut ? T + 1u : T;
     uint8_t* const bytes_gt = reinterpret_cast<uint8_t*>(sh.gt);
     uint8_t* const bytes_eq = reinterpret_cast<uint8_t*>(sh.eq);
 #pragma unroll
@@ -807,9 +817,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
             uint32_t g = 0, q = 0;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const bool in = (v * NT + tid) * 4 + e < n;
-                g |= (in && (cut ? key[v][e] > T : key[v][e] >= T) ? 1u : 0u) << e;
-                q |= (in && key[v][e] == T ? 1u : 0u) << e;
+                g |= (key[v][e] >= from ? 1u : 0u) << e;
+                if (cut) q |= (key[v][e] == T ? 1u : 0u) << e;
             }
             g |= __shfl_down_sync(0xFFFFFFFFu, g, 1) << 4;
             if ((tid & 1) == 0) bytes_gt[(v * NT + tid) / 2] = (uint8_t)g;
@@ -920,15 +929,16 @@ cudaError_t launch_select(const gsa_params_t& p, RowRange rr, const float* score
     a.rr = rr; a.il = il; a.Lq = p.Lq; a.Lk = p.Lk;
     a.k_base = p.k_base; a.k_min = p.k_min; a.k_max = p.k_max; a.k_mode = p.k_mode; a.v_bar = p.v_bar;
 
-    // rows by the number of scores they see: up to 8192, up to 16384, longer
+    // rows by the number of scores they see: up to 4096, 8192, 16384, longer
     const int off = p.Lk - p.Lq;
     auto first_longer = [&](int cap) {                        // first query row that sees more than cap keys, within the range
         const int t = cap - off;
         return t < rr.q_begin ? rr.q_begin : (t > rr.q_begin + rr.R ? rr.q_begin + rr.R : t);
     };
-    const int t8 = first_longer(8192), t16 = first_longer(16384), t_end = rr.q_begin + rr.R;
+    const int t4 = first_longer(4096), t8 = first_longer(8192), t16 = first_longer(16384), t_end = rr.q_begin + rr.R;
     cudaError_t e = cudaSuccess;
-    if (t8 > rr.q_begin) e = launch_short<256, 1>(a, rr.q_begin, t8 - rr.q_begin, st);
+    if (t4 > rr.q_begin) e = launch_short<128, 1>(a, rr.q_begin, t4 - rr.q_begin, st);
+    if (e == cudaSuccess && t8 > t4) e = launch_short<256, 1>(a, t4, t8 - t4, st);
     if (e == cudaSuccess && t16 > t8) e = launch_short<512, 1>(a, t8, t16 - t8, st);
     if (e != cudaSuccess || t16 >= t_end) return e;
     // few long rows: a cluster each, while all of them fit the GPU at once
