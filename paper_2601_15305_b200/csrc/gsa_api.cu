@@ -535,7 +535,7 @@ static int forward_impl(const gsa_params_t* p, const void* Q, const void* K, con
     // Eq. 11, 12, 10 over all rows
     RowRange all{0, p->B, 0, p->Lq};
     e = launch_sparse_attn(*p, all, (const bf16*)Q, (const bf16*)K, Vuse, (const bf16*)g1_logits, g2use, idx,
-                           kt, il, (bf16*)out, wsb + wp.attn_off, st, progress, nullptr, g2_logits != nullptr);
+                           kt, il, (bf16*)out, wsb + wp.attn_off, st, progress, nullptr, g2_logits != nullptr, dense);
     if (g_prof_ev[2]) cudaEventRecord(g_prof_ev[2], st);
     return cuda_rc(e);
 }

@@ -707,14 +707,15 @@ int masked_rows_end(const gsa_params_t& p, const AttnPlan& pl, const RowRange& r
 cudaError_t launch_masked_rows(const gsa_params_t& p, const RowRange& rr, int t_end, const __nv_bfloat16* Q,
                                const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const int32_t* idx,
                                const int32_t* kt, IdxLayout il, __nv_bfloat16* out, void* scratch, size_t scratch_bytes,
-                               cudaStream_t st, AttnProgress* prog, float* lse) {
+                               cudaStream_t st, AttnProgress* prog, float* lse, bool all_visible) {
     const int block = masked_block_rows(p);
     const size_t row_bytes = mask_plan(p, 0, kMaskRowAlign).bytes(p.B) / kMaskRowAlign;
     int64_t per = (int64_t)(scratch_bytes / row_bytes) / block * block;
     if (per < block) return cudaErrorInvalidValue;
     for (int q = rr.q_begin; q < t_end; q += (int)per) {
         const MaskPlan mp = mask_plan(p, q, (int)(t_end - q < per ? t_end - q : per));
-        cudaError_t e = launch_build_masks(p, mp, block, idx, kt, il, (uint4*)scratch, t_dev_status + kStatusGeneralWord, st);
+        cudaError_t e = all_visible ? launch_visible_masks(p, mp, (uint4*)scratch, st)
+                                    : launch_build_masks(p, mp, block, idx, kt, il, (uint4*)scratch, t_dev_status + kStatusGeneralWord, st);
         if (e != cudaSuccess) return e;
         timeline_mark(kStageRangeCuts, st);
         e = launch_masked_attn_fwd(p, mp, (const uint4*)scratch, Q, K, Vg, g1, out, lse, idx, kt, il, t_dev_status, st);
@@ -767,7 +768,8 @@ cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bf
                                const __nv_bfloat16* K, const __nv_bfloat16* V,
                                const __nv_bfloat16* g1, const __nv_bfloat16* g2, const int32_t* idx,
                                const int32_t* kt, IdxLayout il, __nv_bfloat16* out, void* scratch,
-                               cudaStream_t st, AttnProgress* progress, float* lse, bool values_scanned) {
+                               cudaStream_t st, AttnProgress* progress, float* lse, bool values_scanned,
+                               bool all_visible) {
     if (rr.rows() <= 0) return cudaSuccess;
     const AttnPlan pl = plan_attn(p);
     const size_t scratch_bytes = (pl.state_bytes + 255) / 256 * 256 + pl.cuts_bytes;
@@ -780,7 +782,7 @@ cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bf
                 e = launch_check_finite(V, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, t_dev_status + kStatusGeneralWord, st);
             if (e != cudaSuccess) return e;
             e = launch_masked_rows(p, rr, t_end, Q, K, V, g1, idx, kt, il, out, scratch, scratch_bytes, st,
-                                   progress, lse);
+                                   progress, lse, all_visible);
             if (e != cudaSuccess || t_end >= rr.q_begin + rr.R) return e;
             rr.R = rr.q_begin + rr.R - t_end;
             rr.q_begin = t_end;

@@ -39,6 +39,9 @@ inline MaskPlan mask_plan(const gsa_params_t& p, int q0, int rows) {
 cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int block_rows, const int32_t* idx,
                                const int32_t* kt, IdxLayout il, uint4* mask, int32_t* general, cudaStream_t st);
 
+// The same for sets known to hold every visible key (k_mode 3 inside gsa_forward): no set is read.
+cudaError_t launch_visible_masks(const gsa_params_t& p, const MaskPlan& mp, uint4* mask, cudaStream_t st);
+
 // Raises *general if one of n_elems (a multiple of 8) values is infinite or NaN.
 cudaError_t launch_check_finite(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st);
 

@@ -102,6 +102,18 @@ gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restric
     if (at < k || !regular) *general = 1;              // (at < k: an entry past what the row can see, or out of order)
 }
 
+// masks of sets that hold every visible key: nothing to read
+__global__ void __launch_bounds__(256) gsa_visible_masks_kernel(uint4* __restrict__ mask, int64_t n, int row_pitch, int key_tiles,
+                                                                int off, int q0, int rows) {
+    chain_wait();
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    const int r = (int)(i % row_pitch), tile = (int)(i / row_pitch % key_tiles);
+    const int m = r < rows ? off + q0 + r + 1 - tile * kMaskTileKeys : 0;            // keys of the tile that the row sees
+    auto word = [&](int lo) -> uint32_t { return m >= lo + 32 ? 0xFFFFFFFFu : (m > lo ? (1u << (m - lo)) - 1u : 0u); };
+    mask[i] = make_uint4(word(0), word(32), word(64), word(96));
+}
+
 // ---- what the tiles cannot take -----------------------------------------------------------------------------
 // A tile multiplies every value row of its 128 keys, by zero where the key is not in the set, and a bit mask holds a
 // key once.  So a call whose gated values are not all finite (0 * inf), or whose sets are not strictly ascending
@@ -514,6 +526,14 @@ cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int bl
     const dim3 grid((unsigned)(mp.row_pitch / kMaskRowAlign), (unsigned)p.B);
     launch_chained(gsa_build_masks_kernel, grid, kMaskRowAlign * 32, 0, st, idx, kt, mask, il, mp.q0, mp.rows, mp.row_pitch, mp.key_tiles,
                                                                block_rows, p.k_max, p.Lk - p.Lq, general);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_visible_masks(const gsa_params_t& p, const MaskPlan& mp, uint4* mask, cudaStream_t st) {
+    const int64_t n = (int64_t)p.B * mp.key_tiles * mp.row_pitch;
+    launch_chained(gsa_visible_masks_kernel, (unsigned)((n + 255) / 256), 256, 0, st, mask, n, mp.row_pitch, mp.key_tiles,
+                   p.Lk - p.Lq, mp.q0, mp.rows);
     ++g_launches;
     return cudaGetLastError();
 }
