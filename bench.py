@@ -367,8 +367,9 @@ def main():
                 "hbm_gbs": peaks["hbm_gbs"], "frac_hbm": achieved / peaks["hbm_gbs"], "hbm_source": hbm_src,
                 "hbm_gather_gbs": rates["gather_hbm_2GB_piece256_gbs"] if rates else None,
                 "algorithmic_bytes_per_launch": ab, "launch_ms": attn_ms,
-                "note": "one 'launch' = the sparse-attention stage of a forward (range cuts, one kernel launch per 16384-key "
-                        "range, finalize).  The 126 MB L2, not HBM, serves the gather, so frac is taken against the L2's "
+                "note": "one 'launch' = the sparse-attention stage of a forward: masked tiles on the tensor cores for rows that see "
+                        "few enough keys, the gather for the others (range cuts, one kernel launch per 16384-key "
+                        "range, finalize).  All rows are charged the gather's bytes.  The 126 MB L2, not HBM, serves the gather, so frac is taken against the L2's "
                         "measured gather rate; frac_hbm (against the HBM copy bandwidth) exceeds 1 for the same reason"}
     causal_pairs = cfg.B * sum(cfg.Lk - cfg.Lq + t + 1 for t in (0, cfg.Lq - 1)) * cfg.Lq / 2.0
     stages = {"indexer_plus_topk_ms": sel_ms, "sparse_attn_ms": attn_ms,

@@ -371,7 +371,7 @@ void gsa_debug_set_attn_range_keys(int32_t keys);
  * Test knob for the bounded device-side waits: `cycles` is the limit of every wait in SM clock cycles
  * (<= 0 restores the default of 2^31, about a second).  With withhold_first_copy != 0 the copy producer of
  * each tensor-core kernel (gsa_indexer_scores / gsa_forward on the tcgen05 path, gsa_project,
- * gsa_output_projection) leaves out its first copy, so that the wait for it meets a barrier that nothing
+ * gsa_output_projection, the masked tiles of the attention stage and its backward) leaves out its first copy, so that the wait for it meets a barrier that nothing
  * completes: the way to see the give-up path work (status word set, kernel returns, context intact).
  * Process-wide; not meant for production use.
  */
@@ -389,7 +389,7 @@ void gsa_profile_set_events(void *ev_begin, void *ev_selected, void *ev_end);
  * Profiling hook with one interval per launch: `events` is an array of `capacity` cudaEvent_t handles
  * (created by the caller, timing enabled).  Every following gsa_forward records events[0] at entry and the
  * next event behind each stage it enqueues, and writes into the HOST arrays stage_out[i] which stage the
- * interval events[i] .. events[i + 1] belongs to (0 indexer, 1 budget + top-k, 2 value gate, 3 range cuts,
+ * interval events[i] .. events[i + 1] belongs to (0 indexer, 1 budget + top-k, 2 value gate, 3 range cuts or masks,
  * 4 sparse attention, 5 normalise + output gate) and into *count_out the number of intervals.  The events
  * serialise nothing but cost a little: use it for a profiling step, not inside a timed loop.  NULL / 0
  * switches it off.  Process-wide; the caller owns the events and the arrays and reads them after

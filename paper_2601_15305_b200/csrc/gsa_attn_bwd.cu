@@ -1,5 +1,6 @@
 // Backward of sparse gated attention (Eq. 9-12 and Eq. 10 differentiated; the index sets S_t are
-// constants: top-k selection has no derivative and the indexer is trained by its own loss, Sec. 5.1).
+// constants: top-k selection has no derivative and the indexer is trained by its own loss, Sec. 5.1): the gather path, for
+// sets that hold a small share of the visible keys (larger shares: gsa_masked_bwd.cu).
 //
 // With out = o * sigmoid(g1), o = sum_j a_j v'_j, a = softmax_j(scale * q.k_j), v' = V * sigmoid(g2):
 //   do    = dout * sigmoid(g1)

@@ -99,6 +99,13 @@ __device__ __forceinline__ void tma_load_tile(uint32_t dst, const CUtensorMap* t
 // The MMA warp runs converged and one elected lane issues: descriptors then stay in uniform registers.  (A single lane in
 // a branch of its own has to move every operand of every instruction there first: which cost more than
 // a product of M = N = 128, K = 16 takes (64 cycles).  Backward at L = 32K: keys kernel 6.6 -> 6.1 ms, rows 5.7 -> 5.3 ms)
+// Start of a tile kernel: false if the call's inputs rule the tiles out (the plain kernel does the work; the same for every
+// thread).  *timed_out: an earlier CTA or launch of the call gave up on a wait (may differ between threads: use one's).
+__device__ __forceinline__ bool tiles_allowed(const int32_t* dev_status, int* timed_out) {
+    const int32_t st = *reinterpret_cast<const volatile int32_t*>(dev_status);
+    *timed_out = st >= kDevTimeoutTma && st <= kDevTimeoutEpi;
+    return *reinterpret_cast<const volatile int32_t*>(dev_status + kStatusGeneralWord) == 0;
+}
 __device__ __forceinline__ uint32_t elect_lane() {
     uint32_t e;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));

@@ -11,10 +11,10 @@
 // accumulator in TMEM is touched by the softmax warps on a row's first tiles only.  Masked scores are replaced by
 // -inf before the maximum and the exponentials; fp32 everywhere except P (bf16, as in the gather kernel).
 //
-// Bound: the two tiles' softmax chains against their products; 16 exponentials and 4 * 128 * d_h flops per (row, key) column
-// make special-function unit and tensor cores about equally long (1024 cycles per tile at d_h = 128).  Measured at 16 heads
-// of 128 on 8 KV heads: L = 32K 3.92 ms = 1.12 PFLOP/s over the visible pairs (the gather kernel: 19.6 ms), 8K 0.35 ms
-// (4.6 ms), dense 2 x 3072 0.14 ms (2.7 ms).
+// Bound: the serial chain of a tile (scores -> numerators -> product -> next scores); the two tiles' chains fill each other's
+// gaps, with the tensor cores and the special-function unit each busy somewhat over half of the time.  Measured at 16 heads of
+// 128 on 8 KV heads: L = 32K 3.45 ms = 1.27 PFLOP/s over the visible pairs (the gather kernel: 19.6 ms; with a whole tile's
+// numerators handed over at once 3.55), 8K 0.33 ms (4.6 ms), dense 2 x 3072 0.135 ms (2.7 ms).
 //
 // Warps 0-3 / 4-7: softmax and epilogue of tile 0 / 1; warp 8: TMA; warp 9: MMA issue and TMEM allocation; 10, 11
 // only complete their warpgroup.
@@ -197,8 +197,8 @@ __global__ void __launch_bounds__(256) gsa_check_finite_kernel(const uint4* __re
 }
 
 // ---- forward ---------------------------------------------------------------------------------------------
-// Three warpgroups launched at 168 registers a thread; the two softmax groups take 216 (a row's 128 scores live in
-// registers), the copy / MMA group keeps 72: 2 * 216 + 72 = 504 of the 504 the block was launched with.
+// Three warpgroups launched at 168 registers a thread; the two softmax groups take 216 (64 scores of a row and what is made of
+// them live in registers), the copy / MMA group keeps 72: 2 * 216 + 72 = 504 of the 504 the block was launched with.
 constexpr int kFwdThreads = 384;
 
 template <int DH>
@@ -209,7 +209,7 @@ struct FwdSmem {
     static constexpr int SLOTS = DH == 128 ? 5 : 8;                // K / V' tiles in flight
     static constexpr int OFF_RING = 2 * TILE_BYTES;
     static constexpr int OFF_BAR = OFF_RING + SLOTS * TILE_BYTES;
-    static constexpr int N_BARS = 2 * SLOTS + 2 + 2 + 2 + 2 + 1;   // ring full / empty, Q, S, P, O, drain
+    static constexpr int N_BARS = 2 * SLOTS + 2 + 2 + 4 + 2 + 2 + 1;   // ring full / empty, Q, S, P (halves), O, half, drain
     static constexpr int OFF_TMEM = OFF_BAR + N_BARS * 8;
     static constexpr int OFF_ABORT = OFF_TMEM + 8;
     static constexpr int ALLOC = OFF_ABORT + 8 + 1024;
@@ -226,6 +226,7 @@ struct MaskedFwdArgs {
     int32_t Lq, Lk, n_h, n_kv, row_blocks;
     float scale_log2;
     long long wait_cycles;
+    int32_t withhold_first;        // fault injection: the first copy into the ring is left out (its barrier is never completed)
 };
 
 template <int DH, int G>
@@ -252,11 +253,13 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     auto bar_empty = [&](int s) { return bar0 + 8u * (P::SLOTS + s); };
     auto bar_q = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + s); };
     auto bar_s = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 2 + s); };
-    auto bar_p = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 4 + s); };
-    auto bar_o = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 6 + s); };
-    const uint32_t bar_drain = bar0 + 8u * (2 * P::SLOTS + 8);
+    auto bar_p = [&](int s, int p) { return bar0 + 8u * (2 * P::SLOTS + 4 + 2 * s + p); };      // (one completion per tile each)
+    auto bar_o = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 8 + s); };
+    auto bar_h = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 10 + s); };
+    const uint32_t bar_drain = bar0 + 8u * (2 * P::SLOTS + 12);
 
-    if (*a.general) return;                                        // (uniform: written by earlier launches only)
+    int timed_out;
+    if (!tiles_allowed(a.dev_status, &timed_out)) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // (batch element, KV head) outermost, so that the CTAs of a wave share K and V' in the L2; late (long) rows first
     const int blk = a.row_blocks - 1 - (int)(blockIdx.x % a.row_blocks);
@@ -269,9 +272,9 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < P::SLOTS; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(bar_q(s), 1); mbar_init(bar_s(s), 1); mbar_init(bar_p(s), 4); mbar_init(bar_o(s), 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_q(s), 1); mbar_init(bar_s(s), 1); mbar_init(bar_p(s, 0), 4); mbar_init(bar_p(s, 1), 4); mbar_init(bar_o(s), 1); mbar_init(bar_h(s), 1); }
         mbar_init(bar_drain, 1);
-        *s_abort = 0;
+        *s_abort = timed_out;                                      // (then every wait ends at once)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -304,77 +307,83 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         for (int i = 0; i < ntiles; ++i) {
             const uint4 mk = mk_next;
             if (live && i + 1 < ntiles) mk_next = __ldg(mrow + (int64_t)(i + 1) * a.row_pitch);
-            if (!mbar_wait(bar_s(s), i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
-            tc_fence_after();
-            // The reference of the tiles before nearly always still serves, so the numerators are taken against it at once,
-            // 32 columns at a time with the next 32 on their way; only if a selected score then turns out to exceed it
-            // by more than 2^8 (a row's first tiles) is the tile's work done again from the scores, still in registers.
+            if (!(ok = warp_wait(bar_s(s), i & 1, s_abort, a.wait_cycles))) break;
+            // Half a tile at a time, so that the product of the first half's numerators runs under the second half's work.
             const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
-            uint32_t v[4][32];
-            float mx[4];
-            uint64_t sum[2] = {0ull, 0ull};
-            const float neg0 = m_ref == -INFINITY ? 0.f : -m_ref;
-            uint64_t neg2 = pack_f32x2(neg0, neg0);
-            auto numerators = [&](int c) {
-                uint32_t pk[16];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const uint64_t x = fma_f32x2(pack_f32x2(__uint_as_float(v[c][2 * j]), __uint_as_float(v[c][2 * j + 1])), scale2, neg2);
-                    float x0, x1;
-                    unpack_f32x2(x, x0, x1);
-                    x0 = ex2_approx(x0); x1 = ex2_approx(x1);
-                    sum[j & 1] = add_f32x2(sum[j & 1], pack_f32x2(x0, x1));
-                    pk[j] = pack_bf16(x0, x1);
+            for (int p = 0; p < 2; ++p) {
+                // The reference of the tiles before nearly always still serves, so the numerators are taken against it at
+                // once, 32 columns at a time with the next 32 on their way; only if a selected score then turns out to
+                // exceed it by more than 2^8 (a row's first tiles) is the work done again from the scores, still in registers.
+                uint32_t v[2][32];
+                float mx[2];
+                uint64_t sum[2] = {0ull, 0ull};
+                const float neg0 = m_ref == -INFINITY ? 0.f : -m_ref;
+                uint64_t neg2 = pack_f32x2(neg0, neg0);
+                auto numerators = [&](int c) {
+                    uint32_t pk[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const uint64_t x = fma_f32x2(pack_f32x2(__uint_as_float(v[c][2 * j]), __uint_as_float(v[c][2 * j + 1])), scale2, neg2);
+                        float x0, x1;
+                        unpack_f32x2(x, x0, x1);
+                        x0 = ex2_approx(x0); x1 = ex2_approx(x1);
+                        sum[j & 1] = add_f32x2(sum[j & 1], pack_f32x2(x0, x1));
+                        pk[j] = pack_bf16(x0, x1);
+                    }
+                    tc_st16(ts + 32 * p + 16 * c, pk);
+                };
+                tc_ld32(ts + 64 * p, v[0]);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    tc_wait_ld32(v[c]);
+                    if (c == 0) tc_ld32(ts + 64 * p + 32, v[1]);
+                    mx[c] = -INFINITY;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const float x = (mw[2 * p + c] >> j) & 1u ? __uint_as_float(v[c][j]) : -INFINITY;
+                        v[c][j] = __float_as_uint(x);
+                        mx[c] = fmaxf(mx[c], x);
+                    }
+                    // (the numerators of columns 32 n .. go over columns 16 n .., which have been read)
+                    numerators(c);
                 }
-                tc_st16(ts + 16 * c, pk);
-            };
-            tc_ld32(ts, v[0]);
+                const float top = fmaxf(mx[0], mx[1]) * a.scale_log2;
+                if (__any_sync(0xFFFFFFFFu, top > m_ref + 8.0f)) {
+                    const float m_new = fmaxf(m_ref, top);
+                    const float alpha = m_ref == -INFINITY ? 0.f : ex2_approx(m_ref - m_new);
+                    m_ref = m_new;
+                    const float neg1 = m_ref == -INFINITY ? 0.f : -m_ref;
+                    neg2 = pack_f32x2(neg1, neg1);
+                    const uint64_t al2 = pack_f32x2(alpha, alpha);
+                    l2[0] = mul_f32x2(l2[0], al2); l2[1] = mul_f32x2(l2[1], al2);
+                    sum[0] = sum[1] = 0ull;
+                    tc_wait_st();                                  // (the columns are written a second time)
+                    numerators(0);
+                    numerators(1);
+                    if (i > 0 || p > 0) {
+                        // every product into O so far has completed: bar_s says so for the tiles before, bar_h for this one's half
+                        if (p > 0 && !(ok = warp_wait(bar_h(s), i & 1, s_abort, a.wait_cycles))) break;
+                        uint32_t o[16];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                tc_wait_ld32(v[c]);
-                if (c < 3) tc_ld32(ts + 32 * (c + 1), v[c + 1]);
-                mx[c] = -INFINITY;
+                        for (int c = 0; c < DH / 16; ++c) {
+                            tc_ld16(to + 16 * c, o);
+                            tc_wait_ld16(o);
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float x = (mw[c] >> j) & 1u ? __uint_as_float(v[c][j]) : -INFINITY;
-                    v[c][j] = __float_as_uint(x);
-                    mx[c] = fmaxf(mx[c], x);
-                }
-                // (the numerators of these columns go over columns 16 c .. 16 c + 15, which have been read)
-                numerators(c);
-            }
-            const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * a.scale_log2;
-            if (__any_sync(0xFFFFFFFFu, top > m_ref + 8.0f)) {
-                const float m_new = fmaxf(m_ref, top);
-                const float alpha = m_ref == -INFINITY ? 0.f : ex2_approx(m_ref - m_new);
-                m_ref = m_new;
-                const float neg1 = m_ref == -INFINITY ? 0.f : -m_ref;
-                neg2 = pack_f32x2(neg1, neg1);
-                const uint64_t al2 = pack_f32x2(alpha, alpha);
-                l2[0] = mul_f32x2(l2[0], al2); l2[1] = mul_f32x2(l2[1], al2);
-                sum[0] = sum[1] = 0ull;
-                tc_wait_st();                                      // (the columns are written a second time)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) numerators(c);
-                if (i > 0) {                                       // every product into O so far has completed (bar_s)
-                    uint32_t o[16];
-#pragma unroll
-                    for (int c = 0; c < DH / 16; ++c) {
-                        tc_ld16(to + 16 * c, o);
-                        tc_wait_ld16(o);
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
-                        tc_st16(to + 16 * c, o);
+                            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
+                            tc_st16(to + 16 * c, o);
+                        }
                     }
                 }
+                l2[0] = add_f32x2(l2[0], sum[0]); l2[1] = add_f32x2(l2[1], sum[1]);
+                tc_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_p(s, p));
             }
-            l2[0] = add_f32x2(l2[0], sum[0]); l2[1] = add_f32x2(l2[1], sum[1]);
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_p(s));
+            if (!ok) break;
         }
-        if (ok && !mbar_wait(bar_o(s), 0, s_abort, a.wait_cycles)) ok = false;
+        ok = ok && warp_wait(bar_o(s), 0, s_abort, a.wait_cycles);
         if (!ok) {
             if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
         } else {
@@ -423,11 +432,12 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 for (int n = 0; ok && n < 2 * ntiles; ++n) {
                     const int s = n % P::SLOTS;
                     if (!mbar_wait(bar_empty(s), ((n / P::SLOTS) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                    copies_issued = n + 1;
+                    if (n == 0 && a.withhold_first) continue;
                     mbar_expect_tx(bar_full(s), P::TILE_BYTES);
                     for (int c = 0; c < CH; ++c)
                         tma_load_tile(sbase + P::OFF_RING + s * P::TILE_BYTES + c * P::CHUNK_BYTES, (n & 1) ? &tm_v : &tm_k,
                                       c * 64, g, (n >> 1) * kMaskTileKeys, b, bar_full(s));
-                    copies_issued = n + 1;
                 }
                 if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
             }
@@ -447,10 +457,10 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     warp_mma_ss(el, tmem + kTmS + 128 * s, qd + step, kd + step, kIdescS, k > 0);
                 }
             };
-            auto issue_o = [&](int s, int i) {                     // O_s += P_s V'_i
+            auto issue_o = [&](int s, int i, int p) {              // O_s += P_s V'_i, half p of the keys
                 const uint64_t vd = make_mnmajor_desc(slot_addr(2 * i + 1), P::CHUNK_BYTES);
 #pragma unroll
-                for (int k = 0; k < kMaskTileKeys / 16; ++k)       // 16 keys = 2048 bytes of the V' tile, 8 columns of P
+                for (int k = 4 * p; k < 4 * p + 4; ++k)            // 16 keys = 2048 bytes of the V' tile, 8 columns of P
                     warp_mma_ts(el, tmem + kTmO + 128 * s, tmem + kTmS + 128 * s + 8 * k, vd + 128 * k, kIdescO, (i | k) != 0);
             };
             auto release = [&](int n) { warp_commit(el, bar_empty(n % P::SLOTS)); slots_released = n + 1; };
@@ -464,8 +474,11 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 ok = wait_slot(2 * i + 1);
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
-                    if (!ok || !(ok = wait(bar_p(s), i & 1))) break;
-                    issue_o(s, i);
+                    if (!ok || !(ok = wait(bar_p(s, 0), i & 1))) break;
+                    issue_o(s, i, 0);
+                    warp_commit(el, bar_h(s));
+                    if (!(ok = wait(bar_p(s, 1), i & 1))) break;
+                    issue_o(s, i, 1);
                     if (i + 1 < ntiles) {
                         if (s == 0 && !(ok = wait_slot(2 * i + 2))) break;
                         // (in order behind the product that reads P from these columns)
@@ -489,7 +502,7 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         // give-up path: let what was issued complete (each poll is bounded) before shared memory and TMEM are released
         if (warp == 8 && lane == 0) {
             for (int s = 0; s < q_issued; ++s) mbar_drain(bar_q(s), 0);
-            for (int n = max(0, copies_issued - P::SLOTS); n < copies_issued; ++n)
+            for (int n = max(a.withhold_first, copies_issued - P::SLOTS); n < copies_issued; ++n)
                 mbar_drain(bar_full(n % P::SLOTS), (n / P::SLOTS) & 1);
         }
         if (warp == 9) {
@@ -563,6 +576,7 @@ cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, co
     const float sc = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
     a.scale_log2 = sc * 1.4426950408889634f;
     a.wait_cycles = wait_limit_cycles();
+    a.withhold_first = withhold_first_copy() ? 1 : 0;
     const int ctas = sm_count() * 4;
 #define GSA_CASE(DH_, G_)                                                                                              \
     if (p.d_h == DH_ && G == G_) {                                                                                     \

@@ -58,6 +58,7 @@ struct MaskedBwdArgs {
     int32_t pairs_per_cta;         // target kernel: runs of 256 keys per CTA
     float scale, scale_log2;
     long long wait_cycles;
+    int32_t withhold_first;        // fault injection: the first copy of a ring is left out (its barrier is never completed)
 };
 
 // 128-row K-major operand: k-step of 16 columns
@@ -91,9 +92,9 @@ __device__ __forceinline__ void mma_tmem_rows(uint32_t el, uint32_t d, uint32_t 
     const uint32_t bar0 = sbase + PLAN::OFF_BAR;                                                                        \
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-__device__ __forceinline__ uint32_t tile_start(int warp, uint32_t tmem_slot, const uint32_t* s_tmem, volatile int* s_abort) {
+__device__ __forceinline__ uint32_t tile_start(int timed_out, int warp, uint32_t tmem_slot, const uint32_t* s_tmem, volatile int* s_abort) {
     if (threadIdx.x == 0) {
-        *s_abort = 0;
+        *s_abort = timed_out;                                      // (then every wait ends at once)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -156,7 +157,8 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     using T = TileBytes<DH>;
     constexpr int QT = P::QT, ST = P::STAGES;
     constexpr uint32_t kTmS = 0, kTmP = 128, kTmV = 256, kTmK = 384;
-    if (*a.general) return;
+    int timed_out;
+    if (!tiles_allowed(a.dev_status, &timed_out)) return;
     GSA_TILE_PROLOGUE(P)
     auto bar_q = [&](int s) { return bar0 + 8u * s; };                       // Q tile landed
     auto bar_d = [&](int s) { return bar0 + 8u * (ST + s); };                // do tile landed
@@ -187,7 +189,7 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         mbar_init(bar_kv, 1); mbar_init(bar_s, 1); mbar_init(bar_dp, 1); mbar_init(bar_p, 16); mbar_init(bar_ds, 16);
         mbar_init(bar_done, 1); mbar_init(bar_drain, 1);
     }
-    const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
+    const uint32_t tmem = tile_start(timed_out, warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
     int copies = 0, kv_issued = 0, released = 0;
     bool done = false;
 
@@ -205,8 +207,10 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 if (!mbar_wait(bar_free(s), ((i / ST) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
                 const uint32_t dst = sbase + P::OFF_RING + s * 2 * T::TILE;
                 const int z = (i0 + i * SPLIT) * QT;
-                mbar_expect_tx(bar_q(s), T::TILE);
-                for (int c = 0; c < T::CHUNKS; ++c) tma_load_tile(dst + c * T::CHUNK, &tm_q, c * 64, g * G, z, b, bar_q(s));
+                if (i > 0 || !a.withhold_first) {
+                    mbar_expect_tx(bar_q(s), T::TILE);
+                    for (int c = 0; c < T::CHUNKS; ++c) tma_load_tile(dst + c * T::CHUNK, &tm_q, c * 64, g * G, z, b, bar_q(s));
+                }
                 mbar_expect_tx(bar_d(s), T::TILE);
                 for (int c = 0; c < T::CHUNKS; ++c)
                     tma_load_tile(dst + T::TILE + c * T::CHUNK, &tm_do, c * 64, g * G, z, b, bar_d(s));
@@ -268,7 +272,7 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 mk[u] = make_uint4(0u, 0u, 0u, 0u);
                 if (m < QT && rq < a.rows) mk[u] = a.mask[((int64_t)b * a.key_tiles + tile) * a.row_pitch + rq];
             }
-            if (!mbar_wait(bar_statfree(s), ((i / ST) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+            if (!(ok = warp_wait(bar_statfree(s), ((i / ST) & 1) ^ 1, s_abort, a.wait_cycles))) break;
             float* st = reinterpret_cast<float*>(smem + P::OFF_STAT + s * P::STAT_BYTES);
             uint32_t* sm = reinterpret_cast<uint32_t*>(st + 256);
 #pragma unroll
@@ -293,9 +297,8 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             const float* st = reinterpret_cast<const float*>(smem + P::OFF_STAT + s * P::STAT_BYTES) + 32 * part;
             const uint32_t* sm = reinterpret_cast<const uint32_t*>(smem + P::OFF_STAT + s * P::STAT_BYTES + 1024) +
                                  quad * QT + 32 / G * part;
-            if (!mbar_wait(bar_stat(s), (i / ST) & 1, s_abort, a.wait_cycles) ||
-                !mbar_wait(bar_s, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
-            tc_fence_after();
+            if (!(ok = warp_wait(bar_stat(s), (i / ST) & 1, s_abort, a.wait_cycles) &&
+                       warp_wait(bar_s, i & 1, s_abort, a.wait_cycles))) break;
             uint32_t v[32], pk[16];
             tc_ld32(ts, v);
             tc_wait_ld32(v);
@@ -319,8 +322,7 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_p);
 
-            if (!mbar_wait(bar_dp, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
-            tc_fence_after();
+            if (!(ok = warp_wait(bar_dp, i & 1, s_abort, a.wait_cycles))) break;
             uint32_t w[32];
             tc_ld32(tp, w);
             tc_wait_ld32(w);
@@ -340,7 +342,7 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             __syncwarp();
             if (lane == 0) { mbar_arrive(bar_ds); mbar_arrive(bar_statfree(s)); }
         }
-        done = ok && (n == 0 || mbar_wait(bar_done, 0, s_abort, a.wait_cycles));
+        done = ok && (n == 0 || warp_wait(bar_done, 0, s_abort, a.wait_cycles));
         if (!done && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
         tc_fence_after();
     }
@@ -422,7 +424,7 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
              [&] {
                  if (kv_issued) mbar_drain(bar_kv, 0);
                  for (int i = max(0, copies - ST); i < copies; ++i) {
-                     mbar_drain(bar_q(i % ST), (i / ST) & 1);
+                     if (i > 0 || !a.withhold_first) mbar_drain(bar_q(i % ST), (i / ST) & 1);
                      mbar_drain(bar_d(i % ST), (i / ST) & 1);
                  }
              },
@@ -452,7 +454,8 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     using T = TileBytes<DH>;
     constexpr int QT = 128 / G, SL = P::SLOTS;
     constexpr uint32_t kTmS = 0, kTmP = 256, kTmQ = 384;           // S at kTmS + 128 (i & 1)
-    if (*a.general) return;
+    int timed_out;
+    if (!tiles_allowed(a.dev_status, &timed_out)) return;
     GSA_TILE_PROLOGUE(P)
     auto bar_full = [&](int s) { return bar0 + 8u * s; };
     auto bar_empty = [&](int s) { return bar0 + 8u * (SL + s); };
@@ -470,7 +473,7 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         mbar_init(bar_qd, 1); mbar_init(bar_s(0), 1); mbar_init(bar_s(1), 1); mbar_init(bar_dp, 1); mbar_init(bar_read, 16);
         mbar_init(bar_ds, 16); mbar_init(bar_done, 1); mbar_init(bar_drain, 1);
     }
-    const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
+    const uint32_t tmem = tile_start(timed_out, warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
     int copies = 0, qd_issued = 0, k_released = 0, v_released = 0;
 
     if (warp == kCopyWarp) {
@@ -485,11 +488,12 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             for (int e = 0; ok && e < 2 * n; ++e) {
                 const int s = e % SL;
                 if (!mbar_wait(bar_empty(s), ((e / SL) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                copies = e + 1;
+                if (e == 0 && a.withhold_first) continue;
                 mbar_expect_tx(bar_full(s), T::TILE);
                 for (int c = 0; c < T::CHUNKS; ++c)
                     tma_load_tile(sbase + P::OFF_RING + s * T::TILE + c * T::CHUNK, (e & 1) ? &tm_v : &tm_k, c * 64, g,
                                   (e >> 1) * kMaskTileKeys, b, bar_full(s));
-                copies = e + 1;
             }
             if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
         }
@@ -544,8 +548,7 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             const uint32_t mk = mk_next;
             if (live && i + 1 < n) mk_next = __ldg(mrow + (int64_t)(i + 1) * a.row_pitch * 4);
             const uint32_t ts = lane_base + kTmS + 128 * (i & 1) + 32 * part, tp = lane_base + kTmP + 32 * part;
-            if (!mbar_wait(bar_s(i), (i >> 1) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
-            tc_fence_after();
+            if (!(ok = warp_wait(bar_s(i), (i >> 1) & 1, s_abort, a.wait_cycles))) break;
             uint32_t v[32], w[32], pk[16];
             tc_ld32(ts, v);
             tc_wait_ld32(v);
@@ -554,8 +557,7 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 const float x = ex2_approx(fmaf(__uint_as_float(v[j]), a.scale_log2, -l2));
                 v[j] = __float_as_uint((mk >> j) & 1u ? x : 0.f);
             }
-            if (!mbar_wait(bar_dp, i & 1, s_abort, a.wait_cycles)) { ok = false; break; }
-            tc_fence_after();
+            if (!(ok = warp_wait(bar_dp, i & 1, s_abort, a.wait_cycles))) break;
             tc_ld32(tp, w);
             tc_wait_ld32(w);
             tc_fence_before();
@@ -571,7 +573,7 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_ds);
         }
-        if (ok && !mbar_wait(bar_done, 0, s_abort, a.wait_cycles)) ok = false;
+        ok = ok && warp_wait(bar_done, 0, s_abort, a.wait_cycles);
         if (!ok) {
             if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
         } else {
@@ -597,7 +599,7 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     tile_end(warp, lane, tmem, s_abort, bar_drain,
              [&] {
                  if (qd_issued) mbar_drain(bar_qd, 0);
-                 for (int e = max(0, copies - SL); e < copies; ++e) mbar_drain(bar_full(e % SL), (e / SL) & 1);
+                 for (int e = max(a.withhold_first, copies - SL); e < copies; ++e) mbar_drain(bar_full(e % SL), (e / SL) & 1);
              },
              [&] {
                  // (commits arrive in order: the last one of either kind covers the others)
@@ -627,7 +629,8 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     using P = TargetSmem<DH>;
     using T = TileBytes<DH>;
     constexpr int QT = 128 / G;
-    if (*a.general) return;
+    int timed_out;
+    if (!tiles_allowed(a.dev_status, &timed_out)) return;
     const int blk = a.row_blocks - 1 - (int)blockIdx.y, b = blockIdx.z;
     const int r0 = blk * QT, off = a.Lk - a.Lq;
     const int ntiles = min((off + a.q0 + min(r0 + QT, a.rows) + kMaskTileKeys - 1) / kMaskTileKeys, a.key_tiles);
@@ -667,7 +670,7 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
             s_rank[q] = lo;
         }
     }
-    const uint32_t tmem = tile_start(warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
+    const uint32_t tmem = tile_start(timed_out, warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
     int copies = 0, released = 0;
 
     // 640 threads launched at 96 registers: 512 * 104 + 128 * 64 = 61440
@@ -694,8 +697,7 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                 const float neg = -l_next * kLog2e;
                 if (live && g + 1 < a.n_kv) l_next = lse[(g + 1) * G];
                 const uint64_t neg2 = pack_f32x2(neg, neg);
-                if (!mbar_wait(bar_s(s, w), (it >> 1) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
-                tc_fence_after();
+                if (!(ok = warp_wait(bar_s(s, w), (it >> 1) & 1, s_abort, a.wait_cycles))) break;
                 const uint32_t ts = lane_base + 256 * s + 128 * w + 64 * half;
                 uint32_t v[16];
 #pragma unroll
@@ -755,6 +757,8 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                 for (int it = 0; ok && it < n; ++it) {
                     const int s = it & 1, g = it % a.n_kv, pair = pair0 + it / a.n_kv;
                     if (!mbar_wait(bar_empty(s), ((it >> 1) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
+                    copies = it + 1;
+                    if (it == 0 && a.withhold_first) continue;
                     mbar_expect_tx(bar_full(s), P::STAGE);
                     const uint32_t dst = sbase + s * P::STAGE;
                     for (int c = 0; c < T::CHUNKS; ++c) {
@@ -763,7 +767,6 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
                             tma_load_tile(dst + (1 + w) * T::TILE + c * T::CHUNK, &tm_k, c * 64, g, (2 * pair + w) * kMaskTileKeys, b,
                                           bar_full(s));
                     }
-                    copies = it + 1;
                 }
                 if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
             }
@@ -787,7 +790,7 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         }
     }
     tile_end(warp, lane, tmem, s_abort, bar_drain,
-             [&] { for (int i = max(0, copies - 2); i < copies; ++i) mbar_drain(bar_full(i & 1), (i >> 1) & 1); },
+             [&] { for (int i = max(a.withhold_first, copies - 2); i < copies; ++i) mbar_drain(bar_full(i & 1), (i >> 1) & 1); },
              [&] { for (int i = max(0, released - 2); i < released; ++i) mbar_drain(bar_empty(i & 1), (i >> 1) & 1); });
 }
 
@@ -984,6 +987,7 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
     a.scale = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
     a.scale_log2 = a.scale * kLog2e;
     a.wait_cycles = wait_limit_cycles();
+    a.withhold_first = withhold_first_copy() ? 1 : 0;
 #define GSA_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_bwd_t<DH_, G_>(a, p, Q, K, Vg, dOs, (float*)ws, st)
     GSA_CASE(128, 1); GSA_CASE(128, 2); GSA_CASE(128, 4); GSA_CASE(128, 8);
     GSA_CASE(64, 1); GSA_CASE(64, 2); GSA_CASE(64, 4); GSA_CASE(64, 8);

@@ -114,7 +114,7 @@ def test_inputs_that_a_mask_cannot_stand_for(what):
 
 
 # ---- backward ------------------------------------------------------------------------------------------------------
-def _run_bwd(cfg, d, idx, kt, q0, q1, saved_lse):
+def _run_bwd(cfg, d, idx, kt, q0, q1, saved_lse, withhold=False):
     p = gsa.make_params(cfg, q_begin=q0, q_end=q1)
     nan = float("nan")
     out, lse = torch.full_like(d["Q"], nan), torch.full((cfg.B, cfg.Lq, cfg.n_h), nan, dtype=torch.float32, device="cuda")
@@ -125,8 +125,12 @@ def _run_bwd(cfg, d, idx, kt, q0, q1, saved_lse):
     got["pbar"] = torch.full((cfg.B, q1 - q0, cfg.k_max), nan, dtype=torch.float32, device="cuda")
     ws.fill_(0xFF)
     n0 = gsa.gsa_launch_count()
-    gsa.gsa_sparse_gated_attn_bwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], i, k, out, d["dout"], got["dQ"], got["dK"], got["dV"],
-                                  got["dg1"], got["dg2"], ws, pbar=got["pbar"], lse=lse if saved_lse else None)
+    gsa.gsa_debug_set_wait_limit(400_000 if withhold else 0, withhold_first_copy=withhold)
+    try:
+        gsa.gsa_sparse_gated_attn_bwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], i, k, out, d["dout"], got["dQ"], got["dK"], got["dV"],
+                                      got["dg1"], got["dg2"], ws, pbar=got["pbar"], lse=lse if saved_lse else None)
+    finally:
+        gsa.gsa_debug_set_wait_limit(0, withhold_first_copy=False)
     # gate, preparation, two scans, masks, keys, rows, target, three of the plain path (and the statistics' two)
     assert gsa.gsa_launch_count() - n0 == (11 if saved_lse else 13)
     return got, gsa.gsa_device_status(ws)
@@ -189,3 +193,23 @@ def test_masked_backward_leaves_other_inputs_to_the_plain_path(what):
         keys[0, idx[0, 600, :int(kt[0, 600])].long()] = True
         assert bad_keys.any() and not (bad_keys & ~keys).any()
     assert bad_rows.any() and not (bad_rows & ~rows).any()
+
+
+def test_tile_waits_run_out_then_the_next_call_is_correct():
+    """The tile kernels' bounded waits: with the first copy of each ring left out, every kernel gives up, sets the status word
+    and returns; the same calls without the knob are correct."""
+    cfg = CONFIGS["tiny"].with_(name="tile_waits", B=2, Lq=900, Lk=1000, n_h=16, n_kv=8, d_h=128, k_base=150, k_min=1, k_max=209, seed=250)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 251)
+    d = U.to_dev({**x, "dout": x["Q"] * 0.5})
+    gsa.gsa_debug_set_wait_limit(400_000, withhold_first_copy=True)
+    try:
+        status = _run(cfg, d, idx, kt)[2]
+    finally:
+        gsa.gsa_debug_set_wait_limit(0, withhold_first_copy=False)
+    assert status in (1, 2, 3) and _run_bwd(cfg, d, idx, kt, 0, cfg.Lq, True, withhold=True)[1] in (1, 2, 3)
+    torch.cuda.synchronize()
+    out, lse, status = _run(cfg, d, idx, kt)
+    assert status == 0
+    _check(cfg, x, out, lse, idx, kt, _rows(cfg))
+    assert _run_bwd(cfg, d, idx, kt, 0, cfg.Lq, True)[1] == 0
