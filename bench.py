@@ -500,7 +500,7 @@ def main():
         # and KV head (d_h * 2 bytes each); the key-major kernel gathers Q and dout * sigmoid(g1) of every
         # head once per pair (n_h * d_h * 2 bytes each); plus the index sets and their inverse (4 + 4 bytes)
         gather = float(kt_sum) * (2 * cfg.n_kv * cfg.d_h * 2 + 2 * cfg.n_h * cfg.d_h * 2 + 8)
-        backward = {"kernels": "gsa_sparse_attn_bwd_kernel + gsa_sparse_attn_bwd_keys_kernel", "ms": b_ms,
+        backward = {"kernels": "gsa_masked_bwd_* (masked tiles) or gsa_sparse_attn_bwd_* (gather), by the cost models", "ms": b_ms,
                     "bound": "hbm", "algorithmic_bytes": gather, "achieved_gbs": gather / (b_ms * 1e-3) / 1e9,
                     "peak_gbs": peaks["hbm_gbs"], "frac": gather / (b_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                     "ms_recomputing_statistics": b_ms_recompute,

@@ -167,7 +167,7 @@ int gsa_output_projection(const gsa_params_t *p, int32_t d_model, const void *at
  *   lse    [B, Lq, n_h] fp32 or NULL: what gsa_sparse_gated_attn_fwd_lse saved for the same inputs; with it
  *          the sweep over S_t that recomputes the softmax statistics is skipped
  *   ws     workspace of gsa_attn_bwd_workspace_bytes(p) bytes (depends on q_begin / q_end): status word,
- *          V', dout * sigmoid(g1), softmax statistics, and the index sets inverted (key -> query rows)
+ *          V', dout * sigmoid(g1), softmax statistics, and the index sets inverted (key -> query rows) or as masks
  * Returns GSA_ERR_WORKSPACE if ws is too small; nothing is launched on an argument error.
  */
 int gsa_attn_bwd_workspace_bytes(const gsa_params_t *p, size_t *bytes);
