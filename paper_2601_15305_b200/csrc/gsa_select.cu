@@ -58,7 +58,8 @@ struct SelectArgs {
     float v_bar;
 };
 
-// monotone map fp32 -> uint32 (larger float <=> larger key); -0 is folded onto +0
+// monotone map fp32 -> uint32 (larger float <=> larger key); -0 is folded onto +0, and the sum makes every NaN the same
+// one: key 0xFFFFFFFF, above all others.  (-inf has key 0x007FFFFF: no score has key 0.)
 __device__ __forceinline__ uint32_t order_key(float x) {
     const uint32_t b = __float_as_uint(x + 0.0f);
     return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);     // negative: all bits flip; else: sign bit set
@@ -588,11 +589,12 @@ constexpr int short_bins(int NT) { return NT == 128 ? 1024 : 2048; }
 constexpr int short_bins_log2(int NT) { return NT == 128 ? 10 : 11; }
 constexpr int kShortRank = 128;                               // keys of a bin that are ranked directly
 constexpr int kRowCluster = 8;
+constexpr uint32_t kSelOut = 4096;                            // k_max <= 4096
 
 template <int NT>
 struct ShortShared {
     __align__(16) uint32_t hist[short_bins(NT)];
-    int32_t out[4096];                                        // k_max <= 4096
+    int32_t out[kSelOut];
     uint32_t gt[NT], eq[NT];                                  // bitmaps of the slice's positions (32 NT bits)
     uint32_t cand[kShortRank], cand_own[kShortRank];
     double red_a[NT / 32], red_b[NT / 32];
@@ -769,9 +771,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
         want -= sh.found_above;
         lo += fb << shift;
         if (shift == 0) { T = lo; need_eq = want; eq_total = count; break; }
-        hi = min(hi, lo + ((1u << shift) - 1u));
+        const uint32_t left = min(hi - lo, (1u << shift) - 1u);
+        hi = lo + left;                                       // (the last bin's edge may lie past the highest key, a NaN's)
         if (count <= (uint32_t)kShortRank) {
-            const uint32_t left = hi - lo;
 #pragma unroll
             for (int v = 0; v < 8; ++v)
                 if (v * NT * 4 < n) {
@@ -808,7 +810,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
 
     // ---- emission: bitmaps, one scan, ascending positions ----
     const bool cut = eq_total != need_eq;                     // a group of equal keys is cut: lower positions win
-    const uint32_t from = cut ? T + 1u : T;
     uint8_t* const bytes_gt = reinterpret_cast<uint8_t*>(sh.gt);
     uint8_t* const bytes_eq = reinterpret_cast<uint8_t*>(sh.eq);
 #pragma unroll
@@ -817,9 +818,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
             uint32_t g = 0, q = 0;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                g |= (key[v][e] >= from ? 1u : 0u) << e;
+                g |= (key[v][e] >= T ? 1u : 0u) << e;
                 if (cut) q |= (key[v][e] == T ? 1u : 0u) << e;
             }
+            g &= ~q;                                          // (not key >= T + 1: T is the largest number there is in a row of NaN)
             g |= __shfl_down_sync(0xFFFFFFFFu, g, 1) << 4;
             if ((tid & 1) == 0) bytes_gt[(v * NT + tid) / 2] = (uint8_t)g;
             if (cut) {
@@ -857,7 +859,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
         while (q && take) { gw |= q & -q; q &= q - 1u; --take; }
     }
     while (gw) {
-        sh.out[at++] = p0 + tid * 32 + __ffs(gw) - 1;
+        if (at < kSelOut) sh.out[at] = p0 + tid * 32 + __ffs(gw) - 1;
+        ++at;
         gw &= gw - 1u;
     }
     if constexpr (CS > 1) {
