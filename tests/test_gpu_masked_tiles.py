@@ -113,6 +113,42 @@ def test_inputs_that_a_mask_cannot_stand_for(what):
     _check(cfg, x, out, lse, idx, kt, np.unique(np.concatenate([keep, [500]])) if not hit[:, 500].any() else keep)
 
 
+def test_numerators_of_flat_rows_are_rounded_below_one():
+    """Rows whose first tile holds one selected key, with a score a little below all others: the numerators must still fall
+    just below 1, where bf16 is finest.  Against fp64 the output then carries its own rounding (bf16 values with evenly spread
+    logarithms: 1.54e-3 in the 2-norm) and that of the numerators (2^-8 / sqrt 12 over 0.95: 1.19e-3), 1.95e-3 together; just
+    above 1 the numerators' part is 2.2e-3, 2.7e-3 together."""
+    cfg = CONFIGS["tiny"].with_(name="flat", B=1, Lq=1664, Lk=2048, n_h=16, n_kv=8, d_h=128, k_base=300, k_min=1, k_max=419, seed=215)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 216)
+    for t in range(cfg.Lq):                                       # key 0 and nothing else of the first 64 keys
+        s = idx[0, t][idx[0, t] >= 64]
+        idx[0, t] = torch.cat([torch.zeros(1), s, torch.full((cfg.k_max,), -1)])[:cfg.k_max]
+        kt[0, t] = min(cfg.k_max, 1 + len(s))
+    shift = 0.1
+    x["Q"] = (x["Q"].float() + shift).to(torch.bfloat16)
+    x["K"] = (x["K"].float() + 0.2 * shift).to(torch.bfloat16)                         # scores of about 0.033 +- 0.012 in the log2 domain
+    x["K"][:, 0] = 0.0
+    d = U.to_dev(x)
+    p = gsa.make_params(cfg)
+    out = torch.full_like(d["Q"], float("nan"))
+    ws = torch.empty(gsa.gsa_attn_workspace_bytes(p, False), dtype=torch.uint8, device="cuda")
+    n0 = gsa.gsa_launch_count()
+    gsa.gsa_sparse_gated_attn_fwd(p, d["Q"], d["K"], d["V"], d["g1"], None, idx.cuda(), kt.cuda(), out, ws)
+    assert gsa.gsa_launch_count() - n0 == 4 and gsa.gsa_device_status(ws) == 0          # scan of the values, masks, tiles, plain path
+    assert ws.view(torch.int32)[2] == 0                                                 # (the tiles did the work)
+    err = []
+    for t in range(0, cfg.Lq, 4):
+        S = idx[0, t, :int(kt[0, t])].long().cuda()
+        if len(S) < 64:
+            continue
+        k, v = (d[n][0, S].double().repeat_interleave(2, 1) for n in "KV")
+        z = (k * d["Q"][0, t].double()).sum(-1) / cfg.d_h ** 0.5
+        want = (torch.softmax(z, 0)[..., None] * v).sum(0) * torch.sigmoid(d["g1"][0, t].double())
+        err.append(float((out[0, t].double() - want).pow(2).sum() / want.pow(2).sum()))
+    assert len(err) > 200 and np.mean(err) ** 0.5 < 2.1e-3, np.mean(err) ** 0.5
+
+
 # ---- backward ------------------------------------------------------------------------------------------------------
 def _run_bwd(cfg, d, idx, kt, q0, q1, saved_lse, withhold=False):
     p = gsa.make_params(cfg, q_begin=q0, q_end=q1)
