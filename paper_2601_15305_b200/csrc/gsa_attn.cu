@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
                 if (lr0 + q >= rows) break;
 #pragma unroll
                 for (int e = 0; e < G; ++e) {
-                    const bool live = keff[q] > 0 && l[q][e] > 0.f;
+                    const bool live = keff[q] > 0 && l[q][e] != 0.f;      // (a NaN in a selected key shows)
                     const float2 gf = __bfloat1622float2(gl[q][e]);
                     const float v0 = live ? o[q][e] / l[q][e] * fast_sigmoid(gf.x) : 0.f;          // (d, head e)
                     const float v1 = live ? o[q][G + e] / l[q][e] * fast_sigmoid(gf.y) : 0.f;      // (d + 1, head e)
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
 #pragma unroll
                 for (int e = 0; e < G; ++e) {
                     const size_t at = (((size_t)r.b * Lq + r.t) * n_h + g * G + e) * DH + d;
-                    const float v = den[e] > 0.f ? acc[e] / den[e] * fast_sigmoid(__bfloat162float(g1[at])) : 0.f;
+                    const float v = den[e] != 0.f ? acc[e] / den[e] * fast_sigmoid(__bfloat162float(g1[at])) : 0.f;
                     out[at] = __float2bfloat16_rn(v);
                     if (lse && d == 0)
                         lse[((size_t)r.b * Lq + r.t) * n_h + g * G + e] = (mx[e] + log2f(den[e])) * 0.6931471805599453f;

@@ -401,7 +401,7 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             const float l = (la + lb) + (lc + ld);
             const int h = g * G + m % G, t = a.q0 + r;
             const size_t at = (((size_t)b * a.Lq + (live ? t : 0)) * a.n_h + h) * DH;
-            const float inv = l > 0.f ? 1.0f / l : 0.f;            // (an empty set: a zero row)
+            const float inv = l != 0.f ? 1.0f / l : 0.f;           // (an empty set: a zero row; a NaN in a selected key shows)
             if (a.lse && live) a.lse[((size_t)b * a.Lq + t) * a.n_h + h] = (m_ref + log2f(l)) * 0.6931471805599453f;
 #pragma unroll
             for (int c = 0; c < DH / 32; ++c) {
@@ -417,8 +417,8 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const float2 gf = __bfloat1622float2(gp[e]);
-                        const float o0 = l > 0.f ? __uint_as_float(o[q * 8 + 2 * e]) * inv : 0.f;
-                        const float o1 = l > 0.f ? __uint_as_float(o[q * 8 + 2 * e + 1]) * inv : 0.f;
+                        const float o0 = l != 0.f ? __uint_as_float(o[q * 8 + 2 * e]) * inv : 0.f;
+                        const float o1 = l != 0.f ? __uint_as_float(o[q * 8 + 2 * e + 1]) * inv : 0.f;
                         w[e] = pack_bf16(o0 * fast_sigmoid(gf.x), o1 * fast_sigmoid(gf.y));
                     }
                     *reinterpret_cast<uint4*>(a.out + at + c * 32 + q * 8) = make_uint4(w[0], w[1], w[2], w[3]);

@@ -1,0 +1,77 @@
+"""Masked tiles and gather: which of them a call takes, and the same answers from both for inputs that tell them apart."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2601_15305_b200 import binding as gsa
+from paper_2601_15305_b200.inputs import CONFIGS, make_inputs
+
+import gpu_util as U
+from test_gpu_masked_tiles import _sets
+
+pytestmark = pytest.mark.gpu
+
+
+def _fwd(cfg, d, idx, kt, prepass=True):
+    """out, launches, the status head's word that is raised where the tiles leave the work to the gather, status."""
+    p = gsa.make_params(cfg)
+    out = torch.full_like(d["Q"], float("nan"))
+    ws = torch.empty(gsa.gsa_attn_workspace_bytes(p, prepass), dtype=torch.uint8, device="cuda").fill_(0xFF)
+    n0 = gsa.gsa_launch_count()
+    gsa.gsa_sparse_gated_attn_fwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx.cuda(), kt.cuda(), out, ws)
+    n = gsa.gsa_launch_count() - n0
+    status = gsa.gsa_device_status(ws)
+    return out, n, int(ws[:256].view(torch.int32)[2]), status
+
+
+TILES = CONFIGS["tiny"].with_(name="tiles", B=2, Lq=900, Lk=1300, n_h=16, n_kv=8, d_h=128, k_base=300, k_min=1, k_max=419, seed=210)
+
+
+@pytest.mark.parametrize("cfg,prepass,launches", [
+    (TILES, True, 4),                                                                              # gate, masks, tiles, plain path
+    (TILES.with_(name="gather", Lq=700, Lk=4000, k_base=40, k_max=80), True, 3),                  # gate, gather, finalize
+    (TILES.with_(name="fused", Lq=700, Lk=4000, k_base=40, k_max=80), False, 2),
+    (TILES.with_(name="parts", B=3, Lq=2, Lk=3000), False, 2),                                     # decode: sets in segments
+], ids=lambda v: getattr(v, "name", None))
+def test_a_nan_in_a_key_shows_in_the_rows_that_select_it(cfg, prepass, launches):
+    """... in the heads of its KV head, and nowhere else; on every path of the attention stage."""
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 211)
+    x["K"][0, 700, 3, 5] = float("nan")
+    hit = torch.zeros(cfg.B, cfg.Lq, dtype=torch.bool)
+    hit[0] = ((idx[0] == 700) & (torch.arange(cfg.k_max) < kt[0, :, None])).any(-1)
+    if not hit.any():
+        idx[0, 0, 0], kt[0, 0], hit[0, 0] = 700, 1, True
+        idx[0, 0, 1:] = -1
+    out, n, general, status = _fwd(cfg, U.to_dev(x), idx, kt, prepass)
+    assert n == launches and general == 0 and status == 0
+    nan = torch.isnan(out.float().cpu())
+    want = torch.zeros_like(nan)
+    want[:, :, 6:8] = hit[..., None, None]
+    assert (nan == want).all()
+
+
+@pytest.mark.parametrize("jump", [8.5, 9.5, 12.0])
+def test_reference_that_moves_in_either_half_of_a_later_tile(jump):
+    """Two keys of every set exceed all scores before them by `jump` (log2 domain, more than the 2^8 that a reference bears), one
+    in the first and one in the second half of a tile: what was summed before is scaled down by a factor that still counts."""
+    cfg = TILES.with_(name="jump", B=1, Lq=900, Lk=1700)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 212)
+    high = (640 + 17, 1152 + 64 + 9)
+    for t in range(cfg.Lq):
+        s = idx[0, t, :int(kt[0, t])]
+        keys = [k for k in high if k <= cfg.Lk - cfg.Lq + t]
+        s = torch.cat([s[~torch.isin(s, torch.tensor(high, dtype=torch.int32))][:cfg.k_max - 2], torch.tensor(keys, dtype=torch.int32)]).sort().values
+        idx[0, t, :len(s)], idx[0, t, len(s):], kt[0, t] = s, -1, len(s)
+    step = jump * cfg.d_h ** 0.5 / 1.4427 / (0.25 * cfg.d_h)
+    x["Q"] = (x["Q"].float() + 0.5).to(torch.bfloat16)
+    for i, k in enumerate(high):
+        x["K"][:, k] = 0.5 * step * (i + 1)
+    out, n, general, status = _fwd(cfg, U.to_dev(x), idx, kt)
+    assert n == 4 and general == 0 and status == 0
+    rows = np.arange(0, cfg.Lq, 13)
+    want = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx[0][rows].numpy(), kt[0][rows].numpy(), rows,
+                       np.zeros_like(rows))
+    U.check_out(out[0][torch.from_numpy(rows).cuda()].float().cpu().numpy(), want)
