@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
 __global__ void __launch_bounds__(256) gsa_value_gate_kernel(const uint4* __restrict__ V,
                                                              const uint4* __restrict__ g2,
                                                              uint4* __restrict__ Vg, int64_t n_vec,
-                                                             int32_t* nonfinite) {
+                                                             int32_t* untileable) {
     chain_wait();
     uint32_t bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec;
@@ -543,9 +543,9 @@ __global__ void __launch_bounds__(256) gsa_value_gate_kernel(const uint4* __rest
             v2[e] = __floats2bfloat162_rn(vf.x * gate_sigmoid(gf.x), vf.y * gate_sigmoid(gf.y));
         }
         Vg[i] = vv;
-        bad |= nonfinite_bf16x8(vv);
+        bad |= untileable_bf16x8(vv);
     }
-    if (bad && nonfinite) *nonfinite = 1;
+    if (bad && untileable) *untileable = 1;
 }
 
 int g_range_keys = kRangeKeysDefault;
@@ -753,13 +753,13 @@ void set_attn_range_keys(int keys) { g_range_keys = keys >= 1024 ? keys : kRange
 int attn_range_keys() { return g_range_keys; }
 
 cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, __nv_bfloat16* Vg,
-                              int64_t n_elems, cudaStream_t st, int32_t* nonfinite) {
+                              int64_t n_elems, cudaStream_t st, int32_t* untileable) {
     const int64_t n_vec = n_elems / 8;
     if (n_vec <= 0) return cudaSuccess;
     const int blocks = (int)((n_vec + 255) / 256 < sm_count() * 16 ? (n_vec + 255) / 256 : sm_count() * 16);
     launch_chained(gsa_value_gate_kernel, blocks, 256, 0, st, reinterpret_cast<const uint4*>(V),
                                                   reinterpret_cast<const uint4*>(g2),
-                                                  reinterpret_cast<uint4*>(Vg), n_vec, nonfinite);
+                                                  reinterpret_cast<uint4*>(Vg), n_vec, untileable);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -779,7 +779,7 @@ cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bf
         if (t_end > rr.q_begin) {
             cudaError_t e = cudaSuccess;
             if (!values_scanned)
-                e = launch_check_finite(V, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, t_dev_status + kStatusGeneralWord, st);
+                e = launch_check_values(V, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, t_dev_status + kStatusGeneralWord, st);
             if (e != cudaSuccess) return e;
             e = launch_masked_rows(p, rr, t_end, Q, K, V, g1, idx, kt, il, out, scratch, scratch_bytes, st,
                                    progress, lse, all_visible);

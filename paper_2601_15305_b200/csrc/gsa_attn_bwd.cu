@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* 
                                                            const __nv_bfloat16* __restrict__ dout,
                                                            __nv_bfloat16* __restrict__ dOs, __nv_bfloat16* __restrict__ dg1,
                                                            float* __restrict__ delta, RowRange rr, int32_t Lq, int32_t n_h,
-                                                           int32_t* nonfinite /*nullable: raised if do or delta is*/) {
+                                                           int32_t* untileable /*nullable: raised if do or delta is*/) {
     chain_wait();
     constexpr int EPL = DH / 32;
     const int lane = threadIdx.x & 31;
@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* 
     const Vec vdy = *reinterpret_cast<const Vec*>(dout + at), vy = *reinterpret_cast<const Vec*>(out + at),
               vg = *reinterpret_cast<const Vec*>(g1 + at);
     Vec vdo, vdg;
-    float part = 0.f, sum_do = 0.f;
+    float part = 0.f;
+    bool bad = false;
 #pragma unroll
     for (int e = 0; e < EPL; ++e) {
         const float dy = __bfloat162float(vdy.x[e]);
@@ -103,16 +104,15 @@ __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* 
         const float sg = 1.0f / (1.0f + __expf(-__bfloat162float(vg.x[e])));
         vdo.x[e] = __float2bfloat16(dy * sg);
         vdg.x[e] = __float2bfloat16(dy * y * (1.0f - sg));
-        sum_do += dy * sg;
+        bad = bad || !(fabsf(dy * sg) < kTileValueLimit);
         part = fmaf(dy, y, part);
     }
     *reinterpret_cast<Vec*>(dOs + at) = vdo;
     *reinterpret_cast<Vec*>(dg1 + at) = vdg;
-    const float watch = part + sum_do;                                 // (infinities and NaN spread into it)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
     if (lane == 0) delta[qrow * n_h + h] = part;
-    if (nonfinite && !(fabsf(watch) < INFINITY && fabsf(part) < INFINITY)) *nonfinite = 1;
+    if (untileable && (bad || !(fabsf(part) < kTileDeltaLimit))) *untileable = 1;
 }
 
 // first position j of the ascending list S[0 .. n) with S[j] >= x; the whole warp calls it (32 probes a round)
@@ -531,10 +531,10 @@ size_t attn_bwd_range_bytes(const gsa_params_t& p) {
 
 cudaError_t launch_bwd_prep(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* g1, const __nv_bfloat16* out,
                             const __nv_bfloat16* dout, __nv_bfloat16* dOs, __nv_bfloat16* dg1, float* delta,
-                            int32_t* nonfinite, cudaStream_t st) {
+                            int32_t* untileable, cudaStream_t st) {
     const unsigned ctas = (unsigned)(((int64_t)rr.rows() * p.n_h + 7) / 8);
-    if (p.d_h == 128) launch_chained(gsa_bwd_prep_kernel<128>, ctas, 256, 0, st, g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, nonfinite);
-    else launch_chained(gsa_bwd_prep_kernel<64>, ctas, 256, 0, st, g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, nonfinite);
+    if (p.d_h == 128) launch_chained(gsa_bwd_prep_kernel<128>, ctas, 256, 0, st, g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, untileable);
+    else launch_chained(gsa_bwd_prep_kernel<64>, ctas, 256, 0, st, g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, untileable);
     ++g_launches;
     return cudaGetLastError();
 }

@@ -86,17 +86,17 @@ cudaError_t launch_select(const gsa_params_t& p, RowRange rr, const float* score
                           IdxLayout il, int32_t* fallback_rows /*nullable counter*/, cudaStream_t st);
 
 cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, __nv_bfloat16* Vg,
-                              int64_t n_elems, cudaStream_t st, int32_t* nonfinite = nullptr /*raised if a gated value is*/);
+                              int64_t n_elems, cudaStream_t st, int32_t* untileable = nullptr /*raised if a gated value is*/);
 
 // Backward of sparse gated attention.  Query-major half (gsa_attn_bwd.cu): dQ, dg1 for the rows of rr, and
 // per (row, head) do = dout * sigmoid(g1), the softmax statistics lse2 and delta for the key-major half
 // (gsa_attn_bwd_keys.cu), which inverts the index sets inside invert_ws (attn_bwd_invert_bytes) and writes
 // dK, dV, dg2 for every key.
 bool attn_bwd_supported(const gsa_params_t& p);
-// do = dout * sigmoid(g1), dg1 and delta = sum_d dout * out per (row, head); *nonfinite (nullable) is raised if one is not finite
+// do = dout * sigmoid(g1), dg1 and delta = sum_d dout * out per (row, head); *untileable (nullable) is raised if a do or a delta is
 cudaError_t launch_bwd_prep(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* g1, const __nv_bfloat16* out,
                             const __nv_bfloat16* dout, __nv_bfloat16* dOs, __nv_bfloat16* dg1, float* delta,
-                            int32_t* nonfinite, cudaStream_t st);
+                            int32_t* untileable, cudaStream_t st);
 cudaError_t launch_sparse_attn_bwd(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q,
                                    const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1,
                                    const __nv_bfloat16* out, const __nv_bfloat16* dout, const int32_t* idx,
@@ -296,10 +296,14 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) {
     return false;
 }
 
-// nonzero if one of eight bf16 values is infinite or NaN
-__device__ __forceinline__ uint32_t nonfinite_bf16x8(uint4 v) {
-    auto f = [](uint32_t x) -> uint32_t {       // an exponent of all ones carries into the bit above it
-        return (((x & 0x7F807F80u) + 0x00800080u) & 0x80008000u);
+// What the masked tiles must not meet in a row that a set leaves out, because they multiply it by zero: infinities, NaN, and
+// values so large that a product of two rows might overflow before it is multiplied (2^60 each: 128 * 2^120 = 2^127 is finite).
+constexpr float kTileValueLimit = 1152921504606846976.f;         // 2^60
+constexpr float kTileDeltaLimit = 8.507059173023462e37f;         // 2^126: a product below 2^127 and delta still add up
+// nonzero if one of eight bf16 values is that large, infinite or NaN
+__device__ __forceinline__ uint32_t untileable_bf16x8(uint4 v) {
+    auto f = [](uint32_t x) -> uint32_t {       // an exponent field from 127 + 60 on carries into the bit above it
+        return (((x & 0x7F807F80u) + 0x22802280u) & 0x80008000u);
     };
     return f(v.x) | f(v.y) | f(v.z) | f(v.w);
 }

@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256) gsa_visible_masks_kernel(uint4* __restric
 
 // ---- what the tiles cannot take -----------------------------------------------------------------------------
 // A tile multiplies every value row of its 128 keys, by zero where the key is not in the set, and a bit mask holds a
-// key once.  So a call whose gated values are not all finite (0 * inf), or whose sets are not strictly ascending
+// key once.  So a call whose gated values are not all finite and of sane size (untileable_bf16x8), or whose sets are not strictly ascending
 // positions that the row can see, raises the `general` word; the tile kernels then leave at once and this plain
 // kernel (one warp per row and KV head, the set walked entry by entry) does the work.  Otherwise it costs a launch.
 template <int DH, int G>
@@ -191,12 +191,12 @@ gsa_general_attn_kernel(const int32_t* __restrict__ general, const __nv_bfloat16
     }
 }
 
-// raises `general` if a bf16 value is infinite or NaN
-__global__ void __launch_bounds__(256) gsa_check_finite_kernel(const uint4* __restrict__ x, int64_t n_vec, int32_t* general) {
+// raises `general` if a bf16 value is infinite, NaN or too large for the tiles
+__global__ void __launch_bounds__(256) gsa_check_values_kernel(const uint4* __restrict__ x, int64_t n_vec, int32_t* general) {
     chain_wait();
     uint32_t bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * blockDim.x)
-        bad |= nonfinite_bf16x8(__ldg(x + i));
+        bad |= untileable_bf16x8(__ldg(x + i));
     if (bad) *general = 1;
 }
 
@@ -559,10 +559,10 @@ cudaError_t launch_visible_masks(const gsa_params_t& p, const MaskPlan& mp, uint
     return cudaGetLastError();
 }
 
-cudaError_t launch_check_finite(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st) {
+cudaError_t launch_check_values(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st) {
     const int64_t n_vec = n_elems / 8;
     const int64_t want = (n_vec + 255) / 256, cap = (int64_t)sm_count() * 8;
-    launch_chained(gsa_check_finite_kernel, (unsigned)(want < cap ? want : cap), 256, 0, st, reinterpret_cast<const uint4*>(x), n_vec, general);
+    launch_chained(gsa_check_values_kernel, (unsigned)(want < cap ? want : cap), 256, 0, st, reinterpret_cast<const uint4*>(x), n_vec, general);
     ++g_launches;
     return cudaGetLastError();
 }

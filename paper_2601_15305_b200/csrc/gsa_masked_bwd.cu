@@ -959,10 +959,10 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
                               const float* lse_in, void* ws, int32_t* dev_status, cudaStream_t st) {
     int32_t* general = dev_status + kStatusGeneralWord;
     cudaError_t e = launch_bwd_prep(p, rr, g1, out, dout, dOs, dg1, delta, general, st);
-    // (outside the sets the tiles multiply by zero: everything they read has to be finite.  V' and dOs are watched where they
-    // are written; rows of dOs past the range read as zero)
-    if (e == cudaSuccess) e = launch_check_finite(Q, (int64_t)p.B * p.Lq * p.n_h * p.d_h, general, st);
-    if (e == cudaSuccess) e = launch_check_finite(K, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, general, st);
+    // (outside the sets the tiles multiply dP - delta, Q, K and do by zero: all of them have to be finite.  V', do and delta are
+    // watched where they are written; rows of dOs past the range read as zero)
+    if (e == cudaSuccess) e = launch_check_values(Q, (int64_t)p.B * p.Lq * p.n_h * p.d_h, general, st);
+    if (e == cudaSuccess) e = launch_check_values(K, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, general, st);
     const MaskPlan mp = mask_plan(p, rr.q_begin, rr.R);
     uint4* mask = (uint4*)ws;
     if (e == cudaSuccess) e = launch_build_masks(p, mp, masked_block_rows(p), idx, kt, il, mask, general, st);

@@ -75,3 +75,40 @@ def test_reference_that_moves_in_either_half_of_a_later_tile(jump):
     want = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx[0][rows].numpy(), kt[0][rows].numpy(), rows,
                        np.zeros_like(rows))
     U.check_out(out[0][torch.from_numpy(rows).cuda()].float().cpu().numpy(), want)
+
+
+# ---- backward ------------------------------------------------------------------------------------------------------
+BWD = TILES.with_(name="bwd", Lk=1000, k_base=150, k_max=209, seed=240)
+
+
+@pytest.mark.parametrize("what", ["value", "dout"])
+def test_huge_finite_values_that_a_set_leaves_out_do_not_reach_the_gradients(what):
+    """A value row of the lowest bf16 in no set, and a row of dout whose products with the values overflow: the gradients of the
+    rows and keys that do not select them are those of the oracle."""
+    from test_gpu_backward import _compare
+    from test_gpu_masked_tiles import _run_bwd
+    cfg = BWD
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 241)
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(242)) * 0.25).to(torch.bfloat16)
+    if what == "value":
+        x["V"][0, 700] = torch.finfo(torch.bfloat16).min
+        for t in (idx[0] == 700).any(-1).nonzero()[:, 0].tolist():      # (another key in its place)
+            s = set(idx[0, t, :int(kt[0, t])].tolist()) - {700}
+            s |= {next(k for k in range(cfg.Lk) if k not in s and k != 700)}
+            idx[0, t, :len(s)], idx[0, t, len(s):], kt[0, t] = torch.tensor(sorted(s), dtype=torch.int32), -1, len(s)
+    else:
+        key = next(k for k in range(50, cfg.Lk) if k not in set(idx[0, 600].tolist()))
+        x["V"][0, key, 1] *= 64.0
+        dout[0, 600, 3] = (1.0e37 * torch.sign(x["V"][0, key, 1].float())).to(torch.bfloat16)
+    got, status = _run_bwd(cfg, U.to_dev({**x, "dout": dout}), idx, kt, 0, cfg.Lq, True)
+    assert status == 0
+    if what == "value":
+        _compare(cfg, x, got, idx, kt, dout, 0, cfg.Lq)
+        return
+    rows = torch.ones(cfg.B, cfg.Lq, dtype=torch.bool)
+    rows[0, 600] = False
+    keys = torch.ones(cfg.B, cfg.Lk, dtype=torch.bool)
+    keys[0, idx[0, 600, :int(kt[0, 600])].long()] = False
+    for n, live in (("dQ", rows), ("dg1", rows), ("dK", keys), ("dV", keys), ("dg2", keys)):
+        assert torch.isfinite(got[n].float().cpu()[live]).all(), n
