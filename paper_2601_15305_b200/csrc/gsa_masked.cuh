@@ -42,8 +42,10 @@ cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int bl
 // The same for sets known to hold every visible key (k_mode 3 inside gsa_forward): no set is read.
 cudaError_t launch_visible_masks(const gsa_params_t& p, const MaskPlan& mp, uint4* mask, cudaStream_t st);
 
-// Raises *general if one of n_elems (a multiple of 8) values is infinite, NaN or too large (untileable_bf16x8).
-cudaError_t launch_check_values(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st);
+// Raises *general if one of n_elems (a multiple of 8) values is infinite, NaN or too large (untileable_bf16x8); of each of
+// `batches` runs that start batch_stride values (a multiple of 8) apart.
+cudaError_t launch_check_values(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st, int batches = 1,
+                                int64_t batch_stride = 0);
 
 // What a range of rows sees and selects, per KV head: for the choice between the tiles and the gather.  The sets' sizes are on
 // the device; the budget that they centre on stands for them.

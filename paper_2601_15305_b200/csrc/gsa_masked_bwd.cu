@@ -961,7 +961,8 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
     cudaError_t e = launch_bwd_prep(p, rr, g1, out, dout, dOs, dg1, delta, general, st);
     // (outside the sets the tiles multiply dP - delta, Q, K and do by zero: all of them have to be finite.  V', do and delta are
     // watched where they are written; rows of dOs past the range read as zero)
-    if (e == cudaSuccess) e = launch_check_values(Q, (int64_t)p.B * p.Lq * p.n_h * p.d_h, general, st);
+    const int64_t q_row = (int64_t)p.n_h * p.d_h;
+    if (e == cudaSuccess) e = launch_check_values(Q + rr.q_begin * q_row, rr.R * q_row, general, st, p.B, p.Lq * q_row);
     if (e == cudaSuccess) e = launch_check_values(K, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, general, st);
     const MaskPlan mp = mask_plan(p, rr.q_begin, rr.R);
     uint4* mask = (uint4*)ws;

@@ -112,3 +112,25 @@ def test_huge_finite_values_that_a_set_leaves_out_do_not_reach_the_gradients(wha
     keys[0, idx[0, 600, :int(kt[0, 600])].long()] = False
     for n, live in (("dQ", rows), ("dg1", rows), ("dK", keys), ("dV", keys), ("dg2", keys)):
         assert torch.isfinite(got[n].float().cpu()[live]).all(), n
+
+
+def test_rows_outside_the_range_do_not_choose_the_path():
+    """A NaN in a row of Q that the call does not handle (a buffer that another row block has not filled) changes nothing."""
+    from test_gpu_backward import _compare
+    cfg, q0, q1 = BWD, 100, 850
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 243)
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(244)) * 0.25).to(torch.bfloat16)
+    d = U.to_dev({**x, "dout": dout})
+    d["Q"][:, :q0], d["Q"][:, q1:] = float("nan"), float("inf")
+    p = gsa.make_params(cfg, q_begin=q0, q_end=q1)
+    out, lse = torch.empty_like(d["Q"]), torch.empty((cfg.B, cfg.Lq, cfg.n_h), dtype=torch.float32, device="cuda")
+    ws = torch.empty(max(gsa.gsa_attn_workspace_bytes(p, True), gsa.gsa_attn_bwd_workspace_bytes(p)), dtype=torch.uint8, device="cuda")
+    i, k = idx[:, q0:q1].contiguous(), kt[:, q0:q1].contiguous()
+    gsa.gsa_sparse_gated_attn_fwd_lse(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], i.cuda(), k.cuda(), out, lse, ws)
+    got = {n: torch.full_like(d["Q" if n in ("dQ", "dg1") else "K"], float("nan")) for n in ("dQ", "dg1", "dK", "dV", "dg2")}
+    got["pbar"] = torch.empty((cfg.B, q1 - q0, cfg.k_max), dtype=torch.float32, device="cuda")
+    gsa.gsa_sparse_gated_attn_bwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], i.cuda(), k.cuda(), out, d["dout"], got["dQ"], got["dK"],
+                                  got["dV"], got["dg1"], got["dg2"], ws, pbar=got["pbar"], lse=lse)
+    assert gsa.gsa_device_status(ws) == 0 and ws[:256].view(torch.int32)[2] == 0
+    _compare(cfg, x, got, i, k, dout, q0, q1)
