@@ -70,6 +70,10 @@ struct AttnArgs {
     int32_t range, n_cuts;
     float scale_log2;         // sm_scale * log2(e)
     float* lse;               // optional output [B, Lq, n_h]: natural log of sum_j exp(sm_scale * q.k_j) over S_t
+    const int32_t* only_if;   // see left_out
+    int32_t run_if;
+    const __nv_bfloat16* g1;  // DIRECT only
+    __nv_bfloat16* out;
     int32_t* dev_status;      // where an out-of-range index or budget is reported (may be null)
 };
 
@@ -110,10 +114,13 @@ __host__ __device__ __forceinline__ int parts_of(int k_eff, int max_parts) {
     return p < 1 ? 1 : (p > max_parts ? max_parts : p);
 }
 
-template <int DH, int G, bool FUSE_G2>
+// DIRECT: whole sets in one launch, in any order of their entries; rows are normalised, gated and written here instead of through
+// the state (what the masked tiles leave to the gather).
+template <int DH, int G, bool FUSE_G2, bool DIRECT = false>
 __global__ void __launch_bounds__((FUSE_G2 ? kWarpsFused : kWarpsPrefill) * 32, 1)
 gsa_sparse_attn_kernel(const AttnArgs a) {
     chain_wait();
+    if (left_out(a.only_if, a.run_if)) return;
     constexpr int HEAD_BYTES = DH * 2;
     constexpr int NC = DH / 32;                         // 32-d chunks of a head row (one uint4 per thread each)
     constexpr int MT = DH / 16;                         // output m-tiles
@@ -136,7 +143,8 @@ gsa_sparse_attn_kernel(const AttnArgs a) {
     const bool real_cols = 2 * tig < G;                 // this thread's output columns hold real heads
 
     const int rows = a.rr.rows();
-    const int64_t n_items = (int64_t)rows * n_kv * (a.mode == 1 ? a.max_parts : 1);
+    const int mode = DIRECT ? 0 : a.mode;
+    const int64_t n_items = (int64_t)rows * n_kv * (mode == 1 ? a.max_parts : 1);
     const int warps = blockDim.x >> 5;                  // kWarpsPerCta, or fewer where few items are spread over the SMs
     const int64_t warps_total = (int64_t)gridDim.x * warps;
 
@@ -144,14 +152,14 @@ gsa_sparse_attn_kernel(const AttnArgs a) {
         const int g = (int)(item % n_kv);
         int64_t rest = item / n_kv;
         int part = 0;
-        if (a.mode == 1) { part = (int)(rest % a.max_parts); rest /= a.max_parts; }
+        if (mode == 1) { part = (int)(rest % a.max_parts); rest /= a.max_parts; }
         const RowId r = row_of(a.rr, a.il, (int)rest);
         const int k_eff = checked_budget(a.kt[r.irow], a.k_max, a.dev_status);
         int lo, hi, slot = 0;
-        if (a.mode == 0) {
+        if (mode == 0) {
             lo = 0;
             hi = k_eff;
-            if (a.n_cuts > 1) {
+            if (!DIRECT && a.n_cuts > 1) {
                 const int32_t* c = a.cuts + r.irow * a.n_cuts + a.range;
                 lo = c[0];
                 if (a.range + 1 < a.n_cuts) hi = c[1];
@@ -165,7 +173,7 @@ gsa_sparse_attn_kernel(const AttnArgs a) {
             slot = part;
         }
         const int count = hi - lo;
-        if (count <= 0 && !(a.mode == 1)) continue;
+        if (count <= 0 && mode == 0 && !DIRECT) continue;
         const int32_t* __restrict__ idx_seg = a.idx + r.irow * a.k_max + lo;
         const int ntiles = (count + kTileKeys - 1) / kTileKeys;
         float* __restrict__ st = a.state + (((int64_t)slot * a.idx_rows + r.irow) * n_kv + g) * STATE_F;
@@ -184,7 +192,7 @@ gsa_sparse_attn_kernel(const AttnArgs a) {
         // ---- state: O^T[d, head] fragments, running max and sum per head ----------------------
         float o[MT][4];
         float m_run[2], l_run[2];
-        const bool carry_in = a.mode == 0 && lo > 0;
+        const bool carry_in = mode == 0 && !DIRECT && lo > 0;
         if (carry_in && real_cols) {
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt)
@@ -374,7 +382,22 @@ gsa_sparse_attn_kernel(const AttnArgs a) {
             l_run[e] += __shfl_xor_sync(0xFFFFFFFFu, l_run[e], 8);
             l_run[e] += __shfl_xor_sync(0xFFFFFFFFu, l_run[e], 16);
         }
-        if (real_cols) {
+        if (DIRECT) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                if (2 * tig + e >= G) continue;
+                const size_t head = ((size_t)r.b * a.Lq + r.t) * a.n_h + g * G + 2 * tig + e;
+                const bool live = k_eff > 0 && l_run[e] != 0.f;
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf) {
+                        const size_t at = head * DH + mt * 16 + hf * 8 + gid;
+                        a.out[at] = __float2bfloat16_rn(live ? o[mt][hf * 2 + e] / l_run[e] * fast_sigmoid(__bfloat162float(a.g1[at])) : 0.f);
+                    }
+                if (a.lse && gid == 0) a.lse[head] = (m_run[e] + log2f(l_run[e])) * 0.6931471805599453f;
+            }
+        } else if (real_cols) {
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
@@ -395,8 +418,10 @@ gsa_sparse_attn_kernel(const AttnArgs a) {
 // cuts[row][c] = number of selected positions of the row below c * range_keys (c = 0 .. n_cuts-1)
 __global__ void __launch_bounds__(256) gsa_range_cuts_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ kt,
                                                              int32_t* __restrict__ cuts, RowRange rr, IdxLayout il,
-                                                             int k_max, int n_cuts, int range_keys) {
+                                                             int k_max, int n_cuts, int range_keys, const int32_t* only_if,
+                                                             int32_t run_if) {
     chain_wait();
+    if (left_out(only_if, run_if)) return;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)rr.rows() * n_cuts) return;
     const int c = (int)(i % n_cuts);
@@ -422,8 +447,9 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
                                                                 const __nv_bfloat16* __restrict__ g1, __nv_bfloat16* __restrict__ out,
                                                                 RowRange rr, IdxLayout il, int64_t idx_rows, int Lq, int n_h,
                                                                 int n_kv, int k_max, int mode, int max_parts,
-                                                                float* __restrict__ lse) {
+                                                                float* __restrict__ lse, const int32_t* only_if, int32_t run_if) {
     chain_wait();
+    if (left_out(only_if, run_if)) return;
     constexpr int STATE_F = G * (DH + 2);
     const int rows = rr.rows();
     // range mode: kFinRows rows per CTA, all (KV head, d) pairs; parts mode (few rows, several state slots to
@@ -545,7 +571,7 @@ __global__ void __launch_bounds__(256) gsa_value_gate_kernel(const uint4* __rest
         Vg[i] = vv;
         bad |= untileable_bf16x8(vv);
     }
-    if (bad && untileable) *untileable = 1;
+    if (bad && untileable) atomicOr(untileable, kGeneralValues);
 }
 
 int g_range_keys = kRangeKeysDefault;
@@ -598,7 +624,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
     if (pl.mode == 0 && pl.n_ranges > 1) {
         const int64_t n = (int64_t)rr_all.rows() * pl.n_ranges;
         launch_chained(gsa_range_cuts_kernel, (unsigned)((n + 255) / 256), 256, 0, st, a.idx, a.kt, cuts, rr_all, a.il, a.k_max,
-                                                                          pl.n_ranges, g_range_keys);
+                       pl.n_ranges, g_range_keys, a.only_if, a.run_if);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         timeline_mark(kStageRangeCuts, st);
@@ -616,7 +642,8 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
         const dim3 fin_grid = pl.mode == 0 ? dim3((unsigned)((fr.rows() + kFinRows - 1) / kFinRows), 1)
                                            : dim3((unsigned)fr.rows(), (unsigned)a.n_kv);
         launch_chained(gsa_attn_finalize_kernel<DH, G>, fin_grid, pl.mode == 0 ? fin_threads : DH, 0, st,
-            a.state, a.kt, g1, out, fr, a.il, a.idx_rows, p.Lq, p.n_h, p.n_kv, p.k_max, pl.mode, pl.slots, a.lse);
+            a.state, a.kt, g1, out, fr, a.il, a.idx_rows, p.Lq, p.n_h, p.n_kv, p.k_max, pl.mode, pl.slots, a.lse,
+            a.only_if, a.run_if);
         ++g_launches;
         cudaError_t fe = cudaGetLastError();
         timeline_mark(kStageFinalize, st);
@@ -704,32 +731,6 @@ int masked_rows_end(const gsa_params_t& p, const AttnPlan& pl, const RowRange& r
     return t_end;
 }
 
-cudaError_t launch_masked_rows(const gsa_params_t& p, const RowRange& rr, int t_end, const __nv_bfloat16* Q,
-                               const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const int32_t* idx,
-                               const int32_t* kt, IdxLayout il, __nv_bfloat16* out, void* scratch, size_t scratch_bytes,
-                               cudaStream_t st, AttnProgress* prog, float* lse, bool all_visible) {
-    const int block = masked_block_rows(p);
-    const size_t row_bytes = mask_plan(p, 0, kMaskRowAlign).bytes(p.B) / kMaskRowAlign;
-    int64_t per = (int64_t)(scratch_bytes / row_bytes) / block * block;
-    if (per < block) return cudaErrorInvalidValue;
-    for (int q = rr.q_begin; q < t_end; q += (int)per) {
-        const MaskPlan mp = mask_plan(p, q, (int)(t_end - q < per ? t_end - q : per));
-        cudaError_t e = all_visible ? launch_visible_masks(p, mp, (uint4*)scratch, st)
-                                    : launch_build_masks(p, mp, block, idx, kt, il, (uint4*)scratch, t_dev_status + kStatusGeneralWord, st);
-        if (e != cudaSuccess) return e;
-        timeline_mark(kStageRangeCuts, st);
-        e = launch_masked_attn_fwd(p, mp, (const uint4*)scratch, Q, K, Vg, g1, out, lse, idx, kt, il, t_dev_status, st);
-        if (e != cudaSuccess) return e;
-        timeline_mark(kStageAttn, st);
-        if (prog && prog->n < prog->cap && prog->n < 64) {
-            if ((e = cudaEventRecord(prog->events[prog->n], st)) != cudaSuccess) return e;
-            prog->t_lo[prog->n] = q; prog->t_hi[prog->n] = q + mp.rows;
-            ++prog->n;
-        }
-    }
-    return cudaSuccess;
-}
-
 template <int DH, bool FUSE_G2>
 cudaError_t launch_attn_g(const AttnArgs& a, const gsa_params_t& p, const AttnPlan& pl, const __nv_bfloat16* g1,
                           __nv_bfloat16* out, int32_t* cuts, int G, cudaStream_t st, AttnProgress* prog) {
@@ -742,6 +743,85 @@ cudaError_t launch_attn_g(const AttnArgs& a, const gsa_params_t& p, const AttnPl
     return cudaErrorInvalidValue;
 }
 
+// (the cuts lie behind the state)
+template <bool FUSE_G2>
+cudaError_t launch_attn_dh(const AttnArgs& a, const gsa_params_t& p, const AttnPlan& pl, const __nv_bfloat16* g1, __nv_bfloat16* out,
+                           cudaStream_t st, AttnProgress* prog) {
+    int32_t* cuts = reinterpret_cast<int32_t*>((char*)a.state + (pl.state_bytes + 255) / 256 * 256);
+    const int G = p.n_h / p.n_kv;
+    if (p.d_h == 128) return launch_attn_g<128, FUSE_G2>(a, p, pl, g1, out, cuts, G, st, prog);
+    if (p.d_h == 64) return launch_attn_g<64, FUSE_G2>(a, p, pl, g1, out, cuts, G, st, prog);
+    return cudaErrorInvalidValue;
+}
+
+AttnArgs attn_args(const gsa_params_t& p, const AttnPlan& pl, const RowRange& rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                   const __nv_bfloat16* V, const __nv_bfloat16* g2, const int32_t* idx, const int32_t* kt, IdxLayout il,
+                   void* scratch, float* lse) {
+    AttnArgs a;
+    a.lse = lse;
+    a.dev_status = t_dev_status;
+    a.Q = Q; a.K = K; a.V = V; a.g2 = g2; a.idx = idx; a.kt = kt;
+    a.state = reinterpret_cast<float*>(scratch);
+    a.cuts = nullptr;
+    a.rr = rr; a.il = il; a.idx_rows = (int64_t)p.B * p.Lq;
+    a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv; a.k_max = p.k_max;
+    a.mode = pl.mode; a.max_parts = pl.slots; a.range = 0; a.n_cuts = pl.n_ranges;
+    const float sc = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
+    a.scale_log2 = sc * 1.4426950408889634f;
+    a.only_if = nullptr; a.run_if = 0; a.g1 = nullptr; a.out = nullptr;
+    return a;
+}
+
+template <int DH, int G>
+cudaError_t launch_direct_t(const AttnArgs& a, cudaStream_t st) {
+    constexpr int smem = kWarpsPrefill * kVStages * kTileKeys * (DH * 2 + 16);
+    auto kern = gsa_sparse_attn_kernel<DH, G, false, true>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t want = ((int64_t)a.rr.rows() * a.n_kv + kWarpsPrefill - 1) / kWarpsPrefill;
+    launch_chained(kern, (unsigned)(want < sm_count() ? want : sm_count()), kWarpsPrefill * 32, smem, st, a);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_masked_rows(const gsa_params_t& p, const AttnPlan& pl, const RowRange& rr, int t_end, const __nv_bfloat16* Q,
+                               const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const int32_t* idx,
+                               const int32_t* kt, IdxLayout il, __nv_bfloat16* out, void* scratch, size_t scratch_bytes,
+                               cudaStream_t st, AttnProgress* prog, float* lse, bool all_visible) {
+    const int block = masked_block_rows(p);
+    const size_t row_bytes = mask_plan(p, 0, kMaskRowAlign).bytes(p.B) / kMaskRowAlign;
+    int64_t per = (int64_t)(scratch_bytes / row_bytes) / block * block;
+    if (per < block) return cudaErrorInvalidValue;
+    int32_t* const general = t_dev_status + kStatusGeneralWord;
+    for (int q = rr.q_begin; q < t_end; q += (int)per) {
+        const MaskPlan mp = mask_plan(p, q, (int)(t_end - q < per ? t_end - q : per));
+        cudaError_t e = all_visible ? launch_visible_masks(p, mp, (uint4*)scratch, st)
+                                    : launch_build_masks(p, mp, block, idx, kt, il, (uint4*)scratch, general, st);
+        if (e != cudaSuccess) return e;
+        timeline_mark(kStageRangeCuts, st);
+        e = launch_masked_attn_fwd(p, mp, (const uint4*)scratch, Q, K, Vg, g1, out, lse, t_dev_status, st);
+        if (e != cudaSuccess) return e;
+        timeline_mark(kStageAttn, st);
+        // What the tiles have left: the gather, key range by key range if the sets are in order, else whole sets at once.
+        RowRange chunk = rr;
+        chunk.q_begin = q; chunk.R = mp.rows;
+        const bool ranges = pl.mode == 0 && pl.n_ranges > 1;
+        e = launch_attn_direct(p, chunk, Q, K, Vg, g1, idx, kt, il, out, lse, general, ranges ? kRunGeneralSets : kRunAnyGeneral, st);
+        if (e == cudaSuccess && ranges) {
+            AttnArgs a = attn_args(p, pl, chunk, Q, K, Vg, nullptr, idx, kt, il, scratch, lse);
+            a.only_if = general; a.run_if = kRunValuesOnly;
+            e = launch_attn_dh<false>(a, p, pl, g1, out, st, nullptr);
+        }
+        if (e != cudaSuccess) return e;
+        if (prog && prog->n < prog->cap && prog->n < 64) {
+            if ((e = cudaEventRecord(prog->events[prog->n], st)) != cudaSuccess) return e;
+            prog->t_lo[prog->n] = q; prog->t_hi[prog->n] = q + mp.rows;
+            ++prog->n;
+        }
+    }
+    return cudaSuccess;
+}
+
 }  // namespace
 
 size_t attn_scratch_bytes(const gsa_params_t& p) {
@@ -751,6 +831,19 @@ size_t attn_scratch_bytes(const gsa_params_t& p) {
 
 void set_attn_range_keys(int keys) { g_range_keys = keys >= 1024 ? keys : kRangeKeysDefault; }
 int attn_range_keys() { return g_range_keys; }
+
+cudaError_t launch_attn_direct(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                               const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const int32_t* idx, const int32_t* kt, IdxLayout il,
+                               __nv_bfloat16* out, float* lse, const int32_t* only_if, int32_t run_if, cudaStream_t st) {
+    AttnArgs a = attn_args(p, plan_attn(p), rr, Q, K, Vg, nullptr, idx, kt, il, nullptr, lse);
+    a.only_if = only_if; a.run_if = run_if; a.g1 = g1; a.out = out;
+    const int G = p.n_h / p.n_kv;
+#define GSA_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_direct_t<DH_, G_>(a, st)
+    GSA_CASE(128, 1); GSA_CASE(128, 2); GSA_CASE(128, 4); GSA_CASE(128, 8);
+    GSA_CASE(64, 1); GSA_CASE(64, 2); GSA_CASE(64, 4); GSA_CASE(64, 8);
+#undef GSA_CASE
+    return cudaErrorInvalidValue;
+}
 
 cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, __nv_bfloat16* Vg,
                               int64_t n_elems, cudaStream_t st, int32_t* untileable) {
@@ -781,33 +874,15 @@ cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bf
             if (!values_scanned)
                 e = launch_check_values(V, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, t_dev_status + kStatusGeneralWord, st);
             if (e != cudaSuccess) return e;
-            e = launch_masked_rows(p, rr, t_end, Q, K, V, g1, idx, kt, il, out, scratch, scratch_bytes, st,
+            e = launch_masked_rows(p, pl, rr, t_end, Q, K, V, g1, idx, kt, il, out, scratch, scratch_bytes, st,
                                    progress, lse, all_visible);
             if (e != cudaSuccess || t_end >= rr.q_begin + rr.R) return e;
             rr.R = rr.q_begin + rr.R - t_end;
             rr.q_begin = t_end;
         }
     }
-    AttnArgs a;
-    a.lse = lse;
-    a.dev_status = t_dev_status;
-    a.Q = Q; a.K = K; a.V = V; a.g2 = g2; a.idx = idx; a.kt = kt;
-    a.state = reinterpret_cast<float*>(scratch);
-    int32_t* cuts = reinterpret_cast<int32_t*>((char*)scratch + (pl.state_bytes + 255) / 256 * 256);
-    a.cuts = cuts;
-    a.rr = rr; a.il = il; a.idx_rows = (int64_t)p.B * p.Lq;
-    a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv; a.k_max = p.k_max;
-    a.mode = pl.mode; a.max_parts = pl.slots; a.range = 0; a.n_cuts = pl.n_ranges;
-    const float sc = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
-    a.scale_log2 = sc * 1.4426950408889634f;
-    const int G = p.n_h / p.n_kv;
-    if (p.d_h == 128)
-        return g2 ? launch_attn_g<128, true>(a, p, pl, g1, out, cuts, G, st, progress)
-                  : launch_attn_g<128, false>(a, p, pl, g1, out, cuts, G, st, progress);
-    if (p.d_h == 64)
-        return g2 ? launch_attn_g<64, true>(a, p, pl, g1, out, cuts, G, st, progress)
-                  : launch_attn_g<64, false>(a, p, pl, g1, out, cuts, G, st, progress);
-    return cudaErrorInvalidValue;
+    const AttnArgs a = attn_args(p, pl, rr, Q, K, V, g2, idx, kt, il, scratch, lse);
+    return g2 ? launch_attn_dh<true>(a, p, pl, g1, out, st, progress) : launch_attn_dh<false>(a, p, pl, g1, out, st, progress);
 }
 
 }  // namespace gsa

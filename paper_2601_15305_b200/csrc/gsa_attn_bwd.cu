@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* 
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
     if (lane == 0) delta[qrow * n_h + h] = part;
-    if (untileable && (bad || !(fabsf(part) < kTileDeltaLimit))) *untileable = 1;
+    if (untileable && (bad || !(fabsf(part) < kTileDeltaLimit))) atomicOr(untileable, kGeneralValues);
 }
 
 // first position j of the ascending list S[0 .. n) with S[j] >= x; the whole warp calls it (32 probes a round)

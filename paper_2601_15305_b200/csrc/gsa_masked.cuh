@@ -72,12 +72,15 @@ inline RowsWork rows_work(const gsa_params_t& p, int nb, int q0, int rows, int b
 inline int masked_block_rows(const gsa_params_t& p) { return 256 / (p.n_h / p.n_kv); }
 
 // Attention of the rows of mp.  dev_status: the call's status head, whose `general` word says whether the tiles may be
-// used (the masks and the scan of the values come first on the stream); if not, the same launch pair does the rows one
-// set entry at a time.
+// used (the masks and the scan of the values come first on the stream); if not, the launch leaves the rows to the gather.
 cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, const uint4* mask, const __nv_bfloat16* Q,
                                    const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1,
-                                   __nv_bfloat16* out, float* lse, const int32_t* idx, const int32_t* kt, IdxLayout il,
-                                   int32_t* dev_status, cudaStream_t st);
+                                   __nv_bfloat16* out, float* lse, int32_t* dev_status, cudaStream_t st);
+
+// The gather over whole sets in one launch (gsa_attn.cu), run if the word at only_if is one that run_if names (left_out).
+cudaError_t launch_attn_direct(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                               const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const int32_t* idx, const int32_t* kt, IdxLayout il,
+                               __nv_bfloat16* out, float* lse, const int32_t* only_if, int32_t run_if, cudaStream_t st);
 
 // Backward (gsa_masked_bwd.cu): all gradients of the attention stage and the target of the indexer's loss (pbar, zeroed by
 // the caller; may be null).  V: as given, Vg: gated and scanned.  ws: masked_bwd_bytes(p, rr) bytes.

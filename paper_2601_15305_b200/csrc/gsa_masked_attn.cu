@@ -103,7 +103,7 @@ gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restric
         }
         __syncthreads();
     }
-    if (at < k || !regular) *general = 1;              // (at < k: an entry past what the row can see, or out of order)
+    if (at < k || !regular) atomicOr(general, kGeneralSets);              // (at < k: an entry past what the row can see, or out of order)
 }
 
 // masks of sets that hold every visible key: nothing to read
@@ -120,77 +120,9 @@ __global__ void __launch_bounds__(256) gsa_visible_masks_kernel(uint4* __restric
 
 // ---- what the tiles cannot take -----------------------------------------------------------------------------
 // A tile multiplies every value row of its 128 keys, by zero where the key is not in the set, and a bit mask holds a
-// key once.  So a call whose gated values are not all finite and of sane size (untileable_bf16x8), or whose sets are not strictly ascending
-// positions that the row can see, raises the `general` word; the tile kernels then leave at once and this plain
-// kernel (one warp per row and KV head, the set walked entry by entry) does the work.  Otherwise it costs a launch.
-template <int DH, int G>
-__global__ void __launch_bounds__(256)
-gsa_general_attn_kernel(const int32_t* __restrict__ general, const __nv_bfloat16* __restrict__ Q,
-                        const __nv_bfloat16* __restrict__ K, const __nv_bfloat16* __restrict__ V,
-                        const __nv_bfloat16* __restrict__ g1, const int32_t* __restrict__ idx,
-                        const int32_t* __restrict__ kt, IdxLayout il, __nv_bfloat16* __restrict__ out,
-                        float* __restrict__ lse, int32_t* dev_status, int q0, int rows, int B, int Lq, int Lk, int n_kv,
-                        int k_max, float scale_log2) {
-    chain_wait();
-    if (*general == 0) return;
-    constexpr int NV = DH / 32;
-    const int lane = threadIdx.x & 31, n_h = n_kv * G;
-    auto load = [&](const __nv_bfloat16* p, float (&f)[NV]) {
-#pragma unroll
-        for (int c = 0; c < NV; ++c) f[c] = __bfloat162float(p[lane * NV + c]);
-    };
-    const int64_t items = (int64_t)B * rows * n_kv;
-    for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < items; item += (int64_t)gridDim.x * 8) {
-        const int g = (int)(item % n_kv), b = (int)(item / n_kv / rows), t = q0 + (int)(item / n_kv % rows);
-        const int64_t irow = il.row(b, t);
-        const int k = checked_budget(kt[irow], k_max, dev_status);
-        float q[G][NV], o[G][NV], m[G], l[G];
-#pragma unroll
-        for (int e = 0; e < G; ++e) {
-            load(Q + (((size_t)b * Lq + t) * n_h + g * G + e) * DH, q[e]);
-            m[e] = -INFINITY; l[e] = 0.f;
-#pragma unroll
-            for (int c = 0; c < NV; ++c) o[e][c] = 0.f;
-        }
-        for (int j = 0; j < k; ++j) {
-            const int s = checked_pos(idx[irow * k_max + j], Lk, dev_status);
-            const size_t at = (((size_t)b * Lk + s) * n_kv + g) * DH;
-            float kr[NV], vr[NV];
-            load(K + at, kr);
-            load(V + at, vr);
-#pragma unroll
-            for (int e = 0; e < G; ++e) {
-                float z = 0.f;
-#pragma unroll
-                for (int c = 0; c < NV; ++c) z = fmaf(q[e][c], kr[c], z);
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, d);
-                z *= scale_log2;
-                if (z > m[e]) {
-                    const float alpha = exp2f(m[e] - z);
-                    m[e] = z; l[e] *= alpha;
-#pragma unroll
-                    for (int c = 0; c < NV; ++c) o[e][c] *= alpha;
-                }
-                const float pz = exp2f(z - m[e]);
-                l[e] += pz;
-#pragma unroll
-                for (int c = 0; c < NV; ++c) o[e][c] = fmaf(pz, vr[c], o[e][c]);
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < G; ++e) {
-            const size_t at = (((size_t)b * Lq + t) * n_h + g * G + e) * DH;
-            float gl[NV];
-            load(g1 + at, gl);
-#pragma unroll
-            for (int c = 0; c < NV; ++c)
-                out[at + lane * NV + c] = __float2bfloat16_rn(k > 0 ? o[e][c] / l[e] * fast_sigmoid(gl[c]) : 0.f);
-            if (lse && lane == 0) lse[((size_t)b * Lq + t) * n_h + g * G + e] = (m[e] + log2f(l[e])) * 0.6931471805599453f;
-        }
-    }
-}
-
+// key once.  So a call whose gated values are not all finite and of sane size (untileable_bf16x8), or whose sets are not strictly
+// ascending positions that the row can see, raises the `general` word; the tile kernels then leave at once and the gather kernels,
+// enqueued behind them, do the work, at the speed that they have anyway.  Otherwise these cost a launch.
 // raises `general` if a bf16 value is infinite, NaN or too large for the tiles
 __global__ void __launch_bounds__(256) gsa_check_values_kernel(const uint4* __restrict__ x, int64_t n_vec, int64_t batch_vec,
                                                                int ctas_per_batch, int32_t* general) {
@@ -199,7 +131,7 @@ __global__ void __launch_bounds__(256) gsa_check_values_kernel(const uint4* __re
     x += blockIdx.x / ctas_per_batch * batch_vec;
     for (int64_t i = (int64_t)(blockIdx.x % ctas_per_batch) * blockDim.x + threadIdx.x; i < n_vec; i += (int64_t)ctas_per_batch * blockDim.x)
         bad |= untileable_bf16x8(__ldg(x + i));
-    if (bad) *general = 1;
+    if (bad) atomicOr(general, kGeneralValues);
 }
 
 // ---- forward ---------------------------------------------------------------------------------------------
@@ -574,8 +506,7 @@ cudaError_t launch_check_values(const __nv_bfloat16* x, int64_t n_elems, int32_t
 
 cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, const uint4* mask, const __nv_bfloat16* Q,
                                    const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1,
-                                   __nv_bfloat16* out, float* lse, const int32_t* idx, const int32_t* kt, IdxLayout il,
-                                   int32_t* dev_status, cudaStream_t st) {
+                                   __nv_bfloat16* out, float* lse, int32_t* dev_status, cudaStream_t st) {
     const int G = p.n_h / p.n_kv;
     CUtensorMap tq, tk, tv;
     if (!make_heads_tmap(&tq, Q + (size_t)mp.q0 * p.n_h * p.d_h, p.B, p.Lq, mp.rows, p.n_h, p.d_h, 128 / G, G)) return cudaErrorUnknown;
@@ -590,17 +521,7 @@ cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, co
     a.scale_log2 = sc * 1.4426950408889634f;
     a.wait_cycles = wait_limit_cycles();
     a.withhold_first = withhold_first_copy() ? 1 : 0;
-    const int ctas = sm_count() * 4;
-#define GSA_CASE(DH_, G_)                                                                                              \
-    if (p.d_h == DH_ && G == G_) {                                                                                     \
-        cudaError_t e = launch_fwd_t<DH_, G_>(a, p, tq, tk, tv, st);                                                   \
-        if (e != cudaSuccess) return e;                                                                                \
-        launch_chained(gsa_general_attn_kernel<DH_, G_>, ctas, 256, 0, st, a.general, Q, K, Vg, g1, idx, kt, il, out, lse,         \
-                                                               dev_status, mp.q0, mp.rows, p.B, p.Lq, p.Lk, p.n_kv,   \
-                                                               p.k_max, a.scale_log2);                                \
-        ++g_launches;                                                                                                  \
-        return cudaGetLastError();                                                                                     \
-    }
+#define GSA_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_fwd_t<DH_, G_>(a, p, tq, tk, tv, st)
     GSA_CASE(128, 1); GSA_CASE(128, 2); GSA_CASE(128, 4); GSA_CASE(128, 8);
     GSA_CASE(64, 1); GSA_CASE(64, 2); GSA_CASE(64, 4); GSA_CASE(64, 8);
 #undef GSA_CASE

@@ -969,7 +969,8 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
     if (e == cudaSuccess) e = launch_build_masks(p, mp, masked_block_rows(p), idx, kt, il, mask, general, st);
     if (e == cudaSuccess && !lse_in) {
         // the statistics were not saved: the forward's tiles once more (their output goes where dQ is written afterwards)
-        e = launch_masked_attn_fwd(p, mp, mask, Q, K, Vg, g1, dQ, lse_ws, idx, kt, il, dev_status, st);
+        e = launch_masked_attn_fwd(p, mp, mask, Q, K, Vg, g1, dQ, lse_ws, dev_status, st);
+        if (e == cudaSuccess) e = launch_attn_direct(p, rr, Q, K, Vg, g1, idx, kt, il, dQ, lse_ws, general, kRunAnyGeneral, st);
         lse_in = lse_ws;
     }
     if (e != cudaSuccess) return e;

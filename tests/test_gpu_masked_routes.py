@@ -134,3 +134,87 @@ def test_rows_outside_the_range_do_not_choose_the_path():
                                   got["dV"], got["dg1"], got["dg2"], ws, pbar=got["pbar"], lse=lse)
     assert gsa.gsa_device_status(ws) == 0 and ws[:256].view(torch.int32)[2] == 0
     _compare(cfg, x, got, i, k, dout, q0, q1)
+
+
+# ---- what the tiles leave to the gather ----------------------------------------------------------------------------
+SETS, VALUES = 1, 2                              # bits of the status head's word
+
+
+def _irregular(cfg, what, x, idx, kt):
+    """Applies `what` to row 500 of batch element 1 (a set that is otherwise in order and visible) or to the values; returns the
+    bit it raises and the status."""
+    kt[1, 500] = 7
+    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, 700, 800 if cfg.Lk > 1100 else 590], dtype=torch.int32).sort().values
+    idx[1, 500, 7:] = -1
+    n_vis = cfg.Lk - cfg.Lq + 501
+    assert idx[1, 500, 6] < n_vis
+    if what == "unsorted":
+        idx[1, 500, :7] = idx[1, 500, :7].flip(0)
+    elif what == "duplicate":
+        idx[1, 500, 4] = 400
+    elif what == "not_visible":
+        idx[1, 500, 6] = n_vis
+    elif what == "position_too_large":
+        idx[1, 500, 6] = cfg.Lk + 5
+    elif what == "position_negative":
+        idx[1, 500, 0] = -3
+    elif what == "budget_too_large":
+        kt[1, 500] = cfg.k_max + 1
+    elif what == "inf_value":
+        x["V"][0, 700, 3, 5] = float("inf")
+    elif what == "nan_value":
+        x["V"][1, cfg.Lk - 1, 7, 127] = float("nan")
+    elif what == "huge_value":
+        x["V"][1, 0, 0, 0] = -3.0e38
+    status = 6 if what in ("position_too_large", "position_negative", "budget_too_large") else 0
+    return VALUES if "value" in what else (SETS if what else 0), status
+
+
+def _same(a, b):
+    return bool(((a == b) | (torch.isnan(a) & torch.isnan(b))).all())
+
+
+@pytest.mark.parametrize("what", ["unsorted", "duplicate", "not_visible", "position_too_large", "position_negative", "budget_too_large",
+                                  "inf_value", "nan_value", "huge_value", ""])
+def test_the_gather_does_what_the_tiles_leave(what):
+    """Each cause on its own: the call's result is bit for bit that of the gather kernels (which the same call runs when the
+    workspace has no room for the gated values: same sums in the same order)."""
+    cfg = TILES
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 211, empty=[(0, 3)])
+    bit, want_status = _irregular(cfg, what, x, idx, kt)
+    d = U.to_dev(x)
+    out, n, general, status = _fwd(cfg, d, idx, kt)
+    assert (n, general, status) == (4, bit, want_status)
+    out2, n2, _, status2 = _fwd(cfg, d, idx, kt, prepass=False)
+    assert n2 == 2 and status2 == want_status
+    assert _same(out, out2) == bool(what)        # (the tiles' own sums run in another order)
+    assert (out[0, 3] == 0).all()
+
+
+@pytest.mark.parametrize("what", ["unsorted", "inf_value", "nan_value", ""])
+def test_the_gather_does_what_the_tiles_leave_over_several_key_ranges(what):
+    """Key ranges of 1024 keys: sets in order are gathered range by range, others whole; in chunks of rows whose masks fit."""
+    cfg = TILES.with_(name="ranges")
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 211)
+    bit, _ = _irregular(cfg, what, x, idx, kt)
+    gsa.gsa_debug_set_attn_range_keys(1024)
+    try:
+        out, n, general, status = _fwd(cfg, U.to_dev(x), idx, kt)
+    finally:
+        gsa.gsa_debug_set_attn_range_keys(0)
+    # gate, masks, tiles, whole sets; cuts, two ranges, two blocks of finished rows
+    assert (n, general, status) == (4 + 5, bit, 0)
+    hit = torch.zeros(cfg.B, cfg.Lq, dtype=torch.bool)
+    if bit == VALUES:
+        b, key = (0, 700) if what == "inf_value" else (1, cfg.Lk - 1)
+        hit[b] = ((idx[b] == key) & (torch.arange(cfg.k_max) < kt[b, :, None])).any(-1)
+        assert hit.any()
+    bad = ~torch.isfinite(out.float().cpu()).all(-1).all(-1)
+    assert (bad == hit).all()
+    for b in range(cfg.B):
+        rows = np.array([t for t in (*range(0, cfg.Lq, 31), 499, 500, cfg.Lq - 1) if not hit[b, t]])
+        want = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx[b][rows].numpy(), kt[b][rows].numpy(),
+                           rows, np.full_like(rows, b))
+        U.check_out(out[b][torch.from_numpy(rows).cuda()].float().cpu().numpy(), want)
