@@ -810,6 +810,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
 
     // ---- emission: bitmaps, one scan, ascending positions ----
     const bool cut = eq_total != need_eq;                     // a group of equal keys is cut: lower positions win
+    const uint32_t below = cut ? T : T - 1u;                  // (no score has key 0; T + 1 would wrap in a row of NaN)
     uint8_t* const bytes_gt = reinterpret_cast<uint8_t*>(sh.gt);
     uint8_t* const bytes_eq = reinterpret_cast<uint8_t*>(sh.eq);
 #pragma unroll
@@ -818,10 +819,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
             uint32_t g = 0, q = 0;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                g |= (key[v][e] >= T ? 1u : 0u) << e;
+                g |= (key[v][e] > below ? 1u : 0u) << e;
                 if (cut) q |= (key[v][e] == T ? 1u : 0u) << e;
             }
-            g &= ~q;                                          // (not key >= T + 1: T is the largest number there is in a row of NaN)
             g |= __shfl_down_sync(0xFFFFFFFFu, g, 1) << 4;
             if ((tid & 1) == 0) bytes_gt[(v * NT + tid) / 2] = (uint8_t)g;
             if (cut) {
@@ -858,9 +858,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) gsa_select_short_kernel(const S
         uint32_t take = eq_before < need_eq ? need_eq - eq_before : 0u, q = qw;
         while (q && take) { gw |= q & -q; q &= q - 1u; --take; }
     }
+    if (at + (uint32_t)__popc(gw) > kSelOut) gw = 0u;         // (never: at most k_max entries are marked)
     while (gw) {
-        if (at < kSelOut) sh.out[at] = p0 + tid * 32 + __ffs(gw) - 1;
-        ++at;
+        sh.out[at++] = p0 + tid * 32 + __ffs(gw) - 1;
         gw &= gw - 1u;
     }
     if constexpr (CS > 1) {
