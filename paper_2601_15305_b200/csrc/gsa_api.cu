@@ -317,7 +317,7 @@ int gsa_sparse_gated_attn_bwd(const gsa_params_t* p, const void* Q, const void* 
     cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
     if (e == cudaSuccess)
         e = launch_value_gate((const bf16*)V, (const bf16*)g2_logits, Vg, (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st,
-                              t_dev_status + kStatusGeneralWord);
+                              t_dev_status + kStatusGeneralWord, wp.masked ? (const bf16*)K : nullptr);
     IdxLayout il{0, rr.q_begin, rr.R};
     if (e == cudaSuccess && pbar) e = cudaMemsetAsync(pbar, 0, (size_t)rr.rows() * p->k_max * 4, st);
     if (wp.masked) {

@@ -551,10 +551,11 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
 }
 
 // Eq. 9 as a streaming pre-pass: Vg = bf16(V * sigmoid(g2)), 8 elements per thread.
+template <bool WATCH_K>
 __global__ void __launch_bounds__(256) gsa_value_gate_kernel(const uint4* __restrict__ V,
                                                              const uint4* __restrict__ g2,
                                                              uint4* __restrict__ Vg, int64_t n_vec,
-                                                             int32_t* untileable) {
+                                                             int32_t* untileable, const uint4* __restrict__ K) {
     chain_wait();
     uint32_t bad = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec;
@@ -570,6 +571,7 @@ __global__ void __launch_bounds__(256) gsa_value_gate_kernel(const uint4* __rest
         }
         Vg[i] = vv;
         bad |= untileable_bf16x8(vv);
+        if (WATCH_K) bad |= untileable_bf16x8(__ldg(K + i));
     }
     if (bad && untileable) atomicOr(untileable, kGeneralValues);
 }
@@ -846,13 +848,14 @@ cudaError_t launch_attn_direct(const gsa_params_t& p, RowRange rr, const __nv_bf
 }
 
 cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, __nv_bfloat16* Vg,
-                              int64_t n_elems, cudaStream_t st, int32_t* untileable) {
+                              int64_t n_elems, cudaStream_t st, int32_t* untileable, const __nv_bfloat16* K) {
     const int64_t n_vec = n_elems / 8;
     if (n_vec <= 0) return cudaSuccess;
     const int blocks = (int)((n_vec + 255) / 256 < sm_count() * 16 ? (n_vec + 255) / 256 : sm_count() * 16);
-    launch_chained(gsa_value_gate_kernel, blocks, 256, 0, st, reinterpret_cast<const uint4*>(V),
+    launch_chained(K ? gsa_value_gate_kernel<true> : gsa_value_gate_kernel<false>, blocks, 256, 0, st, reinterpret_cast<const uint4*>(V),
                                                   reinterpret_cast<const uint4*>(g2),
-                                                  reinterpret_cast<uint4*>(Vg), n_vec, untileable);
+                                                  reinterpret_cast<uint4*>(Vg), n_vec, untileable,
+                                                  reinterpret_cast<const uint4*>(K));
     ++g_launches;
     return cudaGetLastError();
 }

@@ -47,9 +47,9 @@ struct BwdArgs {
     const int32_t* kt;
     __nv_bfloat16* dQ;
     __nv_bfloat16* dg1;
-    __nv_bfloat16* dOs;           // workspace: do = dout * sigmoid(g1), [B, Lq, n_h, d_h]
+    const __nv_bfloat16* dOs;     // workspace: do = dout * sigmoid(g1), [B, Lq, n_h, d_h]
     float* lse2;                  // workspace: log2-domain log-sum-exp of the scaled logits, [B, Lq, n_h]
-    float* delta;                 // workspace: sum_d dout * out, [B, Lq, n_h]
+    const float* delta;           // workspace: sum_d dout * out, [B, Lq, n_h]
     float* pbar;                  // optional output: mean over the heads of P on S_t, [B, R, k_max], pre-zeroed
     const float* lse_in;          // optional: natural-log softmax statistics saved by the forward pass, [B, Lq, n_h]
     float2* part_ml;              // key ranges: per range (max, sum) of the scaled logits, [n_ranges][B * Lq * n_h]
@@ -62,6 +62,8 @@ struct BwdArgs {
     int32_t Lq, Lk, n_h, n_kv, k_max;
     float scale;
     int32_t* dev_status;          // where an out-of-range index or budget is reported (may be null)
+    const int32_t* only_if;       // LOOP: see left_out
+    int32_t run_if;
 };
 
 __device__ __forceinline__ uint32_t movmatrix_t(uint32_t a) {
@@ -80,9 +82,10 @@ template <int DH>
 __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* __restrict__ g1,
                                                            const __nv_bfloat16* __restrict__ out,
                                                            const __nv_bfloat16* __restrict__ dout,
+                                                           const __nv_bfloat16* __restrict__ Q /*read with untileable only*/,
                                                            __nv_bfloat16* __restrict__ dOs, __nv_bfloat16* __restrict__ dg1,
                                                            float* __restrict__ delta, RowRange rr, int32_t Lq, int32_t n_h,
-                                                           int32_t* untileable /*nullable: raised if do or delta is*/) {
+                                                           int32_t* untileable /*nullable: raised if do, delta or Q is*/) {
     chain_wait();
     constexpr int EPL = DH / 32;
     const int lane = threadIdx.x & 31;
@@ -97,6 +100,11 @@ __global__ void __launch_bounds__(256) gsa_bwd_prep_kernel(const __nv_bfloat16* 
     Vec vdo, vdg;
     float part = 0.f;
     bool bad = false;
+    if (untileable) {
+        const Vec vq = *reinterpret_cast<const Vec*>(Q + at);
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) bad = bad || !(fabsf(__bfloat162float(vq.x[e])) < kTileValueLimit);
+    }
 #pragma unroll
     for (int e = 0; e < EPL; ++e) {
         const float dy = __bfloat162float(vdy.x[e]);
@@ -155,8 +163,7 @@ __global__ void __launch_bounds__(256) gsa_bwd_range_cuts_kernel(const int32_t* 
 // MODE 2: one item = (key range, row, KV head): statistics combined from part_ml, gradient sweep over the
 //         range's part, dQ added into dq32; the items of range 0 also write dg1, do, delta and lse2.
 template <int DH, int G, int MODE>
-__global__ void __launch_bounds__(kBwdWarps * 32, 4) gsa_sparse_attn_bwd_kernel(const BwdArgs a) {
-    chain_wait();
+__device__ __forceinline__ void bwd_item(const BwdArgs& a, const int64_t item) {
     constexpr int ROW = (DH + 8) * 2;                  // bytes of a padded tile row (odd multiple of 16)
     constexpr int KTILE = 16 * ROW, QTILE = 8 * ROW;
     constexpr int STAGE = KTILE;                       // a K tile (V' rows go straight into MMA fragments)
@@ -170,9 +177,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 4) gsa_sparse_attn_bwd_kernel(
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gid = lane >> 2, tig = lane & 3;
-    const int64_t item = (int64_t)blockIdx.x * kBwdWarps + warp;
     const int64_t per_range = (int64_t)a.rr.rows() * a.n_kv;
-    if (item >= per_range * (MODE == 0 ? 1 : a.n_ranges)) return;     // (no block-wide barrier below)
     const int range = MODE == 0 ? 0 : (int)(item / per_range);       // range-major: the warps in flight share a range
     const int64_t rem = item % per_range;
     // long rows first: late rows have the most keys
@@ -459,6 +464,23 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 4) gsa_sparse_attn_bwd_kernel(
     }
 }
 
+// LOOP: a grid that covers the SMs twice, for launches that nearly always return at once (behind the masked tiles).
+template <int DH, int G, int MODE, bool LOOP = false>
+__global__ void __launch_bounds__(kBwdWarps * 32, 4) gsa_sparse_attn_bwd_kernel(const BwdArgs a) {
+    chain_wait();
+    if (LOOP && left_out(a.only_if, a.run_if)) return;
+    const int64_t items = (int64_t)a.rr.rows() * a.n_kv * (MODE == 0 ? 1 : a.n_ranges);
+    int64_t item = (int64_t)blockIdx.x * kBwdWarps + (threadIdx.x >> 5);
+    if (!LOOP) {
+        if (item < items) bwd_item<DH, G, MODE>(a, item);             // (no block-wide barrier inside)
+    } else {
+        for (; item < items; item += (int64_t)gridDim.x * kBwdWarps) {
+            bwd_item<DH, G, MODE>(a, item);
+            __syncwarp();
+        }
+    }
+}
+
 // dQ rows of the range from the fp32 sums
 __global__ void __launch_bounds__(256) gsa_bwd_dq_finish_kernel(const float* __restrict__ dq32,
                                                                 __nv_bfloat16* __restrict__ dQ, RowRange rr,
@@ -474,17 +496,18 @@ __global__ void __launch_bounds__(256) gsa_bwd_dq_finish_kernel(const float* __r
     }
 }
 
-template <int DH, int G, int MODE>
+template <int DH, int G, int MODE, bool LOOP = false>
 cudaError_t launch_bwd_mode(const BwdArgs& a, cudaStream_t st) {
     constexpr int ROW = (DH + 8) * 2;
     constexpr int WARP_SMEM = 2 * 16 * ROW;
     const int smem = kBwdWarps * WARP_SMEM;
-    auto kern = gsa_sparse_attn_bwd_kernel<DH, G, MODE>;
+    auto kern = gsa_sparse_attn_bwd_kernel<DH, G, MODE, LOOP>;
     // (set on every call: the attribute belongs to the current device)
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const int64_t items = (int64_t)a.rr.rows() * a.n_kv * (MODE == 0 ? 1 : a.n_ranges);
-    const int64_t ctas = (items + kBwdWarps - 1) / kBwdWarps;
+    int64_t ctas = (items + kBwdWarps - 1) / kBwdWarps;
+    if (LOOP && ctas > 8 * sm_count()) ctas = 8 * sm_count();         // (two for each of the four places on an SM)
     launch_chained(kern, (unsigned)ctas, kBwdWarps * 32, smem, st, a);
     ++g_launches;
     return cudaGetLastError();
@@ -519,6 +542,19 @@ BwdRanges plan_bwd_ranges(const gsa_params_t& p) {
     return r;
 }
 
+BwdArgs bwd_args(const gsa_params_t& p, const RowRange& rr, const BwdRanges& br, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                 const __nv_bfloat16* Vg, const __nv_bfloat16* dOs, const int32_t* idx, const int32_t* kt, IdxLayout il,
+                 __nv_bfloat16* dQ, float* lse2, const float* delta, float* pbar, const float* lse_in) {
+    BwdArgs a = {};
+    a.range_keys = br.range_keys; a.n_ranges = br.n_ranges; a.total_rows = (int64_t)p.B * p.Lq;
+    a.lse_in = lse_in;
+    a.Q = Q; a.K = K; a.Vg = Vg; a.idx = idx; a.kt = kt; a.dev_status = t_dev_status;
+    a.dQ = dQ; a.dOs = dOs; a.lse2 = lse2; a.delta = delta; a.pbar = pbar; a.rr = rr; a.il = il;
+    a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv; a.k_max = p.k_max;
+    a.scale = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
+    return a;
+}
+
 }  // namespace
 
 size_t attn_bwd_range_bytes(const gsa_params_t& p) {
@@ -530,11 +566,11 @@ size_t attn_bwd_range_bytes(const gsa_params_t& p) {
 }
 
 cudaError_t launch_bwd_prep(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* g1, const __nv_bfloat16* out,
-                            const __nv_bfloat16* dout, __nv_bfloat16* dOs, __nv_bfloat16* dg1, float* delta,
-                            int32_t* untileable, cudaStream_t st) {
+                            const __nv_bfloat16* dout, const __nv_bfloat16* Q, __nv_bfloat16* dOs, __nv_bfloat16* dg1,
+                            float* delta, int32_t* untileable, cudaStream_t st) {
     const unsigned ctas = (unsigned)(((int64_t)rr.rows() * p.n_h + 7) / 8);
-    if (p.d_h == 128) launch_chained(gsa_bwd_prep_kernel<128>, ctas, 256, 0, st, g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, untileable);
-    else launch_chained(gsa_bwd_prep_kernel<64>, ctas, 256, 0, st, g1, out, dout, dOs, dg1, delta, rr, p.Lq, p.n_h, untileable);
+    if (p.d_h == 128) launch_chained(gsa_bwd_prep_kernel<128>, ctas, 256, 0, st, g1, out, dout, Q, dOs, dg1, delta, rr, p.Lq, p.n_h, untileable);
+    else launch_chained(gsa_bwd_prep_kernel<64>, ctas, 256, 0, st, g1, out, dout, Q, dOs, dg1, delta, rr, p.Lq, p.n_h, untileable);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -551,21 +587,30 @@ cudaError_t launch_sparse_attn_bwd(const gsa_params_t& p, RowRange rr, const __n
                                    __nv_bfloat16* dOs, float* lse2, float* delta, float* pbar, const float* lse_in,
                                    void* range_ws, cudaStream_t st) {
     if (rr.rows() <= 0) return cudaSuccess;
-    BwdArgs a;
     const BwdRanges br = plan_bwd_ranges(p);
-    a.range_keys = br.range_keys; a.n_ranges = br.n_ranges; a.total_rows = (int64_t)p.B * p.Lq;
-    a.lse_in = lse_in;
+    BwdArgs a = bwd_args(p, rr, br, Q, K, Vg, dOs, idx, kt, il, dQ, lse2, delta, pbar, lse_in);
     a.part_ml = (float2*)range_ws;
     a.dq32 = (float*)((char*)range_ws + ((size_t)br.n_ranges * a.total_rows * p.n_h * 8 + 255) / 256 * 256);
     a.cuts = (const int32_t*)((char*)a.dq32 + ((size_t)a.total_rows * p.n_h * p.d_h * 4 + 255) / 256 * 256);
-    a.Q = Q; a.K = K; a.Vg = Vg; a.g1 = g1; a.out = out; a.dout = dout; a.idx = idx; a.kt = kt; a.dev_status = t_dev_status;
-    a.dQ = dQ; a.dg1 = dg1; a.dOs = dOs; a.lse2 = lse2; a.delta = delta; a.pbar = pbar; a.rr = rr; a.il = il;
-    a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv; a.k_max = p.k_max;
-    a.scale = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
-    const cudaError_t e0 = launch_bwd_prep(p, rr, g1, out, dout, dOs, dg1, delta, nullptr, st);
+    a.g1 = g1; a.out = out; a.dout = dout; a.dg1 = dg1;
+    const cudaError_t e0 = launch_bwd_prep(p, rr, g1, out, dout, nullptr, dOs, dg1, delta, nullptr, st);
     if (e0 != cudaSuccess) return e0;
     const int G = p.n_h / p.n_kv;
 #define GSA_BWD_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_bwd_t<DH_, G_>(a, st)
+    GSA_BWD_CASE(128, 1); GSA_BWD_CASE(128, 2); GSA_BWD_CASE(128, 4); GSA_BWD_CASE(128, 8);
+    GSA_BWD_CASE(64, 1); GSA_BWD_CASE(64, 2); GSA_BWD_CASE(64, 4); GSA_BWD_CASE(64, 8);
+#undef GSA_BWD_CASE
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_attn_bwd_rows_general(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                                         const __nv_bfloat16* Vg, const __nv_bfloat16* dOs, const int32_t* idx, const int32_t* kt,
+                                         IdxLayout il, __nv_bfloat16* dQ, float* lse2, const float* delta, float* pbar,
+                                         const float* lse_in, const int32_t* general, cudaStream_t st) {
+    BwdArgs a = bwd_args(p, rr, BwdRanges{p.Lk, 1}, Q, K, Vg, dOs, idx, kt, il, dQ, lse2, delta, pbar, lse_in);
+    a.only_if = general; a.run_if = kRunAnyGeneral;
+    const int G = p.n_h / p.n_kv;
+#define GSA_BWD_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_bwd_mode<DH_, G_, 0, true>(a, st)
     GSA_BWD_CASE(128, 1); GSA_BWD_CASE(128, 2); GSA_BWD_CASE(128, 4); GSA_BWD_CASE(128, 8);
     GSA_BWD_CASE(64, 1); GSA_BWD_CASE(64, 2); GSA_BWD_CASE(64, 4); GSA_BWD_CASE(64, 8);
 #undef GSA_BWD_CASE

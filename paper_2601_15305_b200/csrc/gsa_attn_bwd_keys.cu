@@ -20,7 +20,7 @@
 // work items run range-major, (range, key), so that the warps in flight share one range.  The partial
 // sums of a key's ranges then meet in fp32 arrays (one reduction per range and element, not per pair) and
 // a streaming post-pass applies the gate's derivative and rounds.
-#include "gsa_common.cuh"
+#include "gsa_masked.cuh"
 
 namespace gsa {
 
@@ -46,6 +46,7 @@ struct InvArgs {
 
 // one warp per query row: cnt[b * Lk + s] += 1 for every selected s
 __global__ void __launch_bounds__(256) gsa_bwd_count_kernel(const InvArgs a, int32_t* __restrict__ cnt) {
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int64_t lr = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (lr >= a.rr.rows()) return;
@@ -63,6 +64,7 @@ __global__ void __launch_bounds__(256) gsa_bwd_count_kernel(const InvArgs a, int
 // one warp per query row: the row's number goes into the list of every selected key
 __global__ void __launch_bounds__(256) gsa_bwd_fill_kernel(const InvArgs a, int32_t* __restrict__ cur,
                                                            int32_t* __restrict__ rows_of_key) {
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int64_t lr = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (lr >= a.rr.rows()) return;
@@ -103,6 +105,7 @@ __device__ __forceinline__ int32_t block_excl_scan_i32(int32_t v, int32_t* warp_
 // exclusive scan of n counters in three steps: block sums, scan of the block sums, final offsets
 __global__ void __launch_bounds__(kScanThreads) gsa_bwd_scan_sums_kernel(const int32_t* __restrict__ cnt, int64_t n,
                                                                          int32_t* __restrict__ bsum) {
+    chain_wait();
     __shared__ int32_t warp_tot[kScanThreads / 32];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock + threadIdx.x * kScanPerThread;
     int32_t v = 0;
@@ -113,6 +116,7 @@ __global__ void __launch_bounds__(kScanThreads) gsa_bwd_scan_sums_kernel(const i
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 __global__ void __launch_bounds__(kScanThreads) gsa_bwd_scan_top_kernel(int32_t* __restrict__ bsum, int nblk) {
+    chain_wait();
     __shared__ int32_t warp_tot[kScanThreads / 32];
     __shared__ int32_t carry;
     if (threadIdx.x == 0) carry = 0;
@@ -132,6 +136,7 @@ __global__ void __launch_bounds__(kScanThreads) gsa_bwd_scan_final_kernel(const 
                                                                           const int32_t* __restrict__ bsum,
                                                                           int32_t* __restrict__ off,
                                                                           int32_t* __restrict__ cur) {
+    chain_wait();
     __shared__ int32_t warp_tot[kScanThreads / 32];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock + threadIdx.x * kScanPerThread;
     int32_t c[kScanPerThread], v = 0;
@@ -143,6 +148,67 @@ __global__ void __launch_bounds__(kScanThreads) gsa_bwd_scan_final_kernel(const 
     for (int e = 0; e < kScanPerThread; ++e) {
         if (base + e < n) { off[base + e] = run; cur[base + e] = run; }
         run += c[e];
+    }
+}
+
+// ---- the same behind the masked tiles, for what they leave (see left_out) ------------------------------------
+// Fewer and smaller launches, since they nearly always return at once: one counter per (key, row range), whose scan (one CTA) gives
+// every range's boundaries without copies of the cursors; grids that cover the SMs twice (8K rows 21.2 ms, once 22.7; the
+// launches without these bounds 19.0, but each would cost the tiles' calls a pass over empty CTAs).
+__global__ void __launch_bounds__(256) gsa_bwd_count_general_kernel(const InvArgs a, int32_t* __restrict__ cnt, int n_ranges,
+                                                                    int range_rows, float4* __restrict__ sums, int64_t sums_vec,
+                                                                    const int32_t* only_if) {
+    chain_wait();
+    if (left_out(only_if, kRunAnyGeneral)) return;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < sums_vec; i += (int64_t)gridDim.x * 256)
+        sums[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int lane = threadIdx.x & 31;
+    for (int64_t lr = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); lr < a.rr.rows(); lr += (int64_t)gridDim.x * 8) {
+        const int b = a.rr.b0 + (int)(lr / a.rr.R), r = (int)(lr % a.rr.R);
+        const int64_t irow = a.il.row(b, a.rr.q_begin + r);
+        const int ke = clamp_budget(a.kt[irow], a.k_max);
+        for (int j = lane; j < ke; j += 32) {
+            const int32_t s = a.idx[irow * a.k_max + j];
+            if (key_in_range(s, a.Lk)) atomicAdd(cnt + ((int64_t)b * a.Lk + s) * n_ranges + r / range_rows, 1);
+            else report_bad_index(a.dev_status);
+        }
+    }
+}
+__global__ void __launch_bounds__(256) gsa_bwd_fill_general_kernel(const InvArgs a, int32_t* __restrict__ cur, int n_ranges,
+                                                                   int range_rows, int32_t* __restrict__ rows_of_key,
+                                                                   const int32_t* only_if) {
+    chain_wait();
+    if (left_out(only_if, kRunAnyGeneral)) return;
+    const int lane = threadIdx.x & 31;
+    for (int64_t lr = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); lr < a.rr.rows(); lr += (int64_t)gridDim.x * 8) {
+        const int b = a.rr.b0 + (int)(lr / a.rr.R), r = (int)(lr % a.rr.R), t = a.rr.q_begin + r;
+        const int64_t irow = a.il.row(b, t);
+        const int ke = clamp_budget(a.kt[irow], a.k_max);
+        for (int j = lane; j < ke; j += 32) {
+            const int32_t s = a.idx[irow * a.k_max + j];
+            if (key_in_range(s, a.Lk)) rows_of_key[atomicAdd(cur + ((int64_t)b * a.Lk + s) * n_ranges + r / range_rows, 1)] = b * a.Lq + t;
+        }
+    }
+}
+// cnt[0 .. n) -> its exclusive scan, in off and in cnt itself (the cursors)
+__global__ void __launch_bounds__(kScanThreads) gsa_bwd_scan_general_kernel(int32_t* __restrict__ cnt, int64_t n, int32_t* __restrict__ off,
+                                                                            const int32_t* only_if) {
+    chain_wait();
+    if (left_out(only_if, kRunAnyGeneral)) return;
+    __shared__ int32_t warp_tot[kScanThreads / 32];
+    int32_t carry = 0;
+    for (int64_t c0 = 0; c0 < n; c0 += kScanBlock) {
+        const int64_t base = c0 + threadIdx.x * kScanPerThread;
+        int32_t c[kScanPerThread], v = 0, total;
+#pragma unroll
+        for (int e = 0; e < kScanPerThread; ++e) { c[e] = base + e < n ? cnt[base + e] : 0; v += c[e]; }
+        int32_t run = carry + block_excl_scan_i32(v, warp_tot, total);
+#pragma unroll
+        for (int e = 0; e < kScanPerThread; ++e) {
+            if (base + e < n) { off[base + e] = run; cnt[base + e] = run; }
+            run += c[e];
+        }
+        carry += total;
     }
 }
 
@@ -170,6 +236,7 @@ struct KeyArgs {
     int32_t hb_shift;             // log2(HB)
     int32_t NHB;                  // head blocks: n_h / HB
     float scale;
+    const int32_t* only_if;       // LOOP: see left_out
 };
 
 __device__ __forceinline__ uint32_t movmatrix_tk(uint32_t a) {
@@ -183,8 +250,9 @@ __device__ __forceinline__ float ex2_approx_k(float x) {
     return y;
 }
 
-template <int DH, bool PARTIAL>
-__global__ void __launch_bounds__(kKeyWarps * 32) gsa_sparse_attn_bwd_keys_kernel(const KeyArgs a, const int n_ranges) {
+// one item = (row range, key, head block); BY_KEY: off and bnd are [key][range] (bnd: the cursors), not [range][key]
+template <int DH, bool PARTIAL, bool BY_KEY>
+__device__ __forceinline__ void keys_item(const KeyArgs& a, const int n_ranges, const int64_t item) {
     constexpr int ROW = (DH + 8) * 2;                  // bytes of a padded tile row (odd multiple of 16)
     constexpr int TILE16 = 16 * ROW, TILE8 = 8 * ROW;
     constexpr int STAGE = 2 * TILE16;                  // a Q tile and a do tile
@@ -195,14 +263,12 @@ __global__ void __launch_bounds__(kKeyWarps * 32) gsa_sparse_attn_bwd_keys_kerne
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gid = lane >> 2, tig = lane & 3;
-    const int64_t item = (int64_t)blockIdx.x * kKeyWarps + warp;
-    if (item >= a.n_keys * a.NHB * n_ranges) return;   // (no block-wide barrier below)
     // range-major: all keys of query range 0, then range 1, ...
     const int range = (int)(item / (a.n_keys * a.NHB));
     const int64_t key = (item / a.NHB) % a.n_keys;     // b * Lk + s
     const int hb = (int)(item % a.NHB);
-    const int beg = range == 0 ? a.off[key] : a.bnd[(int64_t)(range - 1) * a.n_keys + key];
-    const int end = a.bnd[(int64_t)range * a.n_keys + key];
+    const int beg = BY_KEY ? a.off[key * n_ranges + range] : (range == 0 ? a.off[key] : a.bnd[(int64_t)(range - 1) * a.n_keys + key]);
+    const int end = a.bnd[BY_KEY ? key * n_ranges + range : (int64_t)range * a.n_keys + key];
     if (PARTIAL && beg == end) return;                 // nothing of this key in this range
     const int h_base = hb * a.HB;                      // first head of the block
     const int g_base = h_base / a.G;                   // its KV head = column 0
@@ -360,6 +426,22 @@ __global__ void __launch_bounds__(kKeyWarps * 32) gsa_sparse_attn_bwd_keys_kerne
     }
 }
 
+template <int DH, bool PARTIAL, bool LOOP = false>
+__global__ void __launch_bounds__(kKeyWarps * 32) gsa_sparse_attn_bwd_keys_kernel(const KeyArgs a, const int n_ranges) {
+    chain_wait();
+    if (LOOP && left_out(a.only_if, kRunAnyGeneral)) return;
+    const int64_t items = a.n_keys * a.NHB * n_ranges;
+    int64_t item = (int64_t)blockIdx.x * kKeyWarps + (threadIdx.x >> 5);
+    if (!LOOP) {
+        if (item < items) keys_item<DH, PARTIAL, false>(a, n_ranges, item);       // (no block-wide barrier inside)
+    } else {
+        for (; item < items; item += (int64_t)gridDim.x * kKeyWarps) {
+            keys_item<DH, PARTIAL, true>(a, n_ranges, item);
+            __syncwarp();
+        }
+    }
+}
+
 // dK = bf16(dK32);  dV = bf16(dV'32 * sigmoid(g2));  dg2 = bf16(dV'32 * V * sigmoid'(g2))
 __global__ void __launch_bounds__(256) gsa_attn_bwd_finish_kernel(const float* __restrict__ dK32,
                                                                   const float* __restrict__ dV32,
@@ -367,7 +449,10 @@ __global__ void __launch_bounds__(256) gsa_attn_bwd_finish_kernel(const float* _
                                                                   const __nv_bfloat16* __restrict__ g2,
                                                                   __nv_bfloat16* __restrict__ dK,
                                                                   __nv_bfloat16* __restrict__ dV,
-                                                                  __nv_bfloat16* __restrict__ dg2, int64_t n) {
+                                                                  __nv_bfloat16* __restrict__ dg2, int64_t n,
+                                                                  const int32_t* only_if) {
+    chain_wait();
+    if (left_out(only_if, kRunAnyGeneral)) return;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * 4;
     for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < n; i += stride) {
         const float4 k4 = *reinterpret_cast<const float4*>(dK32 + i);
@@ -391,19 +476,48 @@ __global__ void __launch_bounds__(256) gsa_attn_bwd_finish_kernel(const float* _
     }
 }
 
-template <int DH, bool PARTIAL>
+template <int DH, bool PARTIAL, bool LOOP = false>
 cudaError_t launch_keys_t(const KeyArgs& a, int n_ranges, cudaStream_t st) {
     constexpr int ROW = (DH + 8) * 2;
     constexpr int WARP_SMEM = 4 * 16 * ROW;
     const int smem = kKeyWarps * WARP_SMEM;
+    auto kern = gsa_sparse_attn_bwd_keys_kernel<DH, PARTIAL, LOOP>;
     // (set on every call: the attribute belongs to the current device)
-    {
-        cudaError_t e = cudaFuncSetAttribute(gsa_sparse_attn_bwd_keys_kernel<DH, PARTIAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
     const int64_t items = a.n_keys * a.NHB * n_ranges;
-    const int64_t ctas = (items + kKeyWarps - 1) / kKeyWarps;
-    gsa_sparse_attn_bwd_keys_kernel<DH, PARTIAL><<<(unsigned)ctas, kKeyWarps * 32, smem, st>>>(a, n_ranges);
+    int64_t ctas = (items + kKeyWarps - 1) / kKeyWarps;
+    if (LOOP) {
+        int per_sm = 1;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kKeyWarps * 32, smem)) != cudaSuccess) return e;
+        const int64_t cap = 2ll * sm_count() * (per_sm < 1 ? 1 : per_sm);
+        if (ctas > cap) ctas = cap;
+    }
+    launch_chained(kern, (unsigned)ctas, kKeyWarps * 32, smem, st, a, n_ranges);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+KeyArgs key_args(const gsa_params_t& p, const __nv_bfloat16* Q, const __nv_bfloat16* dOs, const __nv_bfloat16* K,
+                 const __nv_bfloat16* V, const __nv_bfloat16* Vg, const __nv_bfloat16* g2, const float* lse2, const float* delta,
+                 __nv_bfloat16* dK, __nv_bfloat16* dV, __nv_bfloat16* dg2) {
+    KeyArgs a = {};
+    a.Q = Q; a.dOs = dOs; a.K = K; a.V = V; a.Vg = Vg; a.g2 = g2; a.lse2 = lse2; a.delta = delta;
+    a.dK = dK; a.dV = dV; a.dg2 = dg2;
+    a.n_keys = (int64_t)p.B * p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv; a.G = p.n_h / p.n_kv;
+    a.HB = p.n_h < 16 ? p.n_h : 16;
+    a.NHB = p.n_h / a.HB;
+    a.hb_shift = 0;
+    while ((1 << a.hb_shift) < a.HB) ++a.hb_shift;
+    a.scale = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
+    return a;
+}
+
+cudaError_t launch_keys_finish(const float* dK32, const float* dV32, const __nv_bfloat16* V, const __nv_bfloat16* g2, __nv_bfloat16* dK,
+                               __nv_bfloat16* dV, __nv_bfloat16* dg2, int64_t n_elems, const int32_t* only_if, cudaStream_t st) {
+    const int64_t want = (n_elems / 4 + 255) / 256;
+    const int blocks = (int)(want < sm_count() * 16 ? want : sm_count() * 16);
+    launch_chained(gsa_attn_bwd_finish_kernel, blocks, 256, 0, st, dK32, dV32, V, g2, dK, dV, dg2, n_elems, only_if);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -454,12 +568,12 @@ cudaError_t launch_sparse_attn_bwd_keys(const gsa_params_t& p, RowRange rr, cons
     ia.dev_status = t_dev_status;
     const unsigned row_ctas = (unsigned)((rr.rows() + 7) / 8);
     if (rr.rows() > 0) {
-        gsa_bwd_count_kernel<<<row_ctas, 256, 0, st>>>(ia, cnt);
+        launch_chained(gsa_bwd_count_kernel, row_ctas, 256, 0, st, ia, cnt);
         ++g_launches;
     }
-    gsa_bwd_scan_sums_kernel<<<nblk, kScanThreads, 0, st>>>(cnt, n_keys, bsum);
-    gsa_bwd_scan_top_kernel<<<1, kScanThreads, 0, st>>>(bsum, nblk);
-    gsa_bwd_scan_final_kernel<<<nblk, kScanThreads, 0, st>>>(cnt, n_keys, bsum, off, cur);
+    launch_chained(gsa_bwd_scan_sums_kernel, nblk, kScanThreads, 0, st, cnt, n_keys, bsum);
+    launch_chained(gsa_bwd_scan_top_kernel, 1, kScanThreads, 0, st, bsum, nblk);
+    launch_chained(gsa_bwd_scan_final_kernel, nblk, kScanThreads, 0, st, cnt, n_keys, bsum, off, cur);
     g_launches += 3;
     // the lists are filled range by range (in stream order), so every list is grouped by range; the
     // cursors after range r are the boundaries of range r
@@ -469,7 +583,7 @@ cudaError_t launch_sparse_attn_bwd_keys(const gsa_params_t& p, RowRange rr, cons
         ir.rr.q_begin = rr.q_begin + r * range_rows;
         ir.rr.R = rr.R - r * range_rows < range_rows ? rr.R - r * range_rows : range_rows;
         if (ir.rr.rows() > 0) {
-            gsa_bwd_fill_kernel<<<(unsigned)((ir.rr.rows() + 7) / 8), 256, 0, st>>>(ir, cur, rows_of_key);
+            launch_chained(gsa_bwd_fill_kernel, (unsigned)((ir.rr.rows() + 7) / 8), 256, 0, st, ir, cur, rows_of_key);
             ++g_launches;
         }
         e = cudaMemcpyAsync(bnd + (size_t)r * n_keys, cur, (size_t)n_keys * 4, cudaMemcpyDeviceToDevice, st);
@@ -477,30 +591,61 @@ cudaError_t launch_sparse_attn_bwd_keys(const gsa_params_t& p, RowRange rr, cons
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
-    KeyArgs a;
-    a.Q = Q; a.dOs = dOs; a.K = K; a.V = V; a.Vg = Vg; a.g2 = g2; a.lse2 = lse2; a.delta = delta;
-    a.off = off; a.bnd = bnd; a.rows_of_key = rows_of_key; a.dK = dK; a.dV = dV; a.dg2 = dg2;
+    KeyArgs a = key_args(p, Q, dOs, K, V, Vg, g2, lse2, delta, dK, dV, dg2);
+    a.off = off; a.bnd = bnd; a.rows_of_key = rows_of_key;
     a.dK32 = dK32; a.dV32 = dV32;
-    a.n_keys = n_keys; a.n_h = p.n_h; a.n_kv = p.n_kv; a.G = p.n_h / p.n_kv;
-    a.HB = p.n_h < 16 ? p.n_h : 16;
-    a.NHB = p.n_h / a.HB;
-    a.hb_shift = 0;
-    while ((1 << a.hb_shift) < a.HB) ++a.hb_shift;
-    a.scale = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
     if (p.d_h != 128 && p.d_h != 64) return cudaErrorInvalidValue;
     if (n_ranges == 1)
         return p.d_h == 128 ? launch_keys_t<128, false>(a, 1, st) : launch_keys_t<64, false>(a, 1, st);
     if ((e = cudaMemsetAsync(dK32, 0, 2 * ((n_kv_elems * 4 + 255) / 256 * 256), st)) != cudaSuccess) return e;
     e = p.d_h == 128 ? launch_keys_t<128, true>(a, n_ranges, st) : launch_keys_t<64, true>(a, n_ranges, st);
     if (e != cudaSuccess) return e;
-    {
-        const int64_t n_elems = (int64_t)n_kv_elems;
-        const int64_t want = (n_elems / 4 + 255) / 256;
-        const int blocks = (int)(want < sm_count() * 16 ? want : sm_count() * 16);
-        gsa_attn_bwd_finish_kernel<<<blocks, 256, 0, st>>>(dK32, dV32, V, g2, dK, dV, dg2, n_elems);
-        ++g_launches;
-    }
-    return cudaGetLastError();
+    return launch_keys_finish(dK32, dV32, V, g2, dK, dV, dg2, (int64_t)n_kv_elems, nullptr, st);
+}
+
+// counters (and cursors) and offsets per (key, row range), the lists; with several ranges the two fp32 arrays
+size_t attn_bwd_keys_general_zero(const gsa_params_t& p, int32_t rows_per_batch) {
+    return ((size_t)p.B * p.Lk * bwd_ranges(rows_per_batch) * 4 + 15) / 16 * 16;
+}
+size_t attn_bwd_keys_general_bytes(const gsa_params_t& p, int32_t rows_per_batch) {
+    size_t bytes = 2 * attn_bwd_keys_general_zero(p, rows_per_batch) + ((size_t)p.B * rows_per_batch * p.k_max * 4 + 255) / 256 * 256;
+    if (bwd_ranges(rows_per_batch) > 1) bytes += (size_t)p.B * p.Lk * p.n_kv * p.d_h * 8;
+    return bytes;
+}
+
+cudaError_t launch_attn_bwd_keys_general(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q, const __nv_bfloat16* dOs,
+                                         const __nv_bfloat16* K, const __nv_bfloat16* V, const __nv_bfloat16* Vg,
+                                         const __nv_bfloat16* g2, const float* lse2, const float* delta, const int32_t* idx,
+                                         const int32_t* kt, IdxLayout il, void* ws, __nv_bfloat16* dK, __nv_bfloat16* dV,
+                                         __nv_bfloat16* dg2, const int32_t* general, cudaStream_t st) {
+    const int64_t n_keys = (int64_t)p.B * p.Lk, n_elems = n_keys * p.n_kv * p.d_h;
+    const int n_ranges = bwd_ranges(rr.R), range_rows = (rr.R + n_ranges - 1) / n_ranges;
+    const size_t counters = attn_bwd_keys_general_zero(p, rr.R), lists = ((size_t)rr.rows() * p.k_max * 4 + 255) / 256 * 256;
+    int32_t* const cnt = (int32_t*)ws;
+    int32_t* const off = (int32_t*)((char*)ws + counters);
+    int32_t* const rows_of_key = (int32_t*)((char*)off + counters);
+    float* const dK32 = (float*)((char*)rows_of_key + lists);
+    InvArgs ia;
+    ia.idx = idx; ia.kt = kt; ia.rr = rr; ia.il = il; ia.Lq = p.Lq; ia.Lk = p.Lk; ia.k_max = p.k_max;
+    ia.dev_status = t_dev_status;
+    const int64_t want = ((int64_t)rr.rows() + 7) / 8, cap = (int64_t)sm_count() * 8;
+    const unsigned row_ctas = (unsigned)(want < cap ? want : cap);
+    launch_chained(gsa_bwd_count_general_kernel, row_ctas, 256, 0, st, ia, cnt, n_ranges, range_rows, (float4*)dK32,
+                   n_ranges > 1 ? n_elems / 2 : 0, general);
+    launch_chained(gsa_bwd_scan_general_kernel, 1, kScanThreads, 0, st, cnt, n_keys * n_ranges, off, general);
+    launch_chained(gsa_bwd_fill_general_kernel, row_ctas, 256, 0, st, ia, cnt, n_ranges, range_rows, rows_of_key, general);
+    g_launches += 3;
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    KeyArgs a = key_args(p, Q, dOs, K, V, Vg, g2, lse2, delta, dK, dV, dg2);
+    a.off = off; a.bnd = cnt; a.rows_of_key = rows_of_key; a.only_if = general;
+    a.dK32 = dK32; a.dV32 = dK32 + n_elems;
+    if (p.d_h != 128 && p.d_h != 64) return cudaErrorInvalidValue;
+    if (n_ranges == 1)
+        return p.d_h == 128 ? launch_keys_t<128, false, true>(a, 1, st) : launch_keys_t<64, false, true>(a, 1, st);
+    e = p.d_h == 128 ? launch_keys_t<128, true, true>(a, n_ranges, st) : launch_keys_t<64, true, true>(a, n_ranges, st);
+    if (e != cudaSuccess) return e;
+    return launch_keys_finish(dK32, a.dV32, V, g2, dK, dV, dg2, n_elems, general, st);
 }
 
 }  // namespace gsa

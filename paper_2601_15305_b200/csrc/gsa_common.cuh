@@ -89,17 +89,19 @@ cudaError_t launch_select(const gsa_params_t& p, RowRange rr, const float* score
                           IdxLayout il, int32_t* fallback_rows /*nullable counter*/, cudaStream_t st);
 
 cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, __nv_bfloat16* Vg,
-                              int64_t n_elems, cudaStream_t st, int32_t* untileable = nullptr /*raised if a gated value is*/);
+                              int64_t n_elems, cudaStream_t st, int32_t* untileable = nullptr /*raised if a gated value is*/,
+                              const __nv_bfloat16* K = nullptr /*as many values, only watched*/);
 
 // Backward of sparse gated attention.  Query-major half (gsa_attn_bwd.cu): dQ, dg1 for the rows of rr, and
 // per (row, head) do = dout * sigmoid(g1), the softmax statistics lse2 and delta for the key-major half
 // (gsa_attn_bwd_keys.cu), which inverts the index sets inside invert_ws (attn_bwd_invert_bytes) and writes
 // dK, dV, dg2 for every key.
 bool attn_bwd_supported(const gsa_params_t& p);
-// do = dout * sigmoid(g1), dg1 and delta = sum_d dout * out per (row, head); *untileable (nullable) is raised if a do or a delta is
+// do = dout * sigmoid(g1), dg1 and delta = sum_d dout * out per (row, head); *untileable (nullable) is raised if a do, a delta or a
+// value of Q is
 cudaError_t launch_bwd_prep(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* g1, const __nv_bfloat16* out,
-                            const __nv_bfloat16* dout, __nv_bfloat16* dOs, __nv_bfloat16* dg1, float* delta,
-                            int32_t* untileable, cudaStream_t st);
+                            const __nv_bfloat16* dout, const __nv_bfloat16* Q, __nv_bfloat16* dOs, __nv_bfloat16* dg1,
+                            float* delta, int32_t* untileable, cudaStream_t st);
 cudaError_t launch_sparse_attn_bwd(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q,
                                    const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1,
                                    const __nv_bfloat16* out, const __nv_bfloat16* dout, const int32_t* idx,

@@ -42,10 +42,8 @@ cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int bl
 // The same for sets known to hold every visible key (k_mode 3 inside gsa_forward): no set is read.
 cudaError_t launch_visible_masks(const gsa_params_t& p, const MaskPlan& mp, uint4* mask, cudaStream_t st);
 
-// Raises *general if one of n_elems (a multiple of 8) values is infinite, NaN or too large (untileable_bf16x8); of each of
-// `batches` runs that start batch_stride values (a multiple of 8) apart.
-cudaError_t launch_check_values(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st, int batches = 1,
-                                int64_t batch_stride = 0);
+// Raises *general if one of n_elems (a multiple of 8) values is infinite, NaN or too large (untileable_bf16x8).
+cudaError_t launch_check_values(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st);
 
 // What a range of rows sees and selects, per KV head: for the choice between the tiles and the gather.  The sets' sizes are on
 // the device; the budget that they centre on stands for them.
@@ -82,8 +80,23 @@ cudaError_t launch_attn_direct(const gsa_params_t& p, RowRange rr, const __nv_bf
                                const __nv_bfloat16* Vg, const __nv_bfloat16* g1, const int32_t* idx, const int32_t* kt, IdxLayout il,
                                __nv_bfloat16* out, float* lse, const int32_t* only_if, int32_t run_if, cudaStream_t st);
 
+// What the backward's tiles leave to the gather (gsa_attn_bwd.cu, gsa_attn_bwd_keys.cu), run if *general is raised: dQ (and pbar,
+// lse2); then dK, dV, dg2 from the sets inverted inside ws (attn_bwd_keys_general_bytes), whose first attn_bwd_keys_general_zero
+// bytes the tile kernels clear when they leave.
+cudaError_t launch_attn_bwd_rows_general(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,
+                                         const __nv_bfloat16* Vg, const __nv_bfloat16* dOs, const int32_t* idx, const int32_t* kt,
+                                         IdxLayout il, __nv_bfloat16* dQ, float* lse2, const float* delta, float* pbar,
+                                         const float* lse_in, const int32_t* general, cudaStream_t st);
+size_t attn_bwd_keys_general_bytes(const gsa_params_t& p, int32_t rows_per_batch);
+size_t attn_bwd_keys_general_zero(const gsa_params_t& p, int32_t rows_per_batch);
+cudaError_t launch_attn_bwd_keys_general(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q, const __nv_bfloat16* dOs,
+                                         const __nv_bfloat16* K, const __nv_bfloat16* V, const __nv_bfloat16* Vg,
+                                         const __nv_bfloat16* g2, const float* lse2, const float* delta, const int32_t* idx,
+                                         const int32_t* kt, IdxLayout il, void* ws, __nv_bfloat16* dK, __nv_bfloat16* dV,
+                                         __nv_bfloat16* dg2, const int32_t* general, cudaStream_t st);
+
 // Backward (gsa_masked_bwd.cu): all gradients of the attention stage and the target of the indexer's loss (pbar, zeroed by
-// the caller; may be null).  V: as given, Vg: gated and scanned.  ws: masked_bwd_bytes(p, rr) bytes.
+// the caller; may be null).  V: as given, Vg: gated; it and K have been watched (launch_value_gate).  ws: masked_bwd_bytes(p, rr) bytes.
 bool masked_bwd_preferred(const gsa_params_t& p, const RowRange& rr);
 size_t masked_bwd_bytes(const gsa_params_t& p, const RowRange& rr);
 cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,

@@ -124,12 +124,10 @@ __global__ void __launch_bounds__(256) gsa_visible_masks_kernel(uint4* __restric
 // ascending positions that the row can see, raises the `general` word; the tile kernels then leave at once and the gather kernels,
 // enqueued behind them, do the work, at the speed that they have anyway.  Otherwise these cost a launch.
 // raises `general` if a bf16 value is infinite, NaN or too large for the tiles
-__global__ void __launch_bounds__(256) gsa_check_values_kernel(const uint4* __restrict__ x, int64_t n_vec, int64_t batch_vec,
-                                                               int ctas_per_batch, int32_t* general) {
+__global__ void __launch_bounds__(256) gsa_check_values_kernel(const uint4* __restrict__ x, int64_t n_vec, int32_t* general) {
     chain_wait();
     uint32_t bad = 0;
-    x += blockIdx.x / ctas_per_batch * batch_vec;
-    for (int64_t i = (int64_t)(blockIdx.x % ctas_per_batch) * blockDim.x + threadIdx.x; i < n_vec; i += (int64_t)ctas_per_batch * blockDim.x)
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += (int64_t)gridDim.x * blockDim.x)
         bad |= untileable_bf16x8(__ldg(x + i));
     if (bad) atomicOr(general, kGeneralValues);
 }
@@ -493,13 +491,10 @@ cudaError_t launch_visible_masks(const gsa_params_t& p, const MaskPlan& mp, uint
     return cudaGetLastError();
 }
 
-cudaError_t launch_check_values(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st, int batches,
-                                int64_t batch_stride) {
+cudaError_t launch_check_values(const __nv_bfloat16* x, int64_t n_elems, int32_t* general, cudaStream_t st) {
     const int64_t n_vec = n_elems / 8;
-    const int64_t want = (n_vec + 255) / 256, cap = ((int64_t)sm_count() * 8 + batches - 1) / batches;
-    const int per_batch = (int)(want < cap ? want : cap);
-    launch_chained(gsa_check_values_kernel, (unsigned)(per_batch * batches), 256, 0, st, reinterpret_cast<const uint4*>(x), n_vec,
-                   batch_stride / 8, per_batch, general);
+    const int64_t want = (n_vec + 255) / 256, cap = (int64_t)sm_count() * 8;
+    launch_chained(gsa_check_values_kernel, (unsigned)(want < cap ? want : cap), 256, 0, st, reinterpret_cast<const uint4*>(x), n_vec, general);
     ++g_launches;
     return cudaGetLastError();
 }

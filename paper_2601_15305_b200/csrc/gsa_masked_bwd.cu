@@ -57,6 +57,8 @@ struct MaskedBwdArgs {
     int32_t row_blocks;            // of 128 / G queries
     int32_t pairs_per_cta;         // target kernel: runs of 256 keys per CTA
     float scale, scale_log2;
+    uint4* zero;                   // what the general path finds cleared (see launch_attn_bwd_keys_general)
+    int64_t zero_vec;
     long long wait_cycles;
     int32_t withhold_first;        // fault injection: the first copy of a ring is left out (its barrier is never completed)
 };
@@ -158,7 +160,11 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     constexpr int QT = P::QT, ST = P::STAGES;
     constexpr uint32_t kTmS = 0, kTmP = 128, kTmV = 256, kTmK = 384;
     int timed_out;
-    if (!tiles_allowed(a.dev_status, &timed_out)) return;
+    if (!tiles_allowed(a.dev_status, &timed_out)) {                // (no one reads the masks, whose space this is, from here on)
+        for (int64_t i = (int64_t)blockIdx.x * kBwdThreads + threadIdx.x; i < a.zero_vec; i += (int64_t)gridDim.x * kBwdThreads)
+            a.zero[i] = make_uint4(0u, 0u, 0u, 0u);
+        return;
+    }
     GSA_TILE_PROLOGUE(P)
     auto bar_q = [&](int s) { return bar0 + 8u * s; };                       // Q tile landed
     auto bar_d = [&](int s) { return bar0 + 8u * (ST + s); };                // do tile landed
@@ -794,101 +800,9 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
              [&] { for (int i = max(0, released - 2); i < released; ++i) mbar_drain(bar_empty(i & 1), (i >> 1) & 1); });
 }
 
-// ---- what the tiles cannot take (see gsa_general_attn_kernel) -------------------------------------------------------
-// Only when `general` is raised: fp32 sums of dK, dV' by atomics, one warp per (row, KV head), the set entry by entry.
-__global__ void __launch_bounds__(256) gsa_general_bwd_zero_kernel(const int32_t* __restrict__ general, float4* x, int64_t n) {
-    chain_wait();
-    if (*general == 0) return;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
-template <int DH, int G>
-__global__ void __launch_bounds__(256)
-gsa_general_bwd_rows_kernel(const MaskedBwdArgs a, const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K,
-                            const __nv_bfloat16* __restrict__ Vg, const __nv_bfloat16* __restrict__ dOs,
-                            float* __restrict__ dK32, float* __restrict__ dV32) {
-    chain_wait();
-    if (*a.general == 0) return;
-    constexpr int NV = DH / 32;
-    const int lane = threadIdx.x & 31;
-    auto load = [&](const __nv_bfloat16* p, float (&f)[NV]) {
-#pragma unroll
-        for (int c = 0; c < NV; ++c) f[c] = __bfloat162float(p[lane * NV + c]);
-    };
-    auto dot = [&](const float (&x)[NV], const float (&y)[NV]) {
-        float z = 0.f;
-#pragma unroll
-        for (int c = 0; c < NV; ++c) z = fmaf(x[c], y[c], z);
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, d);
-        return z;
-    };
-    const int64_t items = (int64_t)a.B * a.rows * a.n_kv;
-    for (int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); item < items; item += (int64_t)gridDim.x * 8) {
-        const int g = (int)(item % a.n_kv), b = (int)(item / a.n_kv / a.rows), t = a.q0 + (int)(item / a.n_kv % a.rows);
-        const int64_t irow = a.il.row(b, t);
-        const int k = checked_budget(a.kt[irow], a.k_max, a.dev_status);
-        float q[G][NV], d[G][NV], dq[G][NV], l2[G], dl[G];
-#pragma unroll
-        for (int e = 0; e < G; ++e) {
-            const size_t h = ((size_t)b * a.Lq + t) * a.n_h + g * G + e;
-            load(Q + h * DH, q[e]);
-            load(dOs + h * DH, d[e]);
-            l2[e] = a.lse[h] * kLog2e; dl[e] = a.delta[h];
-#pragma unroll
-            for (int c = 0; c < NV; ++c) dq[e][c] = 0.f;
-        }
-        for (int j = 0; j < k; ++j) {
-            const int s = checked_pos(a.idx[irow * a.k_max + j], a.Lk, a.dev_status);
-            const size_t at = (((size_t)b * a.Lk + s) * a.n_kv + g) * DH;
-            float kr[NV], vr[NV], dk[NV], dv[NV], psum = 0.f;
-            load(K + at, kr);
-            load(Vg + at, vr);
-#pragma unroll
-            for (int c = 0; c < NV; ++c) dk[c] = dv[c] = 0.f;
-#pragma unroll
-            for (int e = 0; e < G; ++e) {
-                const float pz = exp2f(fmaf(dot(q[e], kr), a.scale_log2, -l2[e]));
-                const float ds = pz * (dot(d[e], vr) - dl[e]);
-                psum += pz;
-#pragma unroll
-                for (int c = 0; c < NV; ++c) {
-                    dq[e][c] = fmaf(ds, kr[c], dq[e][c]);
-                    dk[c] = fmaf(ds, q[e][c], dk[c]);
-                    dv[c] = fmaf(pz, d[e][c], dv[c]);
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < NV; ++c) {
-                atomicAdd(dK32 + at + lane * NV + c, dk[c]);
-                atomicAdd(dV32 + at + lane * NV + c, dv[c]);
-            }
-            if (a.pbar && lane == 0) atomicAdd(a.pbar + irow * a.k_max + j, psum / (float)a.n_h);      // (zeroed by the caller)
-        }
-#pragma unroll
-        for (int e = 0; e < G; ++e)
-#pragma unroll
-            for (int c = 0; c < NV; ++c)
-                a.dQ[(((size_t)b * a.Lq + t) * a.n_h + g * G + e) * DH + lane * NV + c] = __float2bfloat16_rn(dq[e][c] * a.scale);
-    }
-}
-
-__global__ void __launch_bounds__(256) gsa_general_bwd_finish_kernel(const MaskedBwdArgs a, const float* __restrict__ dK32,
-                                                                     const float* __restrict__ dV32, int64_t n) {
-    chain_wait();
-    if (*a.general == 0) return;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float sg = 1.0f / (1.0f + __expf(-__bfloat162float(a.g2[i])));
-        a.dK[i] = __float2bfloat16_rn(dK32[i] * a.scale);
-        a.dV[i] = __float2bfloat16_rn(dV32[i] * sg);
-        a.dg2[i] = __float2bfloat16_rn(dV32[i] * __bfloat162float(a.V[i]) * sg * (1.0f - sg));
-    }
-}
-
 template <int DH, int G>
 cudaError_t launch_bwd_t(const MaskedBwdArgs& a, const gsa_params_t& p, const __nv_bfloat16* Q, const __nv_bfloat16* K,
-                         const __nv_bfloat16* Vg, const __nv_bfloat16* dOs, float* dKV32, cudaStream_t st) {
+                         const __nv_bfloat16* Vg, const __nv_bfloat16* dOs, cudaStream_t st) {
     CUtensorMap tq, td, tk, tv;
     if (!make_heads_tmap(&tq, Q + (size_t)a.q0 * p.n_h * DH, p.B, p.Lq, a.rows, p.n_h, DH, 128 / G, G)) return cudaErrorUnknown;
     if (!make_heads_tmap(&td, dOs + (size_t)a.q0 * p.n_h * DH, p.B, p.Lq, a.rows, p.n_h, DH, 128 / G, G)) return cudaErrorUnknown;
@@ -915,21 +829,21 @@ cudaError_t launch_bwd_t(const MaskedBwdArgs& a, const gsa_params_t& p, const __
         launch_chained(gsa_masked_target_kernel<DH, G>, grid, kBwdThreads, kSmemT, st, tq, tk, a);
         ++g_launches;
     }
-    const int64_t n = (int64_t)p.B * p.Lk * p.n_kv * DH;
-    const int ctas = sm_count() * 4;
-    launch_chained(gsa_general_bwd_zero_kernel, ctas, 256, 0, st, a.general, reinterpret_cast<float4*>(dKV32), n / 2);
-    launch_chained(gsa_general_bwd_rows_kernel<DH, G>, ctas, 256, 0, st, a, Q, K, Vg, dOs, dKV32, dKV32 + n);
-    launch_chained(gsa_general_bwd_finish_kernel, ctas, 256, 0, st, a, dKV32, dKV32 + n, n);
-    g_launches += 3;
     return cudaGetLastError();
 }
 
 }  // namespace
 
+namespace {
+size_t sets_bytes(const gsa_params_t& p, const RowRange& rr) {           // the masks, or the inverted sets of the general path
+    const size_t masks = mask_plan(p, rr.q_begin, rr.R).bytes(p.B), inv = attn_bwd_keys_general_bytes(p, rr.R);
+    return ((masks > inv ? masks : inv) + 255) / 256 * 256;
+}
+}  // namespace
+
+// then the statistics, for calls that have not saved them
 size_t masked_bwd_bytes(const gsa_params_t& p, const RowRange& rr) {
-    const size_t masks = mask_plan(p, rr.q_begin, rr.R).bytes(p.B);
-    const size_t sums = (size_t)p.B * p.Lk * p.n_kv * p.d_h * 8;
-    return ((masks > sums ? masks : sums) + 255) / 256 * 256;
+    return sets_bytes(p, rr) + ((size_t)p.B * p.Lq * p.n_h * 4 + 255) / 256 * 256;
 }
 
 // Two models in microseconds, as in the forward (masked_rows_end).  Tiles: 1.7 + 1.45 + 1.05 (d_h = 64: 1.3 + 1.1 + 0.9) per
@@ -958,20 +872,18 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
                               __nv_bfloat16* dg2, __nv_bfloat16* dOs, float* lse_ws, float* delta, float* pbar,
                               const float* lse_in, void* ws, int32_t* dev_status, cudaStream_t st) {
     int32_t* general = dev_status + kStatusGeneralWord;
-    cudaError_t e = launch_bwd_prep(p, rr, g1, out, dout, dOs, dg1, delta, general, st);
-    // (outside the sets the tiles multiply dP - delta, Q, K and do by zero: all of them have to be finite.  V', do and delta are
-    // watched where they are written; rows of dOs past the range read as zero)
-    const int64_t q_row = (int64_t)p.n_h * p.d_h;
-    if (e == cudaSuccess) e = launch_check_values(Q + rr.q_begin * q_row, rr.R * q_row, general, st, p.B, p.Lq * q_row);
-    if (e == cudaSuccess) e = launch_check_values(K, (int64_t)p.B * p.Lk * p.n_kv * p.d_h, general, st);
+    // (outside the sets the tiles multiply dP - delta, Q, K and do by zero: all of them have to be finite.  They are watched where
+    // they are read or written first; rows of dOs past the range read as zero)
+    cudaError_t e = launch_bwd_prep(p, rr, g1, out, dout, Q, dOs, dg1, delta, general, st);
     const MaskPlan mp = mask_plan(p, rr.q_begin, rr.R);
     uint4* mask = (uint4*)ws;
     if (e == cudaSuccess) e = launch_build_masks(p, mp, masked_block_rows(p), idx, kt, il, mask, general, st);
     if (e == cudaSuccess && !lse_in) {
         // the statistics were not saved: the forward's tiles once more (their output goes where dQ is written afterwards)
-        e = launch_masked_attn_fwd(p, mp, mask, Q, K, Vg, g1, dQ, lse_ws, dev_status, st);
-        if (e == cudaSuccess) e = launch_attn_direct(p, rr, Q, K, Vg, g1, idx, kt, il, dQ, lse_ws, general, kRunAnyGeneral, st);
-        lse_in = lse_ws;
+        float* const stats = (float*)((char*)ws + sets_bytes(p, rr));
+        e = launch_masked_attn_fwd(p, mp, mask, Q, K, Vg, g1, dQ, stats, dev_status, st);
+        if (e == cudaSuccess) e = launch_attn_direct(p, rr, Q, K, Vg, g1, idx, kt, il, dQ, stats, general, kRunAnyGeneral, st);
+        lse_in = stats;
     }
     if (e != cudaSuccess) return e;
     MaskedBwdArgs a;
@@ -990,11 +902,16 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
     a.scale_log2 = a.scale * kLog2e;
     a.wait_cycles = wait_limit_cycles();
     a.withhold_first = withhold_first_copy() ? 1 : 0;
-#define GSA_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_bwd_t<DH_, G_>(a, p, Q, K, Vg, dOs, (float*)ws, st)
+    a.zero = (uint4*)ws; a.zero_vec = (int64_t)(attn_bwd_keys_general_zero(p, rr.R) / 16);
+    e = cudaErrorInvalidValue;
+#define GSA_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) e = launch_bwd_t<DH_, G_>(a, p, Q, K, Vg, dOs, st)
     GSA_CASE(128, 1); GSA_CASE(128, 2); GSA_CASE(128, 4); GSA_CASE(128, 8);
     GSA_CASE(64, 1); GSA_CASE(64, 2); GSA_CASE(64, 4); GSA_CASE(64, 8);
 #undef GSA_CASE
-    return cudaErrorInvalidValue;
+    if (e == cudaSuccess) e = launch_attn_bwd_rows_general(p, rr, Q, K, Vg, dOs, idx, kt, il, dQ, lse_ws, delta, pbar, lse_in, general, st);
+    if (e == cudaSuccess)
+        e = launch_attn_bwd_keys_general(p, rr, Q, dOs, K, V, Vg, g2, lse_ws, delta, idx, kt, il, ws, dK, dV, dg2, general, st);
+    return e;
 }
 
 }  // namespace gsa

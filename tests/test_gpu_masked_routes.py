@@ -144,10 +144,9 @@ def _irregular(cfg, what, x, idx, kt):
     """Applies `what` to row 500 of batch element 1 (a set that is otherwise in order and visible) or to the values; returns the
     bit it raises and the status."""
     kt[1, 500] = 7
-    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, 700, 800 if cfg.Lk > 1100 else 590], dtype=torch.int32).sort().values
-    idx[1, 500, 7:] = -1
     n_vis = cfg.Lk - cfg.Lq + 501
-    assert idx[1, 500, 6] < n_vis
+    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, n_vis - 41, n_vis - 11], dtype=torch.int32)
+    idx[1, 500, 7:] = -1
     if what == "unsorted":
         idx[1, 500, :7] = idx[1, 500, :7].flip(0)
     elif what == "duplicate":
@@ -218,3 +217,111 @@ def test_the_gather_does_what_the_tiles_leave_over_several_key_ranges(what):
         want = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx[b][rows].numpy(), kt[b][rows].numpy(),
                            rows, np.full_like(rows, b))
         U.check_out(out[b][torch.from_numpy(rows).cuda()].float().cpu().numpy(), want)
+
+
+def _bwd(cfg, d, idx, kt, saved_lse=True, out_of=None):
+    """Gradients, launches of the backward, status head's word, status.  out_of: sets that the forward runs on (default: the same)."""
+    p = gsa.make_params(cfg)
+    nan = float("nan")
+    out, lse = torch.full_like(d["Q"], nan), torch.full((cfg.B, cfg.Lq, cfg.n_h), nan, dtype=torch.float32, device="cuda")
+    ws = torch.empty(max(gsa.gsa_attn_workspace_bytes(p, True), gsa.gsa_attn_bwd_workspace_bytes(p)), dtype=torch.uint8, device="cuda").fill_(0xFF)
+    fi, fk = out_of if out_of else (idx, kt)
+    gsa.gsa_sparse_gated_attn_fwd_lse(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], fi.cuda(), fk.cuda(), out, lse, ws)
+    got = {n: torch.full_like(d["Q" if n in ("dQ", "dg1") else "K"], nan) for n in ("dQ", "dg1", "dK", "dV", "dg2")}
+    got["pbar"] = torch.full((cfg.B, cfg.Lq, cfg.k_max), nan, dtype=torch.float32, device="cuda")
+    ws.fill_(0xFF)
+    n0 = gsa.gsa_launch_count()
+    gsa.gsa_sparse_gated_attn_bwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx.cuda(), kt.cuda(), out, d["dout"], got["dQ"], got["dK"],
+                                  got["dV"], got["dg1"], got["dg2"], ws, pbar=got["pbar"], lse=lse if saved_lse else None)
+    n = gsa.gsa_launch_count() - n0
+    return got, n, int(ws[:256].view(torch.int32)[2]), gsa.gsa_device_status(ws)
+
+
+@pytest.mark.parametrize("what,saved_lse", [("unsorted", True), ("unsorted", False), ("duplicate", True), ("not_visible", True), ("inf_value", True),
+                                            ("huge_value", False), ("inf_key", True), ("nan_query", True), ("inf_dout", True)])
+def test_the_gather_does_what_the_backward_tiles_leave(what, saved_lse):
+    from test_gpu_backward import _compare
+    cfg = BWD
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 241, empty=[(0, 3)])
+    bit, _ = _irregular(cfg, what, x, idx, kt)
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(242)) * 0.25).to(torch.bfloat16)
+    # a value that is not finite reaches the rows that select its key (or its own row) and the keys that those rows select
+    rows = torch.zeros(cfg.B, cfg.Lq, dtype=torch.bool)
+    if what in ("inf_key", "nan_query", "inf_dout"):
+        bit = VALUES
+        if what == "inf_key":
+            x["K"][0, 700, 3, 5] = float("inf")
+        else:
+            (x["Q"] if what == "nan_query" else dout)[0, 640, 3, 5] = float("nan" if what == "nan_query" else "inf")
+            rows[0, 640] = True
+    key = {"inf_value": (0, 700), "inf_key": (0, 700), "huge_value": (1, 0)}.get(what)
+    if key:
+        rows[key[0]] |= ((idx[key[0]] == key[1]) & (torch.arange(cfg.k_max) < kt[key[0], :, None])).any(-1)
+    got, n, general, status = _bwd(cfg, U.to_dev({**x, "dout": dout}), idx, kt, saved_lse)
+    assert (n, general, status) == (11 if saved_lse else 13, bit, 0)
+    if not rows.any():
+        _compare(cfg, x, got, idx, kt, dout, 0, cfg.Lq)
+        return
+    keys = torch.zeros(cfg.B, cfg.Lk, dtype=torch.bool)
+    for b, t in rows.nonzero().tolist():
+        keys[b, idx[b, t, :int(kt[b, t])].long()] = True
+    if what != "huge_value":
+        assert not torch.isfinite(got["dQ"][0].float()).all()
+    # all other rows and keys as the oracle has them, with the value taken out
+    x["V"][~torch.isfinite(x["V"])] = 0
+    x["K"][~torch.isfinite(x["K"])] = 0
+    x["Q"][~torch.isfinite(x["Q"])] = 0
+    if what == "huge_value":
+        x["V"][1, 0, 0, 0] = 0
+    dout[~torch.isfinite(dout)] = 0
+    rb, rt = np.repeat(np.arange(cfg.B), cfg.Lq), np.tile(np.arange(cfg.Lq), cfg.B)
+    want = oracle.attn_bwd(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx.reshape(cfg.B * cfg.Lq, -1).numpy(),
+                           kt.reshape(-1).numpy(), dout.reshape(-1, cfg.n_h, cfg.d_h), rt, rb)
+    for name, bad in (("dQ", rows), ("dg1", rows), ("dK", keys), ("dV", keys), ("dg2", keys)):
+        live = ~bad
+        assert live.sum() > 50
+        g = got[name].float().cpu()[live].numpy()
+        w = want[name].reshape(tuple(got[name].shape))[live.numpy()]
+        assert np.isfinite(g).all() and np.linalg.norm(g - w) <= 8e-3 * np.linalg.norm(w), name
+
+
+@pytest.mark.parametrize("what", ["position_too_large", "position_negative", "budget_too_large"])
+def test_an_entry_out_of_range_is_not_scattered(what):
+    """Such an entry adds nothing to any key: the keys that its row does not select have the gradients of the other rows."""
+    cfg = BWD
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 241)
+    _irregular(cfg, "", x, idx, kt)
+    good = idx.clone(), kt.clone()
+    assert _irregular(cfg, what, x, idx, kt) == (SETS, 6)
+    row = set(good[0][1, 500, :7].tolist())
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(242)) * 0.25).to(torch.bfloat16)
+    got, n, general, status = _bwd(cfg, U.to_dev({**x, "dout": dout}), idx, kt, out_of=good)
+    assert (n, general, status) == (11, SETS, 6)
+    rb, rt = np.repeat(np.arange(cfg.B), cfg.Lq), np.tile(np.arange(cfg.Lq), cfg.B)
+    keep = ~((rb == 1) & (rt == 500))
+    want = oracle.attn_bwd(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], good[0].reshape(cfg.B * cfg.Lq, -1).numpy()[keep],
+                           good[1].reshape(-1).numpy()[keep], dout.reshape(-1, cfg.n_h, cfg.d_h)[torch.from_numpy(keep)], rt[keep], rb[keep])
+    live = torch.tensor([s not in row for s in range(cfg.Lk)])
+    ends = [0, cfg.Lk - 1]                       # what the entry would be clamped to
+    assert live[ends].all()
+    for name in ("dK", "dV", "dg2"):
+        g, w = got[name].float().cpu().numpy()[1], want[name].reshape(tuple(got[name].shape))[1]
+        assert np.linalg.norm(g[live] - w[live]) <= 8e-3 * np.linalg.norm(w[live]), name
+        for s in ends:
+            assert np.abs(g[s] - w[s]).max() <= 8e-3 * np.abs(w[s]).max() + 1e-6, (name, s)
+
+
+def test_the_gather_does_what_the_backward_tiles_leave_over_several_row_ranges():
+    """More than 4096 rows: the lists of a key's rows are cut into ranges whose sums meet in fp32."""
+    from test_gpu_backward import _compare
+    cfg = BWD.with_(name="bwd_ranges", B=1, Lq=4500, Lk=4500, n_h=8, n_kv=4, d_h=64, k_base=300, k_max=350)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 245)
+    idx[0, 4000, :2], kt[0, 4000] = torch.tensor([7, 5], dtype=torch.int32), 2
+    idx[0, 4000, 2:] = -1
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(246)) * 0.25).to(torch.bfloat16)
+    got, n, general, status = _bwd(cfg, U.to_dev({**x, "dout": dout}), idx, kt)
+    assert (n, general, status) == (12, SETS, 0)
+    _compare(cfg, x, got, idx, kt, dout, 0, cfg.Lq)
