@@ -166,8 +166,12 @@ int gsa_output_projection(const gsa_params_t *p, int32_t d_model, const void *at
  *          see below), which this call's second sweep has at hand: one call instead of two
  *   lse    [B, Lq, n_h] fp32 or NULL: what gsa_sparse_gated_attn_fwd_lse saved for the same inputs; with it
  *          the sweep over S_t that recomputes the softmax statistics is skipped
- *   ws     workspace of gsa_attn_bwd_workspace_bytes(p) bytes (depends on q_begin / q_end): status word,
- *          V', dout * sigmoid(g1), softmax statistics, and the index sets inverted (key -> query rows) or as masks
+ *   ws     workspace of gsa_attn_bwd_workspace_bytes(p) bytes: status word, V', dout * sigmoid(g1), softmax
+ *          statistics, and the index sets inverted (key -> query rows) or as masks, whichever is larger where masks
+ *          are the cheaper form.  The size depends on the geometry, q_begin / q_end and k_max, and through that
+ *          choice also on k_base, k_min, k_mode and the current device's number of SMs.  A workspace that holds
+ *          the inverted sets only, sized for other values of those four or for as many other rows, is accepted
+ *          too: the call then works from the inverted sets.
  * Returns GSA_ERR_WORKSPACE if ws is too small; nothing is launched on an argument error.
  */
 int gsa_attn_bwd_workspace_bytes(const gsa_params_t *p, size_t *bytes);

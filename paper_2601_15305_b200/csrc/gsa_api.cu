@@ -263,7 +263,7 @@ struct BwdPlan {
     size_t vg_off, dos_off, lse_off, delta_off, range_off, inv_off, total;
     bool masked;
 };
-static BwdPlan plan_bwd_ws(const gsa_params_t& p, int32_t rows_per_batch) {
+static BwdPlan plan_bwd_ws(const gsa_params_t& p, int32_t rows_per_batch, bool tiles = true) {
     BwdPlan w;
     size_t off = kStatusBytes;
     w.vg_off = off;    off += align_up((size_t)p.B * p.Lk * p.n_kv * p.d_h * 2, 256);
@@ -273,7 +273,7 @@ static BwdPlan plan_bwd_ws(const gsa_params_t& p, int32_t rows_per_batch) {
     w.range_off = off; off += attn_bwd_range_bytes(p);
     // (the inverted index sets, or the masks and what stands in for them where those are the cheaper path)
     const RowRange rr{0, p.B, p.q_begin, rows_per_batch};
-    w.masked = masked_bwd_preferred(p, rr);
+    w.masked = tiles && masked_bwd_preferred(p, rr);
     const size_t inv = attn_bwd_invert_bytes(p, rows_per_batch), msk = w.masked ? masked_bwd_bytes(p, rr) : 0;
     w.inv_off = off;   off += inv > msk ? inv : msk;
     w.total = off;
@@ -305,7 +305,8 @@ int gsa_sparse_gated_attn_bwd(const gsa_params_t* p, const void* Q, const void* 
     const void* ptrs[] = {Q, K, V, g1_logits, g2_logits, idx, out, dout, dQ, dK, dV, dg1, dg2};
     for (const void* q : ptrs) if (!q || !aligned16(q)) return GSA_ERR_INVALID_ARG;
     if (!kt || (pbar && !aligned16(pbar)) || (lse && !aligned16(lse))) return GSA_ERR_INVALID_ARG;
-    const BwdPlan wp = plan_bwd_ws(*p, rr.R);
+    BwdPlan wp = plan_bwd_ws(*p, rr.R);
+    if (wp.masked && ws_bytes < wp.total) wp = plan_bwd_ws(*p, rr.R, false);       // (sized for another budget or another row range)
     if (!ws || !aligned16(ws) || ws_bytes < wp.total) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     char* wsb = (char*)ws;

@@ -325,3 +325,34 @@ def test_the_gather_does_what_the_backward_tiles_leave_over_several_row_ranges()
     got, n, general, status = _bwd(cfg, U.to_dev({**x, "dout": dout}), idx, kt)
     assert (n, general, status) == (12, SETS, 0)
     _compare(cfg, x, got, idx, kt, dout, 0, cfg.Lq)
+
+
+def test_backward_workspace_sized_for_another_budget_is_accepted():
+    """Sized for a budget at which the gather is cheaper and used for one at which the tiles are: the gather does it."""
+    from test_gpu_backward import _compare
+    cfg = BWD
+    small, p = gsa.make_params(cfg, k_base=8, k_min=1), gsa.make_params(cfg)
+    need, want = gsa.gsa_attn_bwd_workspace_bytes(small), gsa.gsa_attn_bwd_workspace_bytes(p)
+    assert need < want
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 247)
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(248)) * 0.25).to(torch.bfloat16)
+    d = U.to_dev({**x, "dout": dout})
+    out, lse = torch.empty_like(d["Q"]), torch.empty((cfg.B, cfg.Lq, cfg.n_h), dtype=torch.float32, device="cuda")
+    wsf = torch.empty(gsa.gsa_attn_workspace_bytes(p, True), dtype=torch.uint8, device="cuda")
+    gsa.gsa_sparse_gated_attn_fwd_lse(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx.cuda(), kt.cuda(), out, lse, wsf)
+    for n_bytes, launches in ((want, 11), (want - 1, 9), (need, 9), (need - 1, None)):
+        ws = torch.empty(want, dtype=torch.uint8, device="cuda").fill_(0xFF)[:n_bytes]
+        got = {n: torch.full_like(d["Q" if n in ("dQ", "dg1") else "K"], float("nan")) for n in ("dQ", "dg1", "dK", "dV", "dg2")}
+        got["pbar"] = torch.full((cfg.B, cfg.Lq, cfg.k_max), float("nan"), dtype=torch.float32, device="cuda")
+        n0 = gsa.gsa_launch_count()
+        run = lambda: gsa.gsa_sparse_gated_attn_bwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx.cuda(), kt.cuda(), out, d["dout"], got["dQ"],
+                                                    got["dK"], got["dV"], got["dg1"], got["dg2"], ws, pbar=got["pbar"], lse=lse)
+        if launches is None:
+            with pytest.raises(gsa.GsaError, match="workspace"):
+                run()
+            assert gsa.gsa_launch_count() == n0
+            continue
+        run()
+        assert gsa.gsa_launch_count() - n0 == launches and gsa.gsa_device_status(ws) == 0
+        _compare(cfg, x, got, idx, kt, dout, 0, cfg.Lq)
