@@ -40,7 +40,8 @@ gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restric
     chain_wait();
     __shared__ __align__(16) uint32_t s_bits[kMaskRowAlign * kMaskRowWords];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int b = blockIdx.y, r0 = blockIdx.x * kMaskRowAlign, r = r0 + warp;
+    const int row_ctas = row_pitch / kMaskRowAlign;      // (batch elements along x: y and z end at 65535)
+    const int b = blockIdx.x / row_ctas, r0 = blockIdx.x % row_ctas * kMaskRowAlign, r = r0 + warp;
     const int blk_end = min((r0 / block_rows + 1) * block_rows, rows);
     const int tiles = min((off + q0 + blk_end + kMaskTileKeys - 1) / kMaskTileKeys, key_tiles);
     const int n_vis = off + q0 + r + 1;
@@ -476,7 +477,7 @@ cudaError_t launch_fwd_t(const MaskedFwdArgs& a, const gsa_params_t& p, const CU
 
 cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int block_rows, const int32_t* idx,
                                const int32_t* kt, IdxLayout il, uint4* mask, int32_t* general, cudaStream_t st) {
-    const dim3 grid((unsigned)(mp.row_pitch / kMaskRowAlign), (unsigned)p.B);
+    const unsigned grid = (unsigned)(mp.row_pitch / kMaskRowAlign) * (unsigned)p.B;
     launch_chained(gsa_build_masks_kernel, grid, kMaskRowAlign * 32, 0, st, idx, kt, mask, il, mp.q0, mp.rows, mp.row_pitch, mp.key_tiles,
                                                                block_rows, p.k_max, p.Lk - p.Lq, general);
     ++g_launches;

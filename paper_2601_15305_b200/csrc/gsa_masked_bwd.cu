@@ -55,7 +55,7 @@ struct MaskedBwdArgs {
     int32_t q0, rows, row_pitch, key_tiles;
     int32_t B, Lq, Lk, n_h, n_kv, k_max;
     int32_t row_blocks;            // of 128 / G queries
-    int32_t pairs_per_cta;         // target kernel: runs of 256 keys per CTA
+    int32_t pairs_per_cta, runs;   // target kernel: runs of that many pairs of key tiles, one per CTA
     float scale, scale_log2;
     uint4* zero;                   // what the general path finds cleared (see launch_attn_bwd_keys_general)
     int64_t zero_vec;
@@ -637,10 +637,12 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
     constexpr int QT = 128 / G;
     int timed_out;
     if (!tiles_allowed(a.dev_status, &timed_out)) return;
-    const int blk = a.row_blocks - 1 - (int)blockIdx.y, b = blockIdx.z;
+    // (runs of keys innermost, then row blocks, then batch elements, all along x: y and z end at 65535)
+    const int run = (int)blockIdx.x % a.runs, rest = (int)blockIdx.x / a.runs;
+    const int blk = a.row_blocks - 1 - rest % a.row_blocks, b = rest / a.row_blocks;
     const int r0 = blk * QT, off = a.Lk - a.Lq;
     const int ntiles = min((off + a.q0 + min(r0 + QT, a.rows) + kMaskTileKeys - 1) / kMaskTileKeys, a.key_tiles);
-    const int pair0 = blockIdx.x * a.pairs_per_cta, pair1 = min(pair0 + a.pairs_per_cta, (ntiles + 1) / 2);
+    const int pair0 = run * a.pairs_per_cta, pair1 = min(pair0 + a.pairs_per_cta, (ntiles + 1) / 2);
     if (pair0 >= pair1) return;
     const int n = (pair1 - pair0) * a.n_kv;                        // steps: (key pair, KV head)
     GSA_TILE_PROLOGUE(P)
@@ -824,9 +826,7 @@ cudaError_t launch_bwd_t(const MaskedBwdArgs& a, const gsa_params_t& p, const __
     launch_chained(gsa_masked_bwd_rows_kernel<DH, G>, (unsigned)(a.row_blocks * p.n_kv * p.B), kBwdThreads, kSmemR, st, tq, td, tk, tv, a);
     g_launches += 2;
     if (a.pbar) {
-        const int pairs = (a.key_tiles + 1) / 2;
-        const dim3 grid((unsigned)((pairs + a.pairs_per_cta - 1) / a.pairs_per_cta), (unsigned)a.row_blocks, (unsigned)p.B);
-        launch_chained(gsa_masked_target_kernel<DH, G>, grid, kBwdThreads, kSmemT, st, tq, tk, a);
+        launch_chained(gsa_masked_target_kernel<DH, G>, (unsigned)a.runs * (unsigned)a.row_blocks * (unsigned)p.B, kBwdThreads, kSmemT, st, tq, tk, a);
         ++g_launches;
     }
     return cudaGetLastError();
@@ -898,6 +898,7 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
     const int64_t pairs = (int64_t)((a.key_tiles + 1) / 2) * a.row_blocks * p.B;
     a.pairs_per_cta = (int)(pairs / 2 / (4 * sm_count()));
     a.pairs_per_cta = a.pairs_per_cta < 1 ? 1 : (a.pairs_per_cta > 8 ? 8 : a.pairs_per_cta);
+    a.runs = ((a.key_tiles + 1) / 2 + a.pairs_per_cta - 1) / a.pairs_per_cta;
     a.scale = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
     a.scale_log2 = a.scale * kLog2e;
     a.wait_cycles = wait_limit_cycles();

@@ -356,3 +356,37 @@ def test_backward_workspace_sized_for_another_budget_is_accepted():
         run()
         assert gsa.gsa_launch_count() - n0 == launches and gsa.gsa_device_status(ws) == 0
         _compare(cfg, x, got, idx, kt, dout, 0, cfg.Lq)
+
+
+def test_more_than_65535_batch_elements():
+    """Attention, its backward and the target over 66000 short sequences: grids whose second and third axes end at 65535."""
+    B, L, nh, dh = 66000, 64, 1, 64
+    p = gsa.make_params(B=B, Lq=L, Lk=L, n_h=nh, n_kv=1, d_h=dh, HI=1, dI=32, k_base=L, k_min=1, k_max=L)
+    g = torch.Generator(device="cuda").manual_seed(260)
+    new = lambda s=1.0: torch.randn(B, L, nh, dh, generator=g, dtype=torch.bfloat16, device="cuda").mul_(s)  # noqa: E731
+    x = {n: new() for n in ("Q", "K", "V", "g1", "g2")}
+    dout = new(0.25)
+    idx = torch.arange(L, dtype=torch.int32, device="cuda").repeat(L, 1)
+    idx = torch.where(idx <= torch.arange(L, device="cuda")[:, None], idx, -1).to(torch.int32).repeat(B, 1, 1)
+    kt = torch.arange(1, L + 1, dtype=torch.int32, device="cuda").repeat(B, 1)
+    out, lse = torch.empty_like(x["Q"]), torch.empty((B, L, nh), dtype=torch.float32, device="cuda")
+    ws = torch.empty(max(gsa.gsa_attn_workspace_bytes(p, True), gsa.gsa_attn_bwd_workspace_bytes(p)), dtype=torch.uint8, device="cuda")
+    n0 = gsa.gsa_launch_count()
+    gsa.gsa_sparse_gated_attn_fwd_lse(p, x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx, kt, out, lse, ws)
+    assert gsa.gsa_launch_count() - n0 in (3, 4) and gsa.gsa_device_status(ws) == 0        # (3: the value gate inside the gather)
+    got = {n: torch.empty_like(x["Q"]) for n in ("Q", "K", "V", "g1", "g2")}
+    pbar = torch.empty((B, L, L), dtype=torch.float32, device="cuda")
+    n0 = gsa.gsa_launch_count()
+    gsa.gsa_sparse_gated_attn_bwd(p, x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx, kt, out, dout, got["Q"], got["K"], got["V"], got["g1"],
+                                  got["g2"], ws, pbar=pbar, lse=lse)
+    assert gsa.gsa_launch_count() - n0 == 11 and gsa.gsa_device_status(ws) == 0
+    at = torch.tensor([0, 1, 65534, 65535, 65536, B - 1], device="cuda")
+    y = {n: x[n][at, :, 0].double().requires_grad_() for n in x}
+    z = (y["Q"] @ y["K"].transpose(1, 2)) / dh ** 0.5
+    P = torch.softmax(z.masked_fill(torch.ones(L, L, dtype=torch.bool, device="cuda").triu(1), -float("inf")), -1)
+    want = (P @ (y["V"] * torch.sigmoid(y["g2"]))) * torch.sigmoid(y["g1"])
+    (want * dout[at, :, 0].double()).sum().backward()
+    rel = lambda a, b: float((a.double() - b).norm() / b.norm())  # noqa: E731
+    assert rel(out[at, :, 0], want.detach()) < 1e-2 and rel(pbar[at], P.detach()) < 2e-3
+    for n in got:
+        assert rel(got[n][at, :, 0], y[n].grad) < 1e-2, n
