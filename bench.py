@@ -37,10 +37,6 @@ UNIT = "tokens/s"
 # special-function operations the indexer's epilogue spends per sigmoid: one exp2 each and one reciprocal
 # shared by the eight heads of a query
 SFU_OPS_PER_SIGMOID = 1.125
-# DRAM bytes (read + written) of the sparse-attention launches of one forward, per workload, from the one-pass
-# ncu capture summarised in profiles/gsa_sparse_attn_kernel_l128k_dram.md (taken with the current kernel,
-# default slab and key ranges); a workload without a capture reports null
-ATTN_DRAM_TRAFFIC = {"l128k": 47.06e9}
 
 
 def measured_peaks():
@@ -115,12 +111,12 @@ def aggregate_over_ranks(ms_local: float, units_local: float):
     return float(t.item()), float(u.item())
 
 
-def attention_bytes(cfg, kt_sum: int) -> float:
-    """Algorithmic bytes of one sparse-attention launch: per selected (t, s) one K row and one V' row of
+def attention_bytes(cfg, kt_sum: int, rows: int) -> float:
+    """Algorithmic bytes of gathering `rows` query rows per batch element with kt_sum selected pairs in all: per selected (t, s) one K row and one V' row of
     all KV heads (2 * n_kv * d_h * 2 B) and one 4-byte index; per token Q, g1 and out (3 * n_h * d_h * 2 B)."""
     per_pair = 2 * cfg.n_kv * cfg.d_h * 2 + 4
     per_tok = 3 * cfg.n_h * cfg.d_h * 2 + 4
-    return float(kt_sum) * per_pair + float(cfg.B * cfg.Lq) * per_tok
+    return float(kt_sum) * per_pair + float(cfg.B * rows) * per_tok
 
 
 def measure_rates(gsa, stream):
@@ -349,28 +345,41 @@ def main():
 
     peaks = measured_peaks()
     rates = None if args.no_rates else measure_rates(gsa, stream)
-    ab = attention_bytes(cfg, kt_sum)
-    achieved = ab / (attn_ms * 1e-3) / 1e9
     hbm_src = f"{peaks['source']} (MEASURED_PEAKS.json hbm_gbs)" if peaks["source"] == "measured" else "fallback 6650 GB/s"
-    # The gather of sparse attention is served by the L2 (key ranges of 16384 keys keep a range's K and V' rows
-    # resident), so the ceiling that binds is the L2's gather rate for 256-byte pieces, measured by the probe
-    # above; the fraction of the HBM copy bandwidth is kept beside it.  `traffic`: DRAM bytes of the launch from
-    # an ncu capture of this kernel (ATTN_DRAM_TRAFFIC), null for workloads without one.
+    # Which rows of the attention stage run as masked tiles and which on the gather (all of them where the value gate runs inside
+    # the gather), and what each part has to do.
+    tile_rows = gsa.gsa_attn_tile_rows(p)[0] if "masked_tiles" in stage_ms else 0
+    off = cfg.Lk - cfg.Lq
+    tile_pairs = cfg.B * (off * tile_rows + tile_rows * (tile_rows + 1) / 2.0)                    # visible (query, key) pairs
+    gather_rows = cfg.Lq - tile_rows
+    kt_gather = int(kt[:, tile_rows:].sum().item())                                               # selected pairs of the other rows
+    gather_ms = sum(stage_ms.get(n, 0.0) for n in ("range_cuts", "sparse_attn", "finalize"))
+    # The gather is served by the L2 (key ranges of 16384 keys keep a range's K and V' rows resident), so the ceiling that binds is
+    # the L2's gather rate for 256-byte pieces, measured by the probe above; the fraction of the HBM copy bandwidth is kept beside it.
     l2_peak = rates["gather_l2_64MB_piece256_gbs"] if rates else None
-    roofline = {"kernel": "gsa_sparse_attn_kernel", "bound": "l2" if rates else "hbm", "achieved": achieved,
-                "peak": l2_peak if rates else peaks["hbm_gbs"], "unit": "GB/s",
-                "frac": achieved / (l2_peak if rates else peaks["hbm_gbs"]), "traffic": ATTN_DRAM_TRAFFIC.get(cfg.name)
-                if args.slab_rows == 0 else None,
-                "peak_source": "measured in this run: gsa_probe_gather, random 256-byte pieces of a 64 MB table (L2-resident)"
-                if rates else hbm_src,
-                "l2_gather_gbs": l2_peak, "frac_l2": achieved / l2_peak if rates else None,
-                "hbm_gbs": peaks["hbm_gbs"], "frac_hbm": achieved / peaks["hbm_gbs"], "hbm_source": hbm_src,
-                "hbm_gather_gbs": rates["gather_hbm_2GB_piece256_gbs"] if rates else None,
-                "algorithmic_bytes_per_launch": ab, "launch_ms": attn_ms,
-                "note": "one 'launch' = the sparse-attention stage of a forward: masked tiles on the tensor cores for rows that see "
-                        "few enough keys, the gather for the others (range cuts, one kernel launch per 16384-key "
-                        "range, finalize).  All rows are charged the gather's bytes.  The 126 MB L2, not HBM, serves the gather, so frac is taken against the L2's "
-                        "measured gather rate; frac_hbm (against the HBM copy bandwidth) exceeds 1 for the same reason"}
+    parts = []
+    if tile_rows:
+        tf = 4.0 * cfg.n_h * cfg.d_h * tile_pairs / (stage_ms["masked_tiles"] * 1e-3) / 1e12
+        parts.append({"kernel": "gsa_masked_attn_fwd_kernel", "bound": "tensor", "achieved": tf, "peak": peaks["bf16_tflops_sustained"],
+                      "unit": "TFLOP/s", "frac": tf / peaks["bf16_tflops_sustained"], "traffic": None,
+                      "peak_source": f"{peaks['source']} bf16_tflops_sustained", "rows": tile_rows, "launch_ms": stage_ms["masked_tiles"],
+                      "selected_share_of_pairs": (kt_sum - kt_gather) / tile_pairs,
+                      "note": "two products over every visible pair of these rows (masks, tiles and the gather launches behind them, "
+                              "which return at once)"})
+    if gather_rows:
+        ab = attention_bytes(cfg, kt_gather, gather_rows)
+        gbs = ab / (gather_ms * 1e-3) / 1e9
+        parts.append({"kernel": "gsa_sparse_attn_kernel", "bound": "l2" if rates else "hbm", "achieved": gbs,
+                      "peak": l2_peak if rates else peaks["hbm_gbs"], "unit": "GB/s",
+                      "frac": gbs / (l2_peak if rates else peaks["hbm_gbs"]), "traffic": None,
+                      "peak_source": "measured in this run: gsa_probe_gather, random 256-byte pieces of a 64 MB table (L2-resident)"
+                      if rates else hbm_src,
+                      "hbm_gbs": peaks["hbm_gbs"], "hbm_source": hbm_src, "rows": gather_rows,
+                      "hbm_gather_gbs": rates["gather_hbm_2GB_piece256_gbs"] if rates else None,
+                      "algorithmic_bytes_per_launch": ab, "launch_ms": gather_ms,
+                      "note": "one 'launch' = the gather's part of the stage: range cuts, one kernel launch per 16384-key range, "
+                              "finalize; the bytes of its own rows"})
+    roofline = max(parts, key=lambda q: q["launch_ms"])
     causal_pairs = cfg.B * sum(cfg.Lk - cfg.Lq + t + 1 for t in (0, cfg.Lq - 1)) * cfg.Lq / 2.0
     stages = {"indexer_plus_topk_ms": sel_ms, "sparse_attn_ms": attn_ms,
               "indexer_causal_tflop": 2.0 * cfg.HI * cfg.dI * causal_pairs / 1e12,
@@ -407,22 +416,24 @@ def main():
         gbs = 3.0 * 2 * cfg.B * cfg.Lk * cfg.n_kv * cfg.d_h / (ms * 1e-3) / 1e9
         roofline_all["value_gate"] = {"kernel": "gsa_value_gate_kernel", "ms": ms, "launches": n, "bound": "hbm",
                                       "achieved_gbs": gbs, "peak_gbs": peaks["hbm_gbs"], "frac": gbs / peaks["hbm_gbs"]}
+    if tile_rows:
+        roofline_all["masked_tiles"] = dict(parts[0], ms=stage_ms["masked_tiles"], launches=stage_launches["masked_tiles"])
     ms, n = per_kernel("sparse_attn")
     if n:
-        gb = float(kt_sum) * (2 * cfg.n_kv * cfg.d_h * 2 + 4)
+        gb = float(kt_gather) * (2 * cfg.n_kv * cfg.d_h * 2 + 4)
         gbs = gb / (ms * 1e-3) / 1e9
         roofline_all["sparse_attn"] = {"kernel": "gsa_sparse_attn_kernel", "ms": ms, "launches": n,
                                        "bound": "l2" if rates else "hbm", "achieved_gbs": gbs,
                                        "peak_gbs": l2_peak if rates else peaks["hbm_gbs"],
                                        "frac": gbs / (l2_peak if rates else peaks["hbm_gbs"]),
                                        "frac_hbm": gbs / peaks["hbm_gbs"],
-                                       "tflops": float(kt_sum) * cfg.n_h * cfg.d_h * 4 / (ms * 1e-3) / 1e12,
-                                       "note": "gathered K and V' rows (+ indices) of the selected pairs; the kernel launches only"}
+                                       "tflops": float(kt_gather) * cfg.n_h * cfg.d_h * 4 / (ms * 1e-3) / 1e12,
+                                       "note": "gathered K and V' rows (+ indices) of the selected pairs of its rows; the kernel launches only"}
     ms, n = per_kernel("finalize")
     if n:
         slots = 1
-        state = cfg.B * cfg.Lq * cfg.n_h * (cfg.d_h + 2) * 4.0 * slots
-        gbs = (state + 2.0 * 2 * cfg.B * cfg.Lq * cfg.n_h * cfg.d_h) / (ms * 1e-3) / 1e9
+        state = cfg.B * gather_rows * cfg.n_h * (cfg.d_h + 2) * 4.0 * slots
+        gbs = (state + 2.0 * 2 * cfg.B * gather_rows * cfg.n_h * cfg.d_h) / (ms * 1e-3) / 1e9
         roofline_all["finalize"] = {"kernel": "gsa_attn_finalize_kernel", "ms": ms, "launches": n, "bound": "hbm",
                                     "achieved_gbs": gbs, "peak_gbs": peaks["hbm_gbs"], "frac": gbs / peaks["hbm_gbs"],
                                     "note": "fp32 softmax state + g1 read, bf16 out written (one state slot per row counted)"}
@@ -496,17 +507,27 @@ def main():
         torch.cuda.synchronize()
         b_ms = be[0].elapsed_time(be[1]) / n_b
         b_ms_recompute = be[1].elapsed_time(be[2])
-        # algorithmic bytes (statistics saved by the forward): the query-major kernel gathers K and V' once per selected (query, key) pair
-        # and KV head (d_h * 2 bytes each); the key-major kernel gathers Q and dout * sigmoid(g1) of every
-        # head once per pair (n_h * d_h * 2 bytes each); plus the index sets and their inverse (4 + 4 bytes)
-        gather = float(kt_sum) * (2 * cfg.n_kv * cfg.d_h * 2 + 2 * cfg.n_h * cfg.d_h * 2 + 8)
-        backward = {"kernels": "gsa_masked_bwd_* (masked tiles) or gsa_sparse_attn_bwd_* (gather), by the cost models", "ms": b_ms,
-                    "bound": "hbm", "algorithmic_bytes": gather, "achieved_gbs": gather / (b_ms * 1e-3) / 1e9,
-                    "peak_gbs": peaks["hbm_gbs"], "frac": gather / (b_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                    "ms_recomputing_statistics": b_ms_recompute,
-                    "tokens_per_s": cfg.B * cfg.Lq / (b_ms * 1e-3), "vs_forward": b_ms / (ms_total / args.steps),
-                    "note": "value gate pre-pass, query-major kernel (dQ, dg1, and the indexer loss's target as a "
-                            "by-product), index-set inversion, key-major kernel (dK, dV, dg2)"}
+        if gsa.gsa_attn_tile_rows(p)[1]:
+            # keys kernel: S, dP, dV', dK; rows kernel: S, dP, dQ; target kernel: S -- eight products over every visible pair
+            flop = 8 * 2.0 * cfg.n_h * cfg.d_h * causal_pairs
+            tf = flop / (b_ms * 1e-3) / 1e12
+            limit = {"kernels": "gsa_masked_bwd_keys_kernel, gsa_masked_bwd_rows_kernel, gsa_masked_target_kernel", "bound": "tensor",
+                     "flops": flop, "achieved_tflops": tf, "peak_tflops": peaks["bf16_tflops_sustained"],
+                     "frac": tf / peaks["bf16_tflops_sustained"],
+                     "note": "value gate, preparation, masks, then dK dV dg2, dQ, and the indexer loss's target as a by-product on masked tiles"}
+        else:
+            # algorithmic bytes (statistics saved by the forward): the query-major kernel gathers K and V' once per selected
+            # (query, key) pair and KV head (d_h * 2 bytes each); the key-major kernel gathers Q and dout * sigmoid(g1) of every
+            # head once per pair (n_h * d_h * 2 bytes each); plus the index sets and their inverse (4 + 4 bytes)
+            gather = float(kt_sum) * (2 * cfg.n_kv * cfg.d_h * 2 + 2 * cfg.n_h * cfg.d_h * 2 + 8)
+            gbs = gather / (b_ms * 1e-3) / 1e9
+            limit = {"kernels": "gsa_sparse_attn_bwd_kernel, gsa_sparse_attn_bwd_keys_kernel", "bound": "l2" if rates else "hbm",
+                     "algorithmic_bytes": gather, "achieved_gbs": gbs, "peak_gbs": l2_peak if rates else peaks["hbm_gbs"],
+                     "frac": gbs / (l2_peak if rates else peaks["hbm_gbs"]),
+                     "note": "value gate pre-pass, query-major kernel (dQ, dg1, and the indexer loss's target as a "
+                             "by-product), index-set inversion, key-major kernel (dK, dV, dg2)"}
+        backward = {**limit, "ms": b_ms, "ms_recomputing_statistics": b_ms_recompute,
+                    "tokens_per_s": cfg.B * cfg.Lq / (b_ms * 1e-3), "vs_forward": b_ms / (ms_total / args.steps)}
         del dout, gq, gk, ws_b, lse
         # the indexer's sparse-phase loss (Eq. 14) on the same index sets: its target, then loss + derivatives
         loss_rows = torch.empty((cfg.B, cfg.Lq), dtype=torch.float32, device="cuda")

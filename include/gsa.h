@@ -355,6 +355,18 @@ int gsa_device_status(const void *ws, void *stream, int32_t *status_out);
  */
 int gsa_select_fallback_rows(const void *ws, void *stream, int32_t *rows_out);
 
+/*
+ * A diagnostic (host call): which way the attention stage goes on the current device for rows [q_begin, q_end).
+ * The library chooses by the geometry, the budget rule's parameters and the number of SMs, not by the data.
+ *   *fwd_rows   the first *fwd_rows of these rows (of every batch element) run as masked dense tiles on the tensor
+ *               cores, the others on the gather.  (None run as tiles in a call whose value gate runs inside the
+ *               gather: decode, or a workspace without room for the gated values.)
+ *   *bwd_tiles  1 if gsa_sparse_gated_attn_bwd runs on tiles
+ * Tiles leave a call to the gather, on the device, if a set is not strictly ascending positions that its row can see, or if
+ * a value that they read is infinite, NaN or at least 2^60 in magnitude (the forward: V'; the backward: Q, K, V', do, delta).
+ */
+int gsa_attn_tile_rows(const gsa_params_t *p, int32_t *fwd_rows, int32_t *bwd_tiles);
+
 /* Number of kernel launches the library has enqueued so far in this process (host counter). */
 int64_t gsa_launch_count(void);
 
@@ -375,8 +387,9 @@ void gsa_debug_set_attn_range_keys(int32_t keys);
  * Test knob for the bounded device-side waits: `cycles` is the limit of every wait in SM clock cycles
  * (<= 0 restores the default of 2^31, about a second).  With withhold_first_copy != 0 the copy producer of
  * each tensor-core kernel (gsa_indexer_scores / gsa_forward on the tcgen05 path, gsa_project,
- * gsa_output_projection, the masked tiles of the attention stage and its backward) leaves out its first copy, so that the wait for it meets a barrier that nothing
- * completes: the way to see the give-up path work (status word set, kernel returns, context intact).
+ * gsa_output_projection, the masked tiles of the attention stage and its backward) leaves out its first copy, so
+ * that the wait for it meets a barrier that nothing completes: the way to see the give-up path work (status word set,
+ * kernel returns, context intact).
  * Process-wide; not meant for production use.
  */
 void gsa_debug_set_wait_limit(int64_t cycles, int32_t withhold_first_copy);
@@ -393,8 +406,8 @@ void gsa_profile_set_events(void *ev_begin, void *ev_selected, void *ev_end);
  * Profiling hook with one interval per launch: `events` is an array of `capacity` cudaEvent_t handles
  * (created by the caller, timing enabled).  Every following gsa_forward records events[0] at entry and the
  * next event behind each stage it enqueues, and writes into the HOST arrays stage_out[i] which stage the
- * interval events[i] .. events[i + 1] belongs to (0 indexer, 1 budget + top-k, 2 value gate, 3 range cuts or masks,
- * 4 sparse attention, 5 normalise + output gate) and into *count_out the number of intervals.  The events
+ * interval events[i] .. events[i + 1] belongs to (0 indexer, 1 budget + top-k, 2 value gate, 3 range cuts,
+ * 4 sparse attention by the gather, 5 normalise + output gate, 6 masks and masked tiles) and into *count_out the number of intervals.  The events
  * serialise nothing but cost a little: use it for a profiling step, not inside a timed loop.  NULL / 0
  * switches it off.  Process-wide; the caller owns the events and the arrays and reads them after
  * synchronising.

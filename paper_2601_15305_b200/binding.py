@@ -25,6 +25,7 @@ EXPORTS = (
     "gsa_attn_bwd_workspace_bytes", "gsa_sparse_gated_attn_bwd", "gsa_vbar_update",
     "gsa_attn_probs_mean", "gsa_indexer_kl_workspace_bytes", "gsa_indexer_kl_bwd", "gsa_sparse_gated_attn_fwd_lse",
     "gsa_profile_set_timeline", "gsa_probe_gather", "gsa_probe_ex2", "gsa_debug_set_wait_limit", "gsa_value_gate",
+    "gsa_attn_tile_rows",
 )
 
 STATIC_SCRATCH_BYTES = 32 << 20     # GSA_STATIC_SCRATCH_BYTES of include/gsa.h
@@ -260,6 +261,13 @@ def gsa_select_fallback_rows(ws, stream=None) -> int:
     return v.value
 
 
+def gsa_attn_tile_rows(p) -> tuple:
+    """(query rows of the forward that run on masked tiles, whether the backward does)."""
+    rows, bwd = ctypes.c_int32(0), ctypes.c_int32(0)
+    _check(lib().gsa_attn_tile_rows(ctypes.byref(p), ctypes.byref(rows), ctypes.byref(bwd)), "gsa_attn_tile_rows")
+    return rows.value, bool(bwd.value)
+
+
 def gsa_launch_count() -> int:
     return int(lib().gsa_launch_count())
 
@@ -272,7 +280,7 @@ def gsa_debug_set_wait_limit(cycles: int = 0, withhold_first_copy: bool = False)
     lib().gsa_debug_set_wait_limit(ctypes.c_int64(cycles), ctypes.c_int32(1 if withhold_first_copy else 0))
 
 
-STAGE_NAMES = ("indexer", "select", "value_gate", "range_cuts", "sparse_attn", "finalize")
+STAGE_NAMES = ("indexer", "select", "value_gate", "range_cuts", "sparse_attn", "finalize", "masked_tiles")
 _timeline_keep = None        # the arrays the library writes into must outlive the calls
 
 

@@ -672,6 +672,17 @@ int gsa_device_status(const void* ws, void* stream, int32_t* status_out) {
     return v == kDevOk ? GSA_OK : (v == kDevBadIndex ? GSA_ERR_INDEX_RANGE : GSA_ERR_DEVICE_TIMEOUT);
 }
 
+int gsa_attn_tile_rows(const gsa_params_t* p, int32_t* fwd_rows, int32_t* bwd_tiles) {
+    int rc = check_params(p);
+    if (rc) return rc;
+    RowRange rr;
+    if ((rc = row_range(p, &rr))) return rc;
+    if (!fwd_rows || !bwd_tiles) return GSA_ERR_INVALID_ARG;
+    *fwd_rows = attn_tile_rows(*p, rr);
+    *bwd_tiles = attn_bwd_supported(*p) && masked_bwd_preferred(*p, rr) ? 1 : 0;
+    return GSA_OK;
+}
+
 int gsa_select_fallback_rows(const void* ws, void* stream, int32_t* rows_out) {
     if (!ws || !rows_out) return GSA_ERR_INVALID_ARG;
     int32_t v = 0;

@@ -629,7 +629,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
                        pl.n_ranges, g_range_keys, a.only_if, a.run_if);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        timeline_mark(kStageRangeCuts, st);
+        if (!a.only_if) timeline_mark(kStageRangeCuts, st);
     }
     a.cuts = cuts;
     a.n_cuts = pl.n_ranges;
@@ -648,7 +648,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
             a.only_if, a.run_if);
         ++g_launches;
         cudaError_t fe = cudaGetLastError();
-        timeline_mark(kStageFinalize, st);
+        if (!a.only_if) timeline_mark(kStageFinalize, st);
         if (fe == cudaSuccess && prog && prog->n < prog->cap && prog->n < 64) {
             fe = cudaEventRecord(prog->events[prog->n], st);
             prog->t_lo[prog->n] = t_lo; prog->t_hi[prog->n] = t_hi;
@@ -676,7 +676,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
         launch_chained(kern, ctas, warps * 32, smem / kWarpsPerCta * warps, st, ar);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        timeline_mark(kStageAttn, st);
+        if (!a.only_if) timeline_mark(kStageAttn, st);
         if (pl.mode == 0 && rg + 1 < pl.n_ranges) {
             // rows whose last visible key lies in this range are complete
             const int64_t t_done = (int64_t)(rg + 1) * g_range_keys - off;
@@ -690,7 +690,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
 
 // First row from which the gather is the cheaper path (rr.q_begin: all of them; its end: none), from two models in
 // microseconds.  Tiles: a CTA takes 2.1 (d_h = 64: 1.9) per key tile of its 256 (row, head) rows and the GPU one CTA per SM,
-// plus 10 for the masks, the start and the plain kernel's launch (measured at L = 32K and 16K).  Gather: 36 ps (24) per pair
+// plus 10 for the masks, the start and the gather's idle launch behind them (measured at L = 32K and 16K).  Gather: 36 ps (24) per pair
 // and KV head, 41 (27) out of several key ranges (measured at L = 16K and 128K for 1, 2, 4 and 8 query heads per KV head),
 // and a warp's own chain of 16-key steps where a call has few rows.
 struct ForwardCosts {
@@ -800,10 +800,8 @@ cudaError_t launch_masked_rows(const gsa_params_t& p, const AttnPlan& pl, const 
         cudaError_t e = all_visible ? launch_visible_masks(p, mp, (uint4*)scratch, st)
                                     : launch_build_masks(p, mp, block, idx, kt, il, (uint4*)scratch, general, st);
         if (e != cudaSuccess) return e;
-        timeline_mark(kStageRangeCuts, st);
         e = launch_masked_attn_fwd(p, mp, (const uint4*)scratch, Q, K, Vg, g1, out, lse, t_dev_status, st);
         if (e != cudaSuccess) return e;
-        timeline_mark(kStageAttn, st);
         // What the tiles have left: the gather, key range by key range if the sets are in order, else whole sets at once.
         RowRange chunk = rr;
         chunk.q_begin = q; chunk.R = mp.rows;
@@ -815,6 +813,7 @@ cudaError_t launch_masked_rows(const gsa_params_t& p, const AttnPlan& pl, const 
             e = launch_attn_dh<false>(a, p, pl, g1, out, st, nullptr);
         }
         if (e != cudaSuccess) return e;
+        timeline_mark(kStageTiles, st);
         if (prog && prog->n < prog->cap && prog->n < 64) {
             if ((e = cudaEventRecord(prog->events[prog->n], st)) != cudaSuccess) return e;
             prog->t_lo[prog->n] = q; prog->t_hi[prog->n] = q + mp.rows;
@@ -858,6 +857,11 @@ cudaError_t launch_value_gate(const __nv_bfloat16* V, const __nv_bfloat16* g2, _
                                                   reinterpret_cast<const uint4*>(K));
     ++g_launches;
     return cudaGetLastError();
+}
+
+int attn_tile_rows(const gsa_params_t& p, RowRange rr) {
+    const AttnPlan pl = plan_attn(p);
+    return masked_rows_end(p, pl, rr, (pl.state_bytes + 255) / 256 * 256 + pl.cuts_bytes) - rr.q_begin;
 }
 
 cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q,

@@ -76,7 +76,7 @@ int sm_count();
 // every launcher records the next event of the caller's array behind the stage it just enqueued and notes
 // which stage the interval that ends there belongs to.
 enum : int32_t { kStageIndexer = 0, kStageSelect = 1, kStageValueGate = 2, kStageRangeCuts = 3, kStageAttn = 4,
-                 kStageFinalize = 5 };
+                 kStageFinalize = 5, kStageTiles = 6 };
 void timeline_mark(int32_t stage, cudaStream_t st);
 
 // ---- stage launchers (host) ----------------------------------------------------------------
@@ -154,6 +154,9 @@ cudaError_t launch_sparse_attn(const gsa_params_t& p, RowRange rr, const __nv_bf
                                AttnProgress* progress = nullptr, float* lse = nullptr,
                                bool values_scanned = false /*launch_value_gate wrote V and watched the status head*/,
                                bool all_visible = false /*launch_all_visible wrote the sets*/);
+
+// query rows from rr.q_begin on that launch_sparse_attn does on masked tiles (V' gated, workspace of attn_scratch_bytes)
+int attn_tile_rows(const gsa_params_t& p, RowRange rr);
 
 // bytes of device scratch launch_sparse_attn needs for `p` (softmax state slots, range cuts)
 size_t attn_scratch_bytes(const gsa_params_t& p);

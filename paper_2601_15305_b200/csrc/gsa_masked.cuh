@@ -114,16 +114,16 @@ __device__ __forceinline__ void tma_load_tile(uint32_t dst, const CUtensorMap* t
         : "memory");
 }
 
-// The MMA warp runs converged and one elected lane issues: descriptors then stay in uniform registers.  (A single lane in
-// a branch of its own has to move every operand of every instruction there first: which cost more than
-// a product of M = N = 128, K = 16 takes (64 cycles).  Backward at L = 32K: keys kernel 6.6 -> 6.1 ms, rows 5.7 -> 5.3 ms)
-// Start of a tile kernel: false if the call's inputs rule the tiles out (the plain kernel does the work; the same for every
+// Start of a tile kernel: false if the call's inputs rule the tiles out (the gather does the work; the same for every
 // thread).  *timed_out: an earlier CTA or launch of the call gave up on a wait (may differ between threads: use one's).
 __device__ __forceinline__ bool tiles_allowed(const int32_t* dev_status, int* timed_out) {
     const int32_t st = *reinterpret_cast<const volatile int32_t*>(dev_status);
     *timed_out = st >= kDevTimeoutTma && st <= kDevTimeoutEpi;
     return *reinterpret_cast<const volatile int32_t*>(dev_status + kStatusGeneralWord) == 0;
 }
+// The MMA warp runs converged and one elected lane issues: descriptors then stay in uniform registers.  (A single lane in
+// a branch of its own has to move every operand of every instruction there first, which cost more than
+// a product of M = N = 128, K = 16 takes (64 cycles).  Backward at L = 32K: keys kernel 6.6 -> 6.1 ms, rows 5.7 -> 5.3 ms.)
 __device__ __forceinline__ uint32_t elect_lane() {
     uint32_t e;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
@@ -174,11 +174,6 @@ __device__ __forceinline__ void warp_commit(uint32_t elected, uint32_t bar) {
         "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]),     \
         "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]),    \
         "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-#define GSA_R32_IN(r)                                                                                               \
-    "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),  \
-        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]),            \
-        "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]),            \
-        "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
 
 // 32 columns of this thread's TMEM lane
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -190,17 +185,9 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr)
         : "memory");
 }
-// waits for every tcgen05.ld of this thread; the registers of r may be used from here on (tc_tie32 for others)
+// waits for every tcgen05.ld of this thread; the registers of r may be used from here on
 __device__ __forceinline__ void tc_wait_ld32(uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" : GSA_R32_TIE(r) : : "memory");
-}
-__device__ __forceinline__ void tc_tie32(uint32_t (&r)[32]) { asm volatile("" : GSA_R32_TIE(r) : : "memory"); }
-__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,"
-        "%29,%30,%31};" ::GSA_R32_IN(r), "r"(taddr)
-        : "memory");
 }
 __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16]) {
     asm volatile(

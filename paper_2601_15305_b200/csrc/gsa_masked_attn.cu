@@ -16,7 +16,7 @@
 // 2.62e-3 with it, 2.64e-3 in the gather kernel; 50 prefill, chunk, dense and training shapes: 0.995 of the gather's on average.
 //
 // Bound: the serial chain of a tile (scores -> numerators -> product -> next scores); the two tiles' chains fill each other's
-// gaps, with the tensor cores and the special-function unit each busy somewhat over half of the time.  Measured at 16 heads of
+// gaps, with the tensor pipe active 42 % and the special-function unit 44 % of the time (8K, profiler).  Measured at 16 heads of
 // 128 on 8 KV heads: L = 32K 3.45 ms = 1.27 PFLOP/s over the visible pairs (the gather kernel: 19.6 ms; with a whole tile's
 // numerators handed over at once 3.55), 8K 0.33 ms (4.6 ms), dense 2 x 3072 0.135 ms (2.7 ms).
 //

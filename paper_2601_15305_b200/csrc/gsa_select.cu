@@ -575,11 +575,11 @@ __global__ void __launch_bounds__(kSelThreads, 2) gsa_select_kernel(const Select
 
 // ---- rows in registers --------------------------------------------------------------------------------------------
 // One CTA of NT threads per row of up to 32 * NT scores, a score's order key in one register (thread t holds scores
-// 4 NT v + 4 t .. + 3), so that nothing of the row is kept in shared memory and four (NT = 256) or two (512) rows share an
-// SM.  One histogram round of the exact key range narrows the threshold to one bin, whose few keys are ranked directly;
+// 4 NT v + 4 t .. + 3), so that nothing of the row is kept in shared memory and eight (NT = 128), four (256) or two (512)
+// rows share an SM (64 registers a thread; 8 to 60 bytes of it are spilled).  One histogram round of the exact key range narrows the threshold to one bin, whose few keys are ranked directly;
 // the selected positions are marked in a bitmap, one scan of its words orders them, and the row is written in whole lines.
 // Bound: the chain of barriers and reductions of a row (about eight, against eighteen of the kernel above), hidden by the
-// other rows of the SM.  Measured on the rows of an 8K prefill (1 .. 8192 scores): 0.130 ms against 0.296 ms in the kernel above.
+// other rows of the SM.  Measured on the rows of an 8K prefill (1 .. 8192 scores): 0.108 ms against 0.296 ms in the kernel above.
 //
 // CS > 1: a cluster of CS CTAs shares a row of up to 32 * NT * CS scores, a contiguous slice each, for calls with so few rows
 // that one CTA per row would leave most of the GPU idle (a decode step).  Moments, histogram, candidates and counts meet

@@ -29,7 +29,7 @@ TILES = CONFIGS["tiny"].with_(name="tiles", B=2, Lq=900, Lk=1300, n_h=16, n_kv=8
 
 
 @pytest.mark.parametrize("cfg,prepass,launches", [
-    (TILES, True, 4),                                                                              # gate, masks, tiles, plain path
+    (TILES, True, 4),                                                                              # gate, masks, tiles, gather
     (TILES.with_(name="gather", Lq=700, Lk=4000, k_base=40, k_max=80), True, 3),                  # gate, gather, finalize
     (TILES.with_(name="fused", Lq=700, Lk=4000, k_base=40, k_max=80), False, 2),
     (TILES.with_(name="parts", B=3, Lq=2, Lk=3000), False, 2),                                     # decode: sets in segments
@@ -390,3 +390,60 @@ def test_more_than_65535_batch_elements():
     assert rel(out[at, :, 0], want.detach()) < 1e-2 and rel(pbar[at], P.detach()) < 2e-3
     for n in got:
         assert rel(got[n][at, :, 0], y[n].grad) < 1e-2, n
+
+
+# ---- rows of one call on both ----------------------------------------------------------------------------------------
+BOTH = CONFIGS["tiny"].with_(name="both", B=2, Lq=8000, Lk=8000, n_h=8, n_kv=8, d_h=64, HI=4, dI=32, k_base=64, k_min=16, k_max=128, seed=270,
+                             v_bar=2.0e-3)
+
+
+@pytest.mark.parametrize("cfg,rows", [
+    (BOTH, (2048, 6000)),                                                               # tiles, then the gather
+    (BOTH.with_(name="gather", B=2, Lq=3000, Lk=3000, n_h=4, n_kv=1, k_max=96, seed=271), (0, 0)),   # the gather alone
+], ids=lambda v: getattr(v, "name", None))
+def test_forward_over_key_ranges_device_and_host_paths(cfg, rows):
+    """Key ranges of 1024 and 2048 keys: attention launches with carried softmax state whose rows are finalised range by range,
+    behind tiles or alone; the host-buffer call streams finished blocks of rows back early."""
+    x = make_inputs(cfg)
+    d = U.to_dev(x)
+    gsa.gsa_debug_set_attn_range_keys(2048 if rows[1] else 1024)
+    try:
+        p = gsa.make_params(cfg)
+        tile_rows = gsa.gsa_attn_tile_rows(p)[0]
+        assert rows[0] <= tile_rows <= rows[1]
+        out, idx, kt, var = U.run_forward(cfg, d)
+        pin = {k: v.pin_memory() for k, v in x.items()}
+        out_h = torch.empty_like(x["Q"]).pin_memory()
+        kt_h = torch.empty((cfg.B, cfg.Lq), dtype=torch.int32).pin_memory()
+        arena = torch.empty(gsa.gsa_forward_host_arena_bytes(p, 0), dtype=torch.uint8, device="cuda")
+        gsa.gsa_forward_host(p, pin["Q"], pin["K"], pin["V"], pin["qI"], pin["kI"], pin["w"], None, pin["g1"], pin["g2"], out_h, kt_h, 0, arena)
+    finally:
+        gsa.gsa_debug_set_attn_range_keys(0)
+    assert torch.equal(out_h.view(torch.int16), out.cpu().view(torch.int16))
+    assert torch.equal(kt_h, kt.cpu())
+    po = U.oracle_params(cfg)
+    for b in range(cfg.B):
+        r = np.unique(np.array([0, 5, 1023, 1024, 2047, 2048, 2999, max(0, tile_rows - 1), tile_rows, cfg.Lq - 1]))
+        o = oracle.forward(po, **x, rows_t=r, rows_b=np.full_like(r, b), want_scores=True)
+        U.check_forward_rows(po, x, o, out[b][r].float().cpu().numpy(), idx[b][r].cpu().numpy(), kt[b][r].cpu().numpy(), r,
+                             np.full_like(r, b), [cfg.Lk - cfg.Lq + int(t) + 1 for t in r])
+
+
+@pytest.mark.parametrize("bad", [False, True])
+def test_values_that_were_gated_before_the_call(bad):
+    """g2 = None: the call's own scan of V decides."""
+    cfg = TILES
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 213)
+    if bad:
+        x["V"][1, 1000, 7, 127] = float("inf")
+    d = {**U.to_dev(x), "g2": None}
+    out, n, general, status = _fwd(cfg, d, idx, kt, prepass=False)
+    assert (n, general, status) == (4, VALUES if bad else 0, 0)            # scan, masks, tiles, gather
+    hit = ((idx[1] == 1000) & (torch.arange(cfg.k_max) < kt[1, :, None])).any(-1) if bad else torch.zeros(cfg.Lq, dtype=torch.bool)
+    assert (torch.isfinite(out[1].float().cpu()).all(-1).all(-1) == ~hit).all() and bool(hit.any()) == bad
+    rows = np.arange(0, cfg.Lq, 31)
+    open_ = torch.zeros_like(x["g2"]) + 40.0                                # (the oracle gates by sigmoid(40) = 1)
+    want = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], open_, idx[0][rows].numpy(), kt[0][rows].numpy(), rows,
+                       np.zeros_like(rows))
+    U.check_out(out[0][torch.from_numpy(rows).cuda()].float().cpu().numpy(), want)

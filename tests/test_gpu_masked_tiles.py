@@ -1,5 +1,5 @@
 """Masked dense tiles of the attention stage against the oracle: sizes at the edges of the 128-key tiles and of the
-128-row tiles, every grouping of query heads, rows without keys, and inputs that the tiles must leave to the plain path."""
+128-row tiles, every grouping of query heads, rows without keys, and inputs that the tiles must leave to the gather."""
 import numpy as np
 import pytest
 import torch
@@ -35,7 +35,7 @@ def _run(cfg, d, idx, kt):
     ws = torch.empty(gsa.gsa_attn_workspace_bytes(p, True), dtype=torch.uint8, device="cuda").fill_(0xFF)
     n0 = gsa.gsa_launch_count()
     gsa.gsa_sparse_gated_attn_fwd_lse(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx.cuda(), kt.cuda(), out, lse, ws)
-    assert gsa.gsa_launch_count() - n0 == 4          # value gate, masks, tiles, plain path (the gather takes 3 here)
+    assert gsa.gsa_launch_count() - n0 == 4          # value gate, masks, tiles, gather (alone it takes 3 here)
     return out, lse, gsa.gsa_device_status(ws)
 
 
@@ -78,12 +78,13 @@ def test_masked_tiles_match_the_oracle(B, Lq, Lk, n_h, n_kv, d_h):
 @pytest.mark.parametrize("what", ["unsorted", "duplicate", "inf_value", "nan_key", "large_scores", "position_too_large", "budget_too_large"])
 def test_inputs_that_a_mask_cannot_stand_for(what):
     """Sets out of order or with an entry twice, and values that are not finite, give what walking the sets gives: a
-    value that is not finite reaches exactly the rows that select it.  Corrupt sets are reported, not followed."""
+    value that is not finite reaches exactly the rows that select it.  Corrupt sets are reported, not followed.  (A NaN in a
+    key and large scores stay on the tiles; test_gpu_masked_routes.py looks at which path each cause takes.)"""
     cfg = CONFIGS["tiny"].with_(name="general", B=2, Lq=900, Lk=1300, n_h=16, n_kv=8, d_h=128, k_base=300, k_min=1, k_max=419, seed=210)
     x = make_inputs(cfg)
     idx, kt = _sets(cfg, 211)
     kt[1, 500] = 7
-    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, 900, 1000], dtype=torch.int32)
+    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, 800, 900], dtype=torch.int32)        # (the row sees 901 keys)
     idx[1, 500, 7:] = -1
     hit = torch.zeros(cfg.B, cfg.Lq, dtype=torch.bool)
     status_want = 0
@@ -135,7 +136,7 @@ def test_numerators_of_flat_rows_are_rounded_below_one():
     ws = torch.empty(gsa.gsa_attn_workspace_bytes(p, False), dtype=torch.uint8, device="cuda")
     n0 = gsa.gsa_launch_count()
     gsa.gsa_sparse_gated_attn_fwd(p, d["Q"], d["K"], d["V"], d["g1"], None, idx.cuda(), kt.cuda(), out, ws)
-    assert gsa.gsa_launch_count() - n0 == 4 and gsa.gsa_device_status(ws) == 0          # scan of the values, masks, tiles, plain path
+    assert gsa.gsa_launch_count() - n0 == 4 and gsa.gsa_device_status(ws) == 0          # scan of the values, masks, tiles, gather
     assert ws.view(torch.int32)[2] == 0                                                 # (the tiles did the work)
     err = []
     for t in range(0, cfg.Lq, 4):
@@ -167,7 +168,7 @@ def _run_bwd(cfg, d, idx, kt, q0, q1, saved_lse, withhold=False):
                                       got["dg1"], got["dg2"], ws, pbar=got["pbar"], lse=lse if saved_lse else None)
     finally:
         gsa.gsa_debug_set_wait_limit(0, withhold_first_copy=False)
-    # gate, preparation, two scans, masks, keys, rows, target, three of the plain path (and the statistics' two)
+    # gate, preparation, masks, keys, rows, target, five of the gather, which return at once (and the statistics' two)
     assert gsa.gsa_launch_count() - n0 == (11 if saved_lse else 13)
     return got, gsa.gsa_device_status(ws)
 
@@ -200,7 +201,7 @@ def test_masked_backward_leaves_other_inputs_to_the_plain_path(what):
     x = make_inputs(cfg)
     idx, kt = _sets(cfg, 241)
     kt[1, 500] = 7
-    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, 700, 800], dtype=torch.int32)
+    idx[1, 500, :7] = torch.tensor([3, 9, 10, 400, 401, 500, 600], dtype=torch.int32)        # (the row sees 601 keys)
     idx[1, 500, 7:] = -1
     dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(242)) * 0.25).to(torch.bfloat16)
     if what == "unsorted":

@@ -213,7 +213,7 @@ def test_topk_l8k_rows_cached_and_global_paths(l8k):
 
 
 def test_topk_long_rows_take_the_uncached_path():
-    """Rows longer than the shared-memory cache (n > ~46K) are re-read from global memory."""
+    """Eight rows of 70000 scores: a cluster each."""
     cfg = CONFIGS["l8k"].with_(name="long", B=1, Lq=8, Lk=70000, seed=12)
     x = make_inputs(cfg)
     d = U.to_dev(x)
@@ -222,9 +222,9 @@ def test_topk_long_rows_take_the_uncached_path():
 
 
 def test_topk_long_rows_that_defeat_the_sample():
-    """Long rows on which the sampled candidate threshold is useless: a handful of score levels (huge
+    """Long rows on which a sampled candidate threshold would be useless: a handful of score levels (huge
     ties), scores increasing with position (every top score sits at the end of the row), a constant row.
-    The kernel must notice (list overflow / too few candidates) and still return the exact set."""
+    Six rows go to the clusters; test_gpu_select_rows.py has the same patterns on the candidate list."""
     cfg = CONFIGS["l8k"].with_(name="degenerate", B=1, Lq=6, Lk=20011, k_base=700, k_min=100, k_max=3000)
     st = U.row_stride(cfg)
     g = torch.Generator().manual_seed(7)
@@ -240,9 +240,9 @@ def test_topk_long_rows_that_defeat_the_sample():
 
 
 def test_topk_long_rows_with_a_tie_cut_and_rows_beyond_the_bitmap():
-    """The two cases in which a long row's set is written by walking the candidate table instead of through
-    the position bitmap: the budget cuts a group of equal scores (scores quantised to 4096 levels: a few equal
-    scores per level, the candidate list does not overflow), and a row of more than 131072 visible scores."""
+    """A budget that cuts a group of equal scores (scores quantised to 4096 levels; five rows: the clusters, the
+    candidate table is walked in test_gpu_select_rows.py), and rows of more than 131072 visible scores, whose
+    sets the list kernel writes by walking the candidate table instead of through the position bitmap."""
     cfg = CONFIGS["l8k"].with_(name="tiecut", B=1, Lq=5, Lk=30011, k_base=900, k_min=100, k_max=3000)
     st = U.row_stride(cfg)
     g = torch.Generator().manual_seed(10)
@@ -257,8 +257,8 @@ def test_topk_long_rows_with_a_tie_cut_and_rows_beyond_the_bitmap():
 
 
 def test_topk_row_lengths_around_the_chunk_and_list_boundaries():
-    """Visible lengths n just below / at / above the short-row limit (8192) and multiples of the 512-score
-    chunk, and rows whose last chunk holds a single score."""
+    """Visible lengths n just below / at / above 8192 (the register kernels of 256 and 512 threads) and multiples
+    of 512; test_gpu_select_rows.py has the lengths above 16384 that the candidate list serves."""
     cfg = CONFIGS["l8k"].with_(name="edges", B=1, Lq=1540, Lk=9730, k_base=900, k_min=64, k_max=2048)
     st = U.row_stride(cfg)
     g = torch.Generator().manual_seed(8)
@@ -523,8 +523,8 @@ def test_forward_host_buffers_match_device_call(tiny):
 
 
 def test_forward_many_key_ranges_device_and_host_paths():
-    """Key ranges of 1024 keys on a 3000-token sequence: three attention launches with carried softmax
-    state, rows finalised range by range; the host-buffer call streams finished rows back early."""
+    """Key ranges of 1024 keys on a 3000-token sequence, whose rows the cost models send to the masked tiles (the gather
+    over several ranges, and both in one call: test_gpu_masked_routes.py); the host-buffer call against the device call."""
     cfg = CONFIGS["tiny"].with_(name="ranges", B=2, Lq=3000, Lk=3000, k_base=300, k_min=64, k_max=600, seed=17,
                                v_bar=2.0e-3)
     x = make_inputs(cfg)

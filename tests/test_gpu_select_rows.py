@@ -1,9 +1,11 @@
-"""Selection on rows held in registers: lengths at the edges of the one-CTA kernels (8192 and 16384 scores) and of the
-clusters' slices, ties cut inside and between slices, and budgets that take everything."""
+"""Selection kernel by kernel.  Rows held in registers: lengths at the edges of the one-CTA kernels (4096, 8192 and 16384 scores) and
+of the clusters' slices, ties cut inside and between slices, budgets that take everything, NaN and infinite scores.  The candidate
+list: many rows of more than 16384 scores."""
 import numpy as np
 import pytest
 import torch
 
+from paper_2601_15305_b200 import binding as gsa
 from paper_2601_15305_b200.inputs import CONFIGS
 
 import gpu_util as U
@@ -76,3 +78,52 @@ def test_rows_with_nan_or_infinite_scores(Lk, Lq, k_max, kind):
             x = sc[0, t, :n].double().numpy()
             want = np.sort(np.lexsort((np.arange(n), -np.where(np.isnan(x), np.inf, x), ~np.isnan(x)))[:k])
             assert (got[:k].numpy() == want).all()
+
+
+# ---- the candidate-list kernel: rows of more than 16384 scores, 38 of them at least (fewer go to the clusters on 148 SMs) ----
+def _list_rows(cfg, sc, rows, k_mode, v_bar):
+    """Compares the listed rows and returns how many of all rows took the whole-row fallback."""
+    _select_and_compare(cfg, sc, rows=rows, k_mode=k_mode, v_bar=v_bar)
+    p = gsa.make_params(cfg, k_mode=k_mode, v_bar=v_bar)
+    idx = torch.empty((1, cfg.Lq, cfg.k_max), device="cuda", dtype=torch.int32)
+    kt = torch.empty((1, cfg.Lq), device="cuda", dtype=torch.int32)
+    ws = torch.zeros(1024, dtype=torch.uint8, device="cuda")
+    gsa.gsa_adaptive_topk(p, sc, sc.shape[-1], idx, kt, None, ws)
+    return gsa.gsa_select_fallback_rows(ws)
+
+
+@pytest.mark.parametrize("pattern", ["five_levels", "two_levels", "increasing", "constant", "decreasing", "late_cluster", "random"])
+def test_list_kernel_on_rows_that_mislead_the_sample(pattern):
+    """Huge ties (more candidates than the list holds: the whole-row fallback), scores in order of position, a late cluster."""
+    cfg = CONFIGS["l8k"].with_(name="list", B=1, Lq=42, Lk=20011, k_base=700, k_min=100, k_max=3000)
+    st, g = U.row_stride(cfg), torch.Generator().manual_seed(7)
+    at = torch.arange(st).float()
+    row = {"five_levels": lambda: torch.randint(0, 5, (st,), generator=g).float() * 0.25 + 1.0,
+           "two_levels": lambda: torch.randint(0, 2, (st,), generator=g).float() * 0.25 + 1.0,
+           "increasing": lambda: at * 1e-4 + 1.0, "constant": lambda: torch.full((st,), 2.5), "decreasing": lambda: at.flip(0) * 1e-4 + 1.0,
+           "late_cluster": lambda: torch.rand(st, generator=g) + (at > st - 3000) * 3.0, "random": lambda: torch.rand(st, generator=g)}[pattern]
+    sc = torch.stack([row() for _ in range(cfg.Lq)])[None].cuda()
+    for k_mode, v_bar in ((2, 1.0), (0, 0.05), (1, 0.05)):
+        fallback = _list_rows(cfg, sc, np.arange(0, cfg.Lq, 6), k_mode, v_bar)
+        if pattern in ("two_levels", "constant"):
+            assert fallback == cfg.Lq
+        if pattern == "random":
+            assert fallback == 0
+
+
+def test_list_kernel_with_a_cut_tie():
+    """The set is written by walking the candidate table instead of through the position bitmap."""
+    cfg = CONFIGS["l8k"].with_(name="list_cut", B=1, Lq=40, Lk=30011, k_base=900, k_min=100, k_max=3000)
+    sc = torch.floor(torch.rand((1, cfg.Lq, U.row_stride(cfg)), generator=torch.Generator().manual_seed(10)) * 4096.0) / 4096.0
+    for k_mode, v_bar in ((2, 1.0), (0, 0.08)):
+        assert _list_rows(cfg, sc.cuda(), np.arange(0, cfg.Lq, 7), k_mode, v_bar) == 0
+
+
+def test_list_kernel_around_the_chunk_boundaries():
+    """Lengths just above 16384 and just below, at and above multiples of the 512-score chunk."""
+    cfg = CONFIGS["l8k"].with_(name="list_edges", B=1, Lq=1540, Lk=16384 + 1540, k_base=900, k_min=64, k_max=2048)
+    sc = (torch.rand((1, cfg.Lq, U.row_stride(cfg)), generator=torch.Generator().manual_seed(8)) ** 4).cuda()
+    # row t sees 16385 + t scores: 16385, 16386 and 16895, 16896 = 33 * 512, 16897, 17408 and one past, 17920, 17921, 17924
+    rows = np.array([0, 1, 510, 511, 512, 1022, 1023, 1024, 1535, 1536, 1539])
+    for k_mode, v_bar in ((0, 0.07), (2, 1.0)):
+        _list_rows(cfg, sc, rows, k_mode, v_bar)
