@@ -357,12 +357,13 @@ int gsa_select_fallback_rows(const void *ws, void *stream, int32_t *rows_out);
 
 /*
  * A diagnostic (host call): which way the attention stage goes on the current device for rows [q_begin, q_end).
- * The library chooses by the geometry, the budget rule's parameters and the number of SMs, not by the data.
+ * The library chooses by the geometry, the budget rule's parameters and the number of SMs; the device then leaves tiles
+ * to the gather where the sets turn out to hold so few pairs that it is cheaper.
  *   *fwd_rows   the first *fwd_rows of these rows (of every batch element) run as masked dense tiles on the tensor
  *               cores, the others on the gather.  (None run as tiles in a call whose value gate runs inside the
  *               gather: decode, or a workspace without room for the gated values.)
  *   *bwd_tiles  1 if gsa_sparse_gated_attn_bwd runs on tiles
- * Tiles leave a call to the gather, on the device, if a set is not strictly ascending positions that its row can see, or if
+ * Tiles also leave a call to the gather if a set is not strictly ascending positions that its row can see, or if
  * a value that they read is infinite, NaN or at least 2^60 in magnitude (the forward: V'; the backward: Q, K, V', do, delta).
  */
 int gsa_attn_tile_rows(const gsa_params_t *p, int32_t *fwd_rows, int32_t *bwd_tiles);

@@ -710,14 +710,25 @@ struct ForwardCosts {
         const double longest = w.selected / ((double)nb * rows) / kTileKeys / (pl.mode == 1 ? pl.slots : 1) * 0.45;
         return (all > longest ? all : longest) + 5.0 + 2.0 * pl.n_ranges;
     }
+    // selected pairs of a chunk of rows below which the gather takes less than seven tenths of the tiles' time
+    double few_pairs(const gsa_params_t& p, const AttnPlan& pl, int nb, int q0, int rows) const {
+        const double us = 0.7 * tiles(p, nb, q0, rows, rows) - 5.0 - 2.0 * pl.n_ranges;
+        const double all = us / (p.n_kv * pair_us), longest = us / 0.45 * kTileKeys * (pl.mode == 1 ? pl.slots : 1) * nb * rows;
+        return all < longest ? all : longest;
+    }
 };
 
-int masked_rows_end(const gsa_params_t& p, const AttnPlan& pl, const RowRange& rr, size_t scratch_bytes) {
-    const int q_end = rr.q_begin + rr.R;
+ForwardCosts forward_costs(const gsa_params_t& p, const AttnPlan& pl) {
     ForwardCosts c;
     c.block = masked_block_rows(p);
     c.tile_us = p.d_h == 128 ? 2.1 : 1.9;
     c.pair_us = (p.d_h == 128 ? 36e-6 : 24e-6) * (pl.n_ranges > 1 ? 41.0 / 36.0 : 1.0);
+    return c;
+}
+
+int masked_rows_end(const gsa_params_t& p, const AttnPlan& pl, const RowRange& rr, size_t scratch_bytes) {
+    const int q_end = rr.q_begin + rr.R;
+    const ForwardCosts c = forward_costs(p, pl);
     const int64_t per = (int64_t)(scratch_bytes / (mask_plan(p, 0, kMaskRowAlign).bytes(p.B) / kMaskRowAlign)) / c.block * c.block;
     if (per < c.block) return rr.q_begin;                          // (no room for the masks of one block of rows)
     // the row that sees so many keys that its share of a block's tiles costs what gathering its set does
@@ -795,10 +806,12 @@ cudaError_t launch_masked_rows(const gsa_params_t& p, const AttnPlan& pl, const 
     int64_t per = (int64_t)(scratch_bytes / row_bytes) / block * block;
     if (per < block) return cudaErrorInvalidValue;
     int32_t* const general = t_dev_status + kStatusGeneralWord;
+    const ForwardCosts costs = forward_costs(p, pl);
     for (int q = rr.q_begin; q < t_end; q += (int)per) {
         const MaskPlan mp = mask_plan(p, q, (int)(t_end - q < per ? t_end - q : per));
         cudaError_t e = all_visible ? launch_visible_masks(p, mp, (uint4*)scratch, st)
-                                    : launch_build_masks(p, mp, block, idx, kt, il, (uint4*)scratch, general, st);
+                                    : launch_build_masks(p, mp, block, idx, kt, il, (uint4*)scratch, t_dev_status,
+                                                         costs.few_pairs(p, pl, rr.nb, q, mp.rows), st);
         if (e != cudaSuccess) return e;
         e = launch_masked_attn_fwd(p, mp, (const uint4*)scratch, Q, K, Vg, g1, out, lse, t_dev_status, st);
         if (e != cudaSuccess) return e;
@@ -809,7 +822,7 @@ cudaError_t launch_masked_rows(const gsa_params_t& p, const AttnPlan& pl, const 
         e = launch_attn_direct(p, chunk, Q, K, Vg, g1, idx, kt, il, out, lse, general, ranges ? kRunGeneralSets : kRunAnyGeneral, st);
         if (e == cudaSuccess && ranges) {
             AttnArgs a = attn_args(p, pl, chunk, Q, K, Vg, nullptr, idx, kt, il, scratch, lse);
-            a.only_if = general; a.run_if = kRunValuesOnly;
+            a.only_if = general; a.run_if = kRunSetsInOrder;
             e = launch_attn_dh<false>(a, p, pl, g1, out, st, nullptr);
         }
         if (e != cudaSuccess) return e;

@@ -32,7 +32,9 @@ constexpr int kStatusFallbackWord = 1;   // int32 word: rows on which top-k sele
 constexpr int kStatusGeneralWord = 2;    // int32 word: nonzero if the call's inputs rule the masked tiles out (gsa_masked.cuh): the
                                          // sum of the bits below
 enum : int32_t { kGeneralSets = 1,       // an index set that a bit mask cannot stand for
-                 kGeneralValues = 2 };   // a value that must not be multiplied by zero
+                 kGeneralValues = 2,     // a value that must not be multiplied by zero
+                 kGeneralFew = 4 };      // the sets turned out so small that the gather is the cheaper path (of one chunk of rows)
+constexpr int kStatusPairsWord = 4;      // two words (64 bits): CTAs of the mask builder and selected pairs that they have counted
 
 // device status word values: which bounded wait of a tensor-core pipeline ran out (copy producer, MMA
 // issuer, epilogue), or that a kernel met an index set entry / budget outside its range
@@ -210,9 +212,9 @@ __device__ __forceinline__ int32_t checked_pos(int32_t s, int32_t Lk, int32_t* d
 
 // Kernels that are enqueued behind the tiles for the inputs that the tiles leave to them: do it, or return at once?  run_if has bit
 // v set for every value v of the `general` word to run at (only_if null: run in any case).  The same for every thread.
-constexpr int32_t kRunAnyGeneral = 0xE, kRunGeneralSets = 0xA, kRunValuesOnly = 0x4;
+constexpr int32_t kRunAnyGeneral = 0xFE, kRunGeneralSets = 0xAA, kRunSetsInOrder = 0x54;
 __device__ __forceinline__ bool left_out(const int32_t* only_if, int32_t run_if) {
-    return only_if && !((run_if >> (*only_if & 3)) & 1);
+    return only_if && !((run_if >> (*only_if & 7)) & 1);
 }
 
 __device__ __forceinline__ float fast_sigmoid(float x) {

@@ -35,9 +35,10 @@ inline MaskPlan mask_plan(const gsa_params_t& p, int q0, int rows) {
 
 // Builds the masks of rows mp.q0 .. of every batch element.  Row r gets the key tiles that the last row of its block
 // of `block_rows` rows (counted from mp.q0) can see.  A set that a mask cannot stand for (not strictly ascending, an
-// entry that the row cannot see, a budget out of range) raises *general.
+// entry that the row cannot see, a budget out of range) raises a bit of the `general` word; so do sets of fewer than few_pairs
+// entries in all (another bit, put down again by the next chunk's masks).
 cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int block_rows, const int32_t* idx,
-                               const int32_t* kt, IdxLayout il, uint4* mask, int32_t* general, cudaStream_t st);
+                               const int32_t* kt, IdxLayout il, uint4* mask, int32_t* dev_status, double few_pairs, cudaStream_t st);
 
 // The same for sets known to hold every visible key (k_mode 3 inside gsa_forward): no set is read.
 cudaError_t launch_visible_masks(const gsa_params_t& p, const MaskPlan& mp, uint4* mask, cudaStream_t st);

@@ -31,13 +31,15 @@ namespace {
 
 // ---- masks -----------------------------------------------------------------------------------------------
 constexpr int kMaskWindowWords = 1024;                 // 32768 keys of every row at a time
+constexpr int kPairsBits = 36;                         // (4 bytes an entry: 2^36 pairs would be 275 GB of sets)
 constexpr int kMaskRowWords = kMaskWindowWords + 4;    // (padded: the rows' pieces of a key tile fall into different banks)
 
 __global__ void __launch_bounds__(kMaskRowAlign * 32)
 gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ kt, uint4* __restrict__ mask,
                        IdxLayout il, int q0, int rows, int row_pitch, int key_tiles, int block_rows, int k_max, int off,
-                       int32_t* __restrict__ general) {
+                       int32_t* dev_status, unsigned long long few_pairs) {
     chain_wait();
+    int32_t* const general = dev_status + kStatusGeneralWord;
     __shared__ __align__(16) uint32_t s_bits[kMaskRowAlign * kMaskRowWords];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row_ctas = row_pitch / kMaskRowAlign;      // (batch elements along x: y and z end at 65535)
@@ -50,6 +52,15 @@ gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restric
     const int32_t* __restrict__ row = idx + irow * k_max;
     const bool vec = (k_max & 3) == 0;                 // rows start on 16-byte boundaries
     uint32_t* const bits = s_bits + warp * kMaskRowWords;
+    // The host chose the tiles by the budget that the sets centre on.  If they hold so few pairs that the gather is cheaper after
+    // all (a normaliser of Eq. 8 far from the scores' variance), the last CTA to count says so, for this chunk of rows: one
+    // atomic per CTA, CTAs in the upper bits and pairs in the lower, sent here and looked at behind the masks.
+    unsigned long long pairs = 0, counted = 0;
+    if (threadIdx.x == 0) {
+        for (int j = 0; j < kMaskRowAlign; ++j)
+            if (r0 + j < rows) pairs += clamp_budget(kt[il.row(b, q0 + r0 + j)], k_max);
+        counted = atomicAdd(reinterpret_cast<unsigned long long*>(dev_status + kStatusPairsWord), (1ull << kPairsBits) + pairs);
+    }
     int at = 0;                                        // entries below `at` have been placed
     bool regular = r >= rows || k == kt[irow];
     for (int w0 = 0; w0 < tiles * 4; w0 += kMaskWindowWords) {
@@ -103,6 +114,11 @@ gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restric
                 *reinterpret_cast<const uint4*>(&s_bits[rr * kMaskRowWords + tile * 4]);
         }
         __syncthreads();
+    }
+    if (threadIdx.x == 0 && (counted >> kPairsBits) == gridDim.x - 1) {
+        *reinterpret_cast<unsigned long long*>(dev_status + kStatusPairsWord) = 0ull;        // (for the next chunk's masks)
+        if ((counted & ((1ull << kPairsBits) - 1)) + pairs < few_pairs) atomicOr(general, kGeneralFew);
+        else atomicAnd(general, ~kGeneralFew);
     }
     if (at < k || !regular) atomicOr(general, kGeneralSets);              // (at < k: an entry past what the row can see, or out of order)
 }
@@ -476,10 +492,10 @@ cudaError_t launch_fwd_t(const MaskedFwdArgs& a, const gsa_params_t& p, const CU
 }  // namespace
 
 cudaError_t launch_build_masks(const gsa_params_t& p, const MaskPlan& mp, int block_rows, const int32_t* idx,
-                               const int32_t* kt, IdxLayout il, uint4* mask, int32_t* general, cudaStream_t st) {
+                               const int32_t* kt, IdxLayout il, uint4* mask, int32_t* dev_status, double few_pairs, cudaStream_t st) {
     const unsigned grid = (unsigned)(mp.row_pitch / kMaskRowAlign) * (unsigned)p.B;
     launch_chained(gsa_build_masks_kernel, grid, kMaskRowAlign * 32, 0, st, idx, kt, mask, il, mp.q0, mp.rows, mp.row_pitch, mp.key_tiles,
-                                                               block_rows, p.k_max, p.Lk - p.Lq, general);
+                                                               block_rows, p.k_max, p.Lk - p.Lq, dev_status, (unsigned long long)(few_pairs > 0.0 ? few_pairs : 0.0));
     ++g_launches;
     return cudaGetLastError();
 }

@@ -12,8 +12,9 @@
 // columns (MN-major) for the sums.
 //
 // Bound: the products and the elementwise work between them in turn.  Measured at L = 32K, 16 heads of 128 on 8 KV heads, mean
-// budget 2048: keys 6.3 ms (four products, 1.4 PFLOP/s), rows 5.3 ms (three, 1.24 PFLOP/s), target 4.9 ms (one, and all the
-// exponentials); the gather kernels took 92 ms for the same.
+// budget 2080: 17.2 ms for a call with its target, 13.3 ms without (seven products, 1.16 PFLOP/s over the visible pairs; the keys
+// kernel somewhat over 6, the rows kernel over 5), so 3.9 ms for the target (one product, and all the exponentials); 8K 1.37 and
+// 1.02 ms.  The gather kernels take 86 and 19.0 ms for a call.
 //
 // Roles in all three: warps 0-15 the elementwise work (four warpgroups side by side, 32 columns of a tile each: with two of
 // them the products waited for it), warp 16 copies, warp 17 MMA issue, 18 and 19 small loads.
@@ -850,10 +851,12 @@ size_t masked_bwd_bytes(const gsa_params_t& p, const RowRange& rr) {
 // 128 x 128 tile in the keys, rows and target kernels, one CTA per SM, 40 for the launches around them (the target is charged
 // whether it is asked for or not).  Gather: 0.115 ps per byte of the K, V', Q and do rows that a pair moves (1.41 ns at 16
 // heads of 128 on 8 KV heads, measured at L = 32K), 20 for its launches.  Fewer row tiles than half of the SMs: the gather.
-bool masked_bwd_preferred(const gsa_params_t& p, const RowRange& rr) {
+namespace {
+struct BackwardCosts { double tiles_us, pair_us, selected; };
+BackwardCosts backward_costs(const gsa_params_t& p, const RowRange& rr) {
     const int G = p.n_h / p.n_kv, block = 128 / G;
     const double ctas = (double)((rr.R + block - 1) / block) * p.n_kv * rr.nb, sms = sm_count();
-    if (2.0 * ctas < sms) return false;
+    if (2.0 * ctas < sms) return {1e30, 0.0, 0.0};
     const RowsWork w = rows_work(p, rr.nb, rr.q_begin, rr.R, block);
     const double all = w.key_tiles * p.n_kv / sms, row_tiles = (double)((rr.R + block - 1) / block);
     const double key_ctas = (double)((p.Lk + kMaskTileKeys - 1) / kMaskTileKeys) * p.n_kv * rr.nb;
@@ -861,8 +864,13 @@ bool masked_bwd_preferred(const gsa_params_t& p, const RowRange& rr) {
     const bool wide = p.d_h == 128;
     const double tiles = (all > keys_chain ? all : keys_chain) * (wide ? 1.7 : 1.3) + (all > w.chain ? all : w.chain) * (wide ? 1.45 : 1.1) +
                          all * (wide ? 1.05 : 0.9) + 40.0;
-    const double gather = w.selected * 4.0 * (p.n_kv + p.n_h) * p.d_h * 0.115e-6 + 20.0;
-    return tiles < gather;
+    return {tiles, 4.0 * (p.n_kv + p.n_h) * p.d_h * 0.115e-6, w.selected};
+}
+}  // namespace
+
+bool masked_bwd_preferred(const gsa_params_t& p, const RowRange& rr) {
+    const BackwardCosts c = backward_costs(p, rr);
+    return c.tiles_us < c.selected * c.pair_us + 20.0;
 }
 
 cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const __nv_bfloat16* Q, const __nv_bfloat16* K,
@@ -877,7 +885,10 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
     cudaError_t e = launch_bwd_prep(p, rr, g1, out, dout, Q, dOs, dg1, delta, general, st);
     const MaskPlan mp = mask_plan(p, rr.q_begin, rr.R);
     uint4* mask = (uint4*)ws;
-    if (e == cudaSuccess) e = launch_build_masks(p, mp, masked_block_rows(p), idx, kt, il, mask, general, st);
+    // sets so small that the gather, in the form that stands behind the tiles, takes less than seven tenths of their time
+    const BackwardCosts costs = backward_costs(p, rr);
+    const double few_pairs = (0.7 * costs.tiles_us - 20.0) / (1.15 * costs.pair_us);
+    if (e == cudaSuccess) e = launch_build_masks(p, mp, masked_block_rows(p), idx, kt, il, mask, dev_status, few_pairs, st);
     if (e == cudaSuccess && !lse_in) {
         // the statistics were not saved: the forward's tiles once more (their output goes where dQ is written afterwards)
         float* const stats = (float*)((char*)ws + sets_bytes(p, rr));

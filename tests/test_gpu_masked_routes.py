@@ -447,3 +447,45 @@ def test_values_that_were_gated_before_the_call(bad):
     want = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], open_, idx[0][rows].numpy(), kt[0][rows].numpy(), rows,
                        np.zeros_like(rows))
     U.check_out(out[0][torch.from_numpy(rows).cuda()].float().cpu().numpy(), want)
+
+
+FEW = 4                                          # the third bit of the word
+
+
+def _small_sets(idx, kt, k):
+    kt = kt.clamp(max=k)
+    return idx.masked_fill(torch.arange(idx.shape[-1]) >= kt[..., None], -1), kt
+
+
+@pytest.mark.parametrize("ranges", [False, True])
+def test_sets_much_smaller_than_the_budget_go_to_the_gather(ranges):
+    """k_base says tiles (a normaliser of Eq. 8 that does not fit the scores): the device sees that the gather is cheaper."""
+    cfg = TILES
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 211, empty=[(0, 3)])
+    d = U.to_dev(x)
+    assert _fwd(cfg, d, idx, kt)[2] == 0
+    idx, kt = _small_sets(idx, kt, 9)
+    if ranges:
+        gsa.gsa_debug_set_attn_range_keys(1024)
+    try:
+        assert gsa.gsa_attn_tile_rows(gsa.make_params(cfg))[0] == cfg.Lq
+        out, n, general, status = _fwd(cfg, d, idx, kt)
+        assert (n, general, status) == (9 if ranges else 4, FEW, 0)
+        assert _same(out, _fwd(cfg, d, idx, kt, prepass=False)[0])        # bit for bit the gather's result
+    finally:
+        gsa.gsa_debug_set_attn_range_keys(0)
+
+
+def test_backward_of_sets_much_smaller_than_the_budget_goes_to_the_gather():
+    from test_gpu_backward import _compare
+    cfg = BWD
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 241, empty=[(0, 3)])
+    dout = (torch.randn(x["Q"].shape, generator=torch.Generator().manual_seed(242)) * 0.25).to(torch.bfloat16)
+    d = U.to_dev({**x, "dout": dout})
+    assert _bwd(cfg, d, idx, kt)[2] == 0
+    idx, kt = _small_sets(idx, kt, 5)
+    got, n, general, status = _bwd(cfg, d, idx, kt)
+    assert (n, general, status) == (11, FEW, 0)
+    _compare(cfg, x, got, idx, kt, dout, 0, cfg.Lq)
