@@ -218,9 +218,11 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     int timed_out;
     if (!tiles_allowed(a.dev_status, &timed_out)) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // (batch element, KV head) outermost, so that the CTAs of a wave share K and V' in the L2; late (long) rows first
-    const int blk = a.row_blocks - 1 - (int)(blockIdx.x % a.row_blocks);
-    const int bh = blockIdx.x / a.row_blocks;
+    // late (long) rows of every (batch element, KV head) first, so that the short ones fill the SMs that come free at the end; the
+    // CTAs of a wave that share K and V' run abreast
+    const int n_bh = gridDim.x / a.row_blocks;
+    const int blk = a.row_blocks - 1 - (int)(blockIdx.x / n_bh);
+    const int bh = blockIdx.x % n_bh;
     const int g = bh % a.n_kv, b = bh / a.n_kv;
     const int r0 = blk * 2 * QT;                                   // first query row of the CTA (from q0)
     const int off = a.Lk - a.Lq;

@@ -175,12 +175,12 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     const uint32_t bar_kv = bar0 + 8u * (5 * ST), bar_s = bar_kv + 8, bar_dp = bar_kv + 16, bar_p = bar_kv + 24,
                    bar_ds = bar_kv + 32, bar_done = bar_kv + 40, bar_drain = bar_kv + 48;
 
-    // early key tiles (the longest) first; (batch element, KV head) outermost.  SPLIT = 2: a cluster of two CTAs shares a tile's
+    // early key tiles (the longest) of every (batch element, KV head) first.  SPLIT = 2: a cluster of two CTAs shares a tile's
     // rows, every other row tile each, for calls whose key tiles leave half of the SMs without work; the second CTA's
     // sums go to the first through distributed shared memory at the end.
     const int part_of = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) : 0;
     const int item = (int)(blockIdx.x / SPLIT);
-    const int tile = item % a.key_tiles, bh = item / a.key_tiles;
+    const int n_bh = (int)(gridDim.x / SPLIT) / a.key_tiles, tile = item / n_bh, bh = item % n_bh;
     const int g = bh % a.n_kv, b = bh / a.n_kv;
     const int off = a.Lk - a.Lq;
     const int r_first = max(0, tile * kMaskTileKeys - off - a.q0);           // first row that sees a key of the tile
@@ -470,7 +470,8 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                    bar_ds = bar_qd + 40, bar_done = bar_qd + 48, bar_drain = bar_qd + 56;
     auto bar_s = [&](int i) { return bar_s0 + 8u * (i & 1); };     // (both buffers may be outstanding)
 
-    const int blk = a.row_blocks - 1 - (int)(blockIdx.x % a.row_blocks), bh = blockIdx.x / a.row_blocks;
+    // late (long) rows of every (batch element, KV head) first
+    const int n_bh = gridDim.x / a.row_blocks, blk = a.row_blocks - 1 - (int)(blockIdx.x / n_bh), bh = blockIdx.x % n_bh;
     const int g = bh % a.n_kv, b = bh / a.n_kv;
     const int r0 = blk * QT, off = a.Lk - a.Lq;
     const int n = min((off + a.q0 + min(r0 + QT, a.rows) + kMaskTileKeys - 1) / kMaskTileKeys, a.key_tiles);
