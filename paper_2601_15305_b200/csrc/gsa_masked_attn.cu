@@ -157,6 +157,9 @@ constexpr int kFwdThreads = 384;
 // its output exact (with 1/16, 2 % more error in dQ and dK, whose dominating terms cancel).  Over spreads of the scores from
 // 0.003 to 3 the finest of 0, 0.02, 0.05, 1/16, 0.1, 0.2 and 0.4 on the whole.
 constexpr float kRefMargin = 0.063362061f;
+// Above this sum of 64 numerators the largest exceeds 2^8: the reference is taken anew.  (The sum is at hand; a maximum of its own
+// costs an instruction a score.  Below it a numerator is at most 2^14, far from any limit of fp32 or bf16.)
+constexpr float kRefSum = 64.f * 256.f;
 
 template <int DH>
 struct FwdSmem {
@@ -166,7 +169,7 @@ struct FwdSmem {
     static constexpr int SLOTS = DH == 128 ? 5 : 8;                // K / V' tiles in flight
     static constexpr int OFF_RING = 2 * TILE_BYTES;
     static constexpr int OFF_BAR = OFF_RING + SLOTS * TILE_BYTES;
-    static constexpr int N_BARS = 2 * SLOTS + 2 + 2 + 4 + 2 + 2 + 1;   // ring full / empty, Q, S, P (halves), O, half, drain
+    static constexpr int N_BARS = 2 * SLOTS + 2 + 4 + 4 + 2 + 1;       // ring full / empty, Q, S (halves), P (halves), g1, drain
     static constexpr int OFF_TMEM = OFF_BAR + N_BARS * 8;
     static constexpr int OFF_ABORT = OFF_TMEM + 8;
     static constexpr int ALLOC = OFF_ABORT + 8 + 1024;
@@ -174,13 +177,12 @@ struct FwdSmem {
 
 struct MaskedFwdArgs {
     const uint4* mask;
-    const __nv_bfloat16* g1;
-    __nv_bfloat16* out;
     float* lse;                    // nullable
     int32_t* dev_status;
     const int32_t* general;
     int32_t q0, rows, row_pitch, key_tiles;      // MaskPlan
     int32_t Lq, Lk, n_h, n_kv, row_blocks;
+    int32_t abreast;               // tile_order
     float scale_log2;
     long long wait_cycles;
     int32_t withhold_first;        // fault injection: the first copy into the ring is left out (its barrier is never completed)
@@ -189,13 +191,15 @@ struct MaskedFwdArgs {
 template <int DH, int G>
 __global__ void __launch_bounds__(kFwdThreads, 1)
 gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                           const __grid_constant__ CUtensorMap tm_v, const MaskedFwdArgs a) {
+                           const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_g,
+                           const __grid_constant__ CUtensorMap tm_o, const MaskedFwdArgs a) {
     chain_wait();
     using P = FwdSmem<DH>;
     constexpr int QT = 128 / G;                                    // queries per M tile
     constexpr int CH = P::CHUNKS;
     constexpr uint32_t kTmS = 0, kTmO = 256;                       // TMEM columns: S / P at kTmS + 128 s, O at kTmO + 128 s
-    constexpr uint32_t kIdescS = make_idesc_bf16(128, kMaskTileKeys);
+    constexpr int HALF = kMaskTileKeys / 2;
+    constexpr uint32_t kIdescS = make_idesc_bf16(128, HALF);
     constexpr uint32_t kIdescO = make_idesc_bf16(128, DH) | kIdescTransB;
 
     extern __shared__ unsigned char dyn_smem_raw[];
@@ -209,20 +213,18 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     auto bar_full = [&](int s) { return bar0 + 8u * s; };
     auto bar_empty = [&](int s) { return bar0 + 8u * (P::SLOTS + s); };
     auto bar_q = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + s); };
-    auto bar_s = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 2 + s); };
-    auto bar_p = [&](int s, int p) { return bar0 + 8u * (2 * P::SLOTS + 4 + 2 * s + p); };      // (one completion per tile each)
-    auto bar_o = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 8 + s); };
-    auto bar_h = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 10 + s); };
+    auto bar_s = [&](int s, int p) { return bar0 + 8u * (2 * P::SLOTS + 2 + 2 * s + p); };      // (completion i: scores of tile i, and
+                                                                                                // the product of tile i - 1's half)
+    auto bar_p = [&](int s, int p) { return bar0 + 8u * (2 * P::SLOTS + 6 + 2 * s + p); };      // (one completion per tile each)
+    auto bar_g = [&](int s) { return bar0 + 8u * (2 * P::SLOTS + 10 + s); };
     const uint32_t bar_drain = bar0 + 8u * (2 * P::SLOTS + 12);
 
     int timed_out;
     if (!tiles_allowed(a.dev_status, &timed_out)) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // late (long) rows of every (batch element, KV head) first, so that the short ones fill the SMs that come free at the end; the
-    // CTAs of a wave that share K and V' run abreast
-    const int n_bh = gridDim.x / a.row_blocks;
-    const int blk = a.row_blocks - 1 - (int)(blockIdx.x / n_bh);
-    const int bh = blockIdx.x % n_bh;
+    int rank, bh;                                                  // (late rows are the long ones)
+    tile_order(blockIdx.x, a.row_blocks, gridDim.x / a.row_blocks, a.abreast, &rank, &bh);
+    const int blk = a.row_blocks - 1 - rank;
     const int g = bh % a.n_kv, b = bh / a.n_kv;
     const int r0 = blk * 2 * QT;                                   // first query row of the CTA (from q0)
     const int off = a.Lk - a.Lq;
@@ -231,7 +233,7 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < P::SLOTS; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(bar_q(s), 1); mbar_init(bar_s(s), 1); mbar_init(bar_p(s, 0), 4); mbar_init(bar_p(s, 1), 4); mbar_init(bar_o(s), 1); mbar_init(bar_h(s), 1); }
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_q(s), 1); mbar_init(bar_g(s), 1); for (int p = 0; p < 2; ++p) { mbar_init(bar_s(s, p), 1); mbar_init(bar_p(s, p), 4); } }
         mbar_init(bar_drain, 1);
         *s_abort = timed_out;                                      // (then every wait ends at once)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -245,7 +247,7 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
-    int copies_issued = 0, q_issued = 0;                           // by the copy producer
+    int copies_issued = 0, q_issued = 0, g_issued = 0;             // by the copy producer
     int slots_released = 0;                                        // by the MMA issuer
 
     if (warp < 8) {
@@ -266,16 +268,16 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         for (int i = 0; i < ntiles; ++i) {
             const uint4 mk = mk_next;
             if (live && i + 1 < ntiles) mk_next = __ldg(mrow + (int64_t)(i + 1) * a.row_pitch);
-            if (!(ok = warp_wait(bar_s(s), i & 1, s_abort, a.wait_cycles))) break;
-            // Half a tile at a time, so that the product of the first half's numerators runs under the second half's work.
             const uint32_t mw[4] = {mk.x, mk.y, mk.z, mk.w};
+            // Half a tile at a time: while one half's numerators are made, the tensor cores take in the other's and score the same
+            // half of the next tile behind it.
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
+                if (!(ok = warp_wait(bar_s(s, p), i & 1, s_abort, a.wait_cycles))) break;
                 // The reference of the tiles before nearly always still serves, so the numerators are taken against it at
-                // once, 32 columns at a time with the next 32 on their way; only if a selected score then turns out to
-                // exceed it by more than 2^8 (a row's first tiles) is the work done again from the scores, still in registers.
+                // once, 32 columns at a time with the next 32 on their way; only if their sum shows that a selected score may exceed
+                // it by more than 2^8 (kRefSum; a row's first tiles) is the work done again from the scores, still in registers.
                 uint32_t v[2][32];
-                float mx[2];
                 uint64_t sum[2] = {0ull, 0ull};
                 const float neg0 = m_ref == -INFINITY ? 0.f : -m_ref;
                 uint64_t neg2 = pack_f32x2(neg0, neg0);
@@ -290,25 +292,27 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                         sum[j & 1] = add_f32x2(sum[j & 1], pack_f32x2(x0, x1));
                         pk[j] = pack_bf16(x0, x1);
                     }
-                    tc_st16(ts + 32 * p + 16 * c, pk);
+                    tc_st16(ts + HALF * p + 16 * c, pk);
                 };
-                tc_ld32(ts + 64 * p, v[0]);
+                tc_ld32(ts + HALF * p, v[0]);
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
                     tc_wait_ld32(v[c]);
-                    if (c == 0) tc_ld32(ts + 64 * p + 32, v[1]);
-                    mx[c] = -INFINITY;
+                    if (c == 0) tc_ld32(ts + HALF * p + 32, v[1]);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const float x = (mw[2 * p + c] >> j) & 1u ? __uint_as_float(v[c][j]) : -INFINITY;
-                        v[c][j] = __float_as_uint(x);
-                        mx[c] = fmaxf(mx[c], x);
-                    }
-                    // (the numerators of columns 32 n .. go over columns 16 n .., which have been read)
+                    for (int j = 0; j < 32; ++j)
+                        if (!((mw[2 * p + c] >> j) & 1u)) v[c][j] = 0xFF800000u;             // -inf
+                    // (the numerators of columns 32 n .. of the half go over its columns 16 n .., which have been read)
                     numerators(c);
                 }
-                const float top = fmaxf(mx[0], mx[1]) * a.scale_log2;
-                if (__any_sync(0xFFFFFFFFu, top > m_ref + 8.0f)) {
+                float a0, a1, a2, a3;
+                unpack_f32x2(sum[0], a0, a1); unpack_f32x2(sum[1], a2, a3);
+                const bool first = m_ref == -INFINITY && (mw[2 * p] | mw[2 * p + 1]) != 0u;
+                if (__any_sync(0xFFFFFFFFu, first || (a0 + a1) + (a2 + a3) > kRefSum)) {
+                    float top = -INFINITY;
+#pragma unroll
+                    for (int j = 0; j < 64; ++j) top = fmaxf(top, __uint_as_float(v[j >> 5][j & 31]));
+                    top *= a.scale_log2;
                     const float m_new = top > m_ref ? top + kRefMargin : m_ref;
                     const float alpha = m_ref == -INFINITY ? 0.f : ex2_approx(m_ref - m_new);
                     m_ref = m_new;
@@ -321,8 +325,8 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                     numerators(0);
                     numerators(1);
                     if (i > 0 || p > 0) {
-                        // every product into O so far has completed: bar_s says so for the tiles before, bar_h for this one's half
-                        if (p > 0 && !(ok = warp_wait(bar_h(s), i & 1, s_abort, a.wait_cycles))) break;
+                        // once the last product handed over has completed, so has every product into O so far
+                        if (!(ok = warp_wait(bar_s(s, p ^ 1), (i + p) & 1, s_abort, a.wait_cycles))) break;
                         uint32_t o[16];
 #pragma unroll
                         for (int c = 0; c < DH / 16; ++c) {
@@ -342,27 +346,29 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             }
             if (!ok) break;
         }
-        ok = ok && warp_wait(bar_o(s), 0, s_abort, a.wait_cycles);
+        // (the last product, and this tile's g1)
+        ok = ok && warp_wait(bar_s(s, 1), ntiles & 1, s_abort, a.wait_cycles) && warp_wait(bar_g(s), 0, s_abort, a.wait_cycles);
         if (!ok) {
             if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
         } else {
-            tc_fence_after();
             float la, lb, lc, ld;
             unpack_f32x2(l2[0], la, lb); unpack_f32x2(l2[1], lc, ld);
             const float l = (la + lb) + (lc + ld);
             const int h = g * G + m % G, t = a.q0 + r;
-            const size_t at = (((size_t)b * a.Lq + (live ? t : 0)) * a.n_h + h) * DH;
             const float inv = l != 0.f ? 1.0f / l : 0.f;           // (an empty set: a zero row; a NaN in a selected key shows)
             if (a.lse && live) a.lse[((size_t)b * a.Lq + t) * a.n_h + h] = (m_ref + log2f(l)) * 0.6931471805599453f;
+            // g1 lies where Q was, in its layout; the output goes over it and out as one box (rows past the last are clipped).
+            // Row by row from and to global memory this took 8.7 us of a CTA's time.
+            unsigned char* const row = smem + s * P::TILE_BYTES + m * 128;
 #pragma unroll
             for (int c = 0; c < DH / 32; ++c) {
                 uint32_t o[32];
                 tc_ld32(to + 32 * c, o);
                 tc_wait_ld32(o);
-                if (!live) continue;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const uint4 gv = *reinterpret_cast<const uint4*>(a.g1 + at + c * 32 + q * 8);
+                    uint4* const at = reinterpret_cast<uint4*>(row + (c >> 1) * P::CHUNK_BYTES + (((4 * (c & 1) + q) ^ (m & 7)) << 4));
+                    const uint4 gv = *at;
                     const __nv_bfloat162* gp = reinterpret_cast<const __nv_bfloat162*>(&gv);
                     uint32_t w[4];
 #pragma unroll
@@ -372,9 +378,14 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                         const float o1 = l != 0.f ? __uint_as_float(o[q * 8 + 2 * e + 1]) * inv : 0.f;
                         w[e] = pack_bf16(o0 * fast_sigmoid(gf.x), o1 * fast_sigmoid(gf.y));
                     }
-                    *reinterpret_cast<uint4*>(a.out + at + c * 32 + q * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+                    *at = make_uint4(w[0], w[1], w[2], w[3]);
                 }
             }
+        }
+        // (every thread of the tile comes here, whether its waits ended well or not)
+        if (tile_results_written(1 + s, 128, ok) && (threadIdx.x & 127) == 0 && r0 + s * QT < a.rows) {
+            for (int c = 0; c < CH; ++c) tma_store_tile(&tm_o, c * 64, g * G, r0 + s * QT, b, sbase + s * P::TILE_BYTES + c * P::CHUNK_BYTES);
+            tma_store_wait();
         }
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
@@ -398,6 +409,15 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                         tma_load_tile(sbase + P::OFF_RING + s * P::TILE_BYTES + c * P::CHUNK_BYTES, (n & 1) ? &tm_v : &tm_k,
                                       c * 64, g, (n >> 1) * kMaskTileKeys, b, bar_full(s));
                 }
+                // the output's gates take Q's place once the last scores have been made
+                const int last = 2 * (ntiles - 1);
+                ok = ok && mbar_wait(bar_empty(last % P::SLOTS), (last / P::SLOTS) & 1, s_abort, a.wait_cycles);
+                for (int s = 0; ok && s < 2; ++s) {
+                    mbar_expect_tx(bar_g(s), P::TILE_BYTES);
+                    for (int c = 0; c < CH; ++c)
+                        tma_load_tile(sbase + s * P::TILE_BYTES + c * P::CHUNK_BYTES, &tm_g, c * 64, g * G, r0 + s * QT, b, bar_g(s));
+                    g_issued = s + 1;
+                }
                 if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
             }
         } else if (warp == 9) {
@@ -407,49 +427,43 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             auto wait = [&](uint32_t bar, uint32_t parity) { return warp_wait(bar, parity, s_abort, a.wait_cycles); };
             auto wait_slot = [&](int n) { return wait(bar_full(n % P::SLOTS), (n / P::SLOTS) & 1); };      // ring entry n has landed
             auto slot_addr = [&](int n) { return sbase + P::OFF_RING + (n % P::SLOTS) * P::TILE_BYTES; };
-            auto issue_s = [&](int s, int i) {                     // S_s = Q_s K_i^T
+            auto issue_s = [&](int s, int i, int p) {              // S_s = Q_s K_i^T, half p of the keys
                 const uint64_t qd = make_kmajor_desc<128>(sbase + s * P::TILE_BYTES);
-                const uint64_t kd = make_kmajor_desc<128>(slot_addr(2 * i));
+                const uint64_t kd = make_kmajor_desc<128>(slot_addr(2 * i) + p * HALF * 128);
 #pragma unroll
                 for (int k = 0; k < DH / 16; ++k) {
                     const uint64_t step = (uint64_t)((k >> 2) * (P::CHUNK_BYTES >> 4) + 2 * (k & 3));
-                    warp_mma_ss(el, tmem + kTmS + 128 * s, qd + step, kd + step, kIdescS, k > 0);
+                    warp_mma_ss(el, tmem + kTmS + 128 * s + HALF * p, qd + step, kd + step, kIdescS, k > 0);
                 }
             };
             auto issue_o = [&](int s, int i, int p) {              // O_s += P_s V'_i, half p of the keys
                 const uint64_t vd = make_mnmajor_desc(slot_addr(2 * i + 1), P::CHUNK_BYTES);
 #pragma unroll
-                for (int k = 4 * p; k < 4 * p + 4; ++k)            // 16 keys = 2048 bytes of the V' tile, 8 columns of P
-                    warp_mma_ts(el, tmem + kTmO + 128 * s, tmem + kTmS + 128 * s + 8 * k, vd + 128 * k, kIdescO, (i | k) != 0);
+                for (int k = 0; k < 4; ++k)                        // 16 keys = 2048 bytes of the V' tile, 8 columns of P
+                    warp_mma_ts(el, tmem + kTmO + 128 * s, tmem + kTmS + 128 * s + HALF * p + 8 * k, vd + 128 * (4 * p + k), kIdescO,
+                                (i | p | k) != 0);
             };
             auto release = [&](int n) { warp_commit(el, bar_empty(n % P::SLOTS)); slots_released = n + 1; };
-            ok = wait_slot(0);
-            for (int s = 0; ok && s < 2; ++s) {
-                ok = wait(bar_q(s), 0);
-                if (ok) { issue_s(s, 0); warp_commit(el, bar_s(s)); }
-            }
+            ok = wait_slot(0) && wait(bar_q(0), 0) && wait(bar_q(1), 0);
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+                if (ok) { issue_s(h & 1, 0, h >> 1); warp_commit(el, bar_s(h & 1, h >> 1)); }
             if (ok) release(0);
             for (int i = 0; ok && i < ntiles; ++i) {
-                ok = wait_slot(2 * i + 1);
+                const bool more = i + 1 < ntiles;
+                ok = wait_slot(2 * i + 1) && (!more || wait_slot(2 * i + 2));
+                // the halves in the order in which the two groups of softmax warps hand them over
 #pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    if (!ok || !(ok = wait(bar_p(s, 0), i & 1))) break;
-                    issue_o(s, i, 0);
-                    warp_commit(el, bar_h(s));
-                    if (!(ok = wait(bar_p(s, 1), i & 1))) break;
-                    issue_o(s, i, 1);
-                    if (i + 1 < ntiles) {
-                        if (s == 0 && !(ok = wait_slot(2 * i + 2))) break;
-                        // (in order behind the product that reads P from these columns)
-                        issue_s(s, i + 1);
-                        warp_commit(el, bar_s(s));
-                    } else {
-                        warp_commit(el, bar_o(s));
-                    }
+                for (int h = 0; h < 4; ++h) {
+                    const int s = h & 1, p = h >> 1;
+                    if (!ok || !(ok = wait(bar_p(s, p), i & 1))) break;
+                    issue_o(s, i, p);
+                    if (more) issue_s(s, i + 1, p);                // (in order behind the product that reads P from these columns)
+                    warp_commit(el, bar_s(s, p));
                 }
                 if (!ok) break;
                 release(2 * i + 1);
-                if (i + 1 < ntiles) release(2 * i + 2);
+                if (more) release(2 * i + 2);
             }
             if (!ok && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
         }
@@ -461,6 +475,7 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
         // give-up path: let what was issued complete (each poll is bounded) before shared memory and TMEM are released
         if (warp == 8 && lane == 0) {
             for (int s = 0; s < q_issued; ++s) mbar_drain(bar_q(s), 0);
+            for (int s = 0; s < g_issued; ++s) mbar_drain(bar_g(s), 0);
             for (int n = max(a.withhold_first, copies_issued - P::SLOTS); n < copies_issued; ++n)
                 mbar_drain(bar_full(n % P::SLOTS), (n / P::SLOTS) & 1);
         }
@@ -481,12 +496,12 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
 
 template <int DH, int G>
 cudaError_t launch_fwd_t(const MaskedFwdArgs& a, const gsa_params_t& p, const CUtensorMap& tq, const CUtensorMap& tk,
-                         const CUtensorMap& tv, cudaStream_t st) {
+                         const CUtensorMap& tv, const CUtensorMap& tg, const CUtensorMap& to, cudaStream_t st) {
     constexpr int kSmem = FwdSmem<DH>::ALLOC;
     auto kern = gsa_masked_attn_fwd_kernel<DH, G>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
     if (e != cudaSuccess) return e;
-    launch_chained(kern, (unsigned)(a.row_blocks * p.n_kv * p.B), kFwdThreads, kSmem, st, tq, tk, tv, a);
+    launch_chained(kern, (unsigned)(a.row_blocks * p.n_kv * p.B), kFwdThreads, kSmem, st, tq, tk, tv, tg, to, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -522,20 +537,24 @@ cudaError_t launch_masked_attn_fwd(const gsa_params_t& p, const MaskPlan& mp, co
                                    const __nv_bfloat16* K, const __nv_bfloat16* Vg, const __nv_bfloat16* g1,
                                    __nv_bfloat16* out, float* lse, int32_t* dev_status, cudaStream_t st) {
     const int G = p.n_h / p.n_kv;
-    CUtensorMap tq, tk, tv;
-    if (!make_heads_tmap(&tq, Q + (size_t)mp.q0 * p.n_h * p.d_h, p.B, p.Lq, mp.rows, p.n_h, p.d_h, 128 / G, G)) return cudaErrorUnknown;
+    CUtensorMap tq, tk, tv, tg, to;
+    const size_t row0 = (size_t)mp.q0 * p.n_h * p.d_h;
+    if (!make_heads_tmap(&tq, Q + row0, p.B, p.Lq, mp.rows, p.n_h, p.d_h, 128 / G, G)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&tg, g1 + row0, p.B, p.Lq, mp.rows, p.n_h, p.d_h, 128 / G, G)) return cudaErrorUnknown;
+    if (!make_heads_tmap(&to, out + row0, p.B, p.Lq, mp.rows, p.n_h, p.d_h, 128 / G, G)) return cudaErrorUnknown;
     if (!make_heads_tmap(&tk, K, p.B, p.Lk, p.Lk, p.n_kv, p.d_h, kMaskTileKeys, 1)) return cudaErrorUnknown;
     if (!make_heads_tmap(&tv, Vg, p.B, p.Lk, p.Lk, p.n_kv, p.d_h, kMaskTileKeys, 1)) return cudaErrorUnknown;
     MaskedFwdArgs a;
-    a.mask = mask; a.g1 = g1; a.out = out; a.lse = lse; a.dev_status = dev_status; a.general = dev_status + kStatusGeneralWord;
+    a.mask = mask; a.lse = lse; a.dev_status = dev_status; a.general = dev_status + kStatusGeneralWord;
     a.q0 = mp.q0; a.rows = mp.rows; a.row_pitch = mp.row_pitch; a.key_tiles = mp.key_tiles;
     a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv;
     a.row_blocks = (mp.rows + masked_block_rows(p) - 1) / masked_block_rows(p);
+    a.abreast = pairs_abreast(p.n_kv * p.B, 4.0 * p.Lk * p.d_h);
     const float sc = p.sm_scale > 0.f ? p.sm_scale : 1.0f / sqrtf((float)p.d_h);
     a.scale_log2 = sc * 1.4426950408889634f;
     a.wait_cycles = wait_limit_cycles();
     a.withhold_first = withhold_first_copy() ? 1 : 0;
-#define GSA_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_fwd_t<DH_, G_>(a, p, tq, tk, tv, st)
+#define GSA_CASE(DH_, G_) if (p.d_h == DH_ && G == G_) return launch_fwd_t<DH_, G_>(a, p, tq, tk, tv, tg, to, st)
     GSA_CASE(128, 1); GSA_CASE(128, 2); GSA_CASE(128, 4); GSA_CASE(128, 8);
     GSA_CASE(64, 1); GSA_CASE(64, 2); GSA_CASE(64, 4); GSA_CASE(64, 8);
 #undef GSA_CASE

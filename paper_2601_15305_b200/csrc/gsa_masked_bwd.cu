@@ -56,6 +56,7 @@ struct MaskedBwdArgs {
     int32_t q0, rows, row_pitch, key_tiles;
     int32_t B, Lq, Lk, n_h, n_kv, k_max;
     int32_t row_blocks;            // of 128 / G queries
+    int32_t abreast_keys, abreast_rows;      // tile_order
     int32_t pairs_per_cta, runs;   // target kernel: runs of that many pairs of key tiles, one per CTA
     float scale, scale_log2;
     uint4* zero;                   // what the general path finds cleared (see launch_attn_bwd_keys_general)
@@ -175,12 +176,13 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     const uint32_t bar_kv = bar0 + 8u * (5 * ST), bar_s = bar_kv + 8, bar_dp = bar_kv + 16, bar_p = bar_kv + 24,
                    bar_ds = bar_kv + 32, bar_done = bar_kv + 40, bar_drain = bar_kv + 48;
 
-    // early key tiles (the longest) of every (batch element, KV head) first.  SPLIT = 2: a cluster of two CTAs shares a tile's
+    // (early key tiles are the long ones)  SPLIT = 2: a cluster of two CTAs shares a tile's
     // rows, every other row tile each, for calls whose key tiles leave half of the SMs without work; the second CTA's
     // sums go to the first through distributed shared memory at the end.
     const int part_of = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) : 0;
     const int item = (int)(blockIdx.x / SPLIT);
-    const int n_bh = (int)(gridDim.x / SPLIT) / a.key_tiles, tile = item / n_bh, bh = item % n_bh;
+    int tile, bh;
+    tile_order(item, a.key_tiles, (int)(gridDim.x / SPLIT) / a.key_tiles, a.abreast_keys, &tile, &bh);
     const int g = bh % a.n_kv, b = bh / a.n_kv;
     const int off = a.Lk - a.Lq;
     const int r_first = max(0, tile * kMaskTileKeys - off - a.q0);           // first row that sees a key of the tile
@@ -470,8 +472,9 @@ gsa_masked_bwd_rows_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                    bar_ds = bar_qd + 40, bar_done = bar_qd + 48, bar_drain = bar_qd + 56;
     auto bar_s = [&](int i) { return bar_s0 + 8u * (i & 1); };     // (both buffers may be outstanding)
 
-    // late (long) rows of every (batch element, KV head) first
-    const int n_bh = gridDim.x / a.row_blocks, blk = a.row_blocks - 1 - (int)(blockIdx.x / n_bh), bh = blockIdx.x % n_bh;
+    int rank, bh;                                                  // (late rows are the long ones)
+    tile_order(blockIdx.x, a.row_blocks, gridDim.x / a.row_blocks, a.abreast_rows, &rank, &bh);
+    const int blk = a.row_blocks - 1 - rank;
     const int g = bh % a.n_kv, b = bh / a.n_kv;
     const int r0 = blk * QT, off = a.Lk - a.Lq;
     const int n = min((off + a.q0 + min(r0 + QT, a.rows) + kMaskTileKeys - 1) / kMaskTileKeys, a.key_tiles);
@@ -905,6 +908,8 @@ cudaError_t launch_masked_bwd(const gsa_params_t& p, const RowRange& rr, const _
     a.B = p.B; a.Lq = p.Lq; a.Lk = p.Lk; a.n_h = p.n_h; a.n_kv = p.n_kv; a.k_max = p.k_max;
     const int G = p.n_h / p.n_kv;
     a.row_blocks = (mp.rows + 128 / G - 1) / (128 / G);
+    a.abreast_keys = pairs_abreast(p.n_kv * p.B, 4.0 * p.Lq * p.d_h * G);        // (Q and do of a pair's heads)
+    a.abreast_rows = pairs_abreast(p.n_kv * p.B, 4.0 * p.Lk * p.d_h);            // (K and V')
     // target kernel: runs of key pairs long enough to pay for a CTA's start, short enough for four CTAs per SM (visible pairs
     // only: half of them in a square range)
     const int64_t pairs = (int64_t)((a.key_tiles + 1) / 2) * a.row_blocks * p.B;
