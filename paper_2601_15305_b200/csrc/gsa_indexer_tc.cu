@@ -8,10 +8,11 @@
 // one key: it reads that key's 256 accumulators, sums the H^I adjacent columns of each query
 // after the sigmoid, and consecutive lanes write consecutive s of a score row (128-byte stores).
 //
-// A CTA works on one query group and a run of key tiles at or below the diagonal (tiles above
-// it are never touched).  Warp roles: warp 0 feeds shared memory by TMA (k^I tiles through a
-// ring of stages, the q^I tile once), warp 1 issues the MMAs and owns the TMEM allocation,
-// warps 2..17 are the epilogue.  Two 256-column accumulators alternate, so the MMAs of tile i+1
+// One CTA per SM, each with the same number of (query group, key tile) pairs at or below the diagonal (tiles above it are never
+// touched): the pairs are numbered group by group and a CTA takes a run of them, which crosses from one group into the next where
+// it has to.  (CTAs of up to 64 tiles of one group, late groups first, left SMs idle at the end: 8K prefill 110 us.)
+// Warp roles: warp 0 feeds shared memory by TMA (k^I tiles through a ring of stages, the q^I tile of every group of the run),
+// warp 1 issues the MMAs and owns the TMEM allocation, warps 2..17 are the epilogue.  Two 256-column accumulators alternate, so the MMAs of tile i+1
 // overlap the epilogue of tile i; the epilogue (exp2 + reciprocal per sigmoid on the
 // special-function unit) is the longer of the two, which is why it gets sixteen warps (four per
 // scheduler), each reading its 64 columns 16 at a time.
@@ -42,7 +43,8 @@ struct TcArgs {
     RowRange rr;
     int32_t Lq, Lk;
     int32_t groups_per_batch;
-    int32_t tiles_per_cta;
+    int64_t tiles_per_batch;       // (query group, key tile) pairs of a batch element, and of the call
+    int64_t tiles;
     long long wait_cycles;         // limit of every bounded wait
     int32_t withhold_q;            // fault injection: the q^I copy is left out, so its barrier is never completed
 };
@@ -52,11 +54,11 @@ struct SmemPlan {
     static constexpr int Q_BYTES = kNCols * DI * 2;
     static constexpr int K_BYTES = kTileKeys * DI * 2;
     static constexpr int OFF_Q = 0;
-    static constexpr int OFF_K = OFF_Q + Q_BYTES;
+    static constexpr int OFF_K = OFF_Q + 2 * Q_BYTES;             // (two groups' q^I tiles in turn)
     static constexpr int OFF_W = OFF_K + kStages * K_BYTES;
-    static constexpr int OFF_B = OFF_W + kNCols * 4;
+    static constexpr int OFF_B = OFF_W + kEpiWarps * kColsPerWarp * 4;
     static constexpr int OFF_BAR = OFF_B + 64;                    // 8-byte aligned
-    static constexpr int N_BARS = 2 * kStages + 1 + 4 + 1;
+    static constexpr int N_BARS = 2 * kStages + 4 + 4 + 1;
     static constexpr int OFF_TMEM = OFF_BAR + N_BARS * 8;
     static constexpr int OFF_ABORT = OFF_TMEM + 8;
     static constexpr int TOTAL = OFF_ABORT + 8;
@@ -139,6 +141,23 @@ __device__ __forceinline__ float gated_head_sum(const uint32_t* x, const float* 
     }
 }
 
+// Key tiles that the query groups of a batch element see.  A group of NQ rows has `off + its rows so far` visible keys at its last row.
+struct TileCount {
+    int32_t off, R, NQ;                    // keys in front of the first row; rows; rows of a group
+    __host__ __device__ int of(int g) const {                                // group g's tiles
+        const int rows = (g + 1) * NQ < R ? (g + 1) * NQ : R;
+        return (off + rows + kTileKeys - 1) / kTileKeys;
+    }
+    // tiles of the groups before g: the sum of ceil((off + NQ j) / 128) over j = 1 .. g (none of these is cut off at R)
+    __host__ __device__ int64_t before(int g) const {
+        if (NQ >= kTileKeys) return (int64_t)g * ((off + kTileKeys - 1) / kTileKeys) + (int64_t)(NQ / kTileKeys) * g * (g + 1) / 2;
+        // with off = 128 a + rest: ceil((rest + NQ j) / 128) = ceil((ceil(rest / NQ) + j) / r), r = 128 / NQ
+        const int a = off / kTileKeys, beta = (off % kTileKeys + NQ - 1) / NQ, r = kTileKeys / NQ;
+        auto u = [r](int64_t n) { const int64_t q = n / r; return r * q * (q + 1) / 2 + (n % r) * (q + 1); };   // sum of ceil(m / r), m <= n
+        return (int64_t)g * a + u(beta + g) - u(beta);
+    }
+};
+
 // instruction descriptor: D fp32, A = B = bf16, both K-major, M = 128, N = 256
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kNCols >> 3) << 17) |
                             ((uint32_t)(kTileKeys >> 4) << 24);
@@ -153,19 +172,28 @@ gsa_indexer_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
     constexpr int KSTEPS = DI / 16;
     constexpr int ROW_BYTES = DI * 2;
 
-    // ---- which work is mine ------------------------------------------------------------------
-    const int g = (int)gridDim.y - 1 - (int)blockIdx.y;               // heavy (late) groups first
-    const int bl = g / a.groups_per_batch;
-    const int tr0 = (g % a.groups_per_batch) * NQ;
-    const int nq = min(NQ, a.rr.R - tr0);
-    const int b = a.rr.b0 + bl;
-    const int t0 = a.rr.q_begin + tr0;
+    // ---- which work is mine: pairs first .. last - 1 ----------------------------------------------------
     const int off = a.Lk - a.Lq;
-    const int n_vis_last = off + t0 + nq;                             // visible keys of the group's last query
-    const int tiles_group = (n_vis_last + kTileKeys - 1) / kTileKeys;
-    const int tile0 = blockIdx.x * a.tiles_per_cta;
-    const int ntiles = min(a.tiles_per_cta, tiles_group - tile0);
-    if (ntiles <= 0) return;                                          // whole CTA, before any barrier
+    const TileCount count{off + a.rr.q_begin, a.rr.R, NQ};
+    const int64_t first = a.tiles * blockIdx.x / gridDim.x, last = a.tiles * (blockIdx.x + 1) / gridDim.x;
+    const int64_t in_batch = first % a.tiles_per_batch;
+    int g_first = 0;                                                  // the group of the first pair
+    for (int lo = 0, hi = a.groups_per_batch - 1; lo <= hi;) {
+        const int mid = (lo + hi) >> 1;
+        if (count.before(mid) <= in_batch) { g_first = mid; lo = mid + 1; } else hi = mid - 1;
+    }
+    // the run, group by group: f(segment, batch element, first row of the group from q_begin, its rows, first key tile, key tiles)
+    auto for_segments = [&](auto f) {
+        int64_t left = last - first;
+        int tile0 = (int)(in_batch - count.before(g_first)), g = g_first, bl = (int)(first / a.tiles_per_batch);
+        for (int seg = 0; left > 0; ++seg) {
+            const int n = (int)min((int64_t)(count.of(g) - tile0), left);
+            if (!f(seg, bl, g * NQ, min(NQ, a.rr.R - g * NQ), tile0, n)) break;
+            left -= n;
+            tile0 = 0;
+            if (++g == a.groups_per_batch) { g = 0; ++bl; }
+        }
+    };
     {   // an earlier CTA gave up: leave, all threads together (one thread reads the word)
         __shared__ int s_go;
         if (threadIdx.x == 0) s_go = *reinterpret_cast<volatile int32_t*>(a.dev_status) == kDevOk;
@@ -179,24 +207,24 @@ gsa_indexer_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
     unsigned char* smem = dyn_smem_raw + pad;
     const uint32_t sbase = raw_u32 + pad;
 
-    float* s_w = reinterpret_cast<float*>(smem + P::OFF_W);
+    float* s_w0 = reinterpret_cast<float*>(smem + P::OFF_W);
     float* s_b = reinterpret_cast<float*>(smem + P::OFF_B);
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + P::OFF_TMEM);
     volatile int* s_abort = reinterpret_cast<volatile int*>(smem + P::OFF_ABORT);
     const uint32_t bar0 = sbase + P::OFF_BAR;
     auto bar_full = [&](int s) { return bar0 + 8u * s; };
     auto bar_empty = [&](int s) { return bar0 + 8u * (kStages + s); };
-    const uint32_t bar_q = bar0 + 8u * (2 * kStages);
-    auto bar_tfull = [&](int i) { return bar0 + 8u * (2 * kStages + 1 + i); };
-    auto bar_tempty = [&](int i) { return bar0 + 8u * (2 * kStages + 3 + i); };
-    const uint32_t bar_drain = bar0 + 8u * (2 * kStages + 5);         // give-up path only
+    auto bar_q = [&](int i) { return bar0 + 8u * (2 * kStages + i); };
+    auto bar_qempty = [&](int i) { return bar0 + 8u * (2 * kStages + 2 + i); };
+    auto bar_tfull = [&](int i) { return bar0 + 8u * (2 * kStages + 4 + i); };
+    auto bar_tempty = [&](int i) { return bar0 + 8u * (2 * kStages + 6 + i); };
+    const uint32_t bar_drain = bar0 + 8u * (2 * kStages + 8);         // give-up path only
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-        mbar_init(bar_q, 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(bar_tfull(i), 1); mbar_init(bar_tempty(i), kEpiWarps); }
+        for (int i = 0; i < 2; ++i) { mbar_init(bar_q(i), 1); mbar_init(bar_qempty(i), 1); mbar_init(bar_tfull(i), 1); mbar_init(bar_tempty(i), kEpiWarps); }
         mbar_init(bar_drain, 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -207,59 +235,61 @@ gsa_indexer_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (warp >= 2) {
-        const int e = threadIdx.x - 64;                               // 0..255 = (query, head) column
-        if (e < kNCols) {
-            const int qi = e / HI, j = e % HI;
-            // (sigmoid path with eight heads: weights pre-scaled by the power of two the head sum leaves over)
-            s_w[e] = qi < nq ? a.w[((size_t)b * a.Lq + t0 + qi) * HI + j] * (RELU ? 1.0f : kWeightScale<HI>) : 0.f;
-            if (e < 8) s_b[e] = (a.bI && e < HI) ? a.bI[e] : 0.f;
-        }
-    }
+    if (threadIdx.x < 8) s_b[threadIdx.x] = (a.bI && threadIdx.x < HI) ? a.bI[threadIdx.x] : 0.f;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *s_tmem;
     // what this thread has put in flight (the copy producer's and the MMA issuer's own counts)
-    int copies_issued = 0, mma_tiles_issued = 0;
-    bool q_issued = false;
+    int copies_issued = 0, mma_tiles_issued = 0, q_issued = 0, q_released = 0;
 
     if (warp == 0) {
         // ================= TMA producer =======================================================
         if (lane == 0) {
-            if (!a.withhold_q) {
-                mbar_expect_tx(bar_q, P::Q_BYTES);
-                tma_load_2d(sbase + P::OFF_Q, &tm_q, 0, (b * a.Lq + t0) * HI, bar_q);
-                q_issued = true;
-            }
-            for (int i = 0; i < ntiles && !*s_abort; ++i) {
-                const int s = i % kStages;
-                if (!mbar_wait(bar_empty(s), ((i / kStages) & 1) ^ 1, s_abort, a.wait_cycles)) break;
-                mbar_expect_tx(bar_full(s), P::K_BYTES);
-                tma_load_2d(sbase + P::OFF_K + s * P::K_BYTES, &tm_k, 0, b * a.Lk + (tile0 + i) * kTileKeys,
-                            bar_full(s));
-                copies_issued = i + 1;
-            }
-            if (copies_issued < ntiles) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
+            bool ok = true;
+            for_segments([&](int seg, int bl, int tr0, int, int tile0, int ntiles) {
+                const int b = a.rr.b0 + bl;
+                if (!(ok = mbar_wait(bar_qempty(seg & 1), ((seg >> 1) & 1) ^ 1, s_abort, a.wait_cycles))) return false;
+                if (!a.withhold_q) {
+                    mbar_expect_tx(bar_q(seg & 1), P::Q_BYTES);
+                    tma_load_2d(sbase + P::OFF_Q + (seg & 1) * P::Q_BYTES, &tm_q, 0, (b * a.Lq + a.rr.q_begin + tr0) * HI, bar_q(seg & 1));
+                    q_issued = seg + 1;
+                }
+                for (int i = 0; i < ntiles; ++i) {
+                    const int s = copies_issued % kStages;
+                    if (!(ok = !*s_abort && mbar_wait(bar_empty(s), ((copies_issued / kStages) & 1) ^ 1, s_abort, a.wait_cycles))) return false;
+                    mbar_expect_tx(bar_full(s), P::K_BYTES);
+                    tma_load_2d(sbase + P::OFF_K + s * P::K_BYTES, &tm_k, 0, b * a.Lk + (tile0 + i) * kTileKeys, bar_full(s));
+                    ++copies_issued;
+                }
+                return true;
+            });
+            if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
         }
     } else if (warp == 1) {
         // ================= MMA issuer =========================================================
         if (lane == 0) {
-            bool ok = mbar_wait(bar_q, 0, s_abort, a.wait_cycles);
-            const uint64_t bdesc = make_kmajor_desc<ROW_BYTES>(sbase + P::OFF_Q);
-            for (int i = 0; ok && i < ntiles; ++i) {
-                const int s = i % kStages, buf = i & 1;
-                if (!mbar_wait(bar_tempty(buf), ((i >> 1) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
-                if (!mbar_wait(bar_full(s), (i / kStages) & 1, s_abort, a.wait_cycles)) { ok = false; break; }
-                tc_fence_after();
-                const uint64_t adesc = make_kmajor_desc<ROW_BYTES>(sbase + P::OFF_K + s * P::K_BYTES);
+            bool ok = true;
+            for_segments([&](int seg, int, int, int, int, int ntiles) {
+                if (!(ok = mbar_wait(bar_q(seg & 1), (seg >> 1) & 1, s_abort, a.wait_cycles))) return false;
+                const uint64_t bdesc = make_kmajor_desc<ROW_BYTES>(sbase + P::OFF_Q + (seg & 1) * P::Q_BYTES);
+                for (int i = 0; i < ntiles; ++i) {
+                    const int n = mma_tiles_issued, s = n % kStages, buf = n & 1;
+                    if (!(ok = mbar_wait(bar_tempty(buf), ((n >> 1) & 1) ^ 1, s_abort, a.wait_cycles))) return false;
+                    if (!(ok = mbar_wait(bar_full(s), (n / kStages) & 1, s_abort, a.wait_cycles))) return false;
+                    tc_fence_after();
+                    const uint64_t adesc = make_kmajor_desc<ROW_BYTES>(sbase + P::OFF_K + s * P::K_BYTES);
 #pragma unroll
-                for (int k = 0; k < KSTEPS; ++k)           // 16 K-elements = 32 bytes = 2 descriptor units
-                    tc_mma_bf16(tmem_base + buf * kNCols, adesc + 2 * k, bdesc + 2 * k, kIdesc, k > 0);
-                tc_commit(bar_empty(s));                   // stage reusable once these MMAs have read it
-                tc_commit(bar_tfull(buf));                 // accumulator ready for the epilogue
-                mma_tiles_issued = i + 1;
-            }
+                    for (int k = 0; k < KSTEPS; ++k)       // 16 K-elements = 32 bytes = 2 descriptor units
+                        tc_mma_bf16(tmem_base + buf * kNCols, adesc + 2 * k, bdesc + 2 * k, kIdesc, k > 0);
+                    tc_commit(bar_empty(s));               // stage reusable once these MMAs have read it
+                    tc_commit(bar_tfull(buf));             // accumulator ready for the epilogue
+                    mma_tiles_issued = n + 1;
+                }
+                tc_commit(bar_qempty(seg & 1));
+                q_released = seg + 1;
+                return true;
+            });
             if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutMma);
         }
     } else {
@@ -272,53 +302,67 @@ gsa_indexer_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         float bias[HI];
 #pragma unroll
         for (int j = 0; j < HI; ++j) bias[j] = RELU ? s_b[j] : fmaf(s_b[j], -1.4426950408889634f, kExpBias<HI>);
-        for (int i = 0; i < ntiles; ++i) {
-            const int buf = i & 1;
-            if (!mbar_wait(bar_tfull(buf), (i >> 1) & 1, s_abort, a.wait_cycles)) {
-                if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
-                break;
-            }
-            tc_fence_after();
-            const int s = (tile0 + i) * kTileKeys + quad * 32 + lane;
-            const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + buf * kNCols + part * kColsPerWarp;
-            // columns are read 16 at a time, the next chunk's load in flight behind the current
-            // chunk's arithmetic
-            float* const out_col = a.scores + ((int64_t)bl * a.rr.R + tr0) * a.row_stride + s;
-            auto do_chunk = [&](const uint32_t (&r)[kChunkCols], int c) {
-                const int q_first = (part * kColsPerWarp + c * kChunkCols) / HI;
-#pragma unroll
-                for (int qq = 0; qq < QPC; ++qq) {
-                    const int qi = q_first + qq;
-                    float wv[HI];
-                    if constexpr (HI >= 4) {
-#pragma unroll
-                        for (int j = 0; j < HI; j += 4) {
-                            const float4 v = *reinterpret_cast<const float4*>(s_w + qi * HI + j);
-                            wv[j] = v.x; wv[j + 1] = v.y; wv[j + 2] = v.z; wv[j + 3] = v.w;
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < HI; ++j) wv[j] = s_w[qi * HI + j];
-                    }
-                    const float acc = gated_head_sum<HI, RELU>(&r[qq * HI], wv, bias);
-                    if (qi < nq && s <= off + t0 + qi) out_col[(int64_t)qi * a.row_stride] = acc;
-                }
-            };
-            uint32_t ra[kChunkCols], rb[kChunkCols];
-            tc_ld16(taddr, ra);
-#pragma unroll
-            for (int c = 0; c < NCHUNK; c += 2) {
-                tc_wait_ld16(ra);
-                tc_ld16(taddr + (c + 1) * kChunkCols, rb);
-                do_chunk(ra, c);
-                tc_wait_ld16(rb);
-                if (c + 2 < NCHUNK) tc_ld16(taddr + (c + 2) * kChunkCols, ra);
-                do_chunk(rb, c + 1);
-            }
-            tc_fence_before();
+        // this warp's columns of the group's weights; eight heads' are scaled by the power of two that the head sum leaves over
+        float* const s_w = s_w0 + ew * kColsPerWarp;
+        int it = 0;
+        for_segments([&](int, int bl, int tr0, int nq, int tile0, int ntiles) {
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_tempty(buf));
-        }
+            for (int e = lane; e < kColsPerWarp; e += 32) {
+                const int qi = (part * kColsPerWarp + e) / HI;
+                s_w[e] = qi < nq ? a.w[((size_t)(a.rr.b0 + bl) * a.Lq + a.rr.q_begin + tr0 + qi) * HI + e % HI] * (RELU ? 1.0f : kWeightScale<HI>)
+                                 : 0.f;
+            }
+            __syncwarp();
+            for (int i = 0; i < ntiles; ++i, ++it) {
+                const int buf = it & 1;
+                if (!__all_sync(0xFFFFFFFFu, mbar_wait(bar_tfull(buf), (it >> 1) & 1, s_abort, a.wait_cycles))) {
+                    if (lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
+                    return false;
+                }
+                tc_fence_after();
+                const int s = (tile0 + i) * kTileKeys + quad * 32 + lane;
+                const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + buf * kNCols + part * kColsPerWarp;
+                // columns are read 16 at a time, the next chunk's load in flight behind the current
+                // chunk's arithmetic
+                float* const out_col = a.scores + ((int64_t)bl * a.rr.R + tr0) * a.row_stride + s;
+                auto do_chunk = [&](const uint32_t (&r)[kChunkCols], int c) {
+                    const int q_first = (part * kColsPerWarp + c * kChunkCols) / HI;
+#pragma unroll
+                    for (int qq = 0; qq < QPC; ++qq) {
+                        const int qi = q_first + qq;
+                        const float* const w = s_w + (c * QPC + qq) * HI;
+                        float wv[HI];
+                        if constexpr (HI >= 4) {
+#pragma unroll
+                            for (int j = 0; j < HI; j += 4) {
+                                const float4 v = *reinterpret_cast<const float4*>(w + j);
+                                wv[j] = v.x; wv[j + 1] = v.y; wv[j + 2] = v.z; wv[j + 3] = v.w;
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < HI; ++j) wv[j] = w[j];
+                        }
+                        const float acc = gated_head_sum<HI, RELU>(&r[qq * HI], wv, bias);
+                        if (qi < nq && s <= off + a.rr.q_begin + tr0 + qi) out_col[(int64_t)qi * a.row_stride] = acc;
+                    }
+                };
+                uint32_t ra[kChunkCols], rb[kChunkCols];
+                tc_ld16(taddr, ra);
+#pragma unroll
+                for (int c = 0; c < NCHUNK; c += 2) {
+                    tc_wait_ld16(ra);
+                    tc_ld16(taddr + (c + 1) * kChunkCols, rb);
+                    do_chunk(ra, c);
+                    tc_wait_ld16(rb);
+                    if (c + 2 < NCHUNK) tc_ld16(taddr + (c + 2) * kChunkCols, ra);
+                    do_chunk(rb, c + 1);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_tempty(buf));
+            }
+            return true;
+        });
     }
 
     tc_fence_before();
@@ -329,7 +373,7 @@ gsa_indexer_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
         // of that may outlive the CTA, whose TMEM and shared memory go to the next one.  All of it completes by
         // itself (nothing issued waits for anything that was not), so these polls end; each is bounded anyway.
         if (warp == 0 && lane == 0) {
-            if (q_issued) mbar_drain(bar_q, 0);
+            for (int i = max(0, q_issued - 2); i < q_issued; ++i) mbar_drain(bar_q(i & 1), (i >> 1) & 1);
             for (int i = max(0, copies_issued - kStages); i < copies_issued; ++i)
                 mbar_drain(bar_full(i % kStages), (i / kStages) & 1);
         }
@@ -340,6 +384,7 @@ gsa_indexer_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_con
                 mbar_drain(bar_empty(i % kStages), (i / kStages) & 1);
             for (int i = max(0, mma_tiles_issued - 2); i < mma_tiles_issued; ++i)
                 mbar_drain(bar_tfull(i & 1), (i >> 1) & 1);
+            for (int i = max(0, q_released - 2); i < q_released; ++i) mbar_drain(bar_qempty(i & 1), (i >> 1) & 1);
         }
         tc_fence_before();
         __syncthreads();
@@ -364,17 +409,12 @@ cudaError_t launch_t(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* qI
     a.w = w; a.bI = bI; a.scores = scores; a.row_stride = row_stride; a.dev_status = dev_status;
     a.rr = rr; a.Lq = p.Lq; a.Lk = p.Lk;
     a.groups_per_batch = (rr.R + NQ - 1) / NQ;
-    const int groups = rr.nb * a.groups_per_batch;
-    const int n_vis_max = p.Lk - p.Lq + rr.q_begin + rr.R;
-    const int tiles_max = (n_vis_max + kTileKeys - 1) / kTileKeys;
-    // enough CTAs to fill the GPU a few times over, but runs long enough to amortise the q^I load
-    int64_t total_tiles = (int64_t)groups * tiles_max;
-    int tpc = (int)(total_tiles / (sm_count() * 4));
-    tpc = tpc < 4 ? 4 : (tpc > 64 ? 64 : tpc);
-    a.tiles_per_cta = tpc;
+    const TileCount count{p.Lk - p.Lq + rr.q_begin, rr.R, NQ};
+    a.tiles_per_batch = count.before(a.groups_per_batch - 1) + count.of(a.groups_per_batch - 1);
+    a.tiles = a.tiles_per_batch * rr.nb;
     a.wait_cycles = wait_limit_cycles();
     a.withhold_q = withhold_first_copy() ? 1 : 0;
-    dim3 grid((tiles_max + tpc - 1) / tpc, groups);
+    const unsigned grid = (unsigned)(a.tiles < sm_count() ? a.tiles : sm_count());
 
     // one CTA per SM: the kernel allocates all 512 TMEM columns, so a second resident CTA would
     // only sit in tcgen05.alloc until the first one leaves
