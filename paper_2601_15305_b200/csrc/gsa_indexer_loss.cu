@@ -15,7 +15,7 @@
 //        dw_i = sum_j dI_j f_ij          db_i += sum_j dX_ij          dq^I^T[c, i] += k^I^T[c, key] dX[key, i]
 //        dk^I[key, c] += dX[key, i] q^I[i, c]   (m16n8k8: the indexer heads are K)
 //    dk^I is a sum over every query that selected the key: d^I fp32 additions per selected pair, done with
-//    red.global.add.v2.f32 into an fp32 array that a streaming pass rounds to bf16 (32 times fewer than the
+//    red.global.add.v4.f32 into an fp32 array that a streaming pass rounds to bf16 (32 times fewer than the
 //    attention's dK would need, which is why that one inverts the index sets instead).
 #include "gsa_common.cuh"
 
@@ -43,8 +43,8 @@ __device__ __forceinline__ void mma_bf16_1688_l(float (&d)[4], uint32_t a0, uint
         : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
         : "r"(a0), "r"(a1), "r"(b0), "f"(0.f), "f"(0.f), "f"(0.f), "f"(0.f));
 }
-__device__ __forceinline__ void red_add_v2_l(float* addr, float x, float y) {
-    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(addr), "f"(x), "f"(y) : "memory");
+__device__ __forceinline__ void red_add_v4_l(float* addr, float x, float y, float z, float w) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
 // ---- the target: mean over the heads of the attention distribution on S_t -----------------------------
@@ -215,20 +215,28 @@ struct KlArgs {
     int32_t* dev_status;          // where an out-of-range index or budget is reported (may be null)
 };
 
-template <int DI, int HI>
+// W: warps of a row.  One warp per row (four rows a CTA) leaves few rows to the latency of their tiles, one after another; four warps
+// share a row's tiles then, and their sums meet in shared memory (launch_kl_t has the rule).
+constexpr int kKlStages = 3;
+constexpr int kKlRowsPerSm = 64;                       // fewer rows an SM, or sets of so many keys: four warps a row
+constexpr int kKlLongSet = 640;
+
+template <int DI, int HI, int W>
 __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const KlArgs a) {
     chain_wait();
+    static_assert(W == 1 || W == kLossWarps, "a warp or the CTA per row");
     constexpr int ROW = (DI + 8) * 2;                  // bytes of a padded tile row (odd multiple of 16)
-    constexpr int KTILE = 16 * ROW, QTILE = 8 * ROW;
-    constexpr int WARP_SMEM = 2 * KTILE + QTILE;       // two k^I stages and the row's q^I tile
+    constexpr int KTILE = 16 * ROW, QTILE = 8 * ROW, ST = kKlStages;
+    constexpr int WARP_SMEM = ST * KTILE + 2 * QTILE;  // k^I stages, and the row's q^I tile twice
     constexpr int KS = DI / 16;
     constexpr int CPR = DI / 8;
     extern __shared__ __align__(16) unsigned char loss_smem[];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gid = lane >> 2, tig = lane & 3;
-    const int64_t item = (int64_t)blockIdx.x * kLossWarps + warp;
-    if (item >= a.rr.rows()) return;                   // (no block-wide barrier below)
+    const int part = W > 1 ? warp : 0;                 // this warp's share of the row's tiles: part, part + W, ...
+    const int64_t item = W > 1 ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * kLossWarps + warp;
+    if (item >= a.rr.rows()) return;                   // (W > 1: one row per CTA, never taken)
     const int lr = a.rr.rows() - 1 - (int)item;        // long rows first
     const int b = a.rr.b0 + lr / a.rr.R, t = a.rr.q_begin + lr % a.rr.R;
     const int64_t qrow = (int64_t)b * a.Lq + t;
@@ -239,12 +247,14 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
 
     unsigned char* const ws = loss_smem + warp * WARP_SMEM;
     const uint32_t st_s32 = (uint32_t)__cvta_generic_to_shared(ws);
-    const uint32_t q_s32 = st_s32 + 2 * KTILE;
-    // q^I of the row as a tile: rows = indexer heads (rows >= HI are zero)
+    const uint32_t q_s32 = st_s32 + ST * KTILE, qp_s32 = q_s32 + QTILE;
+    // q^I of the row as a tile: rows = indexer heads (rows >= HI are zero); and once more with the columns of every 16 in the
+    // order 0 1 4 5 8 9 12 13 | 2 3 6 7 10 11 14 15, so that two column tiles of dk^I leave four neighbours in a lane
     for (int i = lane; i < 8 * DI; i += 32) {
         const int h = i / DI, c = i % DI;
-        reinterpret_cast<__nv_bfloat16*>(ws + 2 * KTILE + h * ROW)[c] =
-            h < HI ? a.qI[(qrow * HI + h) * DI + c] : __float2bfloat16(0.f);
+        const __nv_bfloat16 x = h < HI ? a.qI[(qrow * HI + h) * DI + c] : __float2bfloat16(0.f);
+        reinterpret_cast<__nv_bfloat16*>(ws + ST * KTILE + h * ROW)[c] = x;
+        reinterpret_cast<__nv_bfloat16*>(ws + ST * KTILE + QTILE + h * ROW)[(c & ~15) | ((c & 2) << 2) | ((c & 12) >> 1) | (c & 1)] = x;
     }
     __syncwarp();
     uint32_t qb[2 * KS];                               // B operand of X^T = k^I q^I^T: (k = c, n = head)
@@ -262,7 +272,9 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
     }
 
     const __nv_bfloat16* const kbase = a.kI + (size_t)b * a.Lk * DI;
-    // positions are read a tile ahead of the copies they address: a tile then waits for one memory latency, not for two
+    // copies run two tiles ahead of the work, positions a tile ahead of the copies they address, targets a tile ahead
+    constexpr int STEP = 16 * W;
+    const int j_first = 16 * part;
     auto positions = [&](int j) -> int32_t { return j < ke ? checked_pos(S[min(j + (lane & 15), ke - 1)], a.Lk, a.dev_status) : 0; };
     auto fetch = [&](int j, int stage, int32_t pos16) {
         if (j < ke) {
@@ -276,6 +288,7 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
         }
         cp_async_commit();
     };
+    auto target = [&](int j) -> float { return j < ke ? prow[j] : 0.f; };
     // f(x) and f'(x) of the tile's (key, head) entries, and the keys' scores I (rows gid, gid + 8)
     auto tile_scores = [&](int stage, float (&f)[4], float (&fp)[4], float& I0, float& I1) {
         float x[4] = {0.f, 0.f, 0.f, 0.f};
@@ -293,7 +306,7 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
                 f[i] = fmaxf(v, 0.f);
                 fp[i] = v > 0.f ? 1.f : 0.f;
             } else {
-                f[i] = 1.0f / (1.0f + __expf(-v));
+                f[i] = fast_sigmoid(v);
                 fp[i] = f[i] * (1.0f - f[i]);
             }
         }
@@ -304,44 +317,75 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
     };
 
     // ---- sweep 1: log-sum-exp of the scores, sum pbar, sum pbar I, sum pbar log pbar ------------------
-    float m_run = -INFINITY, l_run = 0.f, s_p = 0.f, s_pi = 0.f, s_plp = 0.f;
-    int32_t pos_next = positions(16);
-    fetch(0, 0, positions(0));
-    for (int j0 = 0, stage = 0; j0 < ke; j0 += 16, stage ^= 1) {
-        fetch(j0 + 16, stage ^ 1, pos_next);
-        pos_next = positions(j0 + 32);
+    // The loss is a small difference of these: every log is taken of a value near one (p k, l / k) and I from the middle of its range, so
+    // that the terms are small, too.
+    const float fk = (float)ke;
+    float I_mid = a.act == 1 ? 0.f : 0.5f * (wv[0] + wv[1]);
+    I_mid += __shfl_xor_sync(0xFFFFFFFFu, I_mid, 1); I_mid += __shfl_xor_sync(0xFFFFFFFFu, I_mid, 2);
+    // Reference of the exponentials, one for the warp.  With sigmoid heads the scores have a bound, the sum of the positive weights:
+    // both sweeps then take the same exponentials, and what they add up to is one to the last bits (a derivative's sum over the
+    // set is a difference of these).  Otherwise it moves when a score exceeds it by 16.
+    float bound = fmaxf(wv[0], 0.f) + fmaxf(wv[1], 0.f), spread = fabsf(wv[0]) + fabsf(wv[1]);
+    bound += __shfl_xor_sync(0xFFFFFFFFu, bound, 1); bound += __shfl_xor_sync(0xFFFFFFFFu, bound, 2);
+    spread += __shfl_xor_sync(0xFFFFFFFFu, spread, 1); spread += __shfl_xor_sync(0xFFFFFFFFu, spread, 2);
+    const bool bounded = a.act != 1 && spread < 60.f;
+    float m_run = bounded ? bound * kLog2eL : -INFINITY, l_run = 0.f, s_p = 0.f, s_pi = 0.f, s_plp = 0.f;
+    int32_t pos_next = positions(j_first + 2 * STEP);
+    fetch(j_first, 0, positions(j_first));
+    fetch(j_first + STEP, 1, positions(j_first + STEP));
+    float p0 = target(j_first + gid), p1 = target(j_first + gid + 8);
+    for (int j0 = j_first, stage = 0; j0 < ke; j0 += STEP, stage = stage + 1 == ST ? 0 : stage + 1) {
+        fetch(j0 + 2 * STEP, stage == 0 ? ST - 1 : stage - 1, pos_next);
+        pos_next = positions(j0 + 3 * STEP);
+        const float n0 = target(j0 + STEP + gid), n1 = target(j0 + STEP + gid + 8);
         const bool v0 = j0 + gid < ke, v1 = j0 + gid + 8 < ke;
-        const float p0 = v0 ? prow[j0 + gid] : 0.f, p1 = v1 ? prow[j0 + gid + 8] : 0.f;
-        cp_async_wait<1>();
+        cp_async_wait<2>();
         __syncwarp();
         float f[4], fp[4], I0, I1;
         tile_scores(stage, f, fp, I0, I1);
-        const float x0 = v0 ? I0 * kLog2eL : -INFINITY, x1 = v1 ? I1 * kLog2eL : -INFINITY;
-        const float m_new = fmaxf(m_run, fmaxf(x0, x1));
-        if (m_new > -INFINITY) {
-            l_run = l_run * ex2_approx_l(m_run - m_new) + ex2_approx_l(x0 - m_new) + ex2_approx_l(x1 - m_new);
-            m_run = m_new;
+        if (!bounded) {
+            float top = fmaxf(v0 ? I0 * kLog2eL : -INFINITY, v1 ? I1 * kLog2eL : -INFINITY);
+            if (__any_sync(0xFFFFFFFFu, top > m_run + 16.f)) {
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+                const float m_new = fmaxf(m_run, top);
+                l_run *= exp2f(m_run - m_new);
+                m_run = m_new;
+            }
         }
+        l_run += (v0 ? ex2_approx_l(fmaf(I0, kLog2eL, -m_run)) : 0.f) + (v1 ? ex2_approx_l(fmaf(I1, kLog2eL, -m_run)) : 0.f);
         s_p += p0 + p1;
-        s_pi += p0 * I0 + p1 * I1;
-        s_plp += (p0 > 0.f ? p0 * __logf(p0) : 0.f) + (p1 > 0.f ? p1 * __logf(p1) : 0.f);
+        s_pi += p0 * (I0 - I_mid) + p1 * (I1 - I_mid);
+        s_plp += (p0 > 0.f ? p0 * __logf(p0 * fk) : 0.f) + (p1 > 0.f ? p1 * __logf(p1 * fk) : 0.f);
+        p0 = n0; p1 = n1;
         __syncwarp();
     }
     cp_async_wait<0>();
     // the four lanes of a key hold the same values: merge across the keys only (lane bits 2..4)
 #pragma unroll
     for (int o = 4; o < 32; o <<= 1) {
-        const float m_o = __shfl_xor_sync(0xFFFFFFFFu, m_run, o);
-        const float l_o = __shfl_xor_sync(0xFFFFFFFFu, l_run, o);
-        const float m_new = fmaxf(m_run, m_o);
-        if (m_new > -INFINITY) l_run = l_run * ex2_approx_l(m_run - m_new) + l_o * ex2_approx_l(m_o - m_new);
-        m_run = m_new;
+        l_run += __shfl_xor_sync(0xFFFFFFFFu, l_run, o);
         s_p += __shfl_xor_sync(0xFFFFFFFFu, s_p, o);
         s_pi += __shfl_xor_sync(0xFFFFFFFFu, s_pi, o);
         s_plp += __shfl_xor_sync(0xFFFFFFFFu, s_plp, o);
     }
-    const float lse2 = m_run + log2f(l_run);           // log2 of sum_j exp(I_j)
-    if (lane == 0) a.loss[irow] = ke > 0 ? s_plp - s_pi + (lse2 / kLog2eL) * s_p : 0.f;
+    if constexpr (W > 1) {
+        __shared__ float s_row[W][5];
+        if (lane == 0) { s_row[warp][0] = m_run; s_row[warp][1] = l_run; s_row[warp][2] = s_p; s_row[warp][3] = s_pi; s_row[warp][4] = s_plp; }
+        __syncthreads();
+        m_run = s_row[0][0]; l_run = s_row[0][1]; s_p = s_row[0][2]; s_pi = s_row[0][3]; s_plp = s_row[0][4];
+#pragma unroll
+        for (int u = 1; u < W; ++u) {                  // (in the same order in every warp: one value of each for the row)
+            const float m_new = fmaxf(m_run, s_row[u][0]);
+            if (m_run != s_row[u][0]) l_run = l_run * exp2f(m_run - m_new) + s_row[u][1] * exp2f(s_row[u][0] - m_new);
+            else l_run += s_row[u][1];
+            m_run = m_new;
+            s_p += s_row[u][2]; s_pi += s_row[u][3]; s_plp += s_row[u][4];
+        }
+    }
+    // softmax(I)_j = 2^(I_j log2 e - m) / l: the small exponents keep what a subtracted log-sum-exp would round away
+    const float soft = s_p / l_run;
+    if (lane == 0 && part == 0) a.loss[irow] = ke > 0 ? s_plp - s_pi + (logf(l_run / fk) + (m_run / kLog2eL - I_mid)) * s_p : 0.f;
     __syncwarp();
 
     // ---- sweep 2: derivatives ----------------------------------------------------------------------------
@@ -349,22 +393,26 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
 #pragma unroll
     for (int mt = 0; mt < KS; ++mt) dq[mt][0] = dq[mt][1] = dq[mt][2] = dq[mt][3] = 0.f;
     float dw_acc[2] = {0.f, 0.f}, db_acc[2] = {0.f, 0.f};
-    int32_t pos_cur = positions(0);
-    pos_next = positions(16);
-    fetch(0, 0, pos_cur);
-    for (int j0 = 0, stage = 0; j0 < ke; j0 += 16, stage ^= 1) {
+    int32_t pos_cur = positions(j_first), pos_1 = positions(j_first + STEP);
+    pos_next = positions(j_first + 2 * STEP);
+    fetch(j_first, 0, pos_cur);
+    fetch(j_first + STEP, 1, pos_1);
+    p0 = target(j_first + gid); p1 = target(j_first + gid + 8);
+    for (int j0 = j_first, stage = 0; j0 < ke; j0 += STEP, stage = stage + 1 == ST ? 0 : stage + 1) {
         const int32_t pos16 = pos_cur;
-        fetch(j0 + 16, stage ^ 1, pos_next);
-        pos_cur = pos_next;
-        pos_next = positions(j0 + 32);
+        fetch(j0 + 2 * STEP, stage == 0 ? ST - 1 : stage - 1, pos_next);
+        pos_cur = pos_1;
+        pos_1 = pos_next;
+        pos_next = positions(j0 + 3 * STEP);
+        const float n0 = target(j0 + STEP + gid), n1 = target(j0 + STEP + gid + 8);
         const bool v0 = j0 + gid < ke, v1 = j0 + gid + 8 < ke;
-        const float p0 = v0 ? prow[j0 + gid] : 0.f, p1 = v1 ? prow[j0 + gid + 8] : 0.f;
-        cp_async_wait<1>();
+        cp_async_wait<2>();
         __syncwarp();
         float f[4], fp[4], I0, I1;
         tile_scores(stage, f, fp, I0, I1);
-        const float dI0 = v0 ? ex2_approx_l(I0 * kLog2eL - lse2) * s_p - p0 : 0.f;
-        const float dI1 = v1 ? ex2_approx_l(I1 * kLog2eL - lse2) * s_p - p1 : 0.f;
+        const float dI0 = v0 ? fmaf(ex2_approx_l(fmaf(I0, kLog2eL, -m_run)), soft, -p0) : 0.f;
+        const float dI1 = v1 ? fmaf(ex2_approx_l(fmaf(I1, kLog2eL, -m_run)), soft, -p1) : 0.f;
+        p0 = n0; p1 = n1;
         float dx[4];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
@@ -386,23 +434,24 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
                 mma_bf16_16816(dq[mt], a0, a1, a2, a3, b0, b1);
             }
         }
-        // dk^I[key, c] += dX[key, head] q^I[head, c]
+        // dk^I[key, c] += dX[key, head] q^I[head, c], 16 bytes of a key's row at a time
         {
             const int32_t key0 = __shfl_sync(0xFFFFFFFFu, pos16, gid), key1 = __shfl_sync(0xFFFFFFFFu, pos16, gid + 8);
-            float* const dk0 = a.dkI32 + ((size_t)b * a.Lk + key0) * DI + 2 * tig;
-            float* const dk1 = a.dkI32 + ((size_t)b * a.Lk + key1) * DI + 2 * tig;
-            const uint32_t boff = q_s32 + (lane & 7) * ROW + (lane >> 3) * 16;
+            float* const dk0 = a.dkI32 + ((size_t)b * a.Lk + key0) * DI + 4 * tig;
+            float* const dk1 = a.dkI32 + ((size_t)b * a.Lk + key1) * DI + 4 * tig;
+            const uint32_t boff = qp_s32 + (lane & 7) * ROW + (lane >> 3) * 16;
 #pragma unroll
             for (int n4 = 0; n4 < DI / 32; ++n4) {
                 uint32_t bq[4];
                 ldmatrix_x4_trans(bq[0], bq[1], bq[2], bq[3], boff + n4 * 64);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float ck[4];
-                    mma_bf16_1688_l(ck, dx_lo, dx_hi, bq[i]);
+                for (int i = 0; i < 4; i += 2) {
+                    float cl[4], ch[4];
+                    mma_bf16_1688_l(cl, dx_lo, dx_hi, bq[i]);
+                    mma_bf16_1688_l(ch, dx_lo, dx_hi, bq[i + 1]);
                     const int col = (n4 * 4 + i) * 8;
-                    if (v0) red_add_v2_l(dk0 + col, ck[0], ck[1]);
-                    if (v1) red_add_v2_l(dk1 + col, ck[2], ck[3]);
+                    if (v0) red_add_v4_l(dk0 + col, cl[0], cl[1], ch[0], ch[1]);
+                    if (v1) red_add_v4_l(dk1 + col, cl[2], cl[3], ch[2], ch[3]);
                 }
             }
         }
@@ -412,12 +461,35 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
 
     // ---- per-row results ------------------------------------------------------------------------------------
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
+    for (int e = 0; e < 2; ++e)
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) {
             dw_acc[e] += __shfl_xor_sync(0xFFFFFFFFu, dw_acc[e], o);
             db_acc[e] += __shfl_xor_sync(0xFFFFFFFFu, db_acc[e], o);
         }
+    if constexpr (W > 1) {
+        static_assert((4 * KS + 4) * 32 * 4 <= ST * KTILE, "a warp's sums fit its stages");
+        float* const mine = reinterpret_cast<float*>(ws) + lane;
+        __syncwarp();
+        if (part > 0) {
+#pragma unroll
+            for (int i = 0; i < 4 * KS; ++i) mine[32 * i] = dq[i >> 2][i & 3];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) { mine[32 * (4 * KS + e)] = dw_acc[e]; mine[32 * (4 * KS + 2 + e)] = db_acc[e]; }
+        }
+        __syncthreads();
+        if (part > 0) return;
+#pragma unroll
+        for (int u = 1; u < W; ++u) {
+            const float* const other = reinterpret_cast<const float*>(loss_smem + u * WARP_SMEM) + lane;
+#pragma unroll
+            for (int i = 0; i < 4 * KS; ++i) dq[i >> 2][i & 3] += other[32 * i];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) { dw_acc[e] += other[32 * (4 * KS + e)]; db_acc[e] += other[32 * (4 * KS + 2 + e)]; }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
         const int h = 2 * tig + e;
         if (h < HI) {
             if (gid == 0) {
@@ -459,11 +531,15 @@ cudaError_t launch_probs_t(const ProbsArgs& a, cudaStream_t st) {
 }
 
 template <int DI, int HI>
-cudaError_t launch_kl_t(const KlArgs& a, cudaStream_t st) {
-    constexpr int smem = kLossWarps * (2 * 16 + 8) * (DI + 8) * 2;
-    auto kern = gsa_indexer_kl_kernel<DI, HI>;
-    const int64_t items = a.rr.rows();
-    launch_chained(kern, (unsigned)((items + kLossWarps - 1) / kLossWarps), kLossWarps * 32, smem, st, a);
+cudaError_t launch_kl_t(const KlArgs& a, int k_base, cudaStream_t st) {
+    constexpr int smem = kLossWarps * (kKlStages * 16 + 2 * 8) * (DI + 8) * 2;
+    const int64_t rows = a.rr.rows();
+    // us with four warps a row and with one: 2 x 2051 rows of 256 keys 68 and 75, 8192 of 2048 1091 and 1212, 32768 of 2048 5018 and
+    // 5153; 4 x 8192 of 400 739 and 706 (start and end of a row show)
+    if (rows < (int64_t)kKlRowsPerSm * sm_count() || k_base >= kKlLongSet)
+        launch_chained(gsa_indexer_kl_kernel<DI, HI, kLossWarps>, (unsigned)rows, kLossWarps * 32, smem, st, a);
+    else
+        launch_chained(gsa_indexer_kl_kernel<DI, HI, 1>, (unsigned)((rows + kLossWarps - 1) / kLossWarps), kLossWarps * 32, smem, st, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -503,7 +579,7 @@ cudaError_t launch_indexer_kl(const gsa_params_t& p, RowRange rr, const __nv_bfl
         a.dqI = dqI; a.dw = dw; a.dkI32 = dkI32; a.dbI = dbI; a.rr = rr; a.il = il;
         a.Lq = p.Lq; a.Lk = p.Lk; a.k_max = p.k_max; a.act = p.act;
         e = cudaErrorInvalidValue;
-#define GSA_KL_CASE(DI_, HI_) if (p.dI == DI_ && p.HI == HI_) e = launch_kl_t<DI_, HI_>(a, st)
+#define GSA_KL_CASE(DI_, HI_) if (p.dI == DI_ && p.HI == HI_) e = launch_kl_t<DI_, HI_>(a, p.k_base, st)
         GSA_KL_CASE(64, 8); GSA_KL_CASE(64, 4); GSA_KL_CASE(64, 2); GSA_KL_CASE(64, 1);
         GSA_KL_CASE(32, 8); GSA_KL_CASE(32, 4); GSA_KL_CASE(32, 2); GSA_KL_CASE(32, 1);
 #undef GSA_KL_CASE
