@@ -665,23 +665,29 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
         }
         mbar_init(bar_drain, 1);
     }
-    if (threadIdx.x >= 512) {
-        // where the CTA's run of keys starts in every query's set
-        const int q = threadIdx.x - 512, r = r0 + q;
-        if (q < QT) {
-            int lo = 0;
-            if (r < a.rows) {
-                const int64_t irow = a.il.row(b, a.q0 + r);
-                const int32_t* __restrict__ set = a.idx + irow * a.k_max;
-                int hi = clamp_budget(a.kt[irow], a.k_max);
-                const int first = pair0 * 2 * kMaskTileKeys;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (set[mid] < first) lo = mid + 1; else hi = mid;
-                }
+    // where the CTA's run of keys starts in every query's set: eight lanes a query, nine ways a step (one thread and two ways took
+    // twelve memory latencies in front of every CTA's work)
+    for (int q0 = 0; q0 < QT; q0 += kBwdThreads / 8) {
+        const int q = q0 + (int)(threadIdx.x >> 3), l8 = lane & 7, r = r0 + q, first = pair0 * 2 * kMaskTileKeys;
+        const bool in = q < QT && r < a.rows;
+        const int64_t irow = in ? a.il.row(b, a.q0 + r) : 0;
+        const int32_t* __restrict__ set = a.idx + irow * a.k_max;
+        int lo = 0, hi = in && first > 0 ? clamp_budget(a.kt[irow], a.k_max) : 0;
+        while (__any_sync(0xFFFFFFFFu, lo < hi)) {
+            const int len = hi - lo;
+            const bool narrow = len > 8;
+            const int at = narrow ? lo + len * (l8 + 1) / 9 : lo + l8;
+            const uint32_t votes = __ballot_sync(0xFFFFFFFFu, at < hi && set[at] < first);
+            const int below = __popc((votes >> (lane & 24)) & 0xFFu);          // (ascending sets: the first `below` probes)
+            if (narrow) {
+                if (below < 8) hi = lo + len * (below + 1) / 9;
+                if (below > 0) lo += len * below / 9 + 1;
+            } else {
+                lo += below;
+                hi = lo;
             }
-            s_rank[q] = lo;
         }
+        if (q < QT && l8 == 0) s_rank[q] = lo;
     }
     const uint32_t tmem = tile_start(timed_out, warp, sbase + P::OFF_TMEM, s_tmem, s_abort);
     int copies = 0, released = 0;
@@ -738,27 +744,35 @@ gsa_masked_target_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_
             }
             const int n0 = __popc(mk0.x) + __popc(mk0.y), n1 = n0 + __popc(mk0.z) + __popc(mk0.w),
                       n2 = n1 + __popc(mk1.x) + __popc(mk1.y);
-            int at = rank + (w ? (half ? n2 : n1) : (half ? n0 : 0));
+            const int at = rank + (w ? (half ? n2 : n1) : (half ? n0 : 0));
             const uint4 mk = w ? mk1 : mk0;
             const uint32_t words[2] = {half ? mk.z : mk.x, half ? mk.w : mk.y};
             rank += n2 + __popc(mk1.z) + __popc(mk1.w);
+            // at every step a lane keeps every other pair of columns and gives its neighbour the rest
+            auto halve = [&](int n, int bit) {
+                const bool odd = (lane >> bit) & 1;
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    float x0, x1;
-                    unpack_f32x2(acc[16 * c + j], x0, x1);
-#pragma unroll
-                    for (int e = 1; e < G; e <<= 1) {
-                        x0 += __shfl_xor_sync(0xFFFFFFFFu, x0, e);
-                        x1 += __shfl_xor_sync(0xFFFFFFFFu, x1, e);
+                for (int j = 0; j < 16; ++j)
+                    if (j < n) {
+                        const uint64_t keep = odd ? acc[2 * j + 1] : acc[2 * j], give = odd ? acc[2 * j] : acc[2 * j + 1];
+                        acc[j] = add_f32x2(keep, __shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)give, 1 << bit));
                     }
-                    const bool mine = (16 * c + j) % G == m % G;
-                    const int p0 = at + __popc(words[c] & ((1u << (2 * j)) - 1u)), p1 = p0 + ((words[c] >> (2 * j)) & 1u);
-                    if (mine && (words[c] >> (2 * j)) & 1u) dst[p0] = x0 * inv_heads;
-                    if (mine && (words[c] >> (2 * j + 1)) & 1u) dst[p1] = x1 * inv_heads;
-                }
-                at += __popc(words[c]);
+            };
+            if constexpr (G >= 2) halve(16, 0);
+            if constexpr (G >= 4) halve(8, 1);
+            if constexpr (G >= 8) halve(4, 2);
+            // pair j now stands for columns 2 c, 2 c + 1 with c = j G + the lane's bits
+            const int at1 = at + __popc(words[0]);
+#pragma unroll
+            for (int j = 0; j < 32 / G; ++j) {
+                const int c = j * G + m % G;                       // (j < 16 / G: in the first word)
+                const uint32_t word = words[j / (16 / G)];
+                const int bit = 2 * c & 31, p0 = (j < 16 / G ? at : at1) + __popc(word & ((1u << bit) - 1u));
+                float x0, x1;
+                unpack_f32x2(acc[j], x0, x1);
+                const uint32_t sel = word >> bit;
+                if (sel & 1u) dst[p0] = x0 * inv_heads;
+                if (sel & 2u) dst[p0 + (sel & 1u)] = x1 * inv_heads;
             }
         }
         if (!ok && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
