@@ -49,8 +49,8 @@ constexpr int kVStages = 2;                // shared-memory stages of a warp's V
                                            // measured at L = 128K: 2 stages 90.2 ms, 3 stages 94.7 ms)
 constexpr int kRangeKeysDefault = 16384;   // keys per L2 range: K + V' rows of 16K tokens = 64 MB at the 1.7B shape
 constexpr int kMaxRanges = 48;
-constexpr int kPartKeys = 128;             // decode: fewest keys worth a parallel segment
-constexpr int kMaxParts = 16;              // most segments (and state slots) per index set
+constexpr int kPartKeys = 32;              // decode: fewest keys worth a parallel segment
+constexpr int kMaxParts = 64;              // most segments (and state slots) per index set
 
 struct AttnArgs {
     const __nv_bfloat16* Q;
@@ -439,8 +439,10 @@ __global__ void __launch_bounds__(256) gsa_range_cuts_kernel(const int32_t* __re
 
 // merge the state slots of a (row, head): out = (sum_p 2^(m_p - M) O_p) / (sum_p 2^(m_p - M) l_p) * sigmoid(g1)
 // A CTA takes kFinRows consecutive query rows; thread = (KV head, d), all G heads of the group.  With a
-// single slot per row (prefill) the loads of all rows are issued before any is used.
+// single slot per row (prefill) the loads of all rows are issued before any is used.  With several (decode) a CTA takes one row
+// and KV head, thread = (one of kFinGroups shares of the slots, d): two memory latencies, whatever the number of slots.
 constexpr int kFinRows = 4;
+constexpr int kFinGroups = 4;
 
 template <int DH, int G>
 __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __restrict__ state, const int32_t* __restrict__ kt,
@@ -452,12 +454,8 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
     if (left_out(only_if, run_if)) return;
     constexpr int STATE_F = G * (DH + 2);
     const int rows = rr.rows();
-    // range mode: kFinRows rows per CTA, all (KV head, d) pairs; parts mode (few rows, several state slots to
-    // merge per row): one row and one KV head per CTA, so that a decode batch still fills the GPU
-    const int rows_per_cta = mode == 0 ? kFinRows : 1;
-    const int lr0 = blockIdx.x * rows_per_cta;
-    const int i_begin = gridDim.y > 1 ? blockIdx.y * DH : 0, i_end = gridDim.y > 1 ? i_begin + DH : n_kv * DH;
     if (mode == 0) {
+        const int lr0 = blockIdx.x * kFinRows;
         // thread = (KV head, two consecutive d): 2 G consecutive floats of the state, bf16 pairs of g1 and out
         for (int i = threadIdx.x; i < n_kv * (DH / 2); i += blockDim.x) {
             const int d = (i % (DH / 2)) * 2;
@@ -509,44 +507,51 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
         }
         return;
     }
-    for (int i = i_begin + threadIdx.x; i < i_end; i += blockDim.x) {
-        const int d = i % DH;
-        const int g = i / DH;
-        {
-            for (int q = 0; q < rows_per_cta && lr0 + q < rows; ++q) {
-                const RowId r = row_of(rr, il, lr0 + q);
-                const int k_eff = clamp_budget(kt[r.irow], k_max);
-                const int np = parts_of(k_eff, max_parts);
-                float acc[G], mx[G], den[G];
+    __shared__ float s_m[kMaxParts * G], s_l[kMaxParts * G], s_top[G], s_den[G], s_acc[kFinGroups][G][DH];
+    const int tid = threadIdx.x, d = tid % DH, grp = tid / DH, warp = tid >> 5, lane = tid & 31;
+    const RowId r = row_of(rr, il, (int)blockIdx.x);
+    const int g = blockIdx.y, k_eff = clamp_budget(kt[r.irow], k_max), np = k_eff > 0 ? parts_of(k_eff, max_parts) : 0;
+    const float* __restrict__ st = state + ((int64_t)r.irow * n_kv + g) * STATE_F;
+    const int64_t slot = idx_rows * n_kv * STATE_F;
+    for (int i = tid; i < np * G; i += kFinGroups * DH) {
+        s_m[i] = st[(i / G) * slot + G * DH + i % G];
+        s_l[i] = st[(i / G) * slot + G * DH + G + i % G];
+    }
+    __syncthreads();
+    static_assert(kFinGroups * DH / 32 >= G, "a warp per head of the group");
+    if (warp < G) {                                            // the slots' weights 2^(m_p - M)
+        float top = -INFINITY, den = 0.f;
+        for (int p = lane; p < np; p += 32) top = fmaxf(top, s_m[p * G + warp]);
 #pragma unroll
-                for (int e = 0; e < G; ++e) { acc[e] = 0.f; den[e] = 0.f; mx[e] = -INFINITY; }
-                if (k_eff > 0) {
-                    for (int p = 0; p < np; ++p) {
-                        const float* st = state + (((int64_t)p * idx_rows + r.irow) * n_kv + g) * STATE_F;
-#pragma unroll
-                        for (int e = 0; e < G; ++e) mx[e] = fmaxf(mx[e], st[G * DH + e]);
-                    }
-                    for (int p = 0; p < np; ++p) {
-                        const float* st = state + (((int64_t)p * idx_rows + r.irow) * n_kv + g) * STATE_F;
-#pragma unroll
-                        for (int e = 0; e < G; ++e) {
-                            const float m = st[G * DH + e];
-                            const float sc = m == -INFINITY ? 0.f : exp2f(m - mx[e]);
-                            acc[e] = fmaf(sc, st[d * G + e], acc[e]);
-                            den[e] = fmaf(sc, st[G * DH + G + e], den[e]);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < G; ++e) {
-                    const size_t at = (((size_t)r.b * Lq + r.t) * n_h + g * G + e) * DH + d;
-                    const float v = den[e] != 0.f ? acc[e] / den[e] * fast_sigmoid(__bfloat162float(g1[at])) : 0.f;
-                    out[at] = __float2bfloat16_rn(v);
-                    if (lse && d == 0)
-                        lse[((size_t)r.b * Lq + r.t) * n_h + g * G + e] = (mx[e] + log2f(den[e])) * 0.6931471805599453f;
-                }
-            }
+        for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+        for (int p = lane; p < np; p += 32) {
+            const float m = s_m[p * G + warp], sc = m == -INFINITY ? 0.f : exp2f(m - top);
+            den = fmaf(sc, s_l[p * G + warp], den);
+            s_m[p * G + warp] = sc;
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xFFFFFFFFu, den, o);
+        if (lane == 0) { s_top[warp] = top; s_den[warp] = den; }
+    }
+    __syncthreads();
+    float acc[G];
+#pragma unroll
+    for (int e = 0; e < G; ++e) acc[e] = 0.f;
+#pragma unroll 4
+    for (int p = grp; p < np; p += kFinGroups)
+#pragma unroll
+        for (int e = 0; e < G; ++e) acc[e] = fmaf(s_m[p * G + e], st[p * slot + d * G + e], acc[e]);
+#pragma unroll
+    for (int e = 0; e < G; ++e) s_acc[grp][e][d] = acc[e];
+    __syncthreads();
+    for (int i = tid; i < G * DH; i += kFinGroups * DH) {
+        const int e = i / DH, c = i % DH;
+        float o = 0.f;
+#pragma unroll
+        for (int u = 0; u < kFinGroups; ++u) o += s_acc[u][e][c];
+        const size_t at = (((size_t)r.b * Lq + r.t) * n_h + g * G + e) * DH + c;
+        out[at] = __float2bfloat16_rn(s_den[e] != 0.f ? o / s_den[e] * fast_sigmoid(__bfloat162float(g1[at])) : 0.f);
+        if (lse && c == 0) lse[((size_t)r.b * Lq + r.t) * n_h + g * G + e] = (s_top[e] + log2f(s_den[e])) * 0.6931471805599453f;
     }
 }
 
@@ -643,7 +648,7 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
         fr.q_begin = t_lo; fr.R = t_hi - t_lo;
         const dim3 fin_grid = pl.mode == 0 ? dim3((unsigned)((fr.rows() + kFinRows - 1) / kFinRows), 1)
                                            : dim3((unsigned)fr.rows(), (unsigned)a.n_kv);
-        launch_chained(gsa_attn_finalize_kernel<DH, G>, fin_grid, pl.mode == 0 ? fin_threads : DH, 0, st,
+        launch_chained(gsa_attn_finalize_kernel<DH, G>, fin_grid, pl.mode == 0 ? fin_threads : kFinGroups * DH, 0, st,
             a.state, a.kt, g1, out, fr, a.il, a.idx_rows, p.Lq, p.n_h, p.n_kv, p.k_max, pl.mode, pl.slots, a.lse,
             a.only_if, a.run_if);
         ++g_launches;
