@@ -57,6 +57,7 @@ gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restric
     // atomic per CTA, CTAs in the upper bits and pairs in the lower, sent here and looked at behind the masks.
     unsigned long long pairs = 0, counted = 0;
     if (threadIdx.x == 0) {
+#pragma unroll
         for (int j = 0; j < kMaskRowAlign; ++j)
             if (r0 + j < rows) pairs += clamp_budget(kt[il.row(b, q0 + r0 + j)], k_max);
         counted = atomicAdd(reinterpret_cast<unsigned long long*>(dev_status + kStatusPairsWord), (1ull << kPairsBits) + pairs);
@@ -69,18 +70,24 @@ gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restric
         __syncwarp();
         const int lo = w0 * 32, hi = min((w0 + words) * 32, n_vis);
         int last = -1;                                 // entry in front of the batch (-1: compared already)
-        while (at < k) {
-            // 256 entries a time, eight consecutive ones per lane: neighbours mostly share a word, which then takes
-            // one shared-memory atomic
-            const int j0 = at + lane * 8;
-            int32_t e[8];
-            if (vec && (at & 3) == 0 && j0 + 8 <= k) {
+        // 256 entries a time, eight consecutive ones per lane: neighbours mostly share a word, which then takes
+        // one shared-memory atomic.  The next 512 are on their way meanwhile.
+        auto load = [&](int32_t (&e)[8], int from) {
+            const int j0 = from + lane * 8;
+            if (vec && (from & 3) == 0 && j0 + 8 <= k) {
                 const int4 a = *reinterpret_cast<const int4*>(row + j0), c = *reinterpret_cast<const int4*>(row + j0 + 4);
                 e[0] = a.x; e[1] = a.y; e[2] = a.z; e[3] = a.w; e[4] = c.x; e[5] = c.y; e[6] = c.z; e[7] = c.w;
             } else {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) e[j] = j0 + j < k ? row[j0 + j] : 0x7FFFFFFF;
             }
+        };
+        int32_t e[8], ahead[2][8];
+        load(e, at);
+        load(ahead[0], at + 256);
+        while (at < k) {
+            load(ahead[1], at + 512);
+            const int j0 = at + lane * 8;
             int before = __shfl_up_sync(0xFFFFFFFFu, e[7], 1);
             if (lane == 0) before = last;
             int taken = 0, word = -1;
@@ -106,6 +113,8 @@ gsa_build_masks_kernel(const int32_t* __restrict__ idx, const int32_t* __restric
             at += taken;
             if (taken < 256) break;
             last = __shfl_sync(0xFFFFFFFFu, e[7], 31);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { e[j] = ahead[0][j]; ahead[0][j] = ahead[1][j]; }
         }
         __syncthreads();
         for (int i = threadIdx.x; i < words / 4 * kMaskRowAlign; i += kMaskRowAlign * 32) {
