@@ -151,11 +151,13 @@ struct KeysSmem {
     static constexpr int ALLOC = OFF_ABORT + 8 + 1024;
 };
 
+struct KeysEndMaps { CUtensorMap v, g2, dk, dv, dg2; };            // V as given and the gate logits; the results
+
 template <int DH, int G, int SPLIT>
 __global__ void __launch_bounds__(kBwdThreads, 1)
 gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
                            const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                           const MaskedBwdArgs a) {
+                           const __grid_constant__ KeysEndMaps end, const MaskedBwdArgs a) {
     chain_wait();
     using P = KeysSmem<DH, G>;
     using T = TileBytes<DH>;
@@ -177,8 +179,8 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                    bar_ds = bar_kv + 32, bar_done = bar_kv + 40, bar_drain = bar_kv + 48;
 
     // (early key tiles are the long ones)  SPLIT = 2: a cluster of two CTAs shares a tile's
-    // rows, every other row tile each, for calls whose key tiles leave half of the SMs without work; the second CTA's
-    // sums go to the first through distributed shared memory at the end.
+    // rows, every other row tile each, for calls whose key tiles leave half of the SMs without work; at the end each sends the
+    // other one of its two sums through distributed shared memory, and the first finishes dK, the second dV and dg2.
     const int part_of = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) : 0;
     const int item = (int)(blockIdx.x / SPLIT);
     int tile, bh;
@@ -188,7 +190,9 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     const int r_first = max(0, tile * kMaskTileKeys - off - a.q0);           // first row that sees a key of the tile
     const int i0 = r_first / QT + part_of;
     // (tiles that no row sees have no masks)
-    const int n = r_first < a.rows && i0 < a.row_blocks ? (a.row_blocks - i0 + SPLIT - 1) / SPLIT : 0;
+    auto row_tiles = [&](int from) { return r_first < a.rows && from < a.row_blocks ? (a.row_blocks - from + SPLIT - 1) / SPLIT : 0; };
+    const int n = row_tiles(i0);
+    const bool makes_k = part_of == 0, makes_v = part_of == SPLIT - 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < ST; ++s) {
@@ -203,26 +207,30 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
     bool done = false;
 
     if (warp == kCopyWarp) {
-        if (lane == 0 && n > 0) {
-            mbar_expect_tx(bar_kv, 2 * T::TILE);
-            for (int c = 0; c < T::CHUNKS; ++c) {
-                tma_load_tile(sbase + P::OFF_K + c * T::CHUNK, &tm_k, c * 64, g, tile * kMaskTileKeys, b, bar_kv);
-                tma_load_tile(sbase + P::OFF_V + c * T::CHUNK, &tm_v, c * 64, g, tile * kMaskTileKeys, b, bar_kv);
+        if (lane == 0) {
+            if (n > 0) {
+                mbar_expect_tx(bar_kv, 2 * T::TILE);
+                for (int c = 0; c < T::CHUNKS; ++c) {
+                    tma_load_tile(sbase + P::OFF_K + c * T::CHUNK, &tm_k, c * 64, g, tile * kMaskTileKeys, b, bar_kv);
+                    tma_load_tile(sbase + P::OFF_V + c * T::CHUNK, &tm_v, c * 64, g, tile * kMaskTileKeys, b, bar_kv);
+                }
+                kv_issued = 1;
             }
-            kv_issued = 1;
             bool ok = true;
-            for (int i = 0; ok && i < n; ++i) {
+            const int entries = n + (makes_v ? 1 : 0);             // the ring's last entry: V and the gate logits, for the end
+            for (int i = 0; ok && i < entries; ++i) {
                 const int s = i % ST;
                 if (!mbar_wait(bar_free(s), ((i / ST) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
                 const uint32_t dst = sbase + P::OFF_RING + s * 2 * T::TILE;
-                const int z = (i0 + i * SPLIT) * QT;
+                const bool rows = i < n;
+                const int z = rows ? (i0 + i * SPLIT) * QT : tile * kMaskTileKeys, h = rows ? g * G : g;
                 if (i > 0 || !a.withhold_first) {
                     mbar_expect_tx(bar_q(s), T::TILE);
-                    for (int c = 0; c < T::CHUNKS; ++c) tma_load_tile(dst + c * T::CHUNK, &tm_q, c * 64, g * G, z, b, bar_q(s));
+                    for (int c = 0; c < T::CHUNKS; ++c) tma_load_tile(dst + c * T::CHUNK, rows ? &tm_q : &end.v, c * 64, h, z, b, bar_q(s));
                 }
                 mbar_expect_tx(bar_d(s), T::TILE);
                 for (int c = 0; c < T::CHUNKS; ++c)
-                    tma_load_tile(dst + T::TILE + c * T::CHUNK, &tm_do, c * 64, g * G, z, b, bar_d(s));
+                    tma_load_tile(dst + T::TILE + c * T::CHUNK, rows ? &tm_do : &end.g2, c * 64, h, z, b, bar_d(s));
                 copies = i + 1;
             }
             if (!ok) atomicCAS(a.dev_status, kDevOk, kDevTimeoutTma);
@@ -351,82 +359,107 @@ gsa_masked_bwd_keys_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             __syncwarp();
             if (lane == 0) { mbar_arrive(bar_ds); mbar_arrive(bar_statfree(s)); }
         }
-        done = ok && (n == 0 || warp_wait(bar_done, 0, s_abort, a.wait_cycles));
+        done = ok && (n == 0 || warp_wait(bar_done, 0, s_abort, a.wait_cycles)) &&
+               (!makes_v || (warp_wait(bar_q(n % ST), (n / ST) & 1, s_abort, a.wait_cycles) &&
+                             warp_wait(bar_d(n % ST), (n / ST) & 1, s_abort, a.wait_cycles)));
         if (!done && lane == 0) atomicCAS(a.dev_status, kDevOk, kDevTimeoutEpi);
         tc_fence_after();
     }
     // ---- sums: dK and dV' of key (quad, lane), columns part * DH / 4 .. of the head ----
-    const int part = (warp & 15) >> 2, quad = warp & 3;
-    const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
-    auto sums = [&](int c, uint32_t (&dk)[16], uint32_t (&dv)[16]) {       // 16 columns
+    const int part = (warp & 15) >> 2, quad = warp & 3, m = quad * 32 + lane;
+    auto sum = [&](uint32_t tm, int c, uint32_t (&x)[16]) {        // 16 columns of one of the sums
         if (n > 0) {
-            tc_ld16(lane_base + kTmK + part * (DH / 4) + 16 * c, dk);
-            tc_wait_ld16(dk);
-            tc_ld16(lane_base + kTmV + part * (DH / 4) + 16 * c, dv);
-            tc_wait_ld16(dv);
+            tc_ld16(tmem + ((uint32_t)(quad * 32) << 16) + tm + part * (DH / 4) + 16 * c, x);
+            tc_wait_ld16(x);
         } else {
 #pragma unroll
-            for (int e = 0; e < 16; ++e) dk[e] = dv[e] = 0u;
+            for (int e = 0; e < 16; ++e) x[e] = 0u;
         }
     };
-    // (the ring of the first CTA is free once both have come here; one float per column and key, lanes side by side)
-    float* const other = reinterpret_cast<float*>(smem + P::OFF_RING) + part * (DH / 4) * 128 + quad * 32 + lane;
+    // what the other CTA sends: one float per column and key, lanes side by side, in the ring's stage behind the last one used
+    auto received = [&](int entries) {
+        return reinterpret_cast<float*>(smem + P::OFF_RING + (entries + 1) % ST * 2 * T::TILE) + part * (DH / 4) * 128 + m;
+    };
     if constexpr (SPLIT > 1) {
         namespace cg = cooperative_groups;
-        static_assert(P::STAGES * 2 * T::TILE >= 2 * DH * 128 * 4, "the second CTA's sums fit the ring");
+        static_assert(2 * T::TILE >= DH * 128 * 4, "a sum fits one stage of the ring");
         cg::this_cluster().sync();
-        if (part_of == 1 && warp < 16 && done) {
-            float* const to = cg::this_cluster().map_shared_rank(other, 0);
+        if (warp < 16 && done) {
+            float* const to = cg::this_cluster().map_shared_rank(received(row_tiles(i0 + 1 - 2 * part_of)), 1 - part_of);
 #pragma unroll
             for (int c = 0; c < DH / 64; ++c) {
-                uint32_t dk[16], dv[16];
-                sums(c, dk, dv);
+                uint32_t x[16];
+                sum(makes_k ? kTmV : kTmK, c, x);
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    to[(16 * c + e) * 128] = __uint_as_float(dk[e]);
-                    to[(DH + 16 * c + e) * 128] = __uint_as_float(dv[e]);
-                }
+                for (int e = 0; e < 16; ++e) to[(16 * c + e) * 128] = __uint_as_float(x[e]);
             }
         }
         cg::this_cluster().sync();
     }
-    if (warp < 16 && part_of == 0 && done) {
-        {
-            const int key = tile * kMaskTileKeys + quad * 32 + lane;
-            const size_t at = (((size_t)b * a.Lk + min(key, a.Lk - 1)) * a.n_kv + g) * DH + part * (DH / 4);
+    if (warp < 16) {
+        // The results go where their tiles lie in shared memory (dK over K, dV over V, dg2 over the logits) and out as boxes; keys past
+        // the last are clipped.
+        unsigned char* const stage = smem + P::OFF_RING + n % ST * 2 * T::TILE;
+        if (done) {
 #pragma unroll
             for (int c = 0; c < DH / 64; ++c) {
-                uint32_t dk[16], dv[16];
-                sums(c, dk, dv);
-                if constexpr (SPLIT > 1) {
+                const int col = part * (DH / 4) + 16 * c;
+                const uint32_t piece0 = (col >> 6) * T::CHUNK + m * 128;
+                auto piece = [&](int q) { return piece0 + (((((col & 63) >> 3) + q) ^ (m & 7)) << 4); };
+                auto whole_sum = [&](uint32_t tm, uint32_t (&x)[16]) {
+                    sum(tm, c, x);
+                    if constexpr (SPLIT > 1) {
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        dk[e] = __float_as_uint(__uint_as_float(dk[e]) + other[(16 * c + e) * 128]);
-                        dv[e] = __float_as_uint(__uint_as_float(dv[e]) + other[(DH + 16 * c + e) * 128]);
+                        for (int e = 0; e < 16; ++e) x[e] = __float_as_uint(__uint_as_float(x[e]) + received(n)[(16 * c + e) * 128]);
+                    }
+                };
+                if (makes_k) {
+                    uint32_t dk[16];
+                    whole_sum(kTmK, dk);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        uint32_t x[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            x[e] = pack_bf16(__uint_as_float(dk[8 * q + 2 * e]) * a.scale, __uint_as_float(dk[8 * q + 2 * e + 1]) * a.scale);
+                        *reinterpret_cast<uint4*>(smem + P::OFF_K + piece(q)) = make_uint4(x[0], x[1], x[2], x[3]);
                     }
                 }
-                if (key >= a.Lk) continue;
+                if (makes_v) {
+                    uint32_t dv[16];
+                    whole_sum(kTmV, dv);
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const size_t p8 = at + 16 * c + 8 * q;
-                    const uint4 vv = *reinterpret_cast<const uint4*>(a.V + p8), gg = *reinterpret_cast<const uint4*>(a.g2 + p8);
-                    const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
-                    const __nv_bfloat162* gp = reinterpret_cast<const __nv_bfloat162*>(&gg);
-                    uint32_t ok_[4], ov[4], og[4];
+                    for (int q = 0; q < 2; ++q) {
+                        uint4* const at_v = reinterpret_cast<uint4*>(stage + piece(q));
+                        uint4* const at_g = reinterpret_cast<uint4*>(stage + T::TILE + piece(q));
+                        const uint4 vv = *at_v, gg = *at_g;
+                        const __nv_bfloat162* vp = reinterpret_cast<const __nv_bfloat162*>(&vv);
+                        const __nv_bfloat162* gp = reinterpret_cast<const __nv_bfloat162*>(&gg);
+                        uint32_t ov[4], og[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 vf = __bfloat1622float2(vp[e]), gf = __bfloat1622float2(gp[e]);
-                        const float s0 = 1.0f / (1.0f + __expf(-gf.x)), s1 = 1.0f / (1.0f + __expf(-gf.y));
-                        const float d0 = __uint_as_float(dv[8 * q + 2 * e]), d1 = __uint_as_float(dv[8 * q + 2 * e + 1]);
-                        ok_[e] = pack_bf16(__uint_as_float(dk[8 * q + 2 * e]) * a.scale, __uint_as_float(dk[8 * q + 2 * e + 1]) * a.scale);
-                        ov[e] = pack_bf16(d0 * s0, d1 * s1);
-                        og[e] = pack_bf16(d0 * vf.x * s0 * (1.0f - s0), d1 * vf.y * s1 * (1.0f - s1));
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 vf = __bfloat1622float2(vp[e]), gf = __bfloat1622float2(gp[e]);
+                            const float s0 = fast_sigmoid(gf.x), s1 = fast_sigmoid(gf.y);
+                            const float d0 = __uint_as_float(dv[8 * q + 2 * e]), d1 = __uint_as_float(dv[8 * q + 2 * e + 1]);
+                            ov[e] = pack_bf16(d0 * s0, d1 * s1);
+                            og[e] = pack_bf16(d0 * vf.x * s0 * (1.0f - s0), d1 * vf.y * s1 * (1.0f - s1));
+                        }
+                        *at_v = make_uint4(ov[0], ov[1], ov[2], ov[3]);
+                        *at_g = make_uint4(og[0], og[1], og[2], og[3]);
                     }
-                    *reinterpret_cast<uint4*>(a.dK + p8) = make_uint4(ok_[0], ok_[1], ok_[2], ok_[3]);
-                    *reinterpret_cast<uint4*>(a.dV + p8) = make_uint4(ov[0], ov[1], ov[2], ov[3]);
-                    *reinterpret_cast<uint4*>(a.dg2 + p8) = make_uint4(og[0], og[1], og[2], og[3]);
                 }
             }
+        }
+        if (tile_results_written(1, 512, done) && threadIdx.x == 0) {
+            for (int c = 0; c < T::CHUNKS; ++c) {
+                if (makes_k) tma_store_tile(&end.dk, c * 64, g, tile * kMaskTileKeys, b, sbase + P::OFF_K + c * T::CHUNK);
+                if (makes_v) {
+                    const uint32_t from = sbase + P::OFF_RING + n % ST * 2 * T::TILE + c * T::CHUNK;
+                    tma_store_tile(&end.dv, c * 64, g, tile * kMaskTileKeys, b, from);
+                    tma_store_tile(&end.dg2, c * 64, g, tile * kMaskTileKeys, b, from + T::TILE);
+                }
+            }
+            tma_store_wait();
         }
     }
     tile_end(warp, lane, tmem, s_abort, bar_drain,
@@ -825,10 +858,13 @@ template <int DH, int G>
 cudaError_t launch_bwd_t(const MaskedBwdArgs& a, const gsa_params_t& p, const __nv_bfloat16* Q, const __nv_bfloat16* K,
                          const __nv_bfloat16* Vg, const __nv_bfloat16* dOs, cudaStream_t st) {
     CUtensorMap tq, td, tk, tv;
+    KeysEndMaps end;
+    auto keys_map = [&](CUtensorMap* tm, const void* x) { return make_heads_tmap(tm, x, p.B, p.Lk, p.Lk, p.n_kv, DH, kMaskTileKeys, 1); };
+    if (!keys_map(&end.v, a.V) || !keys_map(&end.g2, a.g2) || !keys_map(&end.dk, a.dK) || !keys_map(&end.dv, a.dV) ||
+        !keys_map(&end.dg2, a.dg2)) return cudaErrorUnknown;
     if (!make_heads_tmap(&tq, Q + (size_t)a.q0 * p.n_h * DH, p.B, p.Lq, a.rows, p.n_h, DH, 128 / G, G)) return cudaErrorUnknown;
     if (!make_heads_tmap(&td, dOs + (size_t)a.q0 * p.n_h * DH, p.B, p.Lq, a.rows, p.n_h, DH, 128 / G, G)) return cudaErrorUnknown;
-    if (!make_heads_tmap(&tk, K, p.B, p.Lk, p.Lk, p.n_kv, DH, kMaskTileKeys, 1)) return cudaErrorUnknown;
-    if (!make_heads_tmap(&tv, Vg, p.B, p.Lk, p.Lk, p.n_kv, DH, kMaskTileKeys, 1)) return cudaErrorUnknown;
+    if (!keys_map(&tk, K) || !keys_map(&tv, Vg)) return cudaErrorUnknown;
     auto set_smem = [](auto kern, int bytes) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
     constexpr int kSmemK = KeysSmem<DH, G>::ALLOC, kSmemR = RowsSmem<DH>::ALLOC, kSmemT = TargetSmem<DH>::ALLOC;
     static_assert(kSmemK <= 232448 && kSmemR <= 232448 && kSmemT <= 232448, "shared memory of one CTA");
@@ -839,9 +875,9 @@ cudaError_t launch_bwd_t(const MaskedBwdArgs& a, const gsa_params_t& p, const __
     if (e == cudaSuccess) e = set_smem(gsa_masked_target_kernel<DH, G>, kSmemT);
     if (e != cudaSuccess) return e;
     if (split == 2)
-        launch_chained_cluster(2, gsa_masked_bwd_keys_kernel<DH, G, 2>, (unsigned)(key_ctas * 2), kBwdThreads, kSmemK, st, tq, td, tk, tv, a);
+        launch_chained_cluster(2, gsa_masked_bwd_keys_kernel<DH, G, 2>, (unsigned)(key_ctas * 2), kBwdThreads, kSmemK, st, tq, td, tk, tv, end, a);
     else
-        launch_chained(gsa_masked_bwd_keys_kernel<DH, G, 1>, (unsigned)key_ctas, kBwdThreads, kSmemK, st, tq, td, tk, tv, a);
+        launch_chained(gsa_masked_bwd_keys_kernel<DH, G, 1>, (unsigned)key_ctas, kBwdThreads, kSmemK, st, tq, td, tk, tv, end, a);
     launch_chained(gsa_masked_bwd_rows_kernel<DH, G>, (unsigned)(a.row_blocks * p.n_kv * p.B), kBwdThreads, kSmemR, st, tq, td, tk, tv, a);
     g_launches += 2;
     if (a.pbar) {
