@@ -5,8 +5,8 @@
 //     columns n:  q^I (H^I*d^I) | k^I (d^I) | head weights (8, the first H^I used) | g1 logits | g2 logits
 //     q^I, k^I, g1, g2 are rounded to bf16 once; head weights leave as fp32 sigmoid(C).
 //
-// A persistent CTA walks output tiles of 128 tokens x 256 columns.  Warp 0 feeds a ring of shared-
-// memory stages by TMA (a 128 x 64 block of H and a 256 x 64 block of Wt per stage, 128-byte
+// A persistent CTA walks output tiles of 128 tokens x 256 columns (or narrower ones, TileList).  Warp 0 feeds a ring of shared-
+// memory stages by TMA (a 128 x 64 block of H and up to four 64 x 64 blocks of Wt per stage, 128-byte
 // swizzle), warp 1 issues the MMAs (four k-steps per stage) and owns the TMEM allocation, warps
 // 2..9 are the epilogue.  Two 256-column accumulators alternate, so the MMAs of the next tile run
 // while the epilogue converts and stores the current one.  Rows and columns of a tile that fall
@@ -35,7 +35,40 @@ constexpr int kNBars = 2 * kPStages + 4 + 1;
 constexpr int kOffTmem = kOffBar + kNBars * 8;
 constexpr int kOffAbort = kOffTmem + 8;
 constexpr int kSmemTotal = kOffAbort + 8 + 1024;        // slack to align the base to 1024
-constexpr uint32_t kIdescP = make_idesc_bf16(kTileM, kTileN);
+constexpr int kBoxN = 64;                               // columns of one copy of Wt
+
+// Output tiles in the order of their width: all whole ones that fill waves of the SMs; the rest of the whole ones, in halves or quarters
+// if the last wave has room for them; the columns that are left of the last 256.  8192 tokens: 896 whole tiles and 64 of 72 columns,
+// 6.1 waves and a short one instead of 7; the output projection's 512, 3 waves and one of halves instead of 4.  Both calls together
+// 192.8 -> 189.7 us: the GPU is at its power limit there, so that idle SMs cost less than their share.
+struct TileList {
+    int32_t cols;                  // whole column tiles of a token tile
+    int32_t whole, pieces, split, narrow, width_left;      // items of each kind; pieces a tile is cut into; columns left over
+    __host__ __device__ int items() const { return whole + pieces + narrow; }
+    __device__ void get(int i, int* m0, int* n0, int* width) const {
+        if (i < whole + pieces) {
+            const int j = i - whole, t = j < 0 ? i : whole + j / split, w = j < 0 ? kTileN : kTileN / split;
+            *m0 = t / cols * kTileM;
+            *n0 = t % cols * kTileN + (j < 0 ? 0 : j % split * w);
+            *width = w;
+        } else {
+            *m0 = (i - whole - pieces) * kTileM;
+            *n0 = cols * kTileN;
+            *width = width_left;
+        }
+    }
+};
+inline TileList tile_list(int m_tiles, int N, int sms) {
+    TileList l;
+    l.cols = N / kTileN;
+    l.width_left = N % kTileN;
+    l.narrow = l.width_left > 0 ? m_tiles : 0;
+    const int tiles = m_tiles * l.cols, rest = tiles % sms;
+    l.split = rest * 4 + l.narrow <= sms ? 4 : (rest * 2 + l.narrow <= sms ? 2 : 1);
+    l.pieces = l.split > 1 ? rest * l.split : 0;
+    l.whole = l.split > 1 ? tiles - rest : tiles;
+    return l;
+}
 
 struct ProjArgs {
     __nv_bfloat16* qI;
@@ -46,7 +79,7 @@ struct ProjArgs {
     int32_t* dev_status;
     int32_t M, K, N;               // tokens, d_model, stacked output columns
     int32_t n_q, n_k, HI, n_g1, n_g2;
-    int32_t m_tiles, n_tiles;
+    TileList tiles;
     long long wait_cycles;         // limit of every bounded wait
     int32_t withhold_first;        // fault injection: the first stage's copies are left out (its barrier is never completed)
 };
@@ -54,6 +87,7 @@ struct ProjArgs {
 __global__ void __launch_bounds__(kPThreads, 1)
 gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
                    const ProjArgs a) {
+    chain_wait();
     {   // an earlier CTA or launch gave up: leave, all threads together (one thread reads the word)
         __shared__ int s_go;
         if (threadIdx.x == 0) s_go = *reinterpret_cast<volatile int32_t*>(a.dev_status) == kDevOk;
@@ -93,7 +127,7 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
     tc_fence_after();
     const uint32_t tmem_base = *s_tmem;
 
-    const int n_tiles_total = a.m_tiles * a.n_tiles;
+    const int n_tiles_total = a.tiles.items();
     const int kblocks = (a.K + kBlockK - 1) / kBlockK;
     // what this thread has put in flight (the copy producer's and the MMA issuer's own counts)
     uint32_t copies_issued = 0;                            // stages filled so far (all tiles)
@@ -105,7 +139,9 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
         if (lane == 0) {
             bool gave_up = false;
             for (int tile = blockIdx.x; tile < n_tiles_total && !gave_up && !*s_abort; tile += gridDim.x) {
-                const int m0 = (tile / a.n_tiles) * kTileM, n0 = (tile % a.n_tiles) * kTileN;
+                int m0, n0, width;
+                a.tiles.get(tile, &m0, &n0, &width);
+                const int boxes = (width + kBoxN - 1) / kBoxN;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     const uint32_t it = copies_issued;
                     const int s = it % kPStages;
@@ -113,10 +149,11 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
                     if (it == 0 && a.withhold_first) {
                         first_withheld = true;             // (counted as issued; the give-up path skips it)
                     } else {
-                        mbar_expect_tx(bar_full(s), kStageBytes);
+                        mbar_expect_tx(bar_full(s), kA_BYTES + boxes * kBoxN * kBlockK * 2);
                         const uint32_t dst = sbase + s * kStageBytes;
                         tma_load_2d(dst, &tm_h, kb * kBlockK, m0, bar_full(s));
-                        tma_load_2d(dst + kA_BYTES, &tm_w, kb * kBlockK, n0, bar_full(s));
+                        for (int c = 0; c < boxes; ++c)
+                            tma_load_2d(dst + kA_BYTES + c * kBoxN * kBlockK * 2, &tm_w, kb * kBlockK, n0 + c * kBoxN, bar_full(s));
                     }
                     copies_issued = it + 1;
                 }
@@ -130,6 +167,9 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
             bool ok = true;
             for (int tile = blockIdx.x; ok && tile < n_tiles_total; tile += gridDim.x, ++tl) {
                 const int buf = tl & 1;
+                int m0, n0, width;
+                a.tiles.get(tile, &m0, &n0, &width);
+                const uint32_t idesc = make_idesc_bf16(kTileM, (width + 15) / 16 * 16);
                 if (!mbar_wait(bar_tempty(buf), ((tl >> 1) & 1) ^ 1, s_abort, a.wait_cycles)) { ok = false; break; }
                 for (int kb = 0; kb < kblocks; ++kb, ++it) {
                     const int s = it % kPStages;
@@ -139,7 +179,7 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
                     const uint64_t bdesc = make_kmajor_desc<128>(sbase + s * kStageBytes + kA_BYTES);
 #pragma unroll
                     for (int k = 0; k < kBlockK / 16; ++k)      // 16 K-elements = 32 bytes = 2 descriptor units
-                        tc_mma_bf16(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, kIdescP, (kb | k) != 0);
+                        tc_mma_bf16(tmem_base + buf * kTileN, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | k) != 0);
                     tc_commit(bar_empty(s));                    // stage reusable once these MMAs have read it
                     mma_blocks_issued = it + 1;
                 }
@@ -164,11 +204,13 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
                 break;
             }
             tc_fence_after();
-            const int m = (tile / a.n_tiles) * kTileM + quad * 32 + lane;       // this thread's token
-            const int n_base = (tile % a.n_tiles) * kTileN + half * 128;
+            int m0, n0, width;
+            a.tiles.get(tile, &m0, &n0, &width);
+            const int m = m0 + quad * 32 + lane;                                // this thread's token
+            const int n_base = n0 + half * 128, n_end = n0 + width;             // (columns from n_end on are another item's, or nobody's)
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + buf * kTileN + half * 128;
             auto store8 = [&](const uint32_t* r, int n8) {   // 8 consecutive columns starting at n8 (a multiple of 8)
-                if (m >= a.M || n8 >= a.N) return;
+                if (m >= a.M || n8 >= n_end) return;
                 if (n8 >= o_w && n8 < o_g1) {                // head weights: fp32 sigmoid
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
@@ -188,15 +230,16 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
                 *reinterpret_cast<uint4*>(dst) = v;
             };
             uint32_t ra[16], rb[16];
-            tc_ld16(taddr, ra);
+            if (n_base < n_end) tc_ld16(taddr, ra);
 #pragma unroll
             for (int c = 0; c < 8; c += 2) {
+                if (n_base + c * 16 >= n_end) break;
                 tc_wait_ld16(ra);
                 tc_ld16(taddr + (c + 1) * 16, rb);
                 store8(ra, n_base + c * 16);
                 store8(ra + 8, n_base + c * 16 + 8);
                 tc_wait_ld16(rb);
-                if (c + 2 < 8) tc_ld16(taddr + (c + 2) * 16, ra);
+                if (c + 2 < 8 && n_base + (c + 2) * 16 < n_end) tc_ld16(taddr + (c + 2) * 16, ra);
                 store8(rb, n_base + (c + 1) * 16);
                 store8(rb + 8, n_base + (c + 1) * 16 + 8);
             }
@@ -255,18 +298,16 @@ cudaError_t launch_project(const gsa_params_t& p, int d_model, const __nv_bfloat
     a.qI = qI; a.kI = kI; a.w = w; a.g1 = g1; a.g2 = g2; a.dev_status = dev_status;
     a.M = p.B * p.Lk; a.K = d_model; a.N = project_columns(p);
     a.n_q = p.HI * p.dI; a.n_k = p.dI; a.HI = p.HI; a.n_g1 = p.n_h * p.d_h; a.n_g2 = p.n_kv * p.d_h;
-    a.m_tiles = (a.M + kTileM - 1) / kTileM;
-    a.n_tiles = (a.N + kTileN - 1) / kTileN;
+    const int sms = sm_count();
+    a.tiles = tile_list((a.M + kTileM - 1) / kTileM, a.N, sms);
     a.wait_cycles = wait_limit_cycles();
     a.withhold_first = withhold_first_copy() ? 1 : 0;
     CUtensorMap tm_h, tm_w;
     if (!make_kblock_tmap(&tm_h, H, (uint64_t)a.M, (uint64_t)a.K, kTileM)) return cudaErrorUnknown;
-    if (!make_kblock_tmap(&tm_w, Wt, (uint64_t)a.N, (uint64_t)a.K, kTileN)) return cudaErrorUnknown;
+    if (!make_kblock_tmap(&tm_w, Wt, (uint64_t)a.N, (uint64_t)a.K, kBoxN)) return cudaErrorUnknown;
     cudaError_t e = cudaFuncSetAttribute(gsa_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal);
     if (e != cudaSuccess) return e;
-    const int sms = sm_count();
-    const int tiles = a.m_tiles * a.n_tiles;
-    gsa_project_kernel<<<tiles < sms ? tiles : sms, kPThreads, kSmemTotal, st>>>(tm_h, tm_w, a);
+    launch_chained(gsa_project_kernel, (unsigned)(a.tiles.items() < sms ? a.tiles.items() : sms), kPThreads, kSmemTotal, st, tm_h, tm_w, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -280,18 +321,16 @@ cudaError_t launch_gemm_bf16(int M, int K, int N, const __nv_bfloat16* A, const 
     a.qI = C; a.kI = nullptr; a.w = nullptr; a.g1 = nullptr; a.g2 = nullptr; a.dev_status = dev_status;
     a.M = M; a.K = K; a.N = N;
     a.n_q = N; a.n_k = 0; a.HI = 0; a.n_g1 = 0; a.n_g2 = 0;
-    a.m_tiles = (M + kTileM - 1) / kTileM;
-    a.n_tiles = (N + kTileN - 1) / kTileN;
+    const int sms = sm_count();
+    a.tiles = tile_list((M + kTileM - 1) / kTileM, N, sms);
     a.wait_cycles = wait_limit_cycles();
     a.withhold_first = withhold_first_copy() ? 1 : 0;
     CUtensorMap tm_a, tm_b;
     if (!make_kblock_tmap(&tm_a, A, (uint64_t)M, (uint64_t)K, kTileM)) return cudaErrorUnknown;
-    if (!make_kblock_tmap(&tm_b, Bt, (uint64_t)N, (uint64_t)K, kTileN)) return cudaErrorUnknown;
+    if (!make_kblock_tmap(&tm_b, Bt, (uint64_t)N, (uint64_t)K, kBoxN)) return cudaErrorUnknown;
     cudaError_t e = cudaFuncSetAttribute(gsa_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal);
     if (e != cudaSuccess) return e;
-    const int sms = sm_count();
-    const int tiles = a.m_tiles * a.n_tiles;
-    gsa_project_kernel<<<tiles < sms ? tiles : sms, kPThreads, kSmemTotal, st>>>(tm_a, tm_b, a);
+    launch_chained(gsa_project_kernel, (unsigned)(a.tiles.items() < sms ? a.tiles.items() : sms), kPThreads, kSmemTotal, st, tm_a, tm_b, a);
     ++g_launches;
     return cudaGetLastError();
 }
