@@ -21,6 +21,28 @@ int sm_count() {
     }
     return n;
 }
+namespace {
+struct ClearArgs { ClearSpan span[3]; };
+__global__ void __launch_bounds__(256) gsa_clear_kernel(const ClearArgs a) {
+    chain_wait();
+    const size_t first = (size_t)blockIdx.x * 256 + threadIdx.x, step = (size_t)gridDim.x * 256;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const size_t bytes = a.span[s].bytes, vec = (reinterpret_cast<uintptr_t>(a.span[s].p) & 15) == 0 ? bytes / 16 : 0;
+        for (size_t i = first; i < vec; i += step) reinterpret_cast<uint4*>(a.span[s].p)[i] = make_uint4(0u, 0u, 0u, 0u);
+        for (size_t i = vec * 4 + first; i < bytes / 4; i += step) reinterpret_cast<uint32_t*>(a.span[s].p)[i] = 0u;
+    }
+}
+}  // namespace
+
+cudaError_t launch_clear(cudaStream_t st, ClearSpan a, ClearSpan b, ClearSpan c) {
+    ClearArgs args{{a, b, c}};
+    const size_t most = a.bytes > b.bytes ? (a.bytes > c.bytes ? a.bytes : c.bytes) : (b.bytes > c.bytes ? b.bytes : c.bytes);
+    const size_t want = (most / 16 + 255) / 256, cap = (size_t)sm_count() * 8;
+    launch_chained(gsa_clear_kernel, (unsigned)(want < 1 ? 1 : (want < cap ? want : cap)), 256, 0, st, args);
+    return cudaGetLastError();                             // (not counted as a launch, as a memset would not be)
+}
+
 thread_local int32_t* t_dev_status = nullptr;
 static int32_t g_indexer_path = 0;
 static std::atomic<long long> g_wait_cycles{kSpinCycles};
@@ -182,7 +204,7 @@ int gsa_indexer_scores(const gsa_params_t* p, const void* qI, const void* kI, co
     if (!ws || ws_bytes < (size_t)kStatusBytes || !aligned16(ws)) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     t_dev_status = (int32_t*)ws;
-    cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
+    cudaError_t e = launch_clear(st, {ws, (size_t)kStatusBytes});
     if (e != cudaSuccess) return cuda_rc(e);
     return cuda_rc(launch_indexer(*p, rr, (const bf16*)qI, (const bf16*)kI, w, bI, scores, row_stride,
                                   (int32_t*)ws, st));
@@ -208,7 +230,7 @@ int gsa_project(const gsa_params_t* p, int32_t d_model, const void* H, const voi
     if (!ws || ws_bytes < (size_t)kStatusBytes || !aligned16(ws)) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     t_dev_status = (int32_t*)ws;
-    cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
+    cudaError_t e = launch_clear(st, {ws, (size_t)kStatusBytes});
     if (e != cudaSuccess) return cuda_rc(e);
     return cuda_rc(launch_project(*p, d_model, (const bf16*)H, (const bf16*)Wt, (bf16*)qI, (bf16*)kI, w,
                                   (bf16*)g1_logits, (bf16*)g2_logits, (int32_t*)ws, st));
@@ -225,7 +247,7 @@ int gsa_output_projection(const gsa_params_t* p, int32_t d_model, const void* at
     if (!ws || ws_bytes < (size_t)kStatusBytes || !aligned16(ws)) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     t_dev_status = (int32_t*)ws;
-    cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
+    cudaError_t e = launch_clear(st, {ws, (size_t)kStatusBytes});
     if (e != cudaSuccess) return cuda_rc(e);
     return cuda_rc(launch_gemm_bf16(p->B * p->Lq, p->n_h * p->d_h, d_model, (const bf16*)attn_out, (const bf16*)Wo_t,
                                     (bf16*)u, (int32_t*)ws, st));
@@ -243,7 +265,7 @@ int gsa_adaptive_topk(const gsa_params_t* p, const float* scores, int64_t row_st
     int32_t* fb = nullptr;
     t_dev_status = nullptr;
     if (ws && aligned16(ws) && ws_bytes >= (size_t)kStatusBytes) {
-        cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, (cudaStream_t)stream);
+        cudaError_t e = launch_clear((cudaStream_t)stream, {ws, (size_t)kStatusBytes});
         if (e != cudaSuccess) return cuda_rc(e);
         fb = (int32_t*)ws + kStatusFallbackWord;
         t_dev_status = (int32_t*)ws;
@@ -315,12 +337,11 @@ int gsa_sparse_gated_attn_bwd(const gsa_params_t* p, const void* Q, const void* 
     float* lse2 = (float*)(wsb + wp.lse_off);
     float* delta = (float*)(wsb + wp.delta_off);
     t_dev_status = (int32_t*)ws;
-    cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
+    cudaError_t e = launch_clear(st, {ws, (size_t)kStatusBytes}, {pbar, pbar ? (size_t)rr.rows() * p->k_max * 4 : 0});
     if (e == cudaSuccess)
         e = launch_value_gate((const bf16*)V, (const bf16*)g2_logits, Vg, (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st,
                               t_dev_status + kStatusGeneralWord, wp.masked ? (const bf16*)K : nullptr);
     IdxLayout il{0, rr.q_begin, rr.R};
-    if (e == cudaSuccess && pbar) e = cudaMemsetAsync(pbar, 0, (size_t)rr.rows() * p->k_max * 4, st);
     if (wp.masked) {
         if (e == cudaSuccess)
             e = launch_masked_bwd(*p, rr, (const bf16*)Q, (const bf16*)K, (const bf16*)V, Vg, (const bf16*)g1_logits,
@@ -352,7 +373,7 @@ int gsa_attn_probs_mean(const gsa_params_t* p, const void* Q, const void* K, con
     if (!ws || !aligned16(ws) || ws_bytes < (size_t)kStatusBytes) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     t_dev_status = (int32_t*)ws;
-    cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
+    cudaError_t e = launch_clear(st, {ws, (size_t)kStatusBytes});
     IdxLayout il{0, rr.q_begin, rr.R};
     if (e == cudaSuccess) e = launch_attn_probs_mean(*p, rr, (const bf16*)Q, (const bf16*)K, idx, kt, il, pbar, st);
     return cuda_rc(e);
@@ -381,7 +402,8 @@ int gsa_indexer_kl_bwd(const gsa_params_t* p, const void* qI, const void* kI, co
     if (!ws || !aligned16(ws) || ws_bytes < need) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     t_dev_status = (int32_t*)ws;
-    cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
+    // (the fp32 sums of dk^I lie right behind the status head)
+    cudaError_t e = launch_clear(st, {ws, kStatusBytes + (size_t)p->B * p->Lk * p->dI * 4}, {dbI, dbI ? (size_t)p->HI * 4 : 0});
     IdxLayout il{0, rr.q_begin, rr.R};
     if (e == cudaSuccess)
         e = launch_indexer_kl(*p, rr, (const bf16*)qI, (const bf16*)kI, w, bI, idx, kt, il, pbar, loss, (bf16*)dqI,
@@ -422,7 +444,7 @@ static int attn_fwd_impl(const gsa_params_t* p, const void* Q, const void* K, co
     if (!ws || !aligned16(ws) || ws_bytes < attn_ws_bytes(*p, false)) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     t_dev_status = (int32_t*)ws;
-    cudaError_t e0 = cudaMemsetAsync(ws, 0, kStatusBytes, st);
+    cudaError_t e0 = launch_clear(st, {ws, (size_t)kStatusBytes});
     if (e0 != cudaSuccess) return cuda_rc(e0);
     IdxLayout il{0, rr.q_begin, rr.R};
     char* wsb = (char*)ws;
@@ -479,7 +501,7 @@ static int forward_impl(const gsa_params_t* p, const void* Q, const void* K, con
     cudaStream_t st = (cudaStream_t)stream;
     char* wsb = (char*)ws;
     t_dev_status = (int32_t*)ws;
-    cudaError_t e = cudaMemsetAsync(ws, 0, kStatusBytes, st);
+    cudaError_t e = launch_clear(st, {ws, (size_t)kStatusBytes});
     if (e != cudaSuccess) return cuda_rc(e);
 
     float* slab = (float*)(wsb + wp.slab_off);

@@ -71,6 +71,11 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
     return launch_chained_cluster(1, kern, grid, block, smem, st, static_cast<A&&>(args)...);
 }
 
+// Zeroes up to three regions (4-byte aligned, whole words) ahead of a call's kernels.  A kernel of its own, chained like the others:
+// a cudaMemsetAsync stands 2 to 4 us apart from the kernels on either side of it (the three in front of the indexer loss 12 us).
+struct ClearSpan { void* p; size_t bytes; };
+cudaError_t launch_clear(cudaStream_t st, ClearSpan a, ClearSpan b = {nullptr, 0}, ClearSpan c = {nullptr, 0});
+
 // multiprocessors of the current device (cached per device; 148 if the query fails)
 int sm_count();
 
@@ -121,7 +126,7 @@ cudaError_t launch_sparse_attn_bwd_keys(const gsa_params_t& p, RowRange rr, cons
                                         cudaStream_t st);
 // The indexer's sparse-phase loss (gsa_indexer_loss.cu): its target (mean over the heads of the attention
 // distribution on S_t; pbar is zeroed inside) and the loss with its derivatives (dkI32: B * Lk * dI floats
-// of scratch, zeroed inside; dbI may be null).
+// of scratch; dbI may be null; both zeroed by the caller).
 cudaError_t launch_attn_probs_mean(const gsa_params_t& p, RowRange rr, const __nv_bfloat16* Q,
                                    const __nv_bfloat16* K, const int32_t* idx, const int32_t* kt, IdxLayout il,
                                    float* pbar, cudaStream_t st);

@@ -570,9 +570,7 @@ cudaError_t launch_indexer_kl(const gsa_params_t& p, RowRange rr, const __nv_bfl
                               __nv_bfloat16* dqI, __nv_bfloat16* dkI, float* dw, float* dbI, float* dkI32,
                               cudaStream_t st) {
     const int64_t n_k = (int64_t)p.B * p.Lk * p.dI;
-    cudaError_t e = cudaMemsetAsync(dkI32, 0, (size_t)n_k * 4, st);
-    if (e == cudaSuccess && dbI) e = cudaMemsetAsync(dbI, 0, (size_t)p.HI * 4, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     if (rr.rows() > 0) {
         KlArgs a;
         a.qI = qI; a.kI = kI; a.w = w; a.bI = bI; a.idx = idx; a.kt = kt; a.dev_status = t_dev_status; a.pbar = pbar; a.loss = loss;

@@ -91,7 +91,7 @@ extern "C" int gsa_sparse_gated_attn_fwd_static(const gsa_params_t* p, const voi
     // cleared here; the pre-pass overwrites every gated value the attention kernel will read, and the
     // attention kernels write every state slot before they read it.
     t_dev_status = (int32_t*)scratch;
-    e = cudaMemsetAsync(scratch, 0, kStatusBytes, st);
+    e = launch_clear(st, {scratch, (size_t)kStatusBytes});
     if (e == cudaSuccess)
         e = launch_value_gate((const __nv_bfloat16*)V, (const __nv_bfloat16*)g2_logits, Vg,
                           (int64_t)p->B * p->Lk * p->n_kv * p->d_h, st);
