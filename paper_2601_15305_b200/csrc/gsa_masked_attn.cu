@@ -4,25 +4,30 @@
 // One CTA = one KV head and 256 rows, a row being a (query, head of the group) pair: two M = 128 tiles whose chains
 //     S = Q K^T (tcgen05, fp32 in TMEM) -> mask, softmax numerators P (registers) -> P as bf16 into the columns of S
 //     -> O += P V' (tcgen05, A operand in TMEM, V' tile read as it lies: keys are the contraction, d runs along N)
-// run against each other: while four warps work on one tile's scores, the tensor cores run the other's products.  A
-// K and a V' tile are fetched once for both.  Thread = row: no shuffles anywhere.
+// run against each other, by halves of 64 keys: while a half's numerators are made, the tensor cores take in the other halves' and
+// score the same half of the next tile behind each product.  A K and a V' tile are fetched once for both.  Thread = row: no
+// shuffles anywhere.
 //
-// Softmax reference: as in the gather kernel, it moves only when a selected score exceeds it by more than 2^8, so the
+// Softmax reference: it moves only when the numerators' sum shows that a selected score may exceed it by more than 2^8, so the
 // accumulator in TMEM is touched by the softmax warps on a row's first tiles only.  Masked scores are replaced by
-// -inf before the maximum and the exponentials; fp32 everywhere except P (bf16, as in the gather kernel).  The reference is
+// -inf before the exponentials; fp32 everywhere except P (bf16, as in the gather kernel).  The reference is
 // set a little above the maximum it is taken from: that maximum may come from very few keys (a row of 50K keys has three selected
 // ones in its first tile), and where scores are nearly flat half of the row's numerators would then lie just above 1, where bf16
 // is half as fine as just below.  Error of the output against fp64, chunk of 2003 rows at 50021 keys: 2.78e-3 without the margin,
 // 2.62e-3 with it, 2.64e-3 in the gather kernel; 50 prefill, chunk, dense and training shapes: 0.995 of the gather's on average.
 //
-// Bound: the serial chain of a tile (scores -> numerators -> product -> next scores); the two tiles' chains fill each other's
-// gaps, with the tensor pipe active 42 % and the special-function unit 44 % of the time (8K, profiler).  Measured at 16 heads of
-// 128 on 8 KV heads: L = 32K 3.45 ms = 1.27 PFLOP/s over the visible pairs (the gather kernel: 19.6 ms; with a whole tile's
-// numerators handed over at once 3.55), 8K 0.33 ms (4.6 ms), dense 2 x 3072 0.135 ms (2.7 ms).
+// Bound: the tensor pipe and the hand-overs around it.  Per pair of tiles 3270-3390 cycles (a softmax warp: 1790 at the numerators, 490
+// to hand them over, 750 waiting); the products count 2560 of them, for one of N = 64 out of shared memory takes 48 cycles a step of
+// 16 (its A operand alone is 4 KB), not the 32 of its arithmetic.  Whole tiles, with the next scores only behind both halves' product,
+// took 3600, 1500 of it in that wait.  A CTA costs 0.7 us of setup, 1.5 to its first scores and about 2 at its end (8.7 while gates
+// and output went row by row).  Measured at 16 heads of 128 on 8 KV heads: 8K 247 us (319 before the order of tile_order and the halves,
+// the gather kernel 4.6 ms), dense 2 x 3072 100 us (135), L = 32K 3.27 ms = 1.34 PFLOP/s over the visible pairs, at the power limit (3.41;
+// the gather 19.6 ms).  Slower: four softmax warpgroups, a row's halves on two threads (8K 295 us); a share of the exponentials on
+// the FMA pipe (every fourth pair 250 against 252 at 8K, 3.34 against 3.28 ms at 32K; every second 280).
 //
 // Warps 0-3 / 4-7: softmax and epilogue of tile 0 / 1; warp 8: TMA; warp 9: MMA issue and TMEM allocation; 10, 11
 // only complete their warpgroup.
-// TMEM: S0 | S1 (128 columns each, P overlays the first 64) | O0 | O1.
+// TMEM: S0 | S1 (128 columns each, 64 of a half; a half's P overlays its first 32) | O0 | O1.
 #include "gsa_masked.cuh"
 
 namespace gsa {

@@ -13,8 +13,8 @@
 //
 // Bound: the products and the elementwise work between them in turn.  Measured at L = 32K, 16 heads of 128 on 8 KV heads, mean
 // budget 2080: 17.2 ms for a call with its target, 13.3 ms without (seven products, 1.16 PFLOP/s over the visible pairs; the keys
-// kernel somewhat over 6, the rows kernel over 5), so 3.9 ms for the target (one product, and all the exponentials); 8K 1.37 and
-// 1.02 ms.  The gather kernels take 86 and 19.0 ms for a call.
+// kernel somewhat over 6, the rows kernel over 5), so 3.3 ms for the target (one product, and all the exponentials; 3.9 while a thread alone searched a run's start in each set and
+// every lane summed all heads); 8K 1.37 and 1.02 ms.  The gather kernels take 86 and 19.0 ms for a call.
 //
 // Roles in all three: warps 0-15 the elementwise work (four warpgroups side by side, 32 columns of a tile each: with two of
 // them the products waited for it), warp 16 copies, warp 17 MMA issue, 18 and 19 small loads.
