@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(256) gsa_range_cuts_kernel(const int32_t* __re
 // merge the state slots of a (row, head): out = (sum_p 2^(m_p - M) O_p) / (sum_p 2^(m_p - M) l_p) * sigmoid(g1)
 // A CTA takes kFinRows consecutive query rows; thread = (KV head, d), all G heads of the group.  With a
 // single slot per row (prefill) the loads of all rows are issued before any is used.  With several (decode) a CTA takes one row
-// and KV head, thread = (one of kFinGroups shares of the slots, d): two memory latencies, whatever the number of slots.
+// and KV head, thread = (one of kFinGroups shares of the slots, d): one or two memory latencies, whatever the number of slots.
 constexpr int kFinRows = 4;
 constexpr int kFinGroups = 4;
 
@@ -510,10 +510,19 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
     __shared__ float s_m[kMaxParts * G], s_l[kMaxParts * G], s_top[G], s_den[G], s_acc[kFinGroups][G][DH];
     const int tid = threadIdx.x, d = tid % DH, grp = tid / DH, warp = tid >> 5, lane = tid & 31;
     const RowId r = row_of(rr, il, (int)blockIdx.x);
-    const int g = blockIdx.y, k_eff = clamp_budget(kt[r.irow], k_max), np = k_eff > 0 ? parts_of(k_eff, max_parts) : 0;
+    const int g = blockIdx.y;
     const float* __restrict__ st = state + ((int64_t)r.irow * n_kv + g) * STATE_F;
     const int64_t slot = idx_rows * n_kv * STATE_F;
-    for (int i = tid; i < np * G; i += kFinGroups * DH) {
+    // everything that does not depend on another load goes out at once: the budget, every slot's statistics and this thread's share of
+    // the first slots' sums, also of slots that the row does not use (the workspace holds them; their weight stays out of the sums)
+    constexpr int AHEAD = G <= 2 ? 4 : (G == 4 ? 2 : 1);
+    float first[AHEAD][G];
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u)
+#pragma unroll
+        for (int e = 0; e < G; ++e) first[u][e] = grp + u * kFinGroups < max_parts ? st[(grp + u * kFinGroups) * slot + d * G + e] : 0.f;
+    const int k_eff = clamp_budget(kt[r.irow], k_max), np = k_eff > 0 ? parts_of(k_eff, max_parts) : 0;
+    for (int i = tid; i < max_parts * G; i += kFinGroups * DH) {
         s_m[i] = st[(i / G) * slot + G * DH + i % G];
         s_l[i] = st[(i / G) * slot + G * DH + G + i % G];
     }
@@ -537,8 +546,13 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
     float acc[G];
 #pragma unroll
     for (int e = 0; e < G; ++e) acc[e] = 0.f;
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u)
+        if (grp + u * kFinGroups < np)
+#pragma unroll
+            for (int e = 0; e < G; ++e) acc[e] = fmaf(s_m[(grp + u * kFinGroups) * G + e], first[u][e], acc[e]);
 #pragma unroll 4
-    for (int p = grp; p < np; p += kFinGroups)
+    for (int p = grp + AHEAD * kFinGroups; p < np; p += kFinGroups)
 #pragma unroll
         for (int e = 0; e < G; ++e) acc[e] = fmaf(s_m[p * G + e], st[p * slot + d * G + e], acc[e]);
 #pragma unroll
