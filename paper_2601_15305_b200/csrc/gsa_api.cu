@@ -441,6 +441,8 @@ static int attn_fwd_impl(const gsa_params_t* p, const void* Q, const void* K, co
     if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(g1_logits) || !aligned16(out) ||
         !aligned16(idx) || (g2_logits && !aligned16(g2_logits)))
         return GSA_ERR_INVALID_ARG;
+    PartsOfCall parts;
+    if (ws_bytes < attn_ws_bytes(*p, g2_logits && plan_ws(*p, 0).prepass)) t_max_parts = kFewParts;
     if (!ws || !aligned16(ws) || ws_bytes < attn_ws_bytes(*p, false)) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     t_dev_status = (int32_t*)ws;
@@ -496,6 +498,8 @@ static int forward_impl(const gsa_params_t* p, const void* Q, const void* K, con
     if (!dense && (!qI || !kI || !w)) return GSA_ERR_INVALID_ARG;
     const void* ptrs[] = {Q, K, V, qI, kI, w, g1_logits, g2_logits, out, idx_out, kt_out, var_out};
     for (const void* q : ptrs) if (q && !aligned16(q)) return GSA_ERR_INVALID_ARG;
+    PartsOfCall parts;
+    if (ws_bytes < plan_ws(*p, slab_rows).total) t_max_parts = kFewParts;
     const WsPlan wp = plan_ws(*p, slab_rows);
     if (!ws || !aligned16(ws) || ws_bytes < wp.total) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
@@ -594,8 +598,13 @@ int gsa_forward_host(const gsa_params_t* p, const void* Q, const void* K, const 
                      const void* g2_logits, void* out, int32_t* kt_out, int32_t slab_rows, void* arena,
                      size_t arena_bytes, void* stream) {
     size_t need = 0;
+    PartsOfCall parts;
     int rc = gsa_forward_host_arena_bytes(p, slab_rows, &need);
     if (rc) return rc;
+    if (arena_bytes < need) {                              // (forward_impl makes the same choice from what is left for it)
+        t_max_parts = kFewParts;
+        gsa_forward_host_arena_bytes(p, slab_rows, &need);
+    }
     if (!Q || !K || !V || !qI || !kI || !w || !g1_logits || !out) return GSA_ERR_INVALID_ARG;
     if (!arena || !aligned16(arena) || arena_bytes < need) return GSA_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;

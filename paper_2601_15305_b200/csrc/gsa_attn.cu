@@ -50,7 +50,6 @@ constexpr int kVStages = 2;                // shared-memory stages of a warp's V
 constexpr int kRangeKeysDefault = 16384;   // keys per L2 range: K + V' rows of 16K tokens = 64 MB at the 1.7B shape
 constexpr int kMaxRanges = 48;
 constexpr int kPartKeys = 32;              // decode: fewest keys worth a parallel segment
-constexpr int kMaxParts = 64;              // most segments (and state slots) per index set
 
 struct AttnArgs {
     const __nv_bfloat16* Q;
@@ -617,7 +616,7 @@ AttnPlan plan_attn(const gsa_params_t& p) {
     // as many segments per index set as fill the GPU's warp slots once: one wave of longer items beat two waves of
     // shorter ones at the decode workload (attention 0.115 against 0.119 ms)
     int mp = (int)(((int64_t)sm_count() * kWarpsPrefill) / (idx_rows * p.n_kv));
-    mp = mp < 1 ? 1 : (mp > kMaxParts ? kMaxParts : mp);
+    mp = mp < 1 ? 1 : (mp > t_max_parts ? t_max_parts : mp);
     pl.slots = pl.mode == 1 ? mp : 1;
     pl.state_bytes = (size_t)pl.slots * idx_rows * row_state;
     pl.cuts_bytes = pl.mode == 0 && pl.n_ranges > 1 ? (size_t)idx_rows * pl.n_ranges * 4 : 0;
@@ -856,6 +855,8 @@ cudaError_t launch_masked_rows(const gsa_params_t& p, const AttnPlan& pl, const 
 }
 
 }  // namespace
+
+thread_local int t_max_parts = kMaxParts;
 
 size_t attn_scratch_bytes(const gsa_params_t& p) {
     const AttnPlan pl = plan_attn(p);

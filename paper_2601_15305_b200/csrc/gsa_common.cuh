@@ -167,6 +167,14 @@ int attn_tile_rows(const gsa_params_t& p, RowRange rr);
 
 // bytes of device scratch launch_sparse_attn needs for `p` (softmax state slots, range cuts)
 size_t attn_scratch_bytes(const gsa_params_t& p);
+// Most parallel segments of an index set for the call that this host thread is enqueueing (and for the two above).  An entry point
+// whose workspace has no room for the usual number does with the fewer: they are what fewer rows than SMs gain from, no need.
+constexpr int kMaxParts = 64, kFewParts = 16;
+extern thread_local int t_max_parts;
+struct PartsOfCall {
+    PartsOfCall() { t_max_parts = kMaxParts; }
+    ~PartsOfCall() { t_max_parts = kMaxParts; }
+};
 // keys per L2-resident key range of the sparse-attention gather (tuning knob)
 void set_attn_range_keys(int keys);
 int attn_range_keys();

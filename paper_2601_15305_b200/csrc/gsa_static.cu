@@ -67,6 +67,8 @@ extern "C" int gsa_sparse_gated_attn_fwd_static(const gsa_params_t* p, const voi
         !aligned16(idx) || !aligned16(out))
         return GSA_ERR_INVALID_ARG;
 
+    PartsOfCall parts;
+    t_max_parts = kFewParts;                                   // (the array's size is fixed: as much as possible is left to V')
     const size_t vg_bytes = (size_t)p->B * p->Lk * p->n_kv * p->d_h * 2;
     const size_t attn_bytes = (attn_scratch_bytes(*p) + 255) / 256 * 256;
     if (vg_bytes + attn_bytes > kStaticVgBytes) {
