@@ -1,0 +1,118 @@
+"""Where a kernel's work is cut: column widths of the projection's last wave, runs of the indexer's tiles across groups and batch
+elements, warps that share a row of the indexer loss, segments of a decode step's index sets."""
+import numpy as np
+import pytest
+import torch
+
+import gpu_util as U
+import oracle
+from paper_2601_15305_b200 import binding as gsa
+from paper_2601_15305_b200.inputs import CONFIGS, make_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+# rest of the whole tiles on 148 SMs: in quarters (8, 37 tiles), halves (72), whole (80), none (148); 8 .. 248 columns left over
+@pytest.mark.parametrize("M,N", [(1, 8), (130, 264), (1024, 256), (37 * 128, 256), (1024, 2304), (1280, 2048), (148 * 128, 256),
+                                 (999, 760), (300, 1272)])
+def test_gemm_tiles_of_every_width(M, N):
+    p = gsa.make_params(CONFIGS["tiny"].with_(name="gemm", B=1, Lq=M, Lk=M, n_h=4, n_kv=1, d_h=64))
+    gen = torch.Generator(device="cuda").manual_seed(M + N)
+    x = torch.randn(1, M, 4, 64, generator=gen, device="cuda").to(torch.bfloat16)
+    wt = (torch.randn(N, 256, generator=gen, device="cuda") / 16).to(torch.bfloat16)
+    u = torch.full((1, M, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    ws = torch.full((256,), 0xFF, dtype=torch.uint8, device="cuda")
+    gsa.gsa_output_projection(p, N, x, wt, u, ws)
+    torch.cuda.synchronize()
+    assert gsa.gsa_device_status(ws) == 0
+    want = x.reshape(M, 256).double() @ wt.double().T
+    # one rounding to bf16, whose 8 significant bits make half a unit at most 2^-8 of the value, behind fp32 sums of 256 products (each
+    # addition within 2^-24 of a sum of magnitudes below 64)
+    assert ((u[0].double() - want).abs() <= want.abs() / 256 + 64 * 256 * 2.0 ** -24).all()
+
+
+# heads per group of queries: 8, 4 (32 and 64 queries), 2, 1 (128 and 256: several key tiles more from one group to the next)
+@pytest.mark.parametrize("B,Lq,Lk,HI,dI", [(3, 301, 1300, 8, 64), (2, 700, 700, 4, 32), (5, 130, 999, 2, 32), (2, 600, 2500, 1, 64), (1, 5, 129, 8, 32)])
+def test_indexer_runs_cross_groups_and_batch_elements(B, Lq, Lk, HI, dI):
+    cfg = CONFIGS["l8k"].with_(name="runs", B=B, Lq=Lq, Lk=Lk, HI=HI, dI=dI, seed=300 + HI)
+    x = make_inputs(cfg)
+    sc = U.run_scores(cfg, U.to_dev(x)).cpu().numpy()
+    rows = np.arange(Lq)
+    for b in range(B):
+        want = oracle.scores(U.oracle_params(cfg), x["qI"], x["kI"], x["w"], None, rows, np.full_like(rows, b))
+        U.check_scores(sc[b], want, [Lk - Lq + int(t) + 1 for t in rows])
+
+
+# 10000 rows of small sets: a warp per row; the others: four.  weight_scale 40: the scores' bound is too wide to be the reference
+@pytest.mark.parametrize("L,k,weight_scale", [(10000, 40, 1.0), (700, 5, 1.0), (700, 40, 1.0), (700, 40, 40.0)])
+def test_indexer_loss_rows_on_one_and_four_warps(L, k, weight_scale):
+    cfg = CONFIGS["tiny"].with_(name="kl_split", B=1, Lq=L, Lk=L, k_base=k, k_min=k, k_max=2 * k, HI=4, dI=32, seed=310)
+    gen = torch.Generator(device="cuda").manual_seed(311)
+    bf = lambda *s: torch.randn(*s, generator=gen, device="cuda").mul_(32 ** -0.5 * 2).to(torch.bfloat16)  # noqa: E731
+    qI, kI = bf(1, L, 4, 32), bf(1, L, 32)
+    w = torch.rand(1, L, 4, generator=gen, device="cuda") * weight_scale
+    t = torch.arange(L, device="cuda")
+    kt = torch.minimum(t + 1, torch.randint(1, 2 * k + 1, (L,), generator=gen, device="cuda"))
+    order = torch.rand(L, L, generator=gen, device="cuda").masked_fill_(t[None, :] > t[:, None], 2.0)
+    idx = order.argsort(1)[:, :2 * k]
+    idx = idx.masked_fill(torch.arange(2 * k, device="cuda")[None] >= kt[:, None], L).sort(1).values
+    on = idx < L
+    target = torch.rand(L, 2 * k, generator=gen, device="cuda").masked_fill_(~on, 0.0)
+    target /= target.sum(1, keepdim=True)
+    idx32 = torch.where(on, idx, -1).to(torch.int32)[None].contiguous()
+    p = gsa.make_params(cfg)
+    out = dict(loss=torch.empty(1, L, device="cuda"), dqI=torch.empty_like(qI), dkI=torch.empty_like(kI), dw=torch.empty_like(w))
+    ws = torch.full((gsa.gsa_indexer_kl_workspace_bytes(p),), 0xFF, dtype=torch.uint8, device="cuda")
+    gsa.gsa_indexer_kl_bwd(p, qI, kI, w, None, idx32, kt.to(torch.int32)[None].contiguous(), target[None].contiguous(), out["loss"], out["dqI"],
+                           out["dkI"], out["dw"], None, ws)
+    torch.cuda.synchronize()
+    assert gsa.gsa_device_status(ws) == 0
+    q, key, wd = (v[0].double().requires_grad_() for v in (qI, kI, w))
+    scores = (torch.sigmoid(torch.einsum("thc,tkc->tkh", q, key[idx.clamp(max=L - 1)])) * wd[:, None]).sum(-1).masked_fill(~on, -torch.inf)
+    pd = target.double()
+    loss = (torch.where(on, pd * (pd.clamp(min=1e-300).log() - scores.log_softmax(1).masked_fill(~on, 0.0)), 0.0)).sum(1)
+    loss.sum().backward()
+    # fp32 sums of terms of magnitude |I| <= 4 weight_scale and log k; gradients round dX (and the results) to bf16 once
+    assert ((out["loss"][0].double() - loss).abs() <= 2e-3 * loss.abs() + 2e-5 * weight_scale).all()
+    for got, want in ((out["dqI"], q.grad), (out["dkI"], key.grad), (out["dw"], wd.grad)):
+        assert (got[0].double() - want).norm() <= 1e-2 * want.norm()
+
+
+def test_decode_workspace_with_room_for_fewer_segments():
+    """64 state slots are what the size query asks for; 16 are accepted, as are their results; less is refused."""
+    cfg = CONFIGS["decode"].with_(name="room", B=1, Lk=4000, k_base=2048, k_min=2048, k_max=2048, seed=321)
+    x = make_inputs(cfg)
+    d = U.to_dev(x)
+    p = gsa.make_params(cfg)
+    idx = torch.arange(0, 4000, 1, device="cuda").view(-1, 125)[:, :64].reshape(1, 1, -1).to(torch.int32).contiguous()
+    kt = torch.full((1, 1), 2048, dtype=torch.int32, device="cuda")
+    want, slot = gsa.gsa_attn_workspace_bytes(p, False), 8 * 2 * 130 * 4
+    got = {}
+    for name, n in (("all", want), ("few", want - 48 * slot), ("less", want - 48 * slot - 256)):
+        ws = torch.full((n,), 0xFF, dtype=torch.uint8, device="cuda")
+        out = torch.full_like(d["Q"], float("nan"))
+        if name == "less":
+            with pytest.raises(gsa.GsaError):
+                gsa.gsa_sparse_gated_attn_fwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx, kt, out, ws)
+            continue
+        gsa.gsa_sparse_gated_attn_fwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx, kt, out, ws)
+        assert gsa.gsa_device_status(ws) == 0
+        got[name] = out[:, 0].float().cpu().numpy()
+    o = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx[0].cpu().numpy(), kt[0].cpu().numpy(), np.zeros(1, np.int64),
+                    np.zeros(1, np.int64))
+    for v in got.values():
+        U.check_out(v, o)
+
+
+# one, two, 43 (sets of 48 keys a segment) and 64 segments; sequences enough that a set gets four; G = 1 and 8
+@pytest.mark.parametrize("B,k,n_h,n_kv,d_h", [(1, 32, 16, 8, 128), (1, 33, 16, 8, 128), (1, 2049, 16, 8, 128), (1, 2048, 8, 8, 64),
+                                              (2, 500, 8, 1, 128), (40, 130, 32, 8, 64)])
+def test_decode_sets_in_segments(B, k, n_h, n_kv, d_h):
+    cfg = CONFIGS["decode"].with_(name="segments", B=B, Lk=4000, n_h=n_h, n_kv=n_kv, d_h=d_h, k_base=k, k_min=k, k_max=k, seed=320)
+    x = make_inputs(cfg)
+    out, idx, kt, _ = U.run_forward(cfg, U.to_dev(x))
+    rows_b = np.arange(B)
+    o = oracle.forward(U.oracle_params(cfg), **x, rows_t=np.zeros(B, np.int32), rows_b=rows_b, want_scores=True)
+    assert (kt.cpu().numpy() == k).all()
+    U.check_forward_rows(U.oracle_params(cfg), x, o, out[:, 0].float().cpu().numpy(), idx[:, 0].cpu().numpy(), kt[:, 0].cpu().numpy(),
+                         np.zeros(B, np.int64), rows_b, [cfg.Lk] * B)
