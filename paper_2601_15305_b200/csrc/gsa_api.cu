@@ -426,6 +426,8 @@ int gsa_attn_workspace_bytes(const gsa_params_t* p, int32_t with_value_gate_prep
     int rc = check_params(p);
     if (rc) return rc;
     if (!bytes) return GSA_ERR_INVALID_ARG;
+    PartsOfCall parts;
+    t_max_parts = kFewParts;                               // (what the call needs; it splits sets further where it is given more)
     *bytes = attn_ws_bytes(*p, with_value_gate_prepass != 0);
     return GSA_OK;
 }
