@@ -73,10 +73,13 @@ inline int masked_block_rows(const gsa_params_t& p) { return 256 / (p.n_h / p.n_
 // Order of a tile kernel's CTAs: the longest blocks first, of as many (batch element, KV head) pairs abreast as have the tensors
 // that their CTAs stream together in the L2.  One pair after another leaves the last wave to long blocks (8K prefill 319 us of
 // tiles against 276 with all eight heads abreast, dense 2 x 3072 135 against 113); all pairs abreast at every length reads from
-// HBM what the L2 would have had (128K prefill 93.4 ms in all against 94.7, training step of 32K 31.3 against 31.7).
+// HBM what the L2 would have had (128K prefill 93.4 ms in all against 94.7, training step of 32K 31.3 against 31.7).  The groups are
+// of one size: a last group of one pair runs its long blocks alone (8K backward keys kernel, seven pairs and one, 552 us; all eight,
+// whose Q and do are 67 MB, 426; forward at 16K, seven and one, 985, four and four 879).
 inline int pairs_abreast(int pairs, double bytes_each) {
-    const double fit = 64e6 / bytes_each;
-    return fit >= pairs ? pairs : (fit < 1.0 ? 1 : (int)fit);
+    const int fit = 80e6 > bytes_each ? (int)(80e6 / bytes_each) : 1;
+    const int groups = (pairs + fit - 1) / fit;                   // (of one size, so that the last one is no straggler)
+    return (pairs + groups - 1) / groups;
 }
 __device__ __forceinline__ void tile_order(int item, int blocks, int pairs, int abreast, int* block_rank, int* pair) {
     const int group = item / (abreast * blocks), rest = item - group * abreast * blocks, n = min(abreast, pairs - group * abreast);
