@@ -46,6 +46,15 @@ __device__ __forceinline__ void mma_bf16_1688_l(float (&d)[4], uint32_t a0, uint
         : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
         : "r"(a0), "r"(a1), "r"(b0), "f"(0.f), "f"(0.f), "f"(0.f), "f"(0.f));
 }
+// As fast_sigmoid, but a NaN stays one (there the clamp makes it 2^-126): a loss that does not show it goes on as if nothing had
+// happened.  A rounded division in place of rcp.approx costs 8 to 30 % of the kernel and changes no error against fp64 in its second
+// digit (2000 rows of 256 keys, both: loss 1.75e-7, dw 1.0e-6).
+__device__ __forceinline__ float sigmoid_l(float x) {
+    float e, r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(e) : "f"(-kLog2eL * x), "f"(126.f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + ex2_approx_l(e)));
+    return r;
+}
 __device__ __forceinline__ void red_add_v4_l(float* addr, float x, float y, float z, float w) {
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
@@ -309,7 +318,7 @@ __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const K
                 f[i] = fmaxf(v, 0.f);
                 fp[i] = v > 0.f ? 1.f : 0.f;
             } else {
-                f[i] = fast_sigmoid(v);
+                f[i] = sigmoid_l(v);
                 fp[i] = f[i] * (1.0f - f[i]);
             }
         }

@@ -8,6 +8,7 @@ import gpu_util as U
 import oracle
 from paper_2601_15305_b200 import binding as gsa
 from paper_2601_15305_b200.inputs import CONFIGS, make_inputs
+from test_gpu_backward import _run_kl
 
 pytestmark = pytest.mark.gpu
 
@@ -76,6 +77,26 @@ def test_indexer_loss_rows_on_one_and_four_warps(L, k, weight_scale):
     assert ((out["loss"][0].double() - loss).abs() <= 2e-3 * loss.abs() + 2e-5 * weight_scale).all()
     for got, want in ((out["dqI"], q.grad), (out["dkI"], key.grad), (out["dw"], wd.grad)):
         assert (got[0].double() - want).norm() <= 1e-2 * want.norm()
+
+
+# 300 rows: four warps a row; 10000: one
+@pytest.mark.parametrize("L", [300, 10000])
+@pytest.mark.parametrize("where", ["qI", "kI", "w", "bI"])
+def test_a_nan_in_the_indexers_inputs_shows_in_the_loss(L, where):
+    """... and in the head weights' derivative of the rows that meet it, and in no other row's."""
+    cfg, row, key, k = CONFIGS["tiny"].with_(name="kl_nan", B=1, Lq=L, Lk=L, k_base=40, k_min=40, k_max=40, HI=8, dI=64, seed=312), 100, 5, 40
+    gen = torch.Generator(device="cuda").manual_seed(313)
+    bf = lambda *s: torch.randn(*s, generator=gen, device="cuda").mul_(0.125).to(torch.bfloat16)  # noqa: E731
+    d = dict(qI=bf(1, L, 8, 64), kI=bf(1, L, 64), w=torch.rand(1, L, 8, generator=gen, device="cuda"), bI=torch.zeros(8, device="cuda"))
+    t, j = torch.arange(L, device="cuda")[:, None], torch.arange(k, device="cuda")
+    kt = (t[:, 0] + 1).clamp(max=k).to(torch.int32)
+    idx = torch.where(j < kt[:, None], j, -1).to(torch.int32)[None].contiguous()
+    target = torch.where(j < kt[:, None], 1.0 / kt[:, None], 0.0)[None].contiguous()
+    hit = {"qI": t[:, 0] == row, "kI": t[:, 0] >= key, "w": t[:, 0] == row, "bI": t[:, 0] >= 0}[where]
+    d[where][{"qI": (0, row, 2, 7), "kI": (0, key, 7), "w": (0, row, 2), "bI": (3,)}[where]] = float("nan")
+    got = _run_kl(cfg, d, d["bI"], idx, kt[None].contiguous(), target, 0, L)
+    assert (torch.isnan(got["loss"][0]) == hit).all()
+    assert (torch.isnan(got["dw"][0]).any(-1) == hit).all()
 
 
 def test_decode_workspace_with_room_for_more_segments():
