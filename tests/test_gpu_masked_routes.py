@@ -77,6 +77,34 @@ def test_reference_that_moves_in_either_half_of_a_later_tile(jump):
     U.check_out(out[0][torch.from_numpy(rows).cuda()].float().cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("jump,key", [(8.5, 640 + 17), (10.0, 640 + 64 + 17), (11.5, 1152 + 9), (13.5, 1152 + 64 + 9)])
+def test_a_key_that_dominates_its_row_keeps_the_output_exact(jump, key):
+    """One key of every set exceeds all scores before it by `jump` (log2 domain) and alone has a value: the reference has moved to it, so
+    that its numerator is a bf16 value and the output is off by the rounding of the result only."""
+    cfg = TILES.with_(name="needle", B=1, Lq=900, Lk=1700)
+    x = make_inputs(cfg)
+    idx, kt = _sets(cfg, 213)
+    rows = [t for t in range(cfg.Lq) if key <= cfg.Lk - cfg.Lq + t]
+    for t in rows:
+        s = idx[0, t, :int(kt[0, t])]
+        s = torch.cat([s[s != key][:cfg.k_max - 1], torch.tensor([key], dtype=torch.int32)]).sort().values
+        idx[0, t, :len(s)], idx[0, t, len(s):], kt[0, t] = s, -1, len(s)
+    x["Q"] = (x["Q"].float() + 0.5).to(torch.bfloat16)
+    x["K"][:, key] = 2.0 * jump / 1.4427 / cfg.d_h ** 0.5
+    x["V"].zero_()
+    x["V"][:, key] = 1.0
+    x["g1"].fill_(40.0)
+    x["g2"].fill_(40.0)                             # (both gates are one)
+    out, n, general, status = _fwd(cfg, U.to_dev(x), idx, kt)
+    assert n == 4 and general == 0 and status == 0
+    for t in rows[::5]:
+        s = idx[0, t, :int(kt[0, t])].long()
+        k = x["K"][0, s].double().repeat_interleave(cfg.n_h // cfg.n_kv, 1)
+        p = torch.softmax((k * x["Q"][0, t].double()).sum(-1) / cfg.d_h ** 0.5, 0)[s == key][0]
+        # just below one: half a unit of bf16 is 2^-9, behind fp32 sums and exponentials of a few 1e-6
+        assert (out[0, t].double().cpu() - p[:, None]).abs().max() <= 2.0 ** -9 + 2e-5, t
+
+
 # ---- backward ------------------------------------------------------------------------------------------------------
 BWD = TILES.with_(name="bwd", Lk=1000, k_base=150, k_max=209, seed=240)
 
