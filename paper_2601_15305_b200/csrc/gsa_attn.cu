@@ -437,14 +437,26 @@ __global__ void __launch_bounds__(256) gsa_range_cuts_kernel(const int32_t* __re
 }
 
 // merge the state slots of a (row, head): out = (sum_p 2^(m_p - M) O_p) / (sum_p 2^(m_p - M) l_p) * sigmoid(g1)
-// A CTA takes kFinRows consecutive query rows; thread = (KV head, d), all G heads of the group.  With a
-// single slot per row (prefill) the loads of all rows are issued before any is used.  With several (decode) a CTA takes one row
-// and KV head, thread = (one of kFinGroups shares of the slots, d): one or two memory latencies, whatever the number of slots.
+//  * a single slot per row (mode 0, prefill): a CTA takes kFinRows consecutive query rows; thread = (KV head, d), all G heads of the
+//    group.  The loads of all rows are issued before any is used.
+//  * many slots (decode): a CTA takes one row and KV head, thread = (one of kFinGroups shares of the slots, d): one or two memory
+//    latencies, whatever the number of slots.  (In a kernel of its own ptxas gives this form 32 registers in place of 64 and its loads
+//    go out a few at a time: G = 4, 64 slots 12.1 us instead of 10.6.)
+//  * SERIAL, few slots: the same without shares, thread = d, one slot after another: a quarter of the threads and no barriers.  There
+//    are few slots where there are many CTAs (finalize_serial has the line).
 constexpr int kFinRows = 4;
 constexpr int kFinGroups = 4;
 
-template <int DH, int G>
-__global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __restrict__ state, const int32_t* __restrict__ kt,
+// Attention stage in us, shares against serial form, d_h = 128 (64 where four or eight heads share a KV head): 300 rows x 8 KV heads (one
+// slot), 16 keys 31.4 and 18.5, 256 keys 70.0 and 56.9; 64 x 8 (four), 128 keys 16.6 and 15.0, G = 8: 12.4 and 14.7; 56 x 8 (five),
+// 128 keys 16.5 and 14.6, G = 4: 11.1 and 11.9; 40 x 8 (seven), 2048 keys 94.1 and 95.3; 24 x 8 (twelve), sets in one segment 9.6 and 9.1,
+// G = 8: 8.7 and 9.8.
+inline bool finalize_serial(int G, int slots, int slots_used) {
+    return G <= 2 ? slots <= 6 || slots_used == 1 : slots <= 3;
+}
+
+template <int DH, int G, bool SERIAL>
+__global__ void __launch_bounds__(SERIAL ? DH : 1024) gsa_attn_finalize_kernel(const float* __restrict__ state, const int32_t* __restrict__ kt,
                                                                 const __nv_bfloat16* __restrict__ g1, __nv_bfloat16* __restrict__ out,
                                                                 RowRange rr, IdxLayout il, int64_t idx_rows, int Lq, int n_h,
                                                                 int n_kv, int k_max, int mode, int max_parts,
@@ -452,6 +464,34 @@ __global__ void __launch_bounds__(1024) gsa_attn_finalize_kernel(const float* __
     chain_wait();
     if (left_out(only_if, run_if)) return;
     constexpr int STATE_F = G * (DH + 2);
+    if constexpr (SERIAL) {
+        const RowId r = row_of(rr, il, (int)blockIdx.x);
+        const int g = blockIdx.y;
+        const float* __restrict__ st = state + ((int64_t)r.irow * n_kv + g) * STATE_F;
+        const int64_t slot = idx_rows * n_kv * STATE_F;
+        const int d = threadIdx.x;
+        const int k_eff = clamp_budget(kt[r.irow], k_max), np = k_eff > 0 ? parts_of(k_eff, max_parts) : 0;
+        float acc[G], mx[G], den[G];
+#pragma unroll
+        for (int e = 0; e < G; ++e) { acc[e] = 0.f; den[e] = 0.f; mx[e] = -INFINITY; }
+        for (int p = 0; p < np; ++p)
+#pragma unroll
+            for (int e = 0; e < G; ++e) mx[e] = fmaxf(mx[e], st[p * slot + G * DH + e]);
+        for (int p = 0; p < np; ++p)
+#pragma unroll
+            for (int e = 0; e < G; ++e) {
+                const float m = st[p * slot + G * DH + e], sc = m == -INFINITY ? 0.f : exp2f(m - mx[e]);
+                acc[e] = fmaf(sc, st[p * slot + d * G + e], acc[e]);
+                den[e] = fmaf(sc, st[p * slot + G * DH + G + e], den[e]);
+            }
+#pragma unroll
+        for (int e = 0; e < G; ++e) {
+            const size_t at = (((size_t)r.b * Lq + r.t) * n_h + g * G + e) * DH + d;
+            out[at] = __float2bfloat16_rn(den[e] != 0.f ? acc[e] / den[e] * fast_sigmoid(__bfloat162float(g1[at])) : 0.f);
+            if (lse && d == 0) lse[((size_t)r.b * Lq + r.t) * n_h + g * G + e] = (mx[e] + log2f(den[e])) * 0.6931471805599453f;
+        }
+        return;
+    }
     const int rows = rr.rows();
     if (mode == 0) {
         const int lr0 = blockIdx.x * kFinRows;
@@ -661,9 +701,10 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
         fr.q_begin = t_lo; fr.R = t_hi - t_lo;
         const dim3 fin_grid = pl.mode == 0 ? dim3((unsigned)((fr.rows() + kFinRows - 1) / kFinRows), 1)
                                            : dim3((unsigned)fr.rows(), (unsigned)a.n_kv);
-        launch_chained(gsa_attn_finalize_kernel<DH, G>, fin_grid, pl.mode == 0 ? fin_threads : kFinGroups * DH, 0, st,
-            a.state, a.kt, g1, out, fr, a.il, a.idx_rows, p.Lq, p.n_h, p.n_kv, p.k_max, pl.mode, pl.slots, a.lse,
-            a.only_if, a.run_if);
+        const bool serial = pl.mode == 1 && finalize_serial(G, pl.slots, parts_of(p.k_max, pl.slots));
+        launch_chained(serial ? gsa_attn_finalize_kernel<DH, G, true> : gsa_attn_finalize_kernel<DH, G, false>, fin_grid,
+            pl.mode == 0 ? fin_threads : (serial ? DH : kFinGroups * DH), 0, st, a.state, a.kt, g1, out, fr, a.il, a.idx_rows, p.Lq,
+            p.n_h, p.n_kv, p.k_max, pl.mode, pl.slots, a.lse, a.only_if, a.run_if);
         ++g_launches;
         cudaError_t fe = cudaGetLastError();
         if (!a.only_if) timeline_mark(kStageFinalize, st);

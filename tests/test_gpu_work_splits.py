@@ -137,3 +137,16 @@ def test_decode_sets_in_segments(B, k, n_h, n_kv, d_h):
     assert (kt.cpu().numpy() == k).all()
     U.check_forward_rows(U.oracle_params(cfg), x, o, out[:, 0].float().cpu().numpy(), idx[:, 0].cpu().numpy(), kt[:, 0].cpu().numpy(),
                          np.zeros(B, np.int64), rows_b, [cfg.Lk] * B)
+
+
+# slots merged one after another: four; six (G = 1); two, of which a short set fills one; three (G = 8); and in shares: seven, four (G = 4)
+@pytest.mark.parametrize("B,Lq,k,n_h,n_kv,d_h", [(64, 1, 200, 16, 8, 128), (49, 1, 256, 8, 8, 128), (37, 4, 40, 16, 8, 128), (197, 2, 100, 16, 2, 64),
+                                                 (42, 1, 300, 16, 8, 64), (74, 1, 150, 32, 8, 64)])
+def test_merge_of_few_slots(B, Lq, k, n_h, n_kv, d_h):
+    cfg = CONFIGS["decode"].with_(name="merge", B=B, Lq=Lq, Lk=600, n_h=n_h, n_kv=n_kv, d_h=d_h, k_base=k, k_min=k // 2, k_max=k, seed=330)
+    x = make_inputs(cfg)
+    out, idx, kt, _ = U.run_forward(cfg, U.to_dev(x))
+    rows_t, rows_b = np.tile(np.arange(Lq), B), np.repeat(np.arange(B), Lq)
+    o = oracle.attn(U.oracle_params(cfg), x["Q"], x["K"], x["V"], x["g1"], x["g2"], idx.cpu().numpy().reshape(B * Lq, -1), kt.cpu().numpy().reshape(-1),
+                    rows_t, rows_b)
+    U.check_out(out.float().cpu().numpy().reshape(B * Lq, n_h, d_h), o)
