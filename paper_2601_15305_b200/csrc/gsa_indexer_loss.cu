@@ -20,7 +20,7 @@
 //    Bound: latency of the gathered rows and instructions, about 260 a tile and sweep, then the reductions.  8192 rows of 2048 keys
 //    1.09 ms, 32768 rows 5.0 ms, 2 x 2051 of 256 68 us (1.53, 6.49 ms and 91 us with one warp a row, copies one tile ahead, 8-byte
 //    reductions and a division in every sigmoid).
-#include "gsa_common.cuh"
+#include "gsa_masked.cuh"
 
 namespace gsa {
 
@@ -228,10 +228,8 @@ struct KlArgs {
 };
 
 // W: warps of a row.  One warp per row (four rows a CTA) leaves few rows to the latency of their tiles, one after another; four warps
-// share a row's tiles then, and their sums meet in shared memory (launch_kl_t has the rule).
+// share a row's tiles then, and their sums meet in shared memory (kl_four_warps has the rule).
 constexpr int kKlStages = 3;
-constexpr int kKlRowsPerSm = 64;                       // fewer rows an SM, or sets of so many keys: four warps a row
-constexpr int kKlLongSet = 640;
 
 template <int DI, int HI, int W>
 __global__ void __launch_bounds__(kLossWarps * 32) gsa_indexer_kl_kernel(const KlArgs a) {
@@ -542,13 +540,28 @@ cudaError_t launch_probs_t(const ProbsArgs& a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// Four warps a row?  By the keys that a row selects on average, against a line that rises with the rows an SM has: few rows leave warps
+// idle, many pay for the start and the end of a row.  Time with four warps over time with one (d^I = 64; 32):
+//   rows      4 an SM (600)       8 (1200)             24 (3500)           64 (9400)            95 (14000)
+//   32 keys   0.94; 0.97          1.25; 1.10           1.29; 1.19          1.84; 1.28           2.09; 1.35
+//   128       0.77; 0.75          1.00; 0.93           1.00; 1.01          1.20; 1.10           1.25; 1.14
+//   256       0.70; 0.62          0.92; 0.80           0.82; 0.99          1.05; 0.98           1.10; 1.04
+//   768                           0.70; 0.69           0.82; 0.87          0.95; 0.92           0.97; 1.00
+//   2048                                               0.90; 0.82          0.99; 0.82           1.00; 1.66
+// (the last: with d^I = 32 the additions to one key's sums, 22000 rows of 768 keys 2.02.)
+bool kl_four_warps(const gsa_params_t& p, const RowRange& rr) {
+    const double rows = rr.rows(), keys = rows_work(p, rr.nb, rr.q_begin, rr.R, 1).selected / rows, per_sm = rows / sm_count();
+    if (per_sm <= 5) return keys >= 24;
+    if (per_sm <= 9) return keys >= 2 * p.dI;
+    if (per_sm <= 64) return keys >= 3.5 * p.dI;
+    return p.dI >= 64 && keys >= 640;
+}
+
 template <int DI, int HI>
-cudaError_t launch_kl_t(const KlArgs& a, int k_base, cudaStream_t st) {
+cudaError_t launch_kl_t(const KlArgs& a, bool four_warps, cudaStream_t st) {
     constexpr int smem = kLossWarps * (kKlStages * 16 + 2 * 8) * (DI + 8) * 2;
     const int64_t rows = a.rr.rows();
-    // us with four warps a row and with one: 2 x 2051 rows of 256 keys 68 and 75, 8192 of 2048 1091 and 1212, 32768 of 2048 5018 and
-    // 5153; 4 x 8192 of 400 739 and 706 (start and end of a row show)
-    if (rows < (int64_t)kKlRowsPerSm * sm_count() || k_base >= kKlLongSet)
+    if (four_warps)
         launch_chained(gsa_indexer_kl_kernel<DI, HI, kLossWarps>, (unsigned)rows, kLossWarps * 32, smem, st, a);
     else
         launch_chained(gsa_indexer_kl_kernel<DI, HI, 1>, (unsigned)((rows + kLossWarps - 1) / kLossWarps), kLossWarps * 32, smem, st, a);
@@ -589,7 +602,7 @@ cudaError_t launch_indexer_kl(const gsa_params_t& p, RowRange rr, const __nv_bfl
         a.dqI = dqI; a.dw = dw; a.dkI32 = dkI32; a.dbI = dbI; a.rr = rr; a.il = il;
         a.Lq = p.Lq; a.Lk = p.Lk; a.k_max = p.k_max; a.act = p.act;
         e = cudaErrorInvalidValue;
-#define GSA_KL_CASE(DI_, HI_) if (p.dI == DI_ && p.HI == HI_) e = launch_kl_t<DI_, HI_>(a, p.k_base, st)
+#define GSA_KL_CASE(DI_, HI_) if (p.dI == DI_ && p.HI == HI_) e = launch_kl_t<DI_, HI_>(a, kl_four_warps(p, rr), st)
         GSA_KL_CASE(64, 8); GSA_KL_CASE(64, 4); GSA_KL_CASE(64, 2); GSA_KL_CASE(64, 1);
         GSA_KL_CASE(32, 8); GSA_KL_CASE(32, 4); GSA_KL_CASE(32, 2); GSA_KL_CASE(32, 1);
 #undef GSA_KL_CASE

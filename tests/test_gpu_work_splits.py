@@ -79,6 +79,38 @@ def test_indexer_loss_rows_on_one_and_four_warps(L, k, weight_scale):
         assert (got[0].double() - want).norm() <= 1e-2 * want.norm()
 
 
+# four warps a row: few rows, among them some whose set is a tile or less, and many with long sets (of every visible key, too); one
+# warp: short sets.  ReLU and weights of 40: the reference of the exponentials moves
+@pytest.mark.parametrize("L,k,HI,dI,act,weight_scale,k_mode", [
+    (500, 48, 8, 64, 0, 1.0, 0), (500, 48, 8, 64, 1, 1.0, 0), (300, 300, 4, 32, 0, 40.0, 3), (1500, 300, 2, 64, 1, 1.0, 0),
+    (10000, 24, 8, 64, 0, 1.0, 0), (10000, 24, 8, 64, 1, 1.0, 0), (10000, 24, 8, 64, 0, 40.0, 0), (2000, 40, 1, 32, 1, 1.0, 0)])
+def test_indexer_loss_of_both_forms_with_bias(L, k, HI, dI, act, weight_scale, k_mode):
+    cfg = CONFIGS["tiny"].with_(name="kl_forms", B=1, Lq=L, Lk=L, k_base=min(k, 8) if k_mode else k, k_min=1, k_max=k, HI=HI, dI=dI, seed=314)
+    gen = torch.Generator(device="cuda").manual_seed(315)
+    bf = lambda *s: torch.randn(*s, generator=gen, device="cuda").mul_(2 * dI ** -0.5).to(torch.bfloat16)  # noqa: E731
+    d = dict(qI=bf(1, L, HI, dI), kI=bf(1, L, dI), w=torch.rand(1, L, HI, generator=gen, device="cuda") * weight_scale)
+    bI = torch.randn(HI, generator=gen, device="cuda") * 0.2
+    t, j = torch.arange(L, device="cuda")[:, None], torch.arange(k, device="cuda")
+    kt = torch.minimum(t[:, 0] + 1, torch.full((L,), k, device="cuda") if k_mode else torch.randint(1, k + 1, (L,), generator=gen, device="cuda"))
+    idx = j * (t + 1) // kt[:, None]                                  # ascending, spread over what the row sees
+    on = j < kt[:, None]
+    target = torch.rand(L, k, generator=gen, device="cuda").masked_fill_(~on, 0.0)
+    target /= target.sum(1, keepdim=True)
+    got = _run_kl(cfg, d, bI, torch.where(on, idx, -1).to(torch.int32)[None].contiguous(), kt.to(torch.int32)[None].contiguous(),
+                  target[None].contiguous(), 0, L, act=act, k_mode=k_mode)
+    q, key, wd, b = (v.double().requires_grad_() for v in (d["qI"][0], d["kI"][0], d["w"][0], bI))
+    x = torch.einsum("thc,tkc->tkh", q, key[idx.clamp(max=L - 1)]) + b
+    scores = ((torch.relu(x) if act else torch.sigmoid(x)) * wd[:, None]).sum(-1).masked_fill(~on, -torch.inf)
+    pd = target.double()
+    loss = torch.where(on, pd * (pd.clamp(min=1e-300).log() - scores.log_softmax(1).masked_fill(~on, 0.0)), 0.0).sum(1)
+    loss.sum().backward()
+    # fp32 sums of terms of magnitude |I| <= HI weight_scale and log k; gradients round dX (and the results) to bf16 once
+    assert ((got["loss"][0].double() - loss).abs() <= 2e-3 * loss.abs() + 1e-5 * HI * weight_scale).all()
+    for name, want in (("dqI", q.grad), ("dkI", key.grad), ("dw", wd.grad)):
+        assert (got[name][0].double() - want).norm() <= 1e-2 * want.norm(), name
+    assert (got["dbI"].double() - b.grad).norm() <= 1e-2 * b.grad.norm() + 1e-6 * L ** 0.5 * weight_scale
+
+
 # 300 rows: four warps a row; 10000: one
 @pytest.mark.parametrize("L", [300, 10000])
 @pytest.mark.parametrize("where", ["qI", "kI", "w", "bI"])
