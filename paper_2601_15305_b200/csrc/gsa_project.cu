@@ -6,7 +6,7 @@
 //     q^I, k^I, g1, g2 are rounded to bf16 once; head weights leave as fp32 sigmoid(C).
 //
 // A persistent CTA walks output tiles of 128 tokens x 256 columns (or narrower ones, TileList).  Warp 0 feeds a ring of shared-
-// memory stages by TMA (a 128 x 64 block of H and up to four 64 x 64 blocks of Wt per stage, 128-byte
+// memory stages by TMA (a 128 x 64 block of H and a 256 x 64 block of Wt, or 64 x 64 ones, per stage, 128-byte
 // swizzle), warp 1 issues the MMAs (four k-steps per stage) and owns the TMEM allocation, warps
 // 2..9 are the epilogue.  Two 256-column accumulators alternate, so the MMAs of the next tile run
 // while the epilogue converts and stores the current one.  Rows and columns of a tile that fall
@@ -35,18 +35,28 @@ constexpr int kNBars = 2 * kPStages + 4 + 1;
 constexpr int kOffTmem = kOffBar + kNBars * 8;
 constexpr int kOffAbort = kOffTmem + 8;
 constexpr int kSmemTotal = kOffAbort + 8 + 1024;        // slack to align the base to 1024
-constexpr int kBoxN = 64;                               // columns of one copy of Wt
+constexpr int kBoxN = 64;                               // columns of a copy of Wt for tiles that are not whole (a whole one takes a
+                                                        // single copy: four cost 2 to 4 %, 16384 tokens' output 110 us against 107)
 
 // Output tiles in the order of their width: all whole ones that fill waves of the SMs; the rest of the whole ones, in halves or quarters
 // if the last wave has room for them; the columns that are left of the last 256.  8192 tokens: 896 whole tiles and 64 of 72 columns,
 // 6.1 waves and a short one instead of 7; the output projection's 512, 3 waves and one of halves instead of 4.  Both calls together
 // 192.8 -> 189.7 us: the GPU is at its power limit there, so that idle SMs cost less than their share.
+// The columns left over come at the end only while the activations are still in the L2 then: 16384 x 2048 (67 MB) 198.5 us, and 194.4
+// with each token tile's next to its other tiles; 40000 tokens 488 and 466; 5000 (20 MB) 62.6 and 65.8, 12000 (49 MB) 146.7 and 146.5.
+constexpr int64_t kTokensInL2 = 50 << 20;
 struct TileList {
     int32_t cols;                  // whole column tiles of a token tile
+    int32_t among;                 // the columns left over follow each token tile's whole tiles
     int32_t whole, pieces, split, narrow, width_left;      // items of each kind; pieces a tile is cut into; columns left over
     __host__ __device__ int items() const { return whole + pieces + narrow; }
     __device__ void get(int i, int* m0, int* n0, int* width) const {
-        if (i < whole + pieces) {
+        if (among) {
+            const int c = i % (cols + 1);
+            *m0 = i / (cols + 1) * kTileM;
+            *n0 = c * kTileN;
+            *width = c < cols ? kTileN : width_left;
+        } else if (i < whole + pieces) {
             const int j = i - whole, t = j < 0 ? i : whole + j / split, w = j < 0 ? kTileN : kTileN / split;
             *m0 = t / cols * kTileM;
             *n0 = t % cols * kTileN + (j < 0 ? 0 : j % split * w);
@@ -58,7 +68,7 @@ struct TileList {
         }
     }
 };
-inline TileList tile_list(int m_tiles, int N, int sms) {
+inline TileList tile_list(int m_tiles, int N, int K, int sms) {
     TileList l;
     l.cols = N / kTileN;
     l.width_left = N % kTileN;
@@ -67,6 +77,7 @@ inline TileList tile_list(int m_tiles, int N, int sms) {
     l.split = rest * 4 + l.narrow <= sms ? 4 : (rest * 2 + l.narrow <= sms ? 2 : 1);
     l.pieces = l.split > 1 ? rest * l.split : 0;
     l.whole = l.split > 1 ? tiles - rest : tiles;
+    l.among = l.split == 1 && l.narrow > 0 && (int64_t)m_tiles * kTileM * K * 2 > kTokensInL2;
     return l;
 }
 
@@ -86,7 +97,7 @@ struct ProjArgs {
 
 __global__ void __launch_bounds__(kPThreads, 1)
 gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ CUtensorMap tm_w,
-                   const ProjArgs a) {
+                   const __grid_constant__ CUtensorMap tm_w_box, const ProjArgs a) {
     chain_wait();
     {   // an earlier CTA or launch gave up: leave, all threads together (one thread reads the word)
         __shared__ int s_go;
@@ -141,7 +152,9 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
             for (int tile = blockIdx.x; tile < n_tiles_total && !gave_up && !*s_abort; tile += gridDim.x) {
                 int m0, n0, width;
                 a.tiles.get(tile, &m0, &n0, &width);
-                const int boxes = (width + kBoxN - 1) / kBoxN;
+                const bool whole = width == kTileN;
+                const int boxes = whole ? 1 : (width + kBoxN - 1) / kBoxN, bytes = kA_BYTES + (whole ? kTileN : boxes * kBoxN) * kBlockK * 2;
+                const CUtensorMap* const box = whole ? &tm_w : &tm_w_box;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     const uint32_t it = copies_issued;
                     const int s = it % kPStages;
@@ -149,11 +162,11 @@ gsa_project_kernel(const __grid_constant__ CUtensorMap tm_h, const __grid_consta
                     if (it == 0 && a.withhold_first) {
                         first_withheld = true;             // (counted as issued; the give-up path skips it)
                     } else {
-                        mbar_expect_tx(bar_full(s), kA_BYTES + boxes * kBoxN * kBlockK * 2);
+                        mbar_expect_tx(bar_full(s), bytes);
                         const uint32_t dst = sbase + s * kStageBytes;
                         tma_load_2d(dst, &tm_h, kb * kBlockK, m0, bar_full(s));
                         for (int c = 0; c < boxes; ++c)
-                            tma_load_2d(dst + kA_BYTES + c * kBoxN * kBlockK * 2, &tm_w, kb * kBlockK, n0 + c * kBoxN, bar_full(s));
+                            tma_load_2d(dst + kA_BYTES + c * kBoxN * kBlockK * 2, box, kb * kBlockK, n0 + c * kBoxN, bar_full(s));
                     }
                     copies_issued = it + 1;
                 }
@@ -299,15 +312,16 @@ cudaError_t launch_project(const gsa_params_t& p, int d_model, const __nv_bfloat
     a.M = p.B * p.Lk; a.K = d_model; a.N = project_columns(p);
     a.n_q = p.HI * p.dI; a.n_k = p.dI; a.HI = p.HI; a.n_g1 = p.n_h * p.d_h; a.n_g2 = p.n_kv * p.d_h;
     const int sms = sm_count();
-    a.tiles = tile_list((a.M + kTileM - 1) / kTileM, a.N, sms);
+    a.tiles = tile_list((a.M + kTileM - 1) / kTileM, a.N, a.K, sms);
     a.wait_cycles = wait_limit_cycles();
     a.withhold_first = withhold_first_copy() ? 1 : 0;
-    CUtensorMap tm_h, tm_w;
+    CUtensorMap tm_h, tm_w, tm_w_box;
     if (!make_kblock_tmap(&tm_h, H, (uint64_t)a.M, (uint64_t)a.K, kTileM)) return cudaErrorUnknown;
-    if (!make_kblock_tmap(&tm_w, Wt, (uint64_t)a.N, (uint64_t)a.K, kBoxN)) return cudaErrorUnknown;
+    if (!make_kblock_tmap(&tm_w, Wt, (uint64_t)a.N, (uint64_t)a.K, kTileN)) return cudaErrorUnknown;
+    if (!make_kblock_tmap(&tm_w_box, Wt, (uint64_t)a.N, (uint64_t)a.K, kBoxN)) return cudaErrorUnknown;
     cudaError_t e = cudaFuncSetAttribute(gsa_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal);
     if (e != cudaSuccess) return e;
-    launch_chained(gsa_project_kernel, (unsigned)(a.tiles.items() < sms ? a.tiles.items() : sms), kPThreads, kSmemTotal, st, tm_h, tm_w, a);
+    launch_chained(gsa_project_kernel, (unsigned)(a.tiles.items() < sms ? a.tiles.items() : sms), kPThreads, kSmemTotal, st, tm_h, tm_w, tm_w_box, a);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -322,15 +336,16 @@ cudaError_t launch_gemm_bf16(int M, int K, int N, const __nv_bfloat16* A, const 
     a.M = M; a.K = K; a.N = N;
     a.n_q = N; a.n_k = 0; a.HI = 0; a.n_g1 = 0; a.n_g2 = 0;
     const int sms = sm_count();
-    a.tiles = tile_list((M + kTileM - 1) / kTileM, N, sms);
+    a.tiles = tile_list((M + kTileM - 1) / kTileM, N, K, sms);
     a.wait_cycles = wait_limit_cycles();
     a.withhold_first = withhold_first_copy() ? 1 : 0;
-    CUtensorMap tm_a, tm_b;
+    CUtensorMap tm_a, tm_b, tm_b_box;
     if (!make_kblock_tmap(&tm_a, A, (uint64_t)M, (uint64_t)K, kTileM)) return cudaErrorUnknown;
-    if (!make_kblock_tmap(&tm_b, Bt, (uint64_t)N, (uint64_t)K, kBoxN)) return cudaErrorUnknown;
+    if (!make_kblock_tmap(&tm_b, Bt, (uint64_t)N, (uint64_t)K, kTileN)) return cudaErrorUnknown;
+    if (!make_kblock_tmap(&tm_b_box, Bt, (uint64_t)N, (uint64_t)K, kBoxN)) return cudaErrorUnknown;
     cudaError_t e = cudaFuncSetAttribute(gsa_project_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal);
     if (e != cudaSuccess) return e;
-    launch_chained(gsa_project_kernel, (unsigned)(a.tiles.items() < sms ? a.tiles.items() : sms), kPThreads, kSmemTotal, st, tm_a, tm_b, a);
+    launch_chained(gsa_project_kernel, (unsigned)(a.tiles.items() < sms ? a.tiles.items() : sms), kPThreads, kSmemTotal, st, tm_a, tm_b, tm_b_box, a);
     ++g_launches;
     return cudaGetLastError();
 }

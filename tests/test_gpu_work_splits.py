@@ -17,6 +17,16 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("M,N", [(1, 8), (130, 264), (1024, 256), (37 * 128, 256), (1024, 2304), (1280, 2048), (148 * 128, 256),
                                  (999, 760), (300, 1272)])
 def test_gemm_tiles_of_every_width(M, N):
+    _check_gemm(M, N)
+
+
+# more activations than the L2 holds: the columns left over (8, 200) follow each token tile's whole tiles (one, two)
+@pytest.mark.parametrize("M,N", [(103000, 264), (102273, 712)])
+def test_gemm_columns_left_over_beside_the_whole_tiles(M, N):
+    _check_gemm(M, N)
+
+
+def _check_gemm(M, N):
     p = gsa.make_params(CONFIGS["tiny"].with_(name="gemm", B=1, Lq=M, Lk=M, n_h=4, n_kv=1, d_h=64))
     gen = torch.Generator(device="cuda").manual_seed(M + N)
     x = torch.randn(1, M, 4, 64, generator=gen, device="cuda").to(torch.bfloat16)
