@@ -101,6 +101,8 @@ typedef struct gsa_params {
  * Bytes of device workspace gsa_forward (and the per-stage calls) need for `p`.
  * `slab_rows` is the number of query rows whose fp32 score rows gsa_forward keeps
  * resident at a time (0 = library default: about 4 GiB of score rows, at least 32 rows).
+ * The size counts every parallel segment of gsa_sparse_gated_attn_fwd; gsa_forward does with 16 where less is
+ * given and accepts as little as that takes.
  * Host call; writes *bytes.
  */
 int gsa_workspace_bytes(const gsa_params_t *p, int32_t slab_rows, size_t *bytes);
@@ -258,6 +260,13 @@ int gsa_adaptive_topk(const gsa_params_t *p, const float *scores, int64_t row_st
  *       segments).  With gsa_attn_workspace_bytes(p, 1) bytes there is room for the gated values as
  *       well and G2 runs as one streaming pre-pass when that is cheaper than gating the gathered
  *       rows; otherwise the g2 rows are gathered with K and V.
+ *       Calls of few rows (decode) walk a set in parallel segments of at least 32 keys, up to
+ *       n = min(64, 16 * multiprocessors / (B * Lq * n_kv)) of them.  The size that the query returns
+ *       counts at most 16; all n are used if ws has room for the others as well, that is for
+ *       (n - 16) * B * Lq * n_h * (d_h + 2) * 4 bytes more, rounded up to a multiple of 256 (one
+ *       stream with 16 heads of 128: 399360 bytes).  Two calls that differ in that room differ in the rounding
+ *       of their outputs (a segment's softmax numerators are rounded to bf16 against the
+ *       segment's own reference), not in their error; with equal ws_bytes they return the same bits.
  */
 int gsa_attn_workspace_bytes(const gsa_params_t *p, int32_t with_value_gate_prepass, size_t *bytes);
 int gsa_sparse_gated_attn_fwd(const gsa_params_t *p, const void *Q, const void *K, const void *V,
@@ -368,7 +377,8 @@ int gsa_select_fallback_rows(const void *ws, void *stream, int32_t *rows_out);
  */
 int gsa_attn_tile_rows(const gsa_params_t *p, int32_t *fwd_rows, int32_t *bwd_tiles);
 
-/* Number of kernel launches the library has enqueued so far in this process (host counter). */
+/* Number of kernel launches the library has enqueued so far in this process (host counter).  The small kernel that
+ * zeroes a call's status word and sums ahead of its other launches is not counted, as a memset would not be. */
 int64_t gsa_launch_count(void);
 
 /*

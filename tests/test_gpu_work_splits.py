@@ -167,6 +167,30 @@ def test_decode_workspace_with_room_for_more_segments():
         U.check_out(v, o)
 
 
+def test_segments_by_the_room_of_the_workspace():
+    """The 48 state slots behind the first 16 are written if there is room for all of them, and nothing behind those 16 otherwise; calls with
+    equal workspaces return the same bits."""
+    cfg = CONFIGS["decode"].with_(name="room", B=1, Lk=4000, k_base=2048, k_min=2048, k_max=2048, seed=322)
+    d = U.to_dev(make_inputs(cfg))
+    p = gsa.make_params(cfg)
+    idx = torch.arange(0, 4000, 1, device="cuda").view(-1, 125)[:, :64].reshape(1, 1, -1).to(torch.int32).contiguous()
+    kt = torch.full((1, 1), 2048, dtype=torch.int32, device="cuda")
+    want, slot = gsa.gsa_attn_workspace_bytes(p, False), cfg.n_h * (cfg.d_h + 2) * 4
+    assert 256 + 16 * slot <= want < 512 + 16 * slot
+
+    def run(n):
+        ws, out = torch.full((n,), 0xFF, dtype=torch.uint8, device="cuda"), torch.empty_like(d["Q"])
+        gsa.gsa_sparse_gated_attn_fwd(p, d["Q"], d["K"], d["V"], d["g1"], d["g2"], idx, kt, out, ws)
+        assert gsa.gsa_device_status(ws) == 0
+        return out, ws
+
+    out, ws = run(want + 48 * slot)
+    assert (ws[256:256 + 64 * slot].view(64, slot) != 0xFF).any(1).all() and torch.equal(out, run(want + 48 * slot)[0])
+    for n in (want, want + 48 * slot - 256):
+        out, ws = run(n)
+        assert (ws[want:] == 0xFF).all() and torch.equal(out, run(n)[0])
+
+
 # one, two, 43 (sets of 48 keys a segment) and 64 segments; sequences enough that a set gets four; G = 1 and 8
 @pytest.mark.parametrize("B,k,n_h,n_kv,d_h", [(1, 32, 16, 8, 128), (1, 33, 16, 8, 128), (1, 2049, 16, 8, 128), (1, 2048, 8, 8, 64),
                                               (2, 500, 8, 1, 128), (40, 130, 32, 8, 64)])
