@@ -541,20 +541,16 @@ cudaError_t launch_probs_t(const ProbsArgs& a, cudaStream_t st) {
 }
 
 // Four warps a row?  By the keys that a row selects on average, against a line that rises with the rows an SM has: few rows leave warps
-// idle, many pay for the start and the end of a row.  Time with four warps over time with one (d^I = 64; 32):
-//   rows      4 an SM (600)       8 (1200)             24 (3500)           64 (9400)            95 (14000)
-//   32 keys   0.94; 0.97          1.25; 1.10           1.29; 1.19          1.84; 1.28           2.09; 1.35
-//   128       0.77; 0.75          1.00; 0.93           1.00; 1.01          1.20; 1.10           1.25; 1.14
-//   256       0.70; 0.62          0.92; 0.80           0.82; 0.99          1.05; 0.98           1.10; 1.04
-//   768                           0.70; 0.69           0.82; 0.87          0.95; 0.92           0.97; 1.00
-//   2048                                               0.90; 0.82          0.99; 0.82           1.00; 1.66
-// (the last: with d^I = 32 the additions to one key's sums, 22000 rows of 768 keys 2.02.)
+// idle, many pay for the start and the end of a row.  Time with four warps over time with one, on sets that the selection made (average
+// keys: ratio), d^I = 64; with 32 the same within 0.1 but for the shortest sets (1.2 to 1.5 where 64 has 1.5 to 2.4):
+//   rows an SM   3  16: 0.99   40: 0.79    93: 0.60                  41  102: 1.22  202: 1.00  301: 0.92   620: 0.81
+//                5  42: 1.10   66: 0.95   101: 0.78                  81  135: 1.18  285: 0.98  422: 0.94   809: 0.90
+//               11  65: 1.13   99: 0.96   184: 0.82                 162  304: 1.10  456: 1.02  645: 0.98  1953: 0.94
+//               20  65: 1.31  101: 1.09   141: 1.00   199: 0.90     221  400: 1.05                        1800: 0.97
 bool kl_four_warps(const gsa_params_t& p, const RowRange& rr) {
     const double rows = rr.rows(), keys = rows_work(p, rr.nb, rr.q_begin, rr.R, 1).selected / rows, per_sm = rows / sm_count();
-    if (per_sm <= 5) return keys >= 24;
-    if (per_sm <= 9) return keys >= 2 * p.dI;
-    if (per_sm <= 64) return keys >= 3.5 * p.dI;
-    return p.dI >= 64 && keys >= 640;
+    const double line = per_sm <= 5.0 ? 16.0 : 50.0 + 3.0 * per_sm;
+    return keys >= (line < 640.0 ? line : 640.0);
 }
 
 template <int DI, int HI>
