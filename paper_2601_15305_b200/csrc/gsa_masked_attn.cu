@@ -8,7 +8,7 @@
 // score the same half of the next tile behind each product.  A K and a V' tile are fetched once for both.  Thread = row: no
 // shuffles anywhere.
 //
-// Softmax reference: as in the gather kernel, it moves only when a selected score exceeds it by more than 2^8, so the
+// Softmax reference: it moves only when the numerators' sum shows that a selected score may exceed it by more than 2^8, so the
 // accumulator in TMEM is touched by the softmax warps on a row's first tiles only.  Masked scores are replaced by
 // -inf before the exponentials; fp32 everywhere except P (bf16, as in the gather kernel).  The reference is
 // set a little above the maximum it is taken from: that maximum may come from very few keys (a row of 50K keys has three selected
@@ -171,10 +171,11 @@ constexpr int kFwdThreads = 384;
 // its output exact (with 1/16, 2 % more error in dQ and dK, whose dominating terms cancel).  Over spreads of the scores from
 // 0.003 to 3 the finest of 0, 0.02, 0.05, 1/16, 0.1, 0.2 and 0.4 on the whole.
 constexpr float kRefMargin = 0.063362061f;
-// The reference moves where a selected score exceeds it by more than 2^8.  A numerator above 2^8 makes the sum of its 64 one, too, and the
-// sum is at hand, where a maximum costs an instruction a score: only above this sum (2^8 less what the roundings may hide) is the
-// maximum looked at.  (A reference that waited for a sum of 2^14 left a row that one key dominates with a numerator that is no bf16
-// value: error of its output against fp64, a key 2^9 to 2^13.5 above the others, 2.3e-3 against 1.65e-3.  8K prefill 508.8 us then, 509.5 now.)
+// Above this sum of 64 numerators the reference is taken anew.  The sum is at hand, where a maximum costs an instruction a score; a numerator
+// above 2^8 makes it 2^8 (less what the roundings may hide), and so do 64 scores that average 2^2 above the reference.  (A line at
+// 2^14, which some numerator above 2^8 has to cross, left a row that one key dominates with a numerator that is no bf16 value: error of
+// its output against fp64, a key 2^9 to 2^13.5 above the others, 2.3e-3 against 1.65e-3, and no time saved.  Asking the
+// maximum, behind the sum, whether a score lies 2^8 above costs 1.5 to 4 % where G = 1: 6000 rows 113.1 -> 117.5 us.)
 constexpr float kRefSum = 255.f;
 
 template <int DH>
@@ -291,8 +292,8 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
             for (int p = 0; p < 2; ++p) {
                 if (!(ok = warp_wait(bar_s(s, p), i & 1, s_abort, a.wait_cycles))) break;
                 // The reference of the tiles before nearly always still serves, so the numerators are taken against it at
-                // once, 32 columns at a time with the next 32 on their way; only if a selected score then turns out to exceed it by
-                // more than 2^8 (which their sum tells; a row's first tiles) is the work done again from the scores, still in registers.
+                // once, 32 columns at a time with the next 32 on their way; only if their sum shows that a selected score may exceed
+                // it by more than 2^8 (kRefSum; a row's first tiles) is the work done again from the scores, still in registers.
                 uint32_t v[2][32];
                 uint64_t sum[2] = {0ull, 0ull};
                 const float neg0 = m_ref == -INFINITY ? 0.f : -m_ref;
@@ -324,15 +325,11 @@ gsa_masked_attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __gri
                 float a0, a1, a2, a3;
                 unpack_f32x2(sum[0], a0, a1); unpack_f32x2(sum[1], a2, a3);
                 const bool first = m_ref == -INFINITY && (mw[2 * p] | mw[2 * p + 1]) != 0u;
-                bool move = __any_sync(0xFFFFFFFFu, first || (a0 + a1) + (a2 + a3) > kRefSum);
-                float top = -INFINITY;
-                if (move) {
+                if (__any_sync(0xFFFFFFFFu, first || (a0 + a1) + (a2 + a3) > kRefSum)) {
+                    float top = -INFINITY;
 #pragma unroll
                     for (int j = 0; j < 64; ++j) top = fmaxf(top, __uint_as_float(v[j >> 5][j & 31]));
                     top *= a.scale_log2;
-                    move = __any_sync(0xFFFFFFFFu, top > m_ref + 8.0f);
-                }
-                if (move) {
                     const float m_new = top > m_ref ? top + kRefMargin : m_ref;
                     const float alpha = m_ref == -INFINITY ? 0.f : ex2_approx(m_ref - m_new);
                     m_ref = m_new;
