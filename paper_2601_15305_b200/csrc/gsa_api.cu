@@ -22,12 +22,12 @@ int sm_count() {
     return n;
 }
 namespace {
-struct ClearArgs { ClearSpan span[3]; };
+struct ClearArgs { ClearSpan span[2]; };
 __global__ void __launch_bounds__(256) gsa_clear_kernel(const ClearArgs a) {
     chain_wait();
     const size_t first = (size_t)blockIdx.x * 256 + threadIdx.x, step = (size_t)gridDim.x * 256;
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
+    for (int s = 0; s < 2; ++s) {
         const size_t bytes = a.span[s].bytes, vec = (reinterpret_cast<uintptr_t>(a.span[s].p) & 15) == 0 ? bytes / 16 : 0;
         for (size_t i = first; i < vec; i += step) reinterpret_cast<uint4*>(a.span[s].p)[i] = make_uint4(0u, 0u, 0u, 0u);
         for (size_t i = vec * 4 + first; i < bytes / 4; i += step) reinterpret_cast<uint32_t*>(a.span[s].p)[i] = 0u;
@@ -35,9 +35,9 @@ __global__ void __launch_bounds__(256) gsa_clear_kernel(const ClearArgs a) {
 }
 }  // namespace
 
-cudaError_t launch_clear(cudaStream_t st, ClearSpan a, ClearSpan b, ClearSpan c) {
-    ClearArgs args{{a, b, c}};
-    const size_t most = a.bytes > b.bytes ? (a.bytes > c.bytes ? a.bytes : c.bytes) : (b.bytes > c.bytes ? b.bytes : c.bytes);
+cudaError_t launch_clear(cudaStream_t st, ClearSpan a, ClearSpan b) {
+    ClearArgs args{{a, b}};
+    const size_t most = a.bytes > b.bytes ? a.bytes : b.bytes;
     const size_t want = (most / 16 + 255) / 256, cap = (size_t)sm_count() * 8;
     launch_chained(gsa_clear_kernel, (unsigned)(want < 1 ? 1 : (want < cap ? want : cap)), 256, 0, st, args);
     return cudaGetLastError();                             // (not counted as a launch, as a memset would not be)

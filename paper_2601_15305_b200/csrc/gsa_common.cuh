@@ -71,10 +71,10 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
     return launch_chained_cluster(1, kern, grid, block, smem, st, static_cast<A&&>(args)...);
 }
 
-// Zeroes up to three regions (4-byte aligned, whole words) ahead of a call's kernels.  A kernel of its own, chained like the others:
+// Zeroes one or two regions (4-byte aligned, whole words) ahead of a call's kernels.  A kernel of its own, chained like the others:
 // a cudaMemsetAsync stands 2 to 4 us apart from the kernels on either side of it (the three in front of the indexer loss 12 us).
 struct ClearSpan { void* p; size_t bytes; };
-cudaError_t launch_clear(cudaStream_t st, ClearSpan a, ClearSpan b = {nullptr, 0}, ClearSpan c = {nullptr, 0});
+cudaError_t launch_clear(cudaStream_t st, ClearSpan a, ClearSpan b = {nullptr, 0});
 
 // multiprocessors of the current device (cached per device; 148 if the query fails)
 int sm_count();
