@@ -749,7 +749,9 @@ cudaError_t launch_attn_t(AttnArgs a, const gsa_params_t& p, const AttnPlan& pl,
 
 // First row from which the gather is the cheaper path (rr.q_begin: all of them; its end: none), from two models in
 // microseconds.  Tiles: a CTA takes 2.1 (d_h = 64: 1.9) per key tile of its 256 (row, head) rows and the GPU one CTA per SM,
-// plus 10 for the masks, the start and the gather's idle launch behind them (measured at L = 32K and 16K).  Gather: 36 ps (24) per pair
+// plus 10 for the masks, the start and the gather's idle launch behind them (measured at L = 32K and 16K on the kernel of whole tiles; the
+// present one takes 1.7, but a line moved by as much lost where it was tried: 128K, ~120K rows on tiles in place of 96896, 93.6 ms
+// against 95.1).  Gather: 36 ps (24) per pair
 // and KV head, 41 (27) out of several key ranges (measured at L = 16K and 128K for 1, 2, 4 and 8 query heads per KV head),
 // and a warp's own chain of 16-key steps where a call has few rows.
 struct ForwardCosts {

@@ -21,7 +21,7 @@
 // 16 (its A operand alone is 4 KB), not the 32 of its arithmetic.  Whole tiles, with the next scores only behind both halves' product,
 // took 3600, 1500 of it in that wait.  A CTA costs 0.7 us of setup, 1.5 to its first scores and about 2 at its end (8.7 while gates
 // and output went row by row).  Measured at 16 heads of 128 on 8 KV heads: 8K 247 us (319 before the order of tile_order and the halves,
-// the gather kernel 4.6 ms), dense 2 x 3072 100 us (135), L = 32K 3.27 ms = 1.34 PFLOP/s over the visible pairs, at the power limit (3.41;
+// the gather kernel 4.6 ms), dense 2 x 3072 100 us (135), L = 32K 3.27 to 3.37 ms = 1.30 to 1.34 PFLOP/s over the visible pairs, at the power limit (3.41;
 // the gather 19.6 ms).  Slower: four softmax warpgroups, a row's halves on two threads (8K 295 us); a share of the exponentials on
 // the FMA pipe (every fourth pair 250 against 252 at 8K, 3.34 against 3.28 ms at 32K; every second 280).
 //

@@ -12,9 +12,11 @@
 // columns (MN-major) for the sums.
 //
 // Bound: the products and the elementwise work between them in turn.  Measured at L = 32K, 16 heads of 128 on 8 KV heads, mean
-// budget 2080: 17.2 ms for a call with its target, 13.3 ms without (seven products, 1.16 PFLOP/s over the visible pairs; the keys
-// kernel somewhat over 6, the rows kernel over 5), so 3.3 ms for the target (one product, and all the exponentials; 3.9 while a thread alone searched a run's start in each set and
-// every lane summed all heads); 8K 1.37 and 1.02 ms.  The gather kernels take 86 and 19.0 ms for a call.
+// budget 2080: 16.5 ms for a call with its target, 12.9 ms without (seven products, 1.20 PFLOP/s over the visible pairs; the keys
+// kernel somewhat over 6, the rows kernel over 5), so 3.6 ms for the target (one product, and all the exponentials; 0.6 more while a
+// thread alone searched a run's start in each set and every lane summed all heads); 8K 1.18 and 0.85 ms.  The gather kernels take 86
+// and 19.0 ms for a call.  The sigmoids of dV and dg2 by rcp.approx or by a rounded division: the same errors against fp64 to six digits
+// (1500 rows, 8 heads: 2.8377e-3 and 2.7844e-3), up to 2 % of the call for the division.
 //
 // Roles in all three: warps 0-15 the elementwise work (four warpgroups side by side, 32 columns of a tile each: with two of
 // them the products waited for it), warp 16 copies, warp 17 MMA issue, 18 and 19 small loads.
@@ -903,7 +905,7 @@ size_t masked_bwd_bytes(const gsa_params_t& p, const RowRange& rr) {
 
 // Two models in microseconds, as in the forward (masked_rows_end).  Tiles: 1.7 + 1.45 + 1.05 (d_h = 64: 1.3 + 1.1 + 0.9) per
 // 128 x 128 tile in the keys, rows and target kernels, one CTA per SM, 40 for the launches around them (the target is charged
-// whether it is asked for or not).  Gather: 0.115 ps per byte of the K, V', Q and do rows that a pair moves (1.41 ns at 16
+// whether it is asked for or not; measured before the order of the CTAs and the results by TMA, now a tenth less).  Gather: 0.115 ps per byte of the K, V', Q and do rows that a pair moves (1.41 ns at 16
 // heads of 128 on 8 KV heads, measured at L = 32K), 20 for its launches.  Fewer row tiles than half of the SMs: the gather.
 namespace {
 struct BackwardCosts { double tiles_us, pair_us, selected; };

@@ -90,8 +90,8 @@ extern "C" int gsa_sparse_gated_attn_fwd_static(const gsa_params_t* p, const voi
     void* attn_scratch = (char*)scratch + kStatusBytes;
     __nv_bfloat16* Vg = (__nv_bfloat16*)((char*)scratch + kStatusBytes + attn_bytes);
     // The array keeps what the previous call left in it.  The status word must start at zero and is
-    // cleared here; the pre-pass overwrites every gated value the attention kernel will read, and the
-    // attention kernels write every state slot before they read it.
+    // cleared here; the pre-pass overwrites every gated value the attention kernel will read.  Of the
+    // state, the merge may load slots that the call has not written and lets none of them into a sum.
     t_dev_status = (int32_t*)scratch;
     e = launch_clear(st, {scratch, (size_t)kStatusBytes});
     if (e == cudaSuccess)
